@@ -7,6 +7,8 @@
 
 #include <cuda_fp16.h>
 
+#include <vector>
+
 #include "device.cuh"
 
 namespace vtm {
@@ -78,13 +80,53 @@ template <typename TF, typename TV>
 cudaError_t sweep_wide_configure(int R, size_t smem);
 template <typename TF, typename TV>
 cudaError_t launch_sweep_wide(const SweepArgs<TF, TV>& a, int R, int npieces, size_t smem, cudaStream_t st);
+// One segment of a port sweep (port.cu): the tiles (I0, J0) .. (I1, J1) of a subgraph's lower block
+// triangle, row by row.
+struct PortSeg {
+  int64_t s_off;   // the subgraph's first tile
+  int32_t piece;   // index into PortArgs::pieces
+  int32_t I0, J0, I1, J1;
+  int32_t first;   // index of the subgraph's first segment (its segments are consecutive)
+  int32_t nseg;    // segments of the subgraph
+  int64_t part;    // nseg > 1: element offset of the subgraph's partial vectors y, one per segment
+};
+
+// Order of the entries inside a tile of S_j (port.cu).
+enum { kPortPatch8x4 = 0, kPortPatch4x8 = 1, kPortFragments = 2 };
+
+// Shared-memory shape of the port sweep kernel, and which kernel.
+struct PortShape {
+  int vec_elems;   // elements of a padded port vector
+  int pad;         // unused entries after every four ports
+  int op_stride;   // tensor cores: 16-bit entries of a row of the vector operand
+  int layout;      // of S_j's tiles (kPort...)
+  int mma;         // 1: products on the tensor cores
+  int priv;        // 1: an accumulator per warp (R <= 2), 0: one for all
+  int ring;        // 1: shared-memory slots for the tiles in flight (0: no room)
+  int sb;          // strips whose row sums the warps keep between barriers (0: no room)
+  size_t smem;
+};
+
+// Division of a sweep's tiles among CTAs: CTA c takes the segments cta_seg[c] .. cta_seg[c + 1] - 1.
+struct PortPlan {
+  std::vector<PortSeg> segs;
+  std::vector<int32_t> cta_seg;
+  int64_t part_elems = 0;
+};
+
 // Arguments of one sweep in port-response form (port.cu): u = u_base + S_j s per subgraph.
 template <typename T>
 struct PortArgs {
-  const PieceDesc* pieces;     // all subgraphs, one CTA each
+  const PieceDesc* pieces;
+  const PortSeg* segs;
+  const int32_t* cta_seg;      // grid + 1
+  T* s;                        // port vectors of the sweep: ports x R
+  T* part;                     // partial y of the subgraphs with several segments
+  int* ticket;                 // one per segment, zero between sweeps
+  int vec_elems, op_stride, mma, pad, priv, ring, sb;  // PortShape
   const T* S;                  // port responses, lower block triangle of 32 x 32 tiles
   const void* Sh;              // FP32 solvers: the same tiles in IEEE half (nullptr: use S)
-  const float* scale;          // FP16 storage: per stored tile (global tile index), the factor it was divided by
+  const float* scale;          // FP16 storage: per stored tile, the factor it was divided by
   const T* ubase;              // P^T K_j^{-1} b̃_j: ports x R
   const T* wprev;              // outgoing waves of the previous sweep: ends x R
   T* wnext;                    // outgoing waves of this sweep
@@ -92,30 +134,25 @@ struct PortArgs {
   const int32_t* twin;
   const T* invz;
   CoupleRef<T> cpl;            // coupled lines (cpl.ptr == nullptr: none)
-  int det;                     // per-warp column accumulators summed in a fixed order (bitwise
-                               // reproducible); 0: shared-memory atomics
 };
 
-// Shared memory the deterministic SIMT port sweep may take (it keeps three CTAs per SM with FP16
-// storage).
-constexpr size_t kPortDetSmem = 72 * 1024;
-
 __host__ __device__ int64_t port_tiles(int nports);
-size_t port_sweep_smem_bytes(size_t elem, int R, int max_ports, bool det);
-bool port_sweep_det_fits(size_t elem, int R, int max_ports);
+PortShape port_shape(size_t elem, size_t stored, int R, int max_ports);
+PortPlan port_plan(const PieceDesc* pieces, int npieces, size_t elem, size_t stored, int R, int ctas);
 template <typename T>
-cudaError_t port_sweep_configure(int R, size_t smem, bool det);
+cudaError_t port_sweep_configure(int R, const PortShape& sh, bool half, int* ctas_per_sm);
+// Two launches: the port vectors of all nports ports, then the sweep proper.
 template <typename T>
-cudaError_t launch_port_sweep(const PortArgs<T>& a, int R, int npieces, size_t smem, cudaStream_t st);
+cudaError_t launch_port_sweep(const PortArgs<T>& a, int R, int nports, int grid, size_t smem, cudaStream_t st);
 template <typename T>
 cudaError_t launch_gather_port_response(const PieceDesc* pieces, int npieces, const int32_t* port_local, int Rs, int b,
-                                        const T* xc, T* S, cudaStream_t st);
+                                        const T* xc, T* S, int layout, cudaStream_t st);
 template <typename T>
 cudaError_t launch_gather_ports(const PieceDesc* pieces, int npieces, const int32_t* port_local, int R, const T* xc,
                                 T* ubase, cudaStream_t st);
 // FP16 copy (and per-tile scale) of the FP32 port-response tiles.
 cudaError_t launch_port_to_half(const PieceDesc* pieces, int npieces, const float* S, __half* Sh, float* scale,
-                                cudaStream_t st);
+                                const PortShape& from, const PortShape& to, cudaStream_t st);
 
 // Tensor-core port-response sweep for 16 / 32 right-hand sides (port_tc.cu), FP32 solvers.
 struct PortTCArgs {

@@ -7,19 +7,25 @@
 // The outgoing waves are w_out[e] = 2 u_q - w_in[e] (eq. 5.6), exactly as in the band sweep; only
 // the way u is obtained differs.  S_j is symmetric, so only its lower block triangle is stored.
 //
-// Storage of S_j: 32 x 32 tiles (I, J), J <= I, in the order I (I + 1) / 2 + J, from element offset
-// s_off * 1024.  Inside a tile lane L = 4 a + b of the warp owns the 4 x 8 patch of rows
-// 4a .. 4a+3 and columns 8b .. 8b+7; patch entry p = (i mod 4) * 8 + (c mod 8) of element (i, c)
-// sits at ((p / V) * 32 + L) * V + p mod V with V = 16 / sizeof(entry), so that the k-th 16-byte
-// load of all lanes reads 512 contiguous bytes.  The row part T s_J then sums over 4 lanes and the
-// column part T^T s_I over 8 lanes (short reduce-scatters).  Ports beyond n_ports are zero.
+// Storage of S_j: 32 x 32 tiles (I, J), J <= I, in the order I (I + 1) / 2 + J, from tile s_off on;
+// ports beyond n_ports are zero.  Inside a tile the entries lie as the kernel's lanes take them
+// (PortLayout), so that the k-th 16-byte load of all lanes reads 512 contiguous bytes:
+//  * patches: lane 8 a + b owns the 8 x 4 patch of rows 8a .. +7 and columns 4b .. +3 (R <= 2), or
+//    lane 4 a + b the 4 x 8 patch of rows 4a .. +3 and columns 8b .. +7 (R = 4, 8).  The column
+//    part T^T s_I leaves the registers with every tile and sums over the lanes of a column group,
+//    which few columns per lane make short; the row part T s_J stays in registers along a row of
+//    tiles, where few rows per lane take few registers;
+//  * fragments: the 16 x 16 blocks of mma.m16n8k16's A operand (FP32 tiles, R = 4, 8).
 //
-// FP16 storage (FP32 solvers): the same tiles as IEEE half, V = 8, each tile divided by its own
-// largest entry (kept per tile in FP32); products and accumulation stay in FP32 and each tile's two
-// reduced sums are scaled back before they enter y.  It halves the bytes of the sweep; its rounding
-// (2^-11 of each tile's largest entry) is absorbed by the FP64 defect correction, and the solver
-// returns to FP32 storage if a correction step stops gaining a digit.
+// FP16 storage (FP32 solvers): the same tiles as IEEE half, row by row with the 16-byte chunks of a
+// row exchanged for ldmatrix (or as patches), each tile divided by its own largest entry (kept
+// per tile in FP32); the tile's products are scaled back before they enter y.  It halves the bytes
+// of the sweep; its rounding (2^-11 of each tile's largest entry) is absorbed by the FP64 defect
+// correction, and the solver returns to FP32 storage if a correction step stops gaining a digit.
 #include <cuda_fp16.h>
+
+#include <algorithm>
+#include <cmath>
 
 #include "kernels.h"
 
@@ -42,62 +48,98 @@ struct Vec16<double> {
   __device__ static double get(const double2& v, int i) { return i == 0 ? v.x : v.y; }
 };
 
-// Position of element (i, c) of a tile in the patch layout, V entries per 16 bytes.
-__host__ __device__ __forceinline__ int patch_pos(int i, int c, int V) {
-  const int L = (i / 4) * 4 + c / 8, p = (i % 4) * 8 + (c % 8);
+// Rows of a lane's patch.
+__host__ __device__ constexpr int patch_rows(int R) { return R <= 2 ? 8 : 4; }
+
+// Position of element (i, c) of a tile, V entries per 16 bytes.
+__host__ __device__ __forceinline__ int tile_pos(int layout, int i, int c, int V) {
+  if (layout == kPortFragments) {
+    // block (i / 16, c / 16); lane 4 g + t holds rows g, g + 8 and columns 2 t, 2 t + 1 (+ 8): four
+    // pairs in register order (row half, then column half)
+    const int blk = (i >> 4) * 2 + (c >> 4), lane = (i & 7) * 4 + ((c & 7) >> 1);
+    const int pair = ((i >> 3) & 1) + 2 * ((c >> 3) & 1), p = blk * 8 + pair * 2 + (c & 1);
+    return ((p / V) * kNB + lane) * V + p % V;
+  }
+  const int pr = layout == kPortPatch8x4 ? 8 : 4, pc = kNB / pr;
+  const int L = (i / pr) * (kNB / pc) + c / pc, p = (i % pr) * pc + (c % pc);
   return ((p / V) * kNB + L) * V + p % V;
 }
 
-// The raw 16-byte vectors of this lane's patch (kNB entries of type TS), loaded ahead of use.
-template <typename TS>
-struct RawPatch {
-  uint4 v[kNB * sizeof(TS) / 16];
-};
-
-template <typename TS>
-__device__ __forceinline__ void load_raw(const TS* tile, int lane, RawPatch<TS>& r) {
-  const uint4* tp = reinterpret_cast<const uint4*>(tile);
-#pragma unroll
-  for (int k = 0; k < (int)(kNB * sizeof(TS) / 16); ++k) r.v[k] = __ldg(tp + k * kNB + lane);
+// Position of element (i, c) of an FP16 tile stored for ldmatrix: rows of 64 bytes whose four 16-byte
+// chunks are exchanged by the row pair, so that the eight rows of an 8 x 8 matrix hit 32 banks.
+__host__ __device__ __forceinline__ int half_pos(int i, int c) {
+  return i * kNB + (((c >> 3) ^ (i >> 1)) & 3) * 8 + (c & 7);
 }
 
-__device__ __forceinline__ void widen(const RawPatch<float>& r, float (&row)[kNB]) {
+// This lane's patch (kNB entries of type TS, in the tile's patch layout) widened to T.
+__device__ __forceinline__ void load_patch(const float* tile, int lane, float (&p)[kNB]) {
+  const float4* tp = reinterpret_cast<const float4*>(tile);
 #pragma unroll
   for (int k = 0; k < kNB / 4; ++k) {
-    row[4 * k] = __uint_as_float(r.v[k].x);
-    row[4 * k + 1] = __uint_as_float(r.v[k].y);
-    row[4 * k + 2] = __uint_as_float(r.v[k].z);
-    row[4 * k + 3] = __uint_as_float(r.v[k].w);
+    const float4 v = tp[k * kNB + lane];
+    p[4 * k] = v.x, p[4 * k + 1] = v.y, p[4 * k + 2] = v.z, p[4 * k + 3] = v.w;
   }
 }
 
-__device__ __forceinline__ void widen(const RawPatch<double>& r, double (&row)[kNB]) {
+__device__ __forceinline__ void load_patch(const double* tile, int lane, double (&p)[kNB]) {
+  const double2* tp = reinterpret_cast<const double2*>(tile);
 #pragma unroll
   for (int k = 0; k < kNB / 2; ++k) {
-    row[2 * k] = __hiloint2double((int)r.v[k].y, (int)r.v[k].x);
-    row[2 * k + 1] = __hiloint2double((int)r.v[k].w, (int)r.v[k].z);
+    const double2 v = tp[k * kNB + lane];
+    p[2 * k] = v.x, p[2 * k + 1] = v.y;
   }
 }
 
-__device__ __forceinline__ void widen(const RawPatch<__half>& r, float (&row)[kNB]) {
+__device__ __forceinline__ void load_patch(const __half* tile, int lane, float (&p)[kNB]) {
+  const uint4* tp = reinterpret_cast<const uint4*>(tile);
 #pragma unroll
   for (int k = 0; k < kNB / 8; ++k) {
-    const uint32_t w[4] = {r.v[k].x, r.v[k].y, r.v[k].z, r.v[k].w};
+    const uint4 v = tp[k * kNB + lane];
+    const uint32_t w[4] = {v.x, v.y, v.z, v.w};
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
       const float2 f = __half22float2(*reinterpret_cast<const __half2*>(&w[j]));
-      row[k * 8 + 2 * j] = f.x;
-      row[k * 8 + 2 * j + 1] = f.y;
+      p[k * 8 + 2 * j] = f.x;
+      p[k * 8 + 2 * j + 1] = f.y;
     }
   }
 }
 
-__device__ __forceinline__ void tile_of(int t, int& I, int& J) {
-  int i = (int)((sqrtf(8.0f * (float)t + 1.0f) - 1.0f) * 0.5f);
-  while ((i + 1) * (i + 2) / 2 <= t) ++i;
-  while (i * (i + 1) / 2 > t) --i;
-  I = i;
-  J = t - i * (i + 1) / 2;
+// Shared-memory slot of a tile in flight: its patches and, with FP16 storage, the scale once per lane.
+template <typename TS>
+__host__ __device__ constexpr int slot_bytes() {
+  return kNB * kNB * (int)sizeof(TS) + (sizeof(TS) == 2 ? kNB * 4 : 0);
+}
+
+// Tiles in flight per warp.  FP16 tiles with an accumulator per warp: three, which two CTAs per SM
+// have room for (96 KB in flight per SM; one tile and three CTAs keep 48 KB, 0.205 ms per sweep of
+// 128^3 instead of 0.17).
+template <typename TS, bool DEEP>
+__host__ __device__ constexpr int port_depth() {
+  return sizeof(TS) == 2 && DEEP ? 3 : 1;
+}
+
+// This lane's share of a tile on its way to the slot (the caller commits the group).
+template <typename TS>
+__device__ __forceinline__ void fetch_patch(unsigned char* slot, const TS* tile, const float* scale, int lane, uint64_t policy) {
+  const uint32_t d = smem_u32(slot) + lane * 16;
+  const unsigned char* g = reinterpret_cast<const unsigned char*>(tile) + lane * 16;
+#pragma unroll
+  for (int k = 0; k < kNB * (int)sizeof(TS) / 16; ++k)
+    asm volatile("cp.async.cg.shared.global.L2::cache_hint.L2::256B [%0], [%1], 16, %2;" ::"r"(d + k * 512), "l"(g + k * 512), "l"(policy)
+                 : "memory");
+  if constexpr (sizeof(TS) == 2)
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(smem_u32(slot) + kNB * kNB * 2 + lane * 4),
+                 "l"(scale)
+                 : "memory");
+}
+
+// Row and column of tile t.
+__host__ __device__ __forceinline__ void tile_of(int t, int& I, int& J) {
+  I = (int)((sqrtf(8.0f * (float)t + 1.0f) - 1.0f) * 0.5f);
+  while ((I + 1) * (I + 2) / 2 <= t) ++I;
+  while (I * (I + 1) / 2 > t) --I;
+  J = t - I * (I + 1) / 2;
 }
 
 }  // namespace
@@ -111,7 +153,7 @@ __host__ __device__ int64_t port_tiles(int nports) {
 // unit source at port cc (xc holds copies x Rs).  Only tiles with I >= J are written.
 template <typename T>
 __global__ void k_gather_port_response(const PieceDesc* __restrict__ pieces, const int32_t* __restrict__ port_local,
-                                       int Rs, int b, const T* __restrict__ xc, T* __restrict__ S) {
+                                       int Rs, int b, const T* __restrict__ xc, T* __restrict__ S, int layout) {
   const PieceDesc pd = pieces[blockIdx.x];
   constexpr int V = Vec16<T>::V;
   for (int i = threadIdx.x; i < pd.nports * Rs; i += blockDim.x) {
@@ -122,7 +164,7 @@ __global__ void k_gather_port_response(const PieceDesc* __restrict__ pieces, con
     if (I < J) continue;
     const int row = q % kNB, col = cc % kNB;
     const int64_t t = pd.s_off + (int64_t)I * (I + 1) / 2 + J;
-    S[t * kNB * kNB + patch_pos(row, col, V)] =
+    S[t * kNB * kNB + tile_pos(layout, row, col, V)] =
         xc[((size_t)pd.copy_off + port_local[pd.port_off + q]) * Rs + r];
   }
 }
@@ -138,251 +180,1019 @@ __global__ void k_gather_ports(const PieceDesc* __restrict__ pieces, const int32
   }
 }
 
-// One sweep in port-response form, one CTA per subgraph, R right-hand sides.
-// Shared memory: s (n_pad_ports x R), the accumulator y (same size) and, with DET, one accumulator
-// of the same size per warp.  Warp w takes the tiles w, w + 8, ... of the stored lower block
-// triangle (so the eight warps stream neighbouring tiles).  With DET every warp adds its tiles'
-// row and column parts to its own accumulator (in each add the 32 lanes hit 32 different ports),
-// and the accumulators are summed in warp order at the end: identical runs agree bit for bit.
-// Without DET (the accumulators would not fit) the warps add to y with shared-memory atomics.
-template <typename T, typename TS, int R, bool DET>
-__global__ void __launch_bounds__(kSweepThreads, sizeof(TS) == 2 ? 3 : 2) k_port_sweep(const PortArgs<T> a) {
-  extern __shared__ __align__(16) unsigned char smem[];
-  const PieceDesc pd = a.pieces[blockIdx.x];
-  const int np = pd.nports;
-  if (np == 0) return;
-  const int nt = (np + kNB - 1) / kNB;
-  const int npad = nt * kNB;
-  T* sv = reinterpret_cast<T*>(smem);
-  T* yv = sv + (size_t)npad * R;
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  constexpr int kWarps = kSweepThreads / 32;
-  T* const yacc = DET ? yv + (size_t)(1 + warp) * npad * R : yv;  // where this warp adds its parts
-  if constexpr (DET) {
-    for (int i = tid; i < kWarps * npad * R; i += kSweepThreads) yv[(size_t)npad * R + i] = T(0);
-  }
+// Element index of vector entry (port q, column 0) in shared memory.  With pad = 4 (FP32, R >= 4)
+// every group of four ports is followed by four unused entries: a lane reads the 16-byte rows of
+// its patch's columns (8 ports apart) and rows (4 apart), which without the gap all start in the
+// same four banks.
+template <int R>
+__device__ __forceinline__ int vidx(int q, int pad) {
+  return q * R + (q >> 2) * pad;
+}
 
-  // s_q = sum_e w_in[e] / Z_e, w_in[e] = w_prev[twin[e]]; kU entries per thread at a time, their
-  // end ranges, twins and waves loaded in three independent rounds
-  constexpr int kU = 4;
-  for (int i0 = tid; i0 < npad * R; i0 += kSweepThreads * kU) {
-    int e0[kU], e1[kU], tw[kU];
-    T iz[kU];
+template <typename T, int N>
+__device__ __forceinline__ void load_vec(const T* p, T (&v)[N]) {
+  if constexpr (N * sizeof(T) == 16 && sizeof(T) == 4) {
+    const float4 x = *reinterpret_cast<const float4*>(p);
+    v[0] = x.x, v[1] = x.y, v[2] = x.z, v[3] = x.w;
+  } else if constexpr (N == 2 && sizeof(T) == 4) {
+    const float2 x = *reinterpret_cast<const float2*>(p);
+    v[0] = x.x, v[1] = x.y;
+  } else if constexpr (N == 2 && sizeof(T) == 8) {
+    const double2 x = *reinterpret_cast<const double2*>(p);
+    v[0] = x.x, v[1] = x.y;
+  } else {
 #pragma unroll
-    for (int u = 0; u < kU; ++u) {
-      const int q = (i0 + u * kSweepThreads) / R;
-      e0[u] = e1[u] = 0;
-      if (q < np) {
-        e0[u] = a.port_end_ptr[pd.port_off + q];
-        e1[u] = a.port_end_ptr[pd.port_off + q + 1];
-      }
-    }
-#pragma unroll
-    for (int u = 0; u < kU; ++u) {
-      tw[u] = (e1[u] > e0[u]) ? a.twin[e0[u]] : 0;
-      iz[u] = (e1[u] > e0[u]) ? a.invz[e0[u]] : T(0);
-    }
-#pragma unroll
-    for (int u = 0; u < kU; ++u) {
-      const int i = i0 + u * kSweepThreads;
-      if (i >= npad * R) break;
-      const int r = i % R;
-      T acc = (e1[u] > e0[u]) ? a.wprev[(size_t)tw[u] * R + r] * iz[u] : T(0);
-      for (int e = e0[u] + 1; e < e1[u]; ++e) acc += a.wprev[(size_t)a.twin[e] * R + r] * a.invz[e];
-      if (a.cpl.ptr && i / R < np) acc += coupling_current<T, T>(a.cpl, pd.port_off + i / R, r, R, a.wprev);
-      sv[i] = acc;
-      yv[i] = T(0);
-    }
+    for (int i = 0; i < N; ++i) v[i] = p[i];
   }
-  __syncthreads();
+}
 
-  // y = S_j s over the stored lower block triangle: tile (I, J) adds T s_J to y_I and, off the
-  // diagonal, T^T s_I to y_J.
-  const TS* Sb;
-  if constexpr (sizeof(TS) == 2) Sb = static_cast<const TS*>(a.Sh) + pd.s_off * kNB * kNB;
-  else Sb = reinterpret_cast<const TS*>(a.S) + pd.s_off * kNB * kNB;
-  const int64_t ntiles = (int64_t)nt * (nt + 1) / 2;
-  const int pa = lane >> 2, pb = lane & 3;  // patch: rows 4 pa .. +3, columns 8 pb .. +7
-  // each warp keeps the next tile's loads in flight while it works on the current one
-  RawPatch<TS> cur, nxt;
-  // FP16 storage: each tile was divided by its own largest |entry|; the two reduced sums of a
-  // tile are multiplied back before they are added to y
-  const float* tsc = (sizeof(TS) == 2) ? a.scale + pd.s_off : nullptr;
-  T sc_cur = T(1), sc_nxt = T(1);
-  if (warp < ntiles) {
-    load_raw(Sb + (int64_t)warp * kNB * kNB, lane, cur);
-    if constexpr (sizeof(TS) == 2) sc_cur = (T)tsc[warp];
+template <typename T, int N>
+__device__ __forceinline__ void store_vec(T* p, const T (&v)[N]) {
+  if constexpr (N * sizeof(T) == 16 && sizeof(T) == 4) {
+    *reinterpret_cast<float4*>(p) = make_float4(v[0], v[1], v[2], v[3]);
+  } else if constexpr (N == 2 && sizeof(T) == 4) {
+    *reinterpret_cast<float2*>(p) = make_float2(v[0], v[1]);
+  } else if constexpr (N == 2 && sizeof(T) == 8) {
+    *reinterpret_cast<double2*>(p) = make_double2(v[0], v[1]);
+  } else {
+#pragma unroll
+    for (int i = 0; i < N; ++i) p[i] = v[i];
   }
-  for (int t = warp; t < ntiles; t += kWarps) {
-    if (t + kWarps < ntiles) {
-      load_raw(Sb + (int64_t)(t + kWarps) * kNB * kNB, lane, nxt);
-      if constexpr (sizeof(TS) == 2) sc_nxt = (T)tsc[t + kWarps];
-    }
-    int I, J;
-    tile_of(t, I, J);
-    T pt[kNB];
-    widen(cur, pt);
-    cur = nxt;
-    const T sc = sc_cur;
-    sc_cur = sc_nxt;
-    const T* sJ = sv + ((size_t)J * kNB + 8 * pb) * R;
-    const T* sI = sv + ((size_t)I * kNB + 4 * pa) * R;
+}
+
+// Loads that bypass the L1 cache: values that another CTA or the launch before wrote.
+template <typename T, int N>
+__device__ __forceinline__ void load_cg(const T* p, T (&v)[N]) {
+  if constexpr (N == 4 && sizeof(T) == 4) {
+    const float4 x = __ldcg(reinterpret_cast<const float4*>(p));
+    v[0] = x.x, v[1] = x.y, v[2] = x.z, v[3] = x.w;
+  } else if constexpr (N == 2 && sizeof(T) == 4) {
+    const float2 x = __ldcg(reinterpret_cast<const float2*>(p));
+    v[0] = x.x, v[1] = x.y;
+  } else if constexpr (N == 2 && sizeof(T) == 8) {
+    const double2 x = __ldcg(reinterpret_cast<const double2*>(p));
+    v[0] = x.x, v[1] = x.y;
+  } else {
 #pragma unroll
-    for (int r = 0; r < R; ++r) {
-      // row part: 4 partial row sums over this lane's 8 columns, reduce-scattered over the 4 lanes
-      // of the same row group (xor 2, 1): lane (pa, pb) ends with row 4 pa + pb
-      T rp[4];
-#pragma unroll
-      for (int ii = 0; ii < 4; ++ii) {
-        T acc = T(0);
-#pragma unroll
-        for (int jj = 0; jj < 8; ++jj) acc += pt[ii * 8 + jj] * sJ[jj * R + r];
-        rp[ii] = acc;
-      }
-#pragma unroll
-      for (int h = 2; h >= 1; h >>= 1) {
-        const bool upper = (pb & h) != 0;
-#pragma unroll
-        for (int i = 0; i < h; ++i) {
-          const T send = upper ? rp[i] : rp[i + h];
-          const T keep = upper ? rp[i + h] : rp[i];
-          rp[i] = keep + __shfl_xor_sync(0xffffffffu, send, h);
-        }
-      }
-      {
-        const T v = (sizeof(TS) == 2) ? rp[0] * sc : rp[0];
-        T* at = &yacc[((size_t)I * kNB + 4 * pa + pb) * R + r];
-        if constexpr (DET) *at += v;
-        else atomicAdd(at, v);
-      }
-      if (I != J) {
-        // column part: 8 partial column sums over this lane's 4 rows, reduce-scattered over the 8
-        // lanes of the same column group (xor 16, 8, 4): lane (pa, pb) ends with column 8 pb + pa
-        T cp[8];
-#pragma unroll
-        for (int jj = 0; jj < 8; ++jj) {
-          T acc = T(0);
-#pragma unroll
-          for (int ii = 0; ii < 4; ++ii) acc += pt[ii * 8 + jj] * sI[ii * R + r];
-          cp[jj] = acc;
-        }
-#pragma unroll
-        for (int h = 4; h >= 1; h >>= 1) {
-          const bool upper = (pa & h) != 0;
-#pragma unroll
-          for (int i = 0; i < h; ++i) {
-            const T send = upper ? cp[i] : cp[i + h];
-            const T keep = upper ? cp[i + h] : cp[i];
-            cp[i] = keep + __shfl_xor_sync(0xffffffffu, send, 4 * h);
-          }
-        }
-        const T v = (sizeof(TS) == 2) ? cp[0] * sc : cp[0];
-        T* at = &yacc[((size_t)J * kNB + 8 * pb + pa) * R + r];
-        if constexpr (DET) *at += v;
-        else atomicAdd(at, v);
-      }
-    }
+    for (int i = 0; i < N; ++i) v[i] = __ldcg(p + i);
   }
-  __syncthreads();
-  if constexpr (DET) {
-    // y = the warps' accumulators, summed in warp order
-    for (int i = tid; i < npad * R; i += kSweepThreads) {
-      T v = T(0);
+}
+
+// Columns that a thread of the port-vector passes takes at once: 16 bytes of them at most.
+template <typename T, int R>
+__host__ __device__ constexpr int vec_cols() {
+  return R < (int)(16 / sizeof(T)) ? R : (int)(16 / sizeof(T));
+}
+
+// N consecutive entries, 16-byte aligned, in 16-byte loads.
+template <typename T, int N>
+__device__ __forceinline__ void load_run(const T* p, T (&v)[N]) {
+  constexpr int W = 16 / sizeof(T);
 #pragma unroll
-      for (int w = 0; w < kWarps; ++w) v += yv[(size_t)(1 + w) * npad * R + i];
-      yv[i] = v;
+  for (int i = 0; i < N; i += W) {
+    T w[W];
+    load_vec<T, W>(p + i, w);
+#pragma unroll
+    for (int j = 0; j < W; ++j) v[i + j] = w[j];
+  }
+}
+
+// Dependent launch (both kernels of a sweep): wait until the launch before has completed and its
+// writes are visible; let the next launch's CTAs start as this one's leave.
+__device__ __forceinline__ void grid_dep_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void grid_dep_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
+// Sum of N values per lane over the N lanes lane ^ (stride * k): each step halves the values a lane
+// keeps; the lane whose position in the group is k ends with the sum of value k in v[0].
+template <typename T, int N, int RC, int STRIDE>
+__device__ __forceinline__ void reduce_scatter(T (&v)[N][RC], int pos) {
+#pragma unroll
+  for (int h = N / 2; h >= 1; h >>= 1) {
+    const bool upper = (pos & h) != 0;
+#pragma unroll
+    for (int i = 0; i < h; ++i)
+#pragma unroll
+      for (int q = 0; q < RC; ++q) {
+        const T send = upper ? v[i][q] : v[i + h][q];
+        const T keep = upper ? v[i + h][q] : v[i][q];
+        v[i][q] = keep + __shfl_xor_sync(0xffffffffu, send, STRIDE * h);
+      }
+  }
+}
+
+// The end of a segment, for both sweep kernels: y(q, r, v) gives RV columns of the segment's y.  A
+// subgraph of one segment goes straight to its waves; else the partial y goes to scratch and the
+// CTA that finishes the subgraph last (a ticket per subgraph) adds the segments' partials in their
+// order.  Nothing waits, and the order of arrival does not enter the sums: identical runs agree bit
+// for bit.  The waves, w_out[e] = 2 (u_base + y)_q - w_in[e], take kU entries per thread at a time,
+// their partials, end ranges, twins and incoming waves loaded in three independent rounds.
+template <typename T, int R, typename Y>
+__device__ __forceinline__ void finish_segment(const PortArgs<T>& a, const PortSeg& sg, int si, const PieceDesc& pd,
+                                               int rows, int* flag, Y y) {
+  constexpr int RV = vec_cols<T, R>();
+  constexpr int kU = sizeof(T) * RV >= 8 ? 2 : 4, kP = 4;
+  const int tid = threadIdx.x, np = pd.nports;
+  const int npad = (np + kNB - 1) / kNB * kNB;
+  T* const part = a.part + sg.part;  // [nseg][npad * R]
+  if (sg.nseg > 1) {
+    for (int i = tid; i < npad * (R / RV); i += kSweepThreads) {
+      T v[RV] = {};
+      const int q = i / (R / RV), r = i % (R / RV) * RV;
+      if (q < rows) y(q, r, v);
+      store_vec<T, RV>(part + (size_t)(si - sg.first) * npad * R + (size_t)i * RV, v);
+    }
+    __threadfence();
+    __syncthreads();
+    if (tid == 0) {
+      const int n = atomicAdd(a.ticket + sg.first, 1);
+      *flag = n == sg.nseg - 1;
+      if (n == sg.nseg - 1) a.ticket[sg.first] = 0;  // for the next sweep
     }
     __syncthreads();
+    const bool last = *flag != 0;
+    __syncthreads();
+    if (!last) return;
+    __threadfence();
   }
-
-  // w_out[e] = 2 (u_base + y)_q - w_in[e]
-  for (int i0 = tid; i0 < np * R; i0 += kSweepThreads * kU) {
+  const int nv = np * (R / RV);
+  for (int i0 = tid; i0 < nv; i0 += kSweepThreads * kU) {
     int e0[kU], e1[kU], tw[kU];
-    T ub[kU];
+    T uu[kU][RV], ub[kU][RV];
 #pragma unroll
     for (int u = 0; u < kU; ++u) {
       const int i = i0 + u * kSweepThreads;
       e0[u] = e1[u] = 0;
-      ub[u] = T(0);
-      if (i < np * R) {
-        const int q = i / R;
+#pragma unroll
+      for (int c = 0; c < RV; ++c) uu[u][c] = T(0);
+      if (i < nv) {
+        const int q = i / (R / RV), r = i % (R / RV) * RV;
         e0[u] = a.port_end_ptr[pd.port_off + q];
         e1[u] = a.port_end_ptr[pd.port_off + q + 1];
-        ub[u] = a.ubase[(size_t)pd.port_off * R + i];
+        load_cg<T, RV>(a.ubase + (size_t)pd.port_off * R + (size_t)i * RV, ub[u]);
+        if (sg.nseg <= 1) y(q, r, uu[u]);
       }
     }
+    // the segments' partials, kP of them at a time so that their loads do not wait for each other
+    if (sg.nseg > 1)
+      for (int k0 = 0; k0 < sg.nseg; k0 += kP) {
+        T v[kU][kP][RV];
+#pragma unroll
+        for (int u = 0; u < kU; ++u)
+#pragma unroll
+          for (int k = 0; k < kP; ++k) {
+            const int i = i0 + u * kSweepThreads;
+#pragma unroll
+            for (int c = 0; c < RV; ++c) v[u][k][c] = T(0);
+            if (i < nv && k0 + k < sg.nseg) load_cg<T, RV>(part + (size_t)(k0 + k) * npad * R + (size_t)i * RV, v[u][k]);
+          }
+#pragma unroll
+        for (int u = 0; u < kU; ++u)
+#pragma unroll
+          for (int k = 0; k < kP; ++k)
+#pragma unroll
+            for (int c = 0; c < RV; ++c) uu[u][c] += v[u][k][c];
+      }
+#pragma unroll
+    for (int u = 0; u < kU; ++u)
+#pragma unroll
+      for (int c = 0; c < RV; ++c) uu[u][c] += ub[u][c];
 #pragma unroll
     for (int u = 0; u < kU; ++u) tw[u] = (e1[u] > e0[u]) ? a.twin[e0[u]] : 0;
 #pragma unroll
     for (int u = 0; u < kU; ++u) {
       const int i = i0 + u * kSweepThreads;
-      if (i >= np * R) break;
-      const int r = i % R;
-      const T uu = ub[u] + yv[i];
-      a.wnext[(size_t)e0[u] * R + r] = T(2) * uu - a.wprev[(size_t)tw[u] * R + r];
-      for (int e = e0[u] + 1; e < e1[u]; ++e) a.wnext[(size_t)e * R + r] = T(2) * uu - a.wprev[(size_t)a.twin[e] * R + r];
+      if (i >= nv) break;
+      const int r = i % (R / RV) * RV;
+      T w[RV], o[RV];
+      load_cg<T, RV>(a.wprev + (size_t)tw[u] * R + r, w);
+#pragma unroll
+      for (int c = 0; c < RV; ++c) o[c] = T(2) * uu[u][c] - w[c];
+      store_vec<T, RV>(a.wnext + (size_t)e0[u] * R + r, o);
+      for (int e = e0[u] + 1; e < e1[u]; ++e) {
+        load_cg<T, RV>(a.wprev + (size_t)a.twin[e] * R + r, w);
+#pragma unroll
+        for (int c = 0; c < RV; ++c) o[c] = T(2) * uu[u][c] - w[c];
+        store_vec<T, RV>(a.wnext + (size_t)e * R + r, o);
+      }
     }
   }
 }
 
-size_t port_sweep_smem_bytes(size_t elem, int R, int max_ports, bool det) {
+// D += A B, 16 x 8 += 16 x 16 times 16 x 8, FP32 accumulation (HALF: fp16 operands, else bf16).
+template <bool HALF>
+__device__ __forceinline__ void mma16816(float (&d)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1) {
+  if constexpr (HALF)
+    asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, "
+                 "{%0, %1, %2, %3};"
+                 : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
+                 : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
+  else
+    asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, "
+                 "{%0, %1, %2, %3};"
+                 : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
+                 : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
+}
+
+// Four 8 x 8 matrices of 16-bit entries, lane l giving row l % 8 of matrix l / 8; TR: transposed.
+template <bool TR>
+__device__ __forceinline__ void ldmatrix4(uint32_t addr, uint32_t (&v)[4]) {
+  if constexpr (TR)
+    asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0, %1, %2, %3}, [%4];"
+                 : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3])
+                 : "r"(addr)
+                 : "memory");
+  else
+    asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0, %1, %2, %3}, [%4];"
+                 : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3])
+                 : "r"(addr)
+                 : "memory");
+}
+
+__device__ __forceinline__ uint32_t movmatrix(uint32_t a) {
+  uint32_t d;
+  asm volatile("movmatrix.sync.aligned.m8n8.trans.b16 %0, %1;" : "=r"(d) : "r"(a));
+  return d;
+}
+
+// The upper 16 bits of two floats as a pair: bf16 by truncation.
+__device__ __forceinline__ uint32_t upper_pair(float lo, float hi) {
+  return __byte_perm(__float_as_uint(lo), __float_as_uint(hi), 0x7632);
+}
+
+__device__ __forceinline__ float bf16_part(float x) { return __uint_as_float(__float_as_uint(x) & 0xFFFF0000u); }
+
+// Where port p of a strip lies in a row of the vector operand: lane t of a column reads its eight
+// entries (k = 2t, 2t + 1, 2t + 8, 2t + 9 of both 16-row halves) in one 16-byte load.
+__device__ __forceinline__ int operand_pos(int p) {
+  return ((p & 7) >> 1) * 8 + ((p >> 4) * 2 + ((p >> 3) & 1)) * 2 + (p & 1);
+}
+
+// Columns of the MMAs' vector operand.  FP16 tiles: columns 2 r, 2 r + 1 hold the two terms of right-
+// hand side r (hi and lo of s / sigma, sigma_r a power of two at or above the segment's max |s_r|:
+// together 2^-24 of it), so one product takes both and its lane adds them; R = 8 takes two operands.
+// FP32 tiles: S and s both as three bf16 terms (8 + 8 + 8 bits, exact), columns = right-hand sides;
+// the six products of terms above 2^-24 accumulate in order of size.
+template <typename TS, int R>
+__host__ __device__ constexpr int operand_rows() {
+  return sizeof(TS) == 2 ? 2 * R : 3 * R;
+}
+
+// One sweep in port-response form, R right-hand sides.
+//
+// Work split.  A CTA works through segments, runs of consecutive 32 x 32 tiles of one subgraph's
+// stored lower block triangle (PortSeg).  port_plan cuts the tiles of all subgraphs into as many
+// equal shares as CTAs fit on the GPU, so a few large subgraphs fill it as well as many do.  Per
+// segment: the port vector s (k_port_vec) of the rows up to the segment's last strip (a strip is one
+// row of tiles), y = the tiles' products, then finish_segment.
+//
+// PRIV (one or two columns, where eight accumulators of a subgraph's ports fit in shared memory):
+// each warp takes an equal run of the segment's tiles and adds to its own accumulator; nothing
+// couples the warps until the segment's end.  Per tile and lane 64 FMAs per column, 3 shuffles and
+// one shared read-modify-write; the row sums of a strip stay in registers along it.
+// Otherwise one accumulator serves all warps: tile (I, J) belongs to the warp that owns column J
+// (J mod 8 counted forwards and backwards in turn, which gives the warps equally many tiles although
+// the columns get shorter), so the column part is a plain addition by its only writer, and the
+// warps' row sums of `sb` strips are added in warp order between two barriers.
+//
+// Each lane copies its own patches one tile ahead into shared-memory slots that only it reads (cp.async, 16 bytes a piece): no registers hold loads in flight, no lane waits for
+// another, and a segment's first tile arrives while its vectors are read.
+//
+// MMA (FP16 tiles; FP32 tiles with R = 4, 8): the tile's products on the tensor cores
+// (mma.m16n8k16, FP32 accumulation, each tile's sums added in FP32), the transposed ones from
+// ldmatrix.trans or movmatrix.  The SIMT products of an FP16 tile take about 210 instructions per
+// lane (32 conversions, 64 FMAs, shuffles), of an FP32 tile at R = 8 about 980: the issue rate, not
+// the memory, bound those sweeps.
+//
+// What bounds it (GB300): HBM at R = 1, 2 and with FP16 tiles, FP64 arithmetic in FP64 (0.84 of its
+// pipe).  Measured per sweep against one CTA per subgraph with shared-memory atomics (R > 1, FP64) or
+// an accumulator per warp (FP32 / FP16, R = 1): 64^3 in 64 subgraphs 0.116 -> 0.044 ms (FP32, R = 1,
+// 188 MB) and 0.82 -> 0.21 ms (FP64, 376 MB); 101 x 67 x 83 in 288 ragged subgraphs, R = 8, 439 MB:
+// 0.54 -> 0.22 ms; 128^3 in 512 subgraphs, FP16, 1.01 GB: 0.199 -> 0.185 ms (0.80 of the copy
+// bandwidth with the port vectors' own launch; the tiles are read with an evict-first hint, without
+// it 0.198 ms).
+template <typename T, typename TS, int R, bool PRIV, bool MMA>
+__global__ void __launch_bounds__(kSweepThreads, sizeof(T) == 8 ? 1 : 2)
+    k_port_sweep(const PortArgs<T> a) {
+  extern __shared__ __align__(128) unsigned char smem[];
+  constexpr int kWarps = kSweepThreads / 32;
+  constexpr int RC = R >= 2 ? 2 : 1;         // columns per pass
+  constexpr int PR = patch_rows(R), PC = kNB / PR;  // a lane's patch
+  constexpr int RV = vec_cols<T, R>();
+  constexpr int kTile = kNB * kNB;
+  constexpr int kSlot = slot_bytes<TS>();
+  const int pad = PRIV ? 0 : a.pad, sb = a.sb;
+  const bool ring = PRIV || MMA || a.ring != 0;
+  constexpr bool HALF = sizeof(TS) == 2;
+  constexpr int NR = MMA ? operand_rows<TS, R>() : 1;  // rows of the split vector operand
+  constexpr int NB = HALF ? (R + 3) / 4 : 3;           // its 8-column operands per strip
+  __shared__ int smax[MMA && HALF ? R : 1];            // bits of max |s_r| of the segment
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  constexpr int kDepth = port_depth<TS, PRIV && MMA>();
+  unsigned char* const slots = smem + warp * (kDepth * kSlot);
+  T* const sv = reinterpret_cast<T*>(smem + (ring ? kWarps * kDepth * kSlot : 0));
+  uint16_t* const sop = reinterpret_cast<uint16_t*>(sv);    // MMA: s as [NR][op_stride] 16-bit terms
+  T* const yv = MMA ? reinterpret_cast<T*>(sop + NR * a.op_stride) : sv + a.vec_elems;  // PRIV: [kWarps]
+  T* const yw = yv + (PRIV ? (size_t)warp * a.vec_elems : 0);
+  T* const buf = yv + a.vec_elems;                          // not PRIV: [kWarps][sb strips][kNB * R] row sums
+  const int pa = lane / (kNB / PC), pb = lane % (kNB / PC);  // row and column group of the patch
+  const TS* Sall;
+  if constexpr (sizeof(TS) == 2) Sall = static_cast<const TS*>(a.Sh);
+  else Sall = reinterpret_cast<const TS*>(a.S);
+  uint64_t policy;
+  asm volatile("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(policy));
+  grid_dep_launch();
+  bool waited = false;
+
+  for (int si = a.cta_seg[blockIdx.x]; si < a.cta_seg[blockIdx.x + 1]; ++si) {
+    const PortSeg sg = a.segs[si];
+    const PieceDesc pd = a.pieces[sg.piece];
+    const int np = pd.nports;
+    const int I0 = sg.I0, I1 = sg.I1;
+    const int rows = (I1 + 1) * kNB;  // the rows that this segment's tiles touch
+    const TS* const Sb = Sall + sg.s_off * kTile;
+    const float* const tsc = HALF ? a.scale + sg.s_off : nullptr;
+
+    // Walk over this warp's tiles, strip by strip, columns ascending; J < 0 once they are exhausted.
+    struct Walk {
+      int I, J, step, lim, left;
+    };
+    // not PRIV: first own column of strip k.I or of a later one (steps 15 - 2 w and 1 + 2 w in turn)
+    auto strip = [&](Walk& k) {
+      for (;;) {
+        if (k.I > I1) {
+          k.J = -1;
+          return;
+        }
+        k.lim = (k.I == I1) ? sg.J1 : k.I;
+        k.J = warp;
+        k.step = kWarps * 2 - 1 - 2 * warp;
+        if (k.I == I0)
+          while (k.J < sg.J0) {
+            k.J += k.step;
+            k.step = 2 * kWarps - k.step;
+          }
+        if (k.J <= k.lim) return;
+        ++k.I;
+      }
+    };
+    auto next = [&](Walk& k) {
+      if constexpr (PRIV) {
+        if (--k.left == 0) {
+          k.J = -1;
+        } else if (++k.J > k.I) {
+          ++k.I;
+          k.J = 0;
+        }
+      } else {
+        k.J += k.step;
+        k.step = 2 * kWarps - k.step;
+        if (k.J > k.lim) {
+          ++k.I;
+          strip(k);
+        }
+      }
+    };
+    Walk cw;  // the tile being multiplied
+    if constexpr (PRIV) {
+      const int t0 = I0 * (I0 + 1) / 2 + sg.J0, n = I1 * (I1 + 1) / 2 + sg.J1 + 1 - t0;
+      const int f = n * warp / kWarps;
+      cw.left = n * (warp + 1) / kWarps - f;
+      tile_of(t0 + f, cw.I, cw.J);
+      if (cw.left == 0) cw.J = -1;
+    } else {
+      cw.I = I0;
+      strip(cw);
+    }
+    Walk fw = cw;  // the next tile to fetch
+    int slot = 0;  // of the tile being multiplied; its slot takes the tile kDepth ahead
+    auto fetch = [&](int to) {
+      if (fw.J >= 0) {
+        const int64_t t = fw.I * (fw.I + 1) / 2 + fw.J;
+        fetch_patch<TS>(slots + to * kSlot, Sb + t * kTile, HALF ? tsc + t : nullptr, lane, policy);
+        next(fw);
+      }
+      asm volatile("cp.async.commit_group;" ::: "memory");
+    };
+    if (ring)
+#pragma unroll
+      for (int d = 0; d < kDepth; ++d) fetch(d);
+    if (!waited) grid_dep_wait();  // everything above is constant between sweeps
+    waited = true;
+    float sigma[RV];  // MMA, FP16 tiles: the scale of s in the columns this thread writes out
+    if constexpr (MMA) {
+      // s as 16-bit terms, through an FP32 copy in the accumulators' place; then y = 0
+      const T* sp = a.s + (size_t)pd.port_off * R;
+      const int r = tid % (R / RV) * RV;
+      float m[RV] = {};
+      if (HALF && tid < R) smax[tid] = 0;
+#pragma unroll 4
+      for (int i = tid; i < rows * (R / RV); i += kSweepThreads) {
+        T v[RV] = {};
+        if (i / (R / RV) < np) load_cg<T, RV>(sp + (size_t)i * RV, v);
+        store_vec<T, RV>(yv + i * RV, v);
+        if constexpr (HALF)
+#pragma unroll
+          for (int c = 0; c < RV; ++c) m[c] = fmaxf(m[c], fabsf(v[c]));
+      }
+      __syncthreads();
+      if constexpr (HALF) {
+#pragma unroll
+        for (int c = 0; c < RV; ++c) {
+#pragma unroll
+          for (int o = R / RV; o < 32; o <<= 1) m[c] = fmaxf(m[c], __shfl_xor_sync(0xffffffffu, m[c], o));
+          if (lane < R / RV) atomicMax(&smax[r + c], __float_as_int(m[c]));
+        }
+        __syncthreads();
+#pragma unroll
+        for (int c = 0; c < RV; ++c) {
+          int e = 0;
+          const float mm = __int_as_float(smax[r + c]);
+          if (mm > 0.f && isfinite(mm)) frexpf(mm, &e);
+          sigma[c] = ldexpf(1.f, max(-120, e));
+        }
+      }
+      for (int i = tid; i < rows * (R / RV); i += kSweepThreads) {
+        const int q = i / (R / RV);
+        uint16_t* o = sop + (q & ~(kNB - 1)) + operand_pos(q & (kNB - 1));
+        T v[RV];
+        load_vec<T, RV>(yv + i * RV, v);
+#pragma unroll
+        for (int c = 0; c < RV; ++c) {
+          if constexpr (HALF) {
+            const float x = v[c] / sigma[c];
+            const __half hi = __float2half_rn(x);
+            o[(2 * (r + c)) * a.op_stride] = __half_as_ushort(hi);
+            o[(2 * (r + c) + 1) * a.op_stride] = __half_as_ushort(__float2half_rn(x - __half2float(hi)));
+          } else {
+            const float x = v[c], h = bf16_part(x), md = bf16_part(x - h), l = x - h - md;
+            o[(r + c) * a.op_stride] = (uint16_t)(__float_as_uint(h) >> 16);
+            o[(R + r + c) * a.op_stride] = (uint16_t)(__float_as_uint(md) >> 16);
+            o[(2 * R + r + c) * a.op_stride] = (uint16_t)(__float_as_uint(l) >> 16);
+          }
+        }
+      }
+      __syncthreads();
+      constexpr int W = 16 / sizeof(T);
+      const T z4[W] = {};
+      if constexpr (PRIV) {
+        for (int i = lane; i < rows * R / W; i += 32) store_vec<T, W>(yw + i * W, z4);
+      } else {
+        for (int i = tid; i < rows * R / W; i += kSweepThreads) store_vec<T, W>(yv + i * W, z4);
+      }
+    } else {
+      // s and y = 0, RV columns at a time; padding ports are zero
+      const T* sp = a.s + (size_t)pd.port_off * R;
+      const T zero[RV] = {};
+#pragma unroll 4
+      for (int i = tid; i < rows * (R / RV); i += kSweepThreads) {
+        const int q = i / (R / RV), r = i % (R / RV) * RV;
+        T v[RV] = {};
+        if (q < np) load_cg<T, RV>(sp + (size_t)q * R + r, v);
+        store_vec<T, RV>(sv + vidx<R>(q, pad) + r, v);
+        if constexpr (!PRIV) store_vec<T, RV>(yv + vidx<R>(q, pad) + r, zero);
+      }
+      if constexpr (PRIV) {
+        constexpr int W = 16 / sizeof(T);
+        const T z4[W] = {};
+        for (int i = lane; i < rows * R / W; i += 32) store_vec<T, W>(yw + i * W, z4);
+      }
+    }
+    __syncthreads();
+
+    // ---- tensor-core products.  Lane 4 g + t: rows g, g + 8 of a 16-row block, columns 2 t, 2 t + 1.
+    const int fg = lane >> 2, ft = lane & 3;
+    // the vector operand of strip K: registers (k half, k + 8) of both 16-row halves per operand
+    auto operand = [&](int K, uint32_t (&b)[NB][4]) {
+#pragma unroll
+      for (int n = 0; n < NB; ++n) {
+        const int row = HALF ? 8 * n + fg : n * R + fg;
+        const bool on = HALF ? row < NR : fg < R;
+        uint4 v = make_uint4(0u, 0u, 0u, 0u);
+        if (on) v = *reinterpret_cast<const uint4*>(sop + (size_t)row * a.op_stride + K * kNB + ft * 8);
+        b[n][0] = v.x, b[n][1] = v.y, b[n][2] = v.z, b[n][3] = v.w;
+      }
+    };
+    constexpr int ND = HALF ? NB : 1;    // accumulators per 16-row block
+    constexpr int NV = HALF ? ND : 2;    // sums per row that this lane holds
+    // column of the k-th sum of this lane
+    auto out_col = [&](int k) { return HALF ? 4 * k + ft : 2 * ft + k; };
+    // products of the current tile: row sums added to rp[row g, + 8, + 16, + 24], column sums into
+    // the accumulator
+    auto mma_tile = [&](int I, int J, const uint32_t (&bI)[NB][4], float (&rp)[4][NV]) {
+      asm volatile("cp.async.wait_group %0;" ::"n"(kDepth - 1) : "memory");
+      unsigned char* const tile = slots + slot * kSlot;
+      uint32_t bJ[NB][4];
+      operand(J, bJ);
+      float dr[2][ND][4], dc[2][ND][4];
+#pragma unroll
+      for (int h = 0; h < 2; ++h)
+#pragma unroll
+        for (int n = 0; n < ND; ++n)
+#pragma unroll
+          for (int k = 0; k < 4; ++k) dr[h][n][k] = dc[h][n][k] = 0.f;
+      float sc = 1.f;
+      if constexpr (HALF) {
+        sc = reinterpret_cast<const float*>(tile + kNB * kNB * 2)[lane];
+        __syncwarp();  // the other lanes' copies
+        const int row = ((lane >> 3) & 1) * 8 + (lane & 7);
+        const uint32_t base = smem_u32(tile) + row * 64;
+        uint32_t A[4][4], At[4][4];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+          const int mi = k >> 1, chunk = (k & 1) * 2 + (lane >> 4);
+          const uint32_t ad = base + mi * 1024 + (((chunk ^ (row >> 1)) & 3) << 4);
+          ldmatrix4<false>(ad, A[k]);
+          ldmatrix4<true>(ad, At[k]);
+        }
+        __syncwarp();  // every lane is through with the slot
+        fetch(slot);
+        slot = slot + 1 == kDepth ? 0 : slot + 1;
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+          const int mi = k >> 1, ki = k & 1;
+          const uint32_t At2[4] = {At[k][0], At[k][2], At[k][1], At[k][3]};
+#pragma unroll
+          for (int n = 0; n < ND; ++n) {
+            mma16816<true>(dr[mi][n], A[k], bJ[n][2 * ki], bJ[n][2 * ki + 1]);
+            if (I != J) mma16816<true>(dc[ki][n], At2, bI[n][2 * mi], bI[n][2 * mi + 1]);
+          }
+        }
+      } else {
+        float x[kNB];
+        load_patch(reinterpret_cast<const float*>(tile), lane, x);
+        fetch(slot);
+        slot = slot + 1 == kDepth ? 0 : slot + 1;
+        // terms of S from the smallest: a = 2 meets s_hi; a = 1 s_mid, s_hi; a = 0 s_lo, s_mid, s_hi
+#pragma unroll
+        for (int term = 2; term >= 0; --term)
+#pragma unroll
+          for (int k = 0; k < 4; ++k) {
+            const int mi = k >> 1, ki = k & 1;
+            uint32_t A[4], At[4];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+              float p0 = x[8 * k + 2 * u], p1 = x[8 * k + 2 * u + 1];
+              if (term >= 1) p0 -= bf16_part(p0), p1 -= bf16_part(p1);
+              if (term >= 2) p0 -= bf16_part(p0), p1 -= bf16_part(p1);
+              A[u] = upper_pair(p0, p1);
+            }
+            At[0] = movmatrix(A[0]), At[1] = movmatrix(A[2]), At[2] = movmatrix(A[1]), At[3] = movmatrix(A[3]);
+#pragma unroll
+            for (int n = 2 - term; n >= 0; --n) {
+              mma16816<false>(dr[mi][0], A, bJ[n][2 * ki], bJ[n][2 * ki + 1]);
+              if (I != J) mma16816<false>(dc[ki][0], At, bI[n][2 * mi], bI[n][2 * mi + 1]);
+            }
+          }
+      }
+#pragma unroll
+      for (int h = 0; h < 4; ++h)
+#pragma unroll
+        for (int k = 0; k < NV; ++k) {
+          if constexpr (HALF) {
+            const float* d = &dr[h >> 1][k][2 * (h & 1)];
+            rp[h][k] += (d[0] + d[1]) * sc;
+          } else {
+            rp[h][k] += dr[h >> 1][0][2 * (h & 1) + k];
+          }
+        }
+      if (I != J) {
+        if constexpr (HALF) {
+#pragma unroll
+          for (int k = 0; k < NV; ++k)
+            if (out_col(k) < R)
+#pragma unroll
+              for (int h = 0; h < 4; ++h) {
+                const float* d = &dc[h >> 1][k][2 * (h & 1)];
+                yw[(J * kNB + 8 * h + fg) * R + out_col(k)] += (d[0] + d[1]) * sc;
+              }
+        } else if (2 * ft < R) {
+#pragma unroll
+          for (int h = 0; h < 4; ++h) {
+            float2* at = reinterpret_cast<float2*>(yw + (J * kNB + 8 * h + fg) * R + 2 * ft);
+            const float* d = &dc[h >> 1][0][2 * (h & 1)];
+            float2 v = *at;
+            v.x += d[0], v.y += d[1];
+            *at = v;
+          }
+        }
+      }
+    };
+
+    auto wait_patch = [&](int I, int J, T (&pt)[kNB], T& sc) {
+      if (ring) {
+        asm volatile("cp.async.wait_group 0;" ::: "memory");
+        load_patch(reinterpret_cast<const TS*>(slots), lane, pt);
+        if constexpr (sizeof(TS) == 2) sc = reinterpret_cast<const float*>(slots + kNB * kNB * 2)[lane];
+        fetch(0);
+      } else {
+        const TS* t = Sb + (int64_t)(I * (I + 1) / 2 + J) * kTile;
+        load_patch(t, lane, pt);
+        if constexpr (sizeof(TS) == 2) sc = tsc[I * (I + 1) / 2 + J];
+      }
+    };
+    // T s_J into the lane's row sums rp, T^T s_I (off the diagonal) into the accumulator at column J
+    auto multiply = [&](int I, int J, const T (&pt)[kNB], T sc, T (&rp)[PR][R]) {
+#pragma unroll
+      for (int rc = 0; rc < R; rc += RC) {
+        T sI[PR][RC], sJ[PC][RC];
+        if constexpr (R == 1) {
+          load_run(sv + I * kNB + PR * pa, *reinterpret_cast<T(*)[PR]>(&sI[0][0]));
+          load_run(sv + J * kNB + PC * pb, *reinterpret_cast<T(*)[PC]>(&sJ[0][0]));
+        } else {
+#pragma unroll
+          for (int ii = 0; ii < PR; ++ii) load_vec<T, RC>(sv + vidx<R>(I * kNB + PR * pa + ii, pad) + rc, sI[ii]);
+#pragma unroll
+          for (int jj = 0; jj < PC; ++jj) load_vec<T, RC>(sv + vidx<R>(J * kNB + PC * pb + jj, pad) + rc, sJ[jj]);
+        }
+        // FP16 storage: the tile was divided by sc
+        if constexpr (sizeof(TS) == 2) {
+#pragma unroll
+          for (int jj = 0; jj < PC; ++jj)
+#pragma unroll
+            for (int q = 0; q < RC; ++q) sJ[jj][q] *= sc;
+        }
+        T cp[PC][RC];
+#pragma unroll
+        for (int jj = 0; jj < PC; ++jj)
+#pragma unroll
+          for (int q = 0; q < RC; ++q) cp[jj][q] = T(0);
+#pragma unroll
+        for (int ii = 0; ii < PR; ++ii)
+#pragma unroll
+          for (int jj = 0; jj < PC; ++jj)
+#pragma unroll
+            for (int q = 0; q < RC; ++q) {
+              rp[ii][rc + q] += pt[ii * PC + jj] * sJ[jj][q];
+              cp[jj][q] += pt[ii * PC + jj] * sI[ii][q];
+            }
+        if (I != J) {
+          reduce_scatter<T, PC, RC, kNB / PC>(cp, pa);  // lane (pa, pb) ends with column PC pb + pa
+          T* at = yw + vidx<R>(J * kNB + PC * pb + pa, pad) + rc;
+#pragma unroll
+          for (int q = 0; q < RC; ++q) at[q] += (sizeof(TS) == 2) ? cp[0][q] * sc : cp[0][q];
+        }
+      }
+    };
+
+    if constexpr (PRIV) {
+      while (MMA && cw.J >= 0) {
+        const int I = cw.I;
+        uint32_t bI[NB][4];
+        operand(I, bI);
+        float rp[4][NV] = {};
+        do {
+          const int J = cw.J;
+          next(cw);
+          mma_tile(I, J, bI, rp);
+        } while (cw.J >= 0 && cw.I == I);
+        __syncwarp();
+#pragma unroll
+        for (int k = 0; k < NV; ++k)
+          if (out_col(k) < R)
+#pragma unroll
+            for (int h = 0; h < 4; ++h) yw[(I * kNB + 8 * h + fg) * R + out_col(k)] += rp[h][k];
+        __syncwarp();
+      }
+      while (!MMA && cw.J >= 0) {
+        const int I = cw.I;
+        T rp[PR][R];
+#pragma unroll
+        for (int ii = 0; ii < PR; ++ii)
+#pragma unroll
+          for (int r = 0; r < R; ++r) rp[ii][r] = T(0);
+        do {
+          const int J = cw.J;
+          T pt[kNB], sc = T(1);
+          wait_patch(I, J, pt, sc);
+          next(cw);
+          multiply(I, J, pt, sc, rp);
+        } while (cw.J >= 0 && cw.I == I);
+        reduce_scatter<T, PR, R, 1>(rp, pb);  // lane (pa, pb) ends with row PR pa + pb
+        __syncwarp();
+        T* at = yw + (I * kNB + PR * pa + pb) * R;
+#pragma unroll
+        for (int r = 0; r < R; ++r) at[r] += rp[0][r];
+        __syncwarp();
+      }
+      __syncthreads();
+      finish_segment<T, R>(a, sg, si, pd, rows, reinterpret_cast<int*>(sv), [&](int q, int r, T(&v)[RV]) {
+#pragma unroll
+        for (int w = 0; w < kWarps; ++w) {
+          T x[RV];
+          load_vec<T, RV>(yv + (size_t)w * a.vec_elems + q * R + r, x);
+#pragma unroll
+          for (int c = 0; c < RV; ++c) v[c] += x[c];
+        }
+        if constexpr (MMA && HALF)
+#pragma unroll
+          for (int c = 0; c < RV; ++c) v[c] *= sigma[c];
+      });
+    } else {
+      const int sbs = sb > 0 ? sb : 1;
+      for (int Ib = I0; Ib <= I1; Ib += sbs) {
+        const int Ie = min(Ib + sbs, I1 + 1);
+        for (int I = Ib; MMA && I < Ie; ++I) {
+          uint32_t bI[NB][4];
+          operand(I, bI);
+          float rp[4][NV] = {};
+          while (cw.I == I && cw.J >= 0) {
+            const int J = cw.J;
+            next(cw);
+            mma_tile(I, J, bI, rp);
+          }
+          T* o = buf + (size_t)(warp * sb + (I - Ib)) * kNB * R;
+#pragma unroll
+          for (int k = 0; k < NV; ++k)
+            if (out_col(k) < R)
+#pragma unroll
+              for (int h = 0; h < 4; ++h) o[(8 * h + fg) * R + out_col(k)] = rp[h][k];
+        }
+        for (int I = Ib; !MMA && I < Ie; ++I) {
+          T rp[PR][R];
+#pragma unroll
+          for (int ii = 0; ii < PR; ++ii)
+#pragma unroll
+            for (int r = 0; r < R; ++r) rp[ii][r] = T(0);
+          while (cw.I == I && cw.J >= 0) {
+            const int J = cw.J;
+            T pt[kNB], sc = T(1);
+            wait_patch(I, J, pt, sc);
+            next(cw);
+            multiply(I, J, pt, sc, rp);
+          }
+          reduce_scatter<T, PR, R, 1>(rp, pb);  // lane (pa, pb) ends with row PR pa + pb
+          if (sb > 0) {
+            T* o = buf + ((size_t)(warp * sb + (I - Ib)) * kNB + PR * pa + pb) * R;
+#pragma unroll
+            for (int r = 0; r < R; ++r) o[r] = rp[0][r];
+          } else {
+            // no room for the warps' row sums: they take turns
+            for (int w = 0; w < kWarps; ++w) {
+              __syncthreads();
+              if (w == warp) {
+                T* at = yv + vidx<R>(I * kNB + PR * pa + pb, pad);
+#pragma unroll
+                for (int r = 0; r < R; ++r) at[r] += rp[0][r];
+              }
+            }
+            __syncthreads();
+          }
+        }
+        if (sb > 0) {
+          __syncthreads();
+          for (int i = tid; i < (Ie - Ib) * kNB * R; i += kSweepThreads) {
+            T v = T(0);
+#pragma unroll
+            for (int w = 0; w < kWarps; ++w) v += buf[(size_t)w * sb * kNB * R + i];
+            yv[vidx<R>(Ib * kNB + i / R, pad) + i % R] += v;
+          }
+          __syncthreads();
+        }
+      }
+      finish_segment<T, R>(a, sg, si, pd, rows, reinterpret_cast<int*>(sv),
+                           [&](int q, int r, T(&v)[RV]) {
+                             load_vec<T, RV>(yv + vidx<R>(q, pad) + r, v);
+                             if constexpr (MMA && HALF)
+#pragma unroll
+                               for (int c = 0; c < RV; ++c) v[c] *= sigma[c];
+                           });
+    }
+    __syncthreads();
+  }
+  if (!waited) grid_dep_wait();
+}
+
+// The port vectors of a sweep: s_q = sum_e w_in[e] / Z_e (w_in[e] = w_prev[twin[e]], the N2N
+// exchange) plus the coupling currents, one thread per port and RV columns.  Its loads depend on
+// each other in three steps (list ranges, list entries, waves); a kernel of its own has every port
+// of every subgraph in flight at once, and a subgraph that several CTAs work on gathers once.
+template <typename T, int R>
+__global__ void __launch_bounds__(256) k_port_vec(const PortArgs<T> a, int nports) {
+  constexpr int RV = vec_cols<T, R>();
+  grid_dep_launch();
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  const bool live = i < nports * (R / RV);
+  const int q = i / (R / RV), r = i % (R / RV) * RV;
+  int e0 = 0, e1 = 0, k0 = 0, k1 = 0;
+  if (live) {
+    e0 = a.port_end_ptr[q], e1 = a.port_end_ptr[q + 1];
+    if (a.cpl.ptr) k0 = a.cpl.ptr[q], k1 = a.cpl.ptr[q + 1];
+  }
+  T acc[RV] = {}, cc[RV] = {};
+  bool waited = false;  // the lists are constant: only the waves come from the sweep before
+  constexpr int kB = 4;  // list entries loaded together
+  auto list = [&](int lo, int hi, const int32_t* row, const T* coef, T (&sum)[RV]) {
+    for (int k = lo; k < hi; k += kB) {
+      int at[kB];
+      T c[kB], w[kB][RV];
+#pragma unroll
+      for (int j = 0; j < kB; ++j) {
+        at[j] = k + j < hi ? row[k + j] : -1;
+        c[j] = k + j < hi ? coef[k + j] : T(0);
+      }
+      if (!waited) grid_dep_wait();
+      waited = true;
+#pragma unroll
+      for (int j = 0; j < kB; ++j)
+        if (at[j] >= 0) load_cg<T, RV>(a.wprev + (size_t)at[j] * R + r, w[j]);
+#pragma unroll
+      for (int j = 0; j < kB; ++j)
+        if (at[j] >= 0)
+#pragma unroll
+          for (int v = 0; v < RV; ++v) sum[v] += w[j][v] * c[j];
+    }
+  };
+  list(e0, e1, a.twin, a.invz, acc);
+  if (k1 > k0) {
+    list(k0, k1, a.cpl.oth, a.cpl.y, cc);
+#pragma unroll
+    for (int v = 0; v < RV; ++v) acc[v] += cc[v];
+  }
+  if (!waited) grid_dep_wait();
+  if (live) store_vec<T, RV>(a.s + (size_t)q * R + r, acc);
+}
+
+// Shared memory of a sweep and the kernel that goes with it.  Accumulators per warp (R <= 2) if they
+// leave room for two CTAs per SM (one in FP64); the tensor cores for FP16 tiles and for FP32 tiles with R = 4, 8 wherever their operands and
+// slots fit.  Vectors too long for that many CTAs take one, then the SIMT products, then give up
+// the gaps, the slots and the row sums.
+PortShape port_shape(size_t elem, size_t stored, int R, int max_ports) {
   const size_t npad = (size_t)((max_ports + kNB - 1) / kNB) * kNB;
-  return (det ? 2 + kSweepThreads / 32 : 2) * npad * R * elem;
+  constexpr int kWarps = kSweepThreads / 32;
+  const size_t sum = (size_t)kWarps * kNB * R * elem;  // one strip's row sums
+  const size_t slot =
+      (size_t)kWarps * (stored == 2 ? slot_bytes<__half>() : stored == 4 ? slot_bytes<float>() : slot_bytes<double>());
+  const size_t kSmemMax = 226 * 1024;  // the tensor-core kernels have a static part
+  const int per_sm = elem == 8 ? 1 : 2;
+  const size_t all = (228 * 1024) / per_sm - 1024;  // an SM's shared memory, 1 KB per CTA reserved
+  const size_t share = all < kSmemMax ? all : kSmemMax;
+  PortShape p{};
+  auto fit = [&](bool mma, bool priv, int pad, bool ring, int sb, size_t most) {
+    p.mma = mma;
+    p.priv = priv;
+    p.pad = pad;
+    p.ring = ring;
+    p.sb = sb;
+    p.vec_elems = (int)(npad * R + npad / 4 * pad);
+    // rows of the vector operand start half a bank row apart (an odd number of 64-byte strips)
+    p.op_stride = (int)(npad / kNB % 2 ? npad : npad + kNB);
+    const size_t op = (size_t)(stored == 2 ? operand_rows<__half, 1>() : operand_rows<float, 1>()) * R * p.op_stride * 2;
+    const size_t depth = stored == 2 && mma && priv ? port_depth<__half, true>() : 1;
+    p.smem = (ring ? slot * depth : 0) + (mma ? op : p.vec_elems * elem) + (size_t)p.vec_elems * elem * (priv ? kWarps : 1) +
+             sb * sum;
+    p.layout = mma && stored == 4 ? kPortFragments : R <= 2 ? kPortPatch8x4 : kPortPatch4x8;
+    return p.smem <= most;
+  };
+  const bool mma = stored == 2 || (stored == 4 && R >= 4);
+  if (R <= 2 && fit(mma, true, 0, true, 0, share)) return p;
+  if (mma)
+    for (size_t most : {share, kSmemMax})
+      for (int sb : {8, 4, 2, 1})
+        if (fit(true, false, 0, true, sb, most)) return p;
+  const int pad = (elem == 4 && R >= 4) ? 4 : 0;
+  for (size_t most : {share, kSmemMax})
+    for (int sb : {8, 4, 2, 1})
+      if (fit(false, false, pad, true, sb, most)) return p;
+  const size_t all_smem = 227 * 1024;
+  if (fit(false, false, 0, true, 1, all_smem) || fit(false, false, 0, false, 1, all_smem)) return p;
+  fit(false, false, 0, false, 0, all_smem);
+  return p;
 }
 
-bool port_sweep_det_fits(size_t elem, int R, int max_ports) {
-  return port_sweep_smem_bytes(elem, R, max_ports, true) <= kPortDetSmem;
+// Cuts the tiles of all subgraphs, in order, into equal shares for `ctas` CTAs (cut points at whole
+// tiles; a cut that would leave a piece of a subgraph with fewer than kMinSeg tiles moves to the
+// subgraph's end).  Besides its tiles a segment costs about 7 us of latency (its vectors, its
+// partial sums, its waves), which counts as the tiles that one CTA gets through in that time.
+PortPlan port_plan(const PieceDesc* pd, int npieces, size_t elem, size_t stored, int R, int ctas) {
+  constexpr int kMinSeg = 32;
+  const double kSegCost = elem == 8 ? 10.0 : R >= 4 ? 20.0 : 35.0;
+  PortPlan pl;
+  double total = 0;
+  for (int j = 0; j < npieces; ++j)
+    if (pd[j].nports > 0) total += (double)port_tiles(pd[j].nports) + kSegCost;
+  // about one segment per cut more than subgraphs
+  const double share = std::max(1.0, (total + kSegCost * ctas) / std::max(1, ctas));
+  double pos = 0;  // cost placed so far
+  int cta = 0;
+  pl.cta_seg.push_back(0);
+  for (int j = 0; j < npieces; ++j) {
+    if (pd[j].nports <= 0) continue;
+    const int n = (int)port_tiles(pd[j].nports);
+    const int first = (int)pl.segs.size();
+    int t = 0;
+    while (t < n) {
+      pos += kSegCost;
+      const double room = (cta + 1) * share - pos;
+      int take = n - t;
+      if (room < take) {
+        take = std::max(kMinSeg, (int)std::ceil(room));
+        if (n - t - take < kMinSeg) take = n - t;
+      }
+      PortSeg sg{};
+      sg.piece = j;
+      sg.s_off = pd[j].s_off;
+      tile_of(t, sg.I0, sg.J0);
+      tile_of(t + take - 1, sg.I1, sg.J1);
+      sg.first = first;
+      pl.segs.push_back(sg);
+      t += take;
+      pos += take;
+      while (cta + 1 < ctas && pos >= (cta + 1) * share - 1e-9) {
+        ++cta;
+        if (pl.cta_seg.back() != (int)pl.segs.size()) pl.cta_seg.push_back((int)pl.segs.size());
+      }
+    }
+    const int nseg = (int)pl.segs.size() - first;
+    for (int k = first; k < first + nseg; ++k) {
+      pl.segs[k].nseg = nseg;
+      pl.segs[k].part = pl.part_elems;
+    }
+    if (nseg > 1) pl.part_elems += (int64_t)nseg * ((pd[j].nports + kNB - 1) / kNB) * kNB * R;
+  }
+  if (pl.cta_seg.back() != (int)pl.segs.size()) pl.cta_seg.push_back((int)pl.segs.size());
+  return pl;
 }
 
-template <typename T, typename TS, bool DET>
-static cudaError_t port_configure_ts(int R, size_t smem) {
-  const int b = (int)smem;
+template <typename T, typename TS, int R>
+static const void* port_kernel_r(bool priv, bool mma) {
+  constexpr bool can_mma = sizeof(TS) == 2 || (sizeof(TS) == 4 && R >= 4);
+  if constexpr (can_mma) {
+    if constexpr (R <= 2)
+      if (mma && priv) return (const void*)k_port_sweep<T, TS, R, true, true>;
+    if (mma) return (const void*)k_port_sweep<T, TS, R, false, true>;
+  } else if constexpr (R <= 2) {
+    if (priv) return (const void*)k_port_sweep<T, TS, R, true, false>;
+  }
+  return (const void*)k_port_sweep<T, TS, R, false, false>;
+}
+
+template <typename T, typename TS>
+static const void* port_kernel(int R, bool priv, bool mma) {
   switch (R) {
-    case 1: return cudaFuncSetAttribute(k_port_sweep<T, TS, 1, DET>, cudaFuncAttributeMaxDynamicSharedMemorySize, b);
-    case 2: return cudaFuncSetAttribute(k_port_sweep<T, TS, 2, DET>, cudaFuncAttributeMaxDynamicSharedMemorySize, b);
-    case 4: return cudaFuncSetAttribute(k_port_sweep<T, TS, 4, DET>, cudaFuncAttributeMaxDynamicSharedMemorySize, b);
-    case 8: return cudaFuncSetAttribute(k_port_sweep<T, TS, 8, DET>, cudaFuncAttributeMaxDynamicSharedMemorySize, b);
-    default: return cudaErrorInvalidValue;
+    case 1: return port_kernel_r<T, TS, 1>(priv, mma);
+    case 2: return port_kernel_r<T, TS, 2>(priv, mma);
+    case 4: return port_kernel_r<T, TS, 4>(priv, mma);
+    case 8: return port_kernel_r<T, TS, 8>(priv, mma);
+    default: return nullptr;
   }
 }
 
 template <typename T>
-cudaError_t port_sweep_configure(int R, size_t smem, bool det) {
-  cudaError_t e = det ? port_configure_ts<T, T, true>(R, smem) : port_configure_ts<T, T, false>(R, smem);
-  if constexpr (sizeof(T) == 4) {
-    if (e == cudaSuccess) e = det ? port_configure_ts<T, __half, true>(R, smem) : port_configure_ts<T, __half, false>(R, smem);
-  }
+static const void* port_kernel_of(int R, bool priv, bool mma, bool half) {
+  if constexpr (sizeof(T) == 4)
+    if (half) return port_kernel<T, __half>(R, priv, mma);
+  return port_kernel<T, T>(R, priv, mma);
+}
+
+template <typename T>
+cudaError_t port_sweep_configure(int R, const PortShape& sh, bool half, int* ctas_per_sm) {
+  const void* k = port_kernel_of<T>(R, sh.priv, sh.mma, half);
+  if (!k) return cudaErrorInvalidValue;
+  // the limit is the kernel's, not the solver's: the device maximum, whatever solver came last
+  cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                       (sh.mma ? 226 : 227) * 1024);
+  if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(ctas_per_sm, k, kSweepThreads, sh.smem);
   return e;
 }
 
-template <typename T, typename TS, bool DET>
-static cudaError_t port_launch_ts(const PortArgs<T>& a, int R, int npieces, size_t smem, cudaStream_t st) {
-  switch (R) {
-    case 1: k_port_sweep<T, TS, 1, DET><<<npieces, kSweepThreads, smem, st>>>(a); break;
-    case 2: k_port_sweep<T, TS, 2, DET><<<npieces, kSweepThreads, smem, st>>>(a); break;
-    case 4: k_port_sweep<T, TS, 4, DET><<<npieces, kSweepThreads, smem, st>>>(a); break;
-    case 8: k_port_sweep<T, TS, 8, DET><<<npieces, kSweepThreads, smem, st>>>(a); break;
-    default: return cudaErrorInvalidValue;
-  }
-  return cudaGetLastError();
+// A launch whose CTAs may start while the launch before it on the stream still runs (the kernel
+// waits for its results itself, grid_dep_wait).
+template <typename T>
+static cudaError_t launch_dependent(const void* k, int grid, int block, size_t smem, void** args, cudaStream_t st) {
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(grid);
+  cfg.blockDim = dim3(block);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelExC(&cfg, k, args);
 }
 
 template <typename T>
-cudaError_t launch_port_sweep(const PortArgs<T>& a, int R, int npieces, size_t smem, cudaStream_t st) {
-  if (npieces <= 0) return cudaSuccess;
-  if constexpr (sizeof(T) == 4) {
-    if (a.Sh) return a.det ? port_launch_ts<T, __half, true>(a, R, npieces, smem, st)
-                           : port_launch_ts<T, __half, false>(a, R, npieces, smem, st);
-  }
-  return a.det ? port_launch_ts<T, T, true>(a, R, npieces, smem, st) : port_launch_ts<T, T, false>(a, R, npieces, smem, st);
+cudaError_t launch_port_sweep(const PortArgs<T>& a, int R, int nports, int grid, size_t smem, cudaStream_t st) {
+  if (grid <= 0 || nports <= 0) return cudaSuccess;
+  const void* k = port_kernel_of<T>(R, a.priv != 0, a.mma != 0, sizeof(T) == 4 && a.Sh);
+  const void* v = R == 1   ? (const void*)k_port_vec<T, 1>
+                  : R == 2 ? (const void*)k_port_vec<T, 2>
+                  : R == 4 ? (const void*)k_port_vec<T, 4>
+                           : (const void*)k_port_vec<T, 8>;
+  if (!k) return cudaErrorInvalidValue;
+  PortArgs<T> args = a;
+  const int n = nports * std::max(1, R * (int)sizeof(T) / 16);
+  void* av[] = {&args, &nports};
+  cudaError_t e = launch_dependent<T>(v, (n + 255) / 256, 256, 0, av, st);
+  if (e != cudaSuccess) return e;
+  return launch_dependent<T>(k, grid, kSweepThreads, smem, av, st);
 }
 
 // FP16 copy of the FP32 tiles of one subgraph per CTA, one warp per tile: each tile is divided by
-// its largest |entry| (1 if all zero), kept per tile in scale[s_off + t], and re-laid out from the
-// float patch layout ((p/4)*32 + L)*4 + p%4 to the half patch layout ((p/8)*32 + L)*8 + p%8.  A scale
-// per tile keeps the small far-field blocks of S_j at full FP16 precision.
+// its largest |entry| (1 if all zero), kept in scale[], and re-laid out (for ldmatrix, or as patches).  A scale per tile keeps the small far-field blocks of S_j at full FP16 precision.
 __global__ void k_port_to_half(const PieceDesc* __restrict__ pieces, const float* __restrict__ S,
-                               __half* __restrict__ Sh, float* __restrict__ scale) {
+                               __half* __restrict__ Sh, float* __restrict__ scale, int from, int to, int mma) {
   const PieceDesc pd = pieces[blockIdx.x];
   const int64_t nt = port_tiles(pd.nports);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -397,24 +1207,24 @@ __global__ void k_port_to_half(const PieceDesc* __restrict__ pieces, const float
     if (lane == 0) scale[pd.s_off + t] = sc;
     const float inv = 1.f / sc;
     for (int k = lane; k < kNB * kNB; k += 32) {
-      const int L = (k / 4) % kNB, p = (k / 128) * 4 + (k % 4);
-      dst[((p / 8) * kNB + L) * 8 + (p % 8)] = __float2half_rn(src[k] * inv);
+      const int i = k / kNB, c = k % kNB;
+      dst[mma ? half_pos(i, c) : tile_pos(to, i, c, 8)] = __float2half_rn(src[tile_pos(from, i, c, 4)] * inv);
     }
   }
 }
 
 cudaError_t launch_port_to_half(const PieceDesc* pieces, int npieces, const float* S, __half* Sh, float* scale,
-                                cudaStream_t st) {
+                                const PortShape& from, const PortShape& to, cudaStream_t st) {
   if (npieces <= 0) return cudaSuccess;
-  k_port_to_half<<<npieces, kSweepThreads, 0, st>>>(pieces, S, Sh, scale);
+  k_port_to_half<<<npieces, kSweepThreads, 0, st>>>(pieces, S, Sh, scale, from.layout, to.layout, to.mma);
   return cudaGetLastError();
 }
 
 template <typename T>
 cudaError_t launch_gather_port_response(const PieceDesc* pieces, int npieces, const int32_t* port_local, int Rs, int b,
-                                        const T* xc, T* S, cudaStream_t st) {
+                                        const T* xc, T* S, int layout, cudaStream_t st) {
   if (npieces <= 0) return cudaSuccess;
-  k_gather_port_response<T><<<npieces, 256, 0, st>>>(pieces, port_local, Rs, b, xc, S);
+  k_gather_port_response<T><<<npieces, 256, 0, st>>>(pieces, port_local, Rs, b, xc, S, layout);
   return cudaGetLastError();
 }
 
@@ -427,10 +1237,10 @@ cudaError_t launch_gather_ports(const PieceDesc* pieces, int npieces, const int3
 }
 
 #define VTM_PORT_INST(T)                                                                                       \
-  template cudaError_t port_sweep_configure<T>(int, size_t, bool);                                             \
-  template cudaError_t launch_port_sweep<T>(const PortArgs<T>&, int, int, size_t, cudaStream_t);               \
+  template cudaError_t port_sweep_configure<T>(int, const PortShape&, bool, int*);                             \
+  template cudaError_t launch_port_sweep<T>(const PortArgs<T>&, int, int, int, size_t, cudaStream_t);          \
   template cudaError_t launch_gather_port_response<T>(const PieceDesc*, int, const int32_t*, int, int, const T*, \
-                                                      T*, cudaStream_t);                                        \
+                                                      T*, int, cudaStream_t);                                      \
   template cudaError_t launch_gather_ports<T>(const PieceDesc*, int, const int32_t*, int, const T*, T*, cudaStream_t);
 VTM_PORT_INST(float)
 VTM_PORT_INST(double)

@@ -139,9 +139,13 @@ struct vtm_solver {
   bool port_form = false;
   bool port_tc = false;              // R >= 16, FP32: tensor-core port sweep (port_tc.cu)
   DevBuf S, ubase, wzero, wscr;
+  DevBuf port_s;                     // SIMT port sweep: port vectors, ports x R
   bool ubase_ok = false;
-  size_t port_smem = 0;
-  bool port_det = false;             // SIMT port sweep: fixed-order (bitwise reproducible) reduction
+  struct PortDev {                   // SIMT port sweep: shared-memory shape and division of the tiles
+    PortShape sh{};                  // among CTAs, for S_j as stored ([0]) and for its FP16 copy ([1])
+    DevBuf segs, cta_seg, part, ticket;
+    int grid = 0;
+  } port_div[2];
   DevBuf S16, sig16, tc_scratch;     // tensor-core form: fp16 hi / lo blocks, sigma_j, s^T slots
   DevBuf gscale;                     // tensor-core form: sqrt(S_pp) per port (diagonal balance)
   int tc_grid = 0, tc_n4max = 0, tc_tmem_cols = 0;
@@ -939,7 +943,7 @@ static void compute_port_response(vtm_solver* s, int64_t s_tiles) {
         }
       }
       VTM_CUDA(launch_gather_port_response<T>(s->pieces_lo.as<PieceDesc>(), s->np_lo, s->port_local.as<int32_t>(),
-                                              Rs, b, xc32.as<T>(), s->S.as<T>(), st));
+                                              Rs, b, xc32.as<T>(), s->S.as<T>(), s->port_div[0].sh.layout, st));
     }
     VTM_CUDA(cudaStreamSynchronize(st));
   } else {
@@ -957,7 +961,7 @@ static void compute_port_response(vtm_solver* s, int64_t s_tiles) {
         }
       }
       VTM_CUDA(launch_gather_port_response<T>(s->pieces_lo.as<PieceDesc>(), s->np_lo, s->port_local.as<int32_t>(),
-                                              R, b, s->xc.as<T>(), s->S.as<T>(), st));
+                                              R, b, s->xc.as<T>(), s->S.as<T>(), s->port_div[0].sh.layout, st));
     }
     VTM_CUDA(cudaMemsetAsync(s->bt.p, 0, s->bt.bytes, st));
     reset_waves(s);
@@ -1035,7 +1039,19 @@ static void launch_port(vtm_solver* s) {
     }
   }
   PortArgs<T> a;
-  a.det = s->port_det ? 1 : 0;
+  const vtm_solver::PortDev& d = s->port_div[s->port_half ? 1 : 0];
+  a.segs = d.segs.template as<PortSeg>();
+  a.cta_seg = d.cta_seg.template as<int32_t>();
+  a.s = s->port_s.as<T>();
+  a.part = d.part.template as<T>();
+  a.ticket = d.ticket.template as<int>();
+  a.vec_elems = d.sh.vec_elems;
+  a.pad = d.sh.pad;
+  a.op_stride = d.sh.op_stride;
+  a.mma = d.sh.mma;
+  a.priv = d.sh.priv;
+  a.ring = d.sh.ring;
+  a.sb = d.sh.sb;
   a.Sh = s->port_half ? s->Sh.p : nullptr;
   a.scale = s->hscale.as<float>();
   a.pieces = s->pieces_lo.as<PieceDesc>();
@@ -1047,8 +1063,8 @@ static void launch_port(vtm_solver* s) {
   a.twin = s->twin.as<int32_t>();
   a.invz = s->invz_t.as<T>();
   a.cpl = couple_ref<T>(s);
-  VTM_CUDA(launch_port_sweep<T>(a, s->R, s->np_lo, s->port_smem, s->stream));
-  s->launches++;
+  VTM_CUDA(launch_port_sweep<T>(a, s->R, s->nports, d.grid, d.sh.smem, s->stream));
+  s->launches += 2;
 }
 
 // k sweeps in port form: k - 1 port-only sweeps, then one band sweep that also writes x_j.  The
@@ -1069,7 +1085,7 @@ static void port_sweeps_typed(vtm_solver* s, int k) {
 static int64_t launches_per_batch(const vtm_solver* s, int k) {
   const int64_t band = (s->np_lo > 0) + (s->np_hi > 0);
   if (!s->port_form || k < 2) return (int64_t)k * band;
-  const int64_t port = (s->np_lo > 0) + (s->np_hi > 0);
+  const int64_t port = (s->np_lo > 0 ? (s->port_tc ? 1 : 2) : 0) + (s->np_hi > 0);
   return (int64_t)(k - 1) * port + band;
 }
 
@@ -1105,8 +1121,8 @@ static void choose_form(vtm_solver* s, const vtm_setup_opts* o, int64_t s_tiles,
   int tmem_cols = 32;
   while (tmem_cols < n4max * s->R) tmem_cols *= 2;
   const bool tmem_ok = n4max * s->R <= 512 && n4max <= kTcMaxSuper;
-  const bool det = !tc && port_sweep_det_fits(sizeof(T), s->R, max_ports_lo);
-  const size_t smem = tc ? port_tc_smem_bytes(s->R, true) : port_sweep_smem_bytes(sizeof(T), s->R, max_ports_lo, det);
+  const size_t smem =
+      tc ? port_tc_smem_bytes(s->R, true) : port_shape(sizeof(T), sizeof(T), s->R, max_ports_lo).smem;
   // bytes one sweep streams (tensor cores: with the lo half) and the device memory setup needs
   const double s_bytes = tc ? (double)h_bytes : (double)s_tiles * kNB * kNB * sizeof(T);
   const double setup_bytes = tc ? s_bytes + (double)s_tiles * 128.0 * 128.0 * 4.0 : s_bytes;
@@ -1130,11 +1146,25 @@ static void choose_form(vtm_solver* s, const vtm_setup_opts* o, int64_t s_tiles,
   // fill the tail of the launch (all launches over pieces_lo write through global indices only)
   std::stable_sort(lo.begin(), lo.end(), [](const PieceDesc& x, const PieceDesc& y) { return x.nports > y.nports; });
   upload(s->pieces_lo, lo, s->stream);
-  s->port_smem = smem;
+  int dev = 0, nsm = 1;
+  VTM_CUDA(cudaGetDevice(&dev));
+  VTM_CUDA(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
+  auto divide = [&](bool half) {
+    int per_sm = 1;
+    vtm_solver::PortDev& d = s->port_div[half ? 1 : 0];
+    d.sh = port_shape(sizeof(T), half ? sizeof(__half) : sizeof(T), s->R, max_ports_lo);
+    VTM_CUDA(port_sweep_configure<T>(s->R, d.sh, half, &per_sm));
+    const PortPlan pl = port_plan(lo.data(), (int)lo.size(), sizeof(T), half ? sizeof(__half) : sizeof(T), s->R,
+                                  std::max(1, per_sm) * nsm);
+    upload(d.segs, pl.segs, s->stream);
+    upload(d.cta_seg, pl.cta_seg, s->stream);
+    d.part.alloc((size_t)pl.part_elems * sizeof(T));
+    d.ticket.alloc(std::max<size_t>(1, pl.segs.size()) * sizeof(int));
+    VTM_CUDA(cudaMemsetAsync(d.ticket.p, 0, d.ticket.bytes, s->stream));
+    VTM_CUDA(cudaStreamSynchronize(s->stream));  // the uploads read pl
+    d.grid = (int)pl.cta_seg.size() - 1;
+  };
   if (tc) {
-    int dev = 0, nsm = 1;
-    VTM_CUDA(cudaGetDevice(&dev));
-    VTM_CUDA(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
     s->tc_grid = std::min(s->np_lo, nsm);  // one persistent CTA per SM (it holds the SM's tensor memory)
     s->tc_n4max = n4max;
     s->tc_tmem_cols = tmem_cols;
@@ -1150,8 +1180,8 @@ static void choose_form(vtm_solver* s, const vtm_setup_opts* o, int64_t s_tiles,
                                  s->invz_t.as<float>(), couple_ref<float>(s), s->port_rec.as<int4>(), s->stream));
     VTM_CUDA(port_tc_configure(s->R));
   } else {
-    VTM_CUDA(port_sweep_configure<T>(s->R, smem, det));
-    s->port_det = det;
+    s->port_s.alloc((size_t)std::max(1, s->nports) * s->R * sizeof(T));
+    divide(false);
   }
   s->ubase.alloc((size_t)std::max(1, s->nports) * s->R * sizeof(T));
   s->wzero.alloc((size_t)s->E * s->R * sizeof(T));
@@ -1185,8 +1215,9 @@ static void choose_form(vtm_solver* s, const vtm_setup_opts* o, int64_t s_tiles,
     if (!tc && (o->port_storage == VTM_STORE_FP16 || (o->port_storage == VTM_STORE_FP16_AUTO && !l2_resident))) {
       s->Sh.alloc((size_t)s_tiles * kNB * kNB * sizeof(__half));
       s->hscale.alloc((size_t)std::max<int64_t>(1, s_tiles) * sizeof(float));  // one scale per tile
+      divide(true);
       VTM_CUDA(launch_port_to_half(s->pieces_lo.as<PieceDesc>(), s->np_lo, s->S.as<float>(), s->Sh.as<__half>(),
-                                   s->hscale.as<float>(), s->stream));
+                                   s->hscale.as<float>(), s->port_div[0].sh, s->port_div[1].sh, s->stream));
       s->port_half = true;
       s->port_half_auto = (o->port_storage == VTM_STORE_FP16_AUTO);
       s->info.port_bytes = (int64_t)(s_bytes / 2);
