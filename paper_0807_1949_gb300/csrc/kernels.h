@@ -154,6 +154,67 @@ cudaError_t launch_gather_ports(const PieceDesc* pieces, int npieces, const int3
 cudaError_t launch_port_to_half(const PieceDesc* pieces, int npieces, const float* S, __half* Sh, float* scale,
                                 const PortShape& from, const PortShape& to, cudaStream_t st);
 
+// Port sweeps of small systems in one launch, S_j resident in shared memory (port_resident.cu).
+struct ResCta {
+  int64_t s_off;               // the CTA's subgraphs' S_j in the dense storage
+  int32_t s_elems;
+  int32_t vec;                 // ports of the CTA
+  int32_t splits;              // units that share a group of rows
+  int32_t port0, nports;       // into ResPlan::ports
+  int32_t unit0, nunits;       // into ResPlan::units
+};
+struct ResUnit {
+  int32_t s;                   // first row of the unit in the CTA's S (column 0)
+  int32_t stride, n, row0;     // column stride, the subgraph's ports, first row
+  int32_t vec;                 // the subgraph's first port in the CTA's vectors
+  int32_t c0, c1, split;       // columns of the unit
+};
+struct ResPort {
+  int32_t port, vec;           // port (global), its place in the CTA's vectors
+  int32_t e0, e1, w0;          // its ends, the first one's place among the CTA's ends
+};
+struct ResPieceS {
+  int32_t port_off, n, stride;
+  int64_t s;                   // element offset of its dense S_j: entry (i, c) at s + c stride + i
+  int32_t piece;               // index into the subgraphs the plan was made of
+};
+struct ResPlan {
+  bool ok = false;
+  std::vector<ResCta> ctas;
+  std::vector<ResUnit> units;
+  std::vector<ResPort> ports;
+  std::vector<ResPieceS> piece_s;
+  int64_t s_elems = 0;
+  size_t smem = 0;
+};
+template <typename T>
+struct ResArgs {
+  const ResCta* ctas;
+  const ResUnit* units;
+  const ResPort* ports;
+  const T* S;
+  const T* ubase;
+  const T* wprev;              // ends x R: incoming waves of the first sweep
+  T* wout;                     // outgoing waves of the last sweep
+  unsigned long long* xch[2];  // exchange buffers, ends x R words each (FP64: two words), contiguous
+  const int32_t* twin;
+  const T* invz;
+  CoupleRef<T> cpl;
+  int sweeps;
+  int* status;
+  long wait_limit;
+};
+ResPlan res_plan(const PieceDesc* pd, int npieces, size_t elem, int R, int nsm);
+void res_plan_ends(ResPlan& pl, const int32_t* port_end_ptr);  // host copy of the end lists
+template <typename T>
+cudaError_t launch_gather_port_dense(const ResPieceS* ps, int n, const PieceDesc* pieces, const int32_t* port_local,
+                                     int Rs, int b, const T* xc, T* S, cudaStream_t st);
+template <typename T>
+cudaError_t port_resident_configure(int R, size_t smem, int* ctas_per_sm);
+// a.sweeps sweeps in one cooperative launch (after clearing the exchange buffers, xch_bytes in all).
+template <typename T>
+cudaError_t launch_port_resident(const ResArgs<T>& a, int R, int grid, size_t smem, size_t xch_bytes, cudaStream_t st);
+
 // Tensor-core port-response sweep for 16 / 32 right-hand sides (port_tc.cu), FP32 solvers.
 struct PortTCArgs {
   const PieceDesc* pieces;     // subgraphs of the launch (largest first); CTA c takes c, c + grid, ...

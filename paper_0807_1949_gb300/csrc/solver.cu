@@ -146,6 +146,11 @@ struct vtm_solver {
     DevBuf segs, cta_seg, part, ticket;
     int grid = 0;
   } port_div[2];
+  // small systems: S_j resident in shared memory, a batch's sweeps in one launch (port_resident.cu)
+  bool resident = false;
+  DevBuf res_ctas, res_units, res_ports, res_ps, res_xch;
+  int res_grid = 0, res_pieces = 0;
+  size_t res_smem = 0;
   DevBuf S16, sig16, tc_scratch;     // tensor-core form: fp16 hi / lo blocks, sigma_j, s^T slots
   DevBuf gscale;                     // tensor-core form: sqrt(S_pp) per port (diagonal balance)
   int tc_grid = 0, tc_n4max = 0, tc_tmem_cols = 0;
@@ -884,7 +889,7 @@ template <typename T>
 static void compute_port_response(vtm_solver* s, int64_t s_tiles) {
   cudaStream_t st = s->stream;
   const int np = s->npieces;
-  s->S.alloc((size_t)s_tiles * kNB * kNB * sizeof(T));
+  if (!s->resident) s->S.alloc((size_t)s_tiles * kNB * kNB * sizeof(T));
   VTM_CUDA(cudaMemsetAsync(s->S.p, 0, s->S.bytes, st));
   const size_t kSmemMax = 227 * 1024;
   int st_lo = 0;
@@ -942,8 +947,12 @@ static void compute_port_response(vtm_solver* s, int64_t s_tiles) {
           VTM_CUDA((launch_sweep_wide<T, T>(a, Rs, s->np_lo, sm_lo, st)));
         }
       }
-      VTM_CUDA(launch_gather_port_response<T>(s->pieces_lo.as<PieceDesc>(), s->np_lo, s->port_local.as<int32_t>(),
-                                              Rs, b, xc32.as<T>(), s->S.as<T>(), s->port_div[0].sh.layout, st));
+      if (s->resident)
+        VTM_CUDA(launch_gather_port_dense<T>(s->res_ps.as<ResPieceS>(), s->res_pieces, s->pieces_lo.as<PieceDesc>(),
+                                             s->port_local.as<int32_t>(), Rs, b, xc32.as<T>(), s->S.as<T>(), st));
+      else
+        VTM_CUDA(launch_gather_port_response<T>(s->pieces_lo.as<PieceDesc>(), s->np_lo, s->port_local.as<int32_t>(),
+                                                Rs, b, xc32.as<T>(), s->S.as<T>(), s->port_div[0].sh.layout, st));
     }
     VTM_CUDA(cudaStreamSynchronize(st));
   } else {
@@ -953,6 +962,11 @@ static void compute_port_response(vtm_solver* s, int64_t s_tiles) {
       VTM_CUDA(launch_unit_rhs<T>(s->pieces.as<PieceDesc>(), np, s->port_local.as<int32_t>(), R, b, s->bt.as<T>(), st));
       reset_waves(s);
       sweeps_typed<T>(s, 1);
+      if (s->resident) {
+        VTM_CUDA(launch_gather_port_dense<T>(s->res_ps.as<ResPieceS>(), s->res_pieces, s->pieces_lo.as<PieceDesc>(),
+                                             s->port_local.as<int32_t>(), R, b, s->xc.as<T>(), s->S.as<T>(), st));
+        continue;
+      }
       if constexpr (sizeof(T) == 4) {
         if (s->port_tc) {
           VTM_CUDA(launch_gather_port_blocks(s->pieces_lo.as<PieceDesc>(), s->np_lo, s->port_local.as<int32_t>(), R, b,
@@ -1067,10 +1081,39 @@ static void launch_port(vtm_solver* s) {
   s->launches += 2;
 }
 
+// k port sweeps of a small system in one launch.
+template <typename T>
+static void launch_resident(vtm_solver* s, int k) {
+  ResArgs<T> a;
+  a.ctas = s->res_ctas.as<ResCta>();
+  a.units = s->res_units.as<ResUnit>();
+  a.ports = s->res_ports.as<ResPort>();
+  a.S = s->S.as<T>();
+  a.ubase = s->ubase.as<T>();
+  a.wprev = s->w[s->cur].as<T>();
+  a.wout = s->w[(s->cur + k) & 1].as<T>();
+  a.xch[0] = s->res_xch.as<unsigned long long>();
+  a.xch[1] = a.xch[0] + s->res_xch.bytes / 16;
+  a.twin = s->twin.as<int32_t>();
+  a.invz = s->invz_t.as<T>();
+  a.cpl = couple_ref<T>(s);
+  a.sweeps = k;
+  a.status = s->status.as<int>();
+  a.wait_limit = std::max(s->wait_limit, 65536L);  // a poll is one load here (about 1 us), not a suspended wait
+  VTM_CUDA(launch_port_resident<T>(a, s->R, s->res_grid, s->res_smem, s->res_xch.bytes, s->stream));
+  s->launches++;
+  s->cur = (s->cur + k) & 1;
+}
+
 // k sweeps in port form: k - 1 port-only sweeps, then one band sweep that also writes x_j.  The
 // flagged subgraphs (FP32 solvers) take their FP64 band sweep in every sweep.
 template <typename T>
 static void port_sweeps_typed(vtm_solver* s, int k) {
+  if (s->resident) {
+    if (k > 1) launch_resident<T>(s, k - 1);
+    if (k > 0) sweeps_typed<T>(s, 1);
+    return;
+  }
   for (int i = 0; i + 1 < k; ++i) {
     if (s->np_lo > 0) launch_port<T>(s);
     if constexpr (sizeof(T) == 4) {
@@ -1085,6 +1128,7 @@ static void port_sweeps_typed(vtm_solver* s, int k) {
 static int64_t launches_per_batch(const vtm_solver* s, int k) {
   const int64_t band = (s->np_lo > 0) + (s->np_hi > 0);
   if (!s->port_form || k < 2) return (int64_t)k * band;
+  if (s->resident) return 1 + band;
   const int64_t port = (s->np_lo > 0 ? (s->port_tc ? 1 : 2) : 0) + (s->np_hi > 0);
   return (int64_t)(k - 1) * port + band;
 }
@@ -1142,13 +1186,40 @@ static void choose_form(vtm_solver* s, const vtm_setup_opts* o, int64_t s_tiles,
   s->port_form = true;
   s->port_tc = tc;
   s->info.sweep_form = VTM_FORM_PORT;
+  int dev = 0, nsm = 1;
+  VTM_CUDA(cudaGetDevice(&dev));
+  VTM_CUDA(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
   // largest subgraphs first: the block scheduler starts CTAs in index order, so the smallest ones
   // fill the tail of the launch (all launches over pieces_lo write through global indices only)
   std::stable_sort(lo.begin(), lo.end(), [](const PieceDesc& x, const PieceDesc& y) { return x.nports > y.nports; });
   upload(s->pieces_lo, lo, s->stream);
-  int dev = 0, nsm = 1;
-  VTM_CUDA(cudaGetDevice(&dev));
-  VTM_CUDA(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
+  // Systems whose S_j all fit into the SMs' shared memory keep them there (port_resident.cu): up to
+  // about 30 MB in FP32.  Not with subgraphs that need their FP64 band sweep every sweep, nor where
+  // the caller asked for FP16 storage.
+  if (s->np_hi == 0 && o->port_storage != VTM_STORE_FP16) {
+    ResPlan rp = res_plan(lo.data(), (int)lo.size(), sizeof(T), s->R, nsm);
+    int per_sm = 0;
+    if (rp.ok) VTM_CUDA(port_resident_configure<T>(s->R, rp.smem, &per_sm));
+    if (per_sm > 0) {
+      s->resident = true;
+      s->port_tc = false;
+      std::vector<int32_t> ends(s->nports + 1);
+      VTM_CUDA(cudaMemcpyAsync(ends.data(), s->port_end_ptr.p, ends.size() * sizeof(int32_t), cudaMemcpyDeviceToHost,
+                               s->stream));
+      VTM_CUDA(cudaStreamSynchronize(s->stream));
+      res_plan_ends(rp, ends.data());
+      upload(s->res_ctas, rp.ctas, s->stream);
+      upload(s->res_units, rp.units, s->stream);
+      upload(s->res_ports, rp.ports, s->stream);
+      upload(s->res_ps, rp.piece_s, s->stream);
+      VTM_CUDA(cudaStreamSynchronize(s->stream));  // the uploads read rp
+      s->res_grid = (int)rp.ctas.size();
+      s->res_pieces = (int)rp.piece_s.size();
+      s->res_smem = rp.smem;
+      s->res_xch.alloc((size_t)2 * s->E * s->R * (sizeof(T) / 4) * sizeof(unsigned long long));
+      s->S.alloc((size_t)rp.s_elems * sizeof(T));
+    }
+  }
   auto divide = [&](bool half) {
     int per_sm = 1;
     vtm_solver::PortDev& d = s->port_div[half ? 1 : 0];
@@ -1164,7 +1235,8 @@ static void choose_form(vtm_solver* s, const vtm_setup_opts* o, int64_t s_tiles,
     VTM_CUDA(cudaStreamSynchronize(s->stream));  // the uploads read pl
     d.grid = (int)pl.cta_seg.size() - 1;
   };
-  if (tc) {
+  if (s->resident) {
+  } else if (tc) {
     s->tc_grid = std::min(s->np_lo, nsm);  // one persistent CTA per SM (it holds the SM's tensor memory)
     s->tc_n4max = n4max;
     s->tc_tmem_cols = tmem_cols;
@@ -1194,7 +1266,7 @@ static void choose_form(vtm_solver* s, const vtm_setup_opts* o, int64_t s_tiles,
     // FP16_AUTO only where the sweep streams S_j from HBM: responses that stay in the 126 MB L2
     // gain nothing from half the bytes and would pay the extra sweeps of FP16 rounding
     const bool l2_resident = s_bytes <= 96.0 * (1 << 20);
-    if (tc) {
+    if (tc && !s->resident) {
       // fp16 hi / lo blocks of S_j / sigma_j from the FP32 setup blocks, which are then released
       VTM_CUDA(cudaMemsetAsync(s->S16.p, 0, s->S16.bytes, s->stream));
       VTM_CUDA(launch_port_blocks_to_f16(s->pieces_lo.as<PieceDesc>(), s->np_lo, s->S.as<float>(),
@@ -1212,7 +1284,7 @@ static void choose_form(vtm_solver* s, const vtm_setup_opts* o, int64_t s_tiles,
         s->info.port_storage_bits = 16;
       }
     }
-    if (!tc && (o->port_storage == VTM_STORE_FP16 || (o->port_storage == VTM_STORE_FP16_AUTO && !l2_resident))) {
+    if (!tc && !s->resident && (o->port_storage == VTM_STORE_FP16 || (o->port_storage == VTM_STORE_FP16_AUTO && !l2_resident))) {
       s->Sh.alloc((size_t)s_tiles * kNB * kNB * sizeof(__half));
       s->hscale.alloc((size_t)std::max<int64_t>(1, s_tiles) * sizeof(float));  // one scale per tile
       divide(true);
@@ -1231,7 +1303,8 @@ static void choose_form(vtm_solver* s, const vtm_setup_opts* o, int64_t s_tiles,
   VTM_CUDA(cudaEventCreate(&e1));
   port_sweeps_typed<T>(s, 2);
   VTM_CUDA(cudaEventRecord(e0, s->stream));
-  for (int i = 0; i < 3; ++i) {
+  if (s->resident) launch_resident<T>(s, 3);
+  for (int i = 0; i < 3 && !s->resident; ++i) {
     if (s->np_lo > 0) launch_port<T>(s);
     s->cur ^= 1;
   }
