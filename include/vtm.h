@@ -224,10 +224,11 @@ typedef struct vtm_setup_opts {
                               reports VTM_ERR_TIMEOUT (0 = 4194304)                          */
   int32_t withhold_slab;   /* testing only: the sweep never issues the copy of this factor slab
                               of each subgraph, so that wait runs out (0 = off; k>0 = slab k-1) */
-  int32_t sweep_variant;   /* 0 or 1: single-block sweep (the autotuner picks the staging depth);
-                              2: pipelined sweep (nrhs <= 2; VTM_ERR_INVALID if no staging depth
-                              fits).  The pipelined schedule is never chosen automatically: it
-                              measured slower on every workload tried.
+  int32_t sweep_variant;   /* nrhs <= 8: 0: the pipelined sweep for FP32 solvers where it is the faster
+                              one (three factor slabs fit in shared memory, and nrhs > 1 or no more
+                              subgraphs than SMs), else the single-block sweep; 1: single-block
+                              sweep; 2: pipelined sweep (nrhs <= 2; VTM_ERR_INVALID if no staging
+                              depth fits).  The autotuner picks the staging depth.
                               3: FP32, nrhs 16 / 32: the multi-RHS band sweep on the SIMT cores
                               only (by default its products run on the tensor cores when every
                               half-bandwidth is at most 384)                                   */
@@ -299,8 +300,8 @@ typedef struct vtm_solver_info {
   double sweep_ms;             /* autotuner's device time of one sweep (all subgraphs)        */
   int32_t flagged_pieces;      /* FP32 solvers: subgraphs refactored and swept in FP64 because
                                   their FP32 pivots broke down or kept < 1e-5 of the diagonal  */
-  int32_t sweep_variant;       /* 0: one CTA works each block step in turn; 1: pipelined (warp 0
-                                  finishes block k while the others prepare block k+1)        */
+  int32_t sweep_variant;       /* 0: one CTA works each block step in turn; 1: pipelined (chain
+                                  warps finish block k while the others prepare block k+1)    */
   int32_t sweep_form;          /* VTM_FORM_BAND or VTM_FORM_PORT (after AUTO was resolved)    */
   int64_t port_bytes;          /* PORT: bytes of the port responses S_j one sweep streams     */
   double port_setup_ms;        /* PORT: device time of computing S_j (unit-source solves)     */

@@ -148,4 +148,43 @@ __device__ __forceinline__ T coupling_current(const CoupleRef<TV>& c, int port, 
   return acc;
 }
 
+// acc = sum of w_in[e] / Z_e over the ends of a port plus its coupling currents, R right-hand sides.
+// List entries and the waves they point to are loaded four at a time, so that a port waits for three
+// rounds of loads and not for one per entry.
+template <typename T, int R>
+__device__ __forceinline__ void port_inflow(const int32_t* port_end_ptr, const int32_t* twin, const T* invz,
+                                            const CoupleRef<T>& cpl, const T* w, int port, T (&acc)[R]) {
+  constexpr int kB = 4;
+  const int e0 = port_end_ptr[port], e1 = port_end_ptr[port + 1];
+  const int c0 = cpl.ptr ? cpl.ptr[port] : 0, c1 = cpl.ptr ? cpl.ptr[port + 1] : 0;
+  T cc[R];
+#pragma unroll
+  for (int r = 0; r < R; ++r) acc[r] = cc[r] = T(0);
+  auto list = [&](int lo, int hi, const int32_t* place, const T* coef, T(&sum)[R]) {
+    for (int k = lo; k < hi; k += kB) {
+      int at[kB];
+      T y[kB];
+#pragma unroll
+      for (int j = 0; j < kB; ++j) {
+        at[j] = k + j < hi ? place[k + j] : -1;
+        y[j] = k + j < hi ? coef[k + j] : T(0);
+      }
+      T v[kB][R];
+#pragma unroll
+      for (int j = 0; j < kB; ++j)
+#pragma unroll
+        for (int r = 0; r < R; ++r) v[j][r] = at[j] >= 0 ? w[(size_t)at[j] * R + r] : T(0);
+#pragma unroll
+      for (int j = 0; j < kB; ++j)
+        if (at[j] >= 0)
+#pragma unroll
+          for (int r = 0; r < R; ++r) sum[r] += v[j][r] * y[j];
+    }
+  };
+  list(e0, e1, twin, invz, acc);
+  list(c0, c1, cpl.oth, cpl.y, cc);
+#pragma unroll
+  for (int r = 0; r < R; ++r) acc[r] += cc[r];
+}
+
 }  // namespace vtm

@@ -51,14 +51,15 @@ cudaError_t sweep_occupancy(int R, size_t smem, int* ctas_per_sm);
 template <typename TF, typename TV>
 cudaError_t launch_sweep(const SweepArgs<TF, TV>& a, int R, int npieces, size_t smem, cudaStream_t st);
 
-// Pipelined variant (R = 1, 2): warp 0 finishes block k while warps 1-7 prepare block k+1.
-size_t sweep_pipe_smem_bytes(size_t elem, int R, int stages, int slot_elems, int ys_elems, int win_elems);
-template <typename TF, typename TV>
-cudaError_t sweep_pipe_configure(int R, size_t smem);
-template <typename TF, typename TV>
+// Pipelined variant: chain warps finish block k while the others prepare block k+1.
+constexpr size_t kPipeSmemMax = 226 * 1024;  // dynamic shared memory the kernel may take
+size_t sweep_pipe_smem_bytes(size_t elem, int R, int stages, int slot_elems, int ys_elems);
+template <typename T>
+cudaError_t sweep_pipe_configure(int R);
+template <typename T>
 cudaError_t sweep_pipe_occupancy(int R, size_t smem, int* ctas_per_sm);
-template <typename TF, typename TV>
-cudaError_t launch_sweep_pipe(const SweepArgs<TF, TV>& a, int R, int npieces, size_t smem, cudaStream_t st);
+template <typename T>
+cudaError_t launch_sweep_pipe(const SweepArgs<T, T>& a, int R, int npieces, size_t smem, cudaStream_t st);
 
 // Multi-RHS sweep with the band products on the tensor cores (R = 16, 32; FP32 solvers): the factor
 // of each subgraph, balanced and split into fp16 hi / lo panels of 128-row groups, built once from

@@ -117,7 +117,7 @@ struct vtm_solver {
   int64_t wt_bytes = 0;
   int wt_max_groups = 0;
   DevBuf wt;
-  bool pipe = false;                 // R <= 2: pipelined sweep kernel chosen by the autotuner
+  bool pipe = false;                 // R <= 8: pipelined sweep kernel
   struct Cand {
     int stages;
     bool pipe;
@@ -210,7 +210,7 @@ void reset_waves(vtm_solver* s);
 
 static size_t sweep_smem_for(const vtm_solver* s, size_t elem, int stages, bool pipe = false) {
   if (s->wide) return sweep_wide_smem_bytes(elem, s->R, stages, s->slot_elems, s->cap);
-  if (pipe) return sweep_pipe_smem_bytes(elem, s->R, stages, s->slot_elems, s->ys_elems, s->win_elems);
+  if (pipe) return sweep_pipe_smem_bytes(elem, s->R, stages, s->slot_elems, s->ys_elems);
   return sweep_smem_bytes(elem, s->R, stages, s->slot_elems, s->ys_elems, s->win_elems);
 }
 void line_features(const vtm_partition* p, float* out);
@@ -632,25 +632,34 @@ static void setup_typed(const vtm_partition* p, const vtm_setup_opts* o, vtm_sol
   s->cap = 64;
   while (s->cap < max_Wp - 1 + kNB) s->cap *= 2;
   // deeper rings for thin bands: a slab of a 2D subgraph is a few KB, and hiding DRAM latency takes
-  // several of them in flight (the mbarrier area holds up to kMaxStages)
-  size_t pipe_cap = 0;
+  // several of them in flight (the mbarrier area holds up to kMaxStages).  FP32 solvers
+  // take the pipelined sweep (see k_sweep_pipe) where it has room for three slabs (two in work, one in
+  // flight), with one right-hand side only up to one subgraph per SM: beyond that two single-block
+  // CTAs per SM hide each other's chains (128^3 in 512 subgraphs 0.95 ms, pipelined 1.01; 64^3 in 64:
+  // 0.38 and 0.25; 288 ragged subgraphs with 8 right-hand sides 1.22 and 0.50).  In FP64 the chain warp
+  // has one quarter of the SM's FP64 units (32^2: 38 us, pipelined 81).  Only the staging depth is
+  // tuned, never the variant: the variants add in different orders, and two identical solvers must
+  // agree bit for bit.
+  int dev = 0, nsm = 1;
+  VTM_CUDA(cudaGetDevice(&dev));
+  VTM_CUDA(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
+  const bool pipe_auto = o->sweep_variant == 0 && sizeof(T) == 4 && (R > 1 || np <= nsm);
+  std::vector<vtm_solver::Cand> single;
+  bool pipes = false;
   for (int st2 : {2, 3, 4, 6, 8, 12, kMaxStages}) {
     const size_t b = sweep_smem_for(s, sizeof(T), st2, false);
     if (b <= kSmemMax) {
       stage_cands.push_back(st2);
-      if (o->sweep_variant != 2) s->cands.push_back({st2, false});
+      single.push_back({st2, false});
       smem_cap = std::max(smem_cap, b);
     }
-    // the pipelined schedule measured slower than the single-block one on every workload tried, so
-    // the autotuner only considers it when it is asked for explicitly
-    if (!s->wide && R <= 2 && st2 >= 3 && o->sweep_variant == 2) {
-      const size_t bp = sweep_smem_for(s, sizeof(T), st2, true);
-      if (bp <= kSmemMax) {
-        s->cands.push_back({st2, true});
-        pipe_cap = std::max(pipe_cap, bp);
-      }
+    if (!s->wide && st2 >= 3 && (pipe_auto || (o->sweep_variant == 2 && R <= 2)) &&
+        sweep_smem_for(s, sizeof(T), st2, true) <= kPipeSmemMax) {
+      s->cands.push_back({st2, true});
+      pipes = true;
     }
   }
+  if (!pipes && o->sweep_variant != 2) s->cands = single;
   if (stage_cands.empty())
     fail(VTM_ERR_INVALID, "a subgraph is too large for the shared-memory sweep (n_j, bandwidth or nrhs too big)");
   if (s->cands.empty())
@@ -660,7 +669,7 @@ static void setup_typed(const vtm_partition* p, const vtm_setup_opts* o, vtm_sol
   s->sweep_smem = sweep_smem_for(s, sizeof(T), s->stages);
   if (s->wide) VTM_CUDA((sweep_wide_configure<T, T>(R, smem_cap)));
   else VTM_CUDA((sweep_configure<T, T>(R, smem_cap)));
-  if (pipe_cap > 0) VTM_CUDA((sweep_pipe_configure<T, T>(R, pipe_cap)));
+  if (pipes) VTM_CUDA(sweep_pipe_configure<T>(R));
 
   // ---- vertex -> copies (for assembly)
   std::vector<int64_t> vc_ptr(p->n + 1, 0), vc_copy(C);
@@ -812,8 +821,9 @@ static void launch_one(vtm_solver* s, const SweepArgs<TF, TV>& a, int np, size_t
     }
   }
   if (s->wide) VTM_CUDA((launch_sweep_wide<TF, TV>(a, s->R, np, smem, s->stream)));
-  else if (pipe) VTM_CUDA((launch_sweep_pipe<TF, TV>(a, s->R, np, smem, s->stream)));
-  else VTM_CUDA((launch_sweep<TF, TV>(a, s->R, np, smem, s->stream)));
+  else if (pipe) {
+    if constexpr (std::is_same_v<TF, TV>) VTM_CUDA(launch_sweep_pipe<TF>(a, s->R, np, smem, s->stream));
+  } else VTM_CUDA((launch_sweep<TF, TV>(a, s->R, np, smem, s->stream)));
   s->launches++;
 }
 
@@ -869,7 +879,7 @@ static void autotune_sweep(vtm_solver* s) {
   s->info.sweep_variant = best_pipe ? 1 : 0;
   int occ = 1;
   if (!s->wide && !s->pipe) VTM_CUDA((sweep_occupancy<T, T>(s->R, s->sweep_smem, &occ)));
-  if (s->pipe) VTM_CUDA((sweep_pipe_occupancy<T, T>(s->R, s->sweep_smem, &occ)));
+  if (s->pipe) VTM_CUDA(sweep_pipe_occupancy<T>(s->R, s->sweep_smem, &occ));
   s->info.sweep_stages = best_st;
   s->info.sweep_ctas_per_sm = occ;
   s->info.sweep_ms = best;

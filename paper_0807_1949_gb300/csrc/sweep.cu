@@ -230,32 +230,97 @@ __global__ void __launch_bounds__(kSweepThreads, 2) k_sweep(const SweepArgs<T, T
 }
 
 // ------------------------------------------------------------------------------------------------
-// Pipelined variant (R = 1, 2): per 32-row block step the chain warp (warp 0) finishes block k --
-// the 32 columns next to the block ("near"), the partial sum prepared one step earlier ("far"), the
-// inverted diagonal block -- while warps 1-7 compute the far part of block k+1 from the next slab.
-// Forward: near columns [k0-32, k0), far columns < k0-32; backward (rows of U): near columns
-// [k0+32, k0+64), far columns >= k0+64.  Both halves read disjoint rows of the vector, so one CTA
-// barrier per block step is enough.  Needs two slabs resident (stages >= 3 keeps one in flight).
-constexpr int kFarThreads = kSweepThreads - 32;
-constexpr int kFarPerRow = kFarThreads / kNB;  // 7 threads per row of the next block
+// Pipelined variant: per 32-row block step the chain warps finish block k -- the 32 columns next to
+// the block ("near"), the partial sums prepared one step earlier ("far"), the inverted diagonal
+// block -- while the far warps compute the far part of block k + 1.  Forward: near columns
+// [k0 - 32, k0), far columns < k0 - 32; backward (rows of U): near columns [k0 + 32, k0 + 64), far
+// columns >= k0 + 64.  Both halves read disjoint rows of the vector, and every chain warp keeps its
+// own right-hand sides, whose near values it wrote itself, so one CTA barrier per block step is
+// enough.  Needs two slabs resident (stages >= 3 keeps one in flight).
+//
+// A lane owns a row of the block and takes its columns in step with the other lanes: column d of row
+// r lies at r (Wp - 1) + d (plus a constant), an odd stride, so the 32 lanes hit 32 banks, and the
+// vector entry of a column is one broadcast load for all rows and R right-hand sides.  (With eight
+// lanes per row, k_sweep, every product needs its own vector load, and each block step three barriers
+// and two chains of shuffles.)
+//
+// What bounds it: HBM with many subgraphs; with few, the chain of block steps (near part, diagonal
+// block, one barrier: about 0.25 us at R = 1 against 0.9 - 1.2 us per step of k_sweep).
+constexpr int kChainWarps[9] = {0, 1, 1, 0, 2, 0, 0, 0, 4};
 
-template <typename T, typename TV, int R>
-__global__ void __launch_bounds__(kSweepThreads, 1) k_sweep_pipe(const SweepArgs<T, TV> a) {
+template <int R>
+struct Chain {
+  static constexpr int NC = kChainWarps[R];              // chain warps
+  static constexpr int RP = R / NC;                      // right-hand sides of each
+  static constexpr int NF = kSweepThreads / 32 - NC;     // far warps
+};
+
+template <typename T, int N>
+__device__ __forceinline__ void load_n(const T* p, T (&v)[N]) {
+  if constexpr (sizeof(T) == 4 && N % 4 == 0) {
+#pragma unroll
+    for (int i = 0; i < N; i += 4) {
+      const float4 x = *reinterpret_cast<const float4*>(p + i);
+      v[i] = x.x, v[i + 1] = x.y, v[i + 2] = x.z, v[i + 3] = x.w;
+    }
+  } else if constexpr (sizeof(T) == 4 && N == 2) {
+    const float2 x = *reinterpret_cast<const float2*>(p);
+    v[0] = x.x, v[1] = x.y;
+  } else if constexpr (sizeof(T) == 8 && N % 2 == 0) {
+#pragma unroll
+    for (int i = 0; i < N; i += 2) {
+      const double2 x = *reinterpret_cast<const double2*>(p + i);
+      v[i] = x.x, v[i + 1] = x.y;
+    }
+  } else {
+#pragma unroll
+    for (int i = 0; i < N; ++i) v[i] = p[i];
+  }
+}
+
+// acc[q] += sum over columns d0 <= d < d1 (d0, d1 multiples of 4) of l[d] v[d][q], where column d of
+// this lane's row counts if keep(d).  v: the entry of column 0, its RP values of the R per row; for
+// R = 1 the rows of four columns are one 16-byte load.
+template <typename T, int R, int RP, typename K>
+__device__ __forceinline__ void dot_columns(const T* l, const T* v, int d0, int d1, K keep, T (&acc)[4][RP]) {
+  for (int d = d0; d < d1; d += 4) {
+    T x[4][RP];
+    if constexpr (R == 1) {
+      T y[4];
+      load_n<T, 4>(v + d, y);
+#pragma unroll
+      for (int j = 0; j < 4; ++j) x[j][0] = y[j];
+    } else {
+#pragma unroll
+      for (int j = 0; j < 4; ++j) load_n<T, RP>(v + (d + j) * R, x[j]);
+    }
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      const T e = l[d + j];
+      const T f = keep(d + j) ? e : T(0);
+#pragma unroll
+      for (int q = 0; q < RP; ++q) acc[j][q] += f * x[j][q];
+    }
+  }
+}
+
+template <typename T, int R>
+__global__ void __launch_bounds__(kSweepThreads, 2) k_sweep_pipe(const SweepArgs<T, T> a) {
   extern __shared__ __align__(128) unsigned char smem[];
   __shared__ int abort_flag;
+  constexpr int NC = Chain<R>::NC, RP = Chain<R>::RP, NF = Chain<R>::NF;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const PieceDesc pd = a.pieces[blockIdx.x];
   const int S = a.stages;
   uint64_t* bars = reinterpret_cast<uint64_t*>(smem);
   T* ring = reinterpret_cast<T*>(smem + 128);
-  T* ys = ring + (size_t)S * a.slot_elems;
-  T* win = ys + a.ys_elems;
-  T* farp = win + a.win_elems;                        // [2][kFarPerRow][kNB][R]
-  T* tbuf = farp + 2 * kFarPerRow * kNB * R;          // [kNB][R]
-  constexpr int kFarBuf = kFarPerRow * kNB * R;
-
-  const int Wp = pd.Wp;
+  T* farp = ring + (size_t)S * a.slot_elems;          // [2][NF][kNB][R]
+  T* tbuf = farp + 2 * NF * kNB * R;                  // [NC][kNB][RP]
+  const int Wp = pd.Wp, w = pd.w;
   const int off = Wp - 1;
+  T* ys = tbuf + kNB * R;                             // Wp zero rows, n_pad rows, Wp + 4 zero rows
+  constexpr int kFarBuf = NF * kNB * R;
+
   const int nblk = pd.n_pad / kNB;
   const int total = 2 * nblk;
   const uint32_t slab_bytes = (uint32_t)(kNB * Wp * sizeof(T));
@@ -281,166 +346,114 @@ __global__ void __launch_bounds__(kSweepThreads, 1) k_sweep_pipe(const SweepArgs
     for (int s = 0; s < S && s < total; ++s) issue(s);
 
   // ---- prologue: r_j = b̃_j + sum_e w_in[e] / Z_e at the port rows; far part of block 0 is zero
-  for (int i = tid; i < off * R; i += kSweepThreads) {
-    ys[i] = T(0);
-    ys[(size_t)(off + pd.n_pad) * R + i] = T(0);
+  for (int i = tid; i < (Wp + 4) * R; i += kSweepThreads) {
+    if (i < Wp * R) ys[i] = T(0);
+    ys[(size_t)(Wp + pd.n_pad) * R + i] = T(0);  // the last far columns are rounded up to fours
   }
   for (int i = tid; i < kFarBuf; i += kSweepThreads) farp[i] = T(0);
-  const TV* btp = a.bt + (size_t)pd.copy_off * R;
-  for (int i = tid; i < pd.n_pad * R; i += kSweepThreads) ys[(size_t)off * R + i] = (i < pd.n * R) ? (T)btp[i] : T(0);
+  const T* btp = a.bt + (size_t)pd.copy_off * R;
+#pragma unroll 8
+  for (int i = tid; i < pd.n_pad * R; i += kSweepThreads) ys[(size_t)Wp * R + i] = (i < pd.n * R) ? btp[i] : T(0);
   __syncthreads();
   for (int q = tid; q < pd.nports; q += kSweepThreads) {
     const int l = a.port_local[pd.port_off + q];
-    const int e0 = a.port_end_ptr[pd.port_off + q], e1 = a.port_end_ptr[pd.port_off + q + 1];
     T acc[R];
+    port_inflow<T, R>(a.port_end_ptr, a.twin, a.invz, a.cpl, a.wprev, pd.port_off + q, acc);
 #pragma unroll
-    for (int rr = 0; rr < R; ++rr) acc[rr] = T(0);
-    for (int e = e0; e < e1; ++e) {
-      const int tw = a.twin[e];
-      const T iz = (T)a.invz[e];
-#pragma unroll
-      for (int rr = 0; rr < R; ++rr) {
-        const T w = (T)a.wprev[(size_t)tw * R + rr];
-        win[(e - pd.end_off) * R + rr] = w;
-        acc[rr] += w * iz;
-      }
-    }
-    if (a.cpl.ptr)
-#pragma unroll
-      for (int rr = 0; rr < R; ++rr) acc[rr] += coupling_current<T, TV>(a.cpl, pd.port_off + q, rr, R, a.wprev);
-#pragma unroll
-    for (int rr = 0; rr < R; ++rr) ys[(size_t)(off + l) * R + rr] += acc[rr];
+    for (int rr = 0; rr < R; ++rr) ys[(size_t)(Wp + l) * R + rr] += acc[rr];
   }
   __syncthreads();
 
-  int s = 0;
+  const int r = lane;
+  const int nfar = w > kNB ? (w - kNB + 3) / 4 * 4 : 0;  // far columns, in fours
+  const bool whole = off >= 2 * kNB - 1;  // the near columns lie inside every row's storage
+  int s = 0, slot = 0;                    // slot, phase of item s
+  uint32_t phase = 0;
   for (; s < total; ++s) {
     const int par = s & 1;
-    if (warp == 0) {
-      // ---- chain: finish item s (block k0), one row per lane
-      if (!mbar_wait_bounded(&bars[s % S], (uint32_t)((s / S) & 1), a.wait_limit)) abort_flag = 1;
-      const T* L = ring + (size_t)(s % S) * a.slot_elems;
+    const int slot1 = slot + 1 == S ? 0 : slot + 1;  // of item s + 1
+    const uint32_t phase1 = slot + 1 == S ? phase ^ 1u : phase;
+    if (warp < NC) {
+      // ---- chain: finish item s (block k0) for this warp's right-hand sides
+      if (!mbar_wait_bounded(&bars[slot], phase, a.wait_limit)) abort_flag = 1;
+      const T* L = ring + (size_t)slot * a.slot_elems;
       const bool fwd = s < nblk;
       const int k0 = (fwd ? s : total - 1 - s) * kNB;
-      const int r = lane;
-      const T* Lr = L + r * Wp;
-      T near[R];
+      const int q0 = warp * RP;
+      T* yk = ys + (size_t)(Wp + k0) * R + q0;  // the block's rows
+      const T* Lr = L + r * off + (fwd ? off : 0);  // entry of column d at Lr[d]
+      T acc[4][RP];
 #pragma unroll
-      for (int rr = 0; rr < R; ++rr) near[rr] = T(0);
-      if (fwd) {
-        const int pbeg = max(0, off - r - kNB), pend = off - r;
-        const T* yb = ys + (size_t)(k0 + r) * R;
-        for (int p = pbeg; p < pend; ++p) {
-          const T l = Lr[p];
+      for (int j = 0; j < 4; ++j)
 #pragma unroll
-          for (int rr = 0; rr < R; ++rr) near[rr] += l * yb[(size_t)p * R + rr];
-        }
-      } else {
-        const int pbeg = kNB - r, pend = min(Wp, 2 * kNB - r);
-        const T* xb = ys + (size_t)(k0 + r + off) * R;
-        for (int p = pbeg; p < pend; ++p) {
-          const T u = Lr[p];
+        for (int q = 0; q < RP; ++q) acc[j][q] = T(0);
+      const T* fp = farp + par * kFarBuf + r * R + q0;
 #pragma unroll
-          for (int rr = 0; rr < R; ++rr) near[rr] += u * xb[(size_t)p * R + rr];
-        }
+      for (int h = 0; h < NF; ++h) {
+        T f[RP];
+        load_n<T, RP>(fp + h * kNB * R, f);
+#pragma unroll
+        for (int q = 0; q < RP; ++q) acc[h & 3][q] += f[q];
       }
-      const T* fp = farp + par * kFarBuf;
+      if (whole) {
+        const int d0 = fwd ? -kNB : kNB;
+        dot_columns<T, R, RP>(Lr + d0, yk + d0 * R, 0, kNB, [](int) { return true; }, acc);
+      } else if (fwd) {
+        dot_columns<T, R, RP>(Lr, yk, -kNB, 0, [&](int d) { return d + off >= r; }, acc);
+      } else {
+        dot_columns<T, R, RP>(Lr, yk, kNB, 2 * kNB, [&](int d) { return d - r <= off; }, acc);
+      }
+      T* tb = tbuf + warp * kNB * RP;
+      {
+        T y0[RP];
+        load_n<T, RP>(yk + r * R, y0);
 #pragma unroll
-      for (int rr = 0; rr < R; ++rr) {
-        T far = T(0);
-#pragma unroll
-        for (int h = 0; h < kFarPerRow; ++h) far += fp[(h * kNB + r) * R + rr];
-        tbuf[r * R + rr] = ys[(size_t)(k0 + r + off) * R + rr] - far - near[rr];
+        for (int q = 0; q < RP; ++q) tb[r * RP + q] = y0[q] - ((acc[0][q] + acc[1][q]) + (acc[2][q] + acc[3][q]));
       }
       __syncwarp();
-      T y[R];
 #pragma unroll
-      for (int rr = 0; rr < R; ++rr) y[rr] = T(0);
-      if (fwd) {
-        const T* Li = Lr + off - r;  // inv(L_KK)[r][c] at Li[c], c <= r
-        for (int c = 0; c <= r; ++c) {
-          const T l = Li[c];
+      for (int j = 0; j < 4; ++j)
 #pragma unroll
-          for (int rr = 0; rr < R; ++rr) y[rr] += l * tbuf[c * R + rr];
-        }
-      } else {
-        const T* Ui = Lr - r;        // inv(U_KK)[r][c] at Ui[c], c >= r
-        for (int c = r; c < kNB; ++c) {
-          const T u = Ui[c];
+        for (int q = 0; q < RP; ++q) acc[j][q] = T(0);
+      // inv(L_KK)[r][c], c <= r (backward: inv(U_KK)[r][c], c >= r)
+      if (fwd) dot_columns<T, RP, RP>(Lr, tb, 0, kNB, [&](int c) { return c <= r; }, acc);
+      else dot_columns<T, RP, RP>(Lr, tb, 0, kNB, [&](int c) { return c >= r; }, acc);
 #pragma unroll
-          for (int rr = 0; rr < R; ++rr) y[rr] += u * tbuf[c * R + rr];
-        }
-      }
-#pragma unroll
-      for (int rr = 0; rr < R; ++rr) ys[(size_t)(k0 + r + off) * R + rr] = y[rr];
+      for (int q = 0; q < RP; ++q) yk[r * R + q] = (acc[0][q] + acc[1][q]) + (acc[2][q] + acc[3][q]);
     } else if (s + 1 < total) {
-      // ---- far part of item s+1 from its slab (values complete at the start of step s)
-      const int s1 = s + 1;
-      if (!mbar_wait_bounded(&bars[s1 % S], (uint32_t)((s1 / S) & 1), a.wait_limit)) abort_flag = 1;
-      const T* L1 = ring + (size_t)(s1 % S) * a.slot_elems;
+      // ---- far part of item s + 1 from its slab (values complete at the start of step s)
+      const int s1 = s + 1, f = warp - NC;
+      if (!mbar_wait_bounded(&bars[slot1], phase1, a.wait_limit)) abort_flag = 1;
+      const T* L1 = ring + (size_t)slot1 * a.slot_elems;
       const bool fwd1 = s1 < nblk;
       const int k1 = (fwd1 ? s1 : total - 1 - s1) * kNB;
-      const int t2 = tid - 32;
-      const int r = t2 / kFarPerRow, h = t2 % kFarPerRow;
-      const T* Lr = L1 + r * Wp;
-      T acc[R];
+      const T* yk = ys + (size_t)(Wp + k1) * R;
+      const T* Lr = L1 + r * off + (fwd1 ? off : 0);
+      T acc[4][R];
 #pragma unroll
-      for (int rr = 0; rr < R; ++rr) acc[rr] = T(0);
-      if constexpr (sizeof(T) == 4 && R == 1) {
-        float a0 = 0.f, a1 = 0.f, a2 = 0.f, a3 = 0.f;
-        const float4* L4 = reinterpret_cast<const float4*>(Lr);
-        if (fwd1) {
-          const int pend = off - r - kNB;  // far positions [0, pend)
-          const float* yb = reinterpret_cast<const float*>(ys) + (k1 + r);
-          for (int q = h; 4 * q < pend; q += kFarPerRow) {
-            const float4 l = L4[q];
-            const int p = 4 * q;
-            a0 = fmaf(l.x, yb[p], a0);
-            if (p + 1 < pend) a1 = fmaf(l.y, yb[p + 1], a1);
-            if (p + 2 < pend) a2 = fmaf(l.z, yb[p + 2], a2);
-            if (p + 3 < pend) a3 = fmaf(l.w, yb[p + 3], a3);
-          }
-        } else {
-          const int pbeg = 2 * kNB - r;    // far positions [pbeg, Wp)
-          const float* xb = reinterpret_cast<const float*>(ys) + (k1 + r + off);
-          for (int q = (pbeg >> 2) + h; q < (Wp >> 2); q += kFarPerRow) {
-            const float4 u = L4[q];
-            const int p = 4 * q;
-            if (p >= pbeg) a0 = fmaf(u.x, xb[p], a0);
-            if (p + 1 >= pbeg) a1 = fmaf(u.y, xb[p + 1], a1);
-            if (p + 2 >= pbeg) a2 = fmaf(u.z, xb[p + 2], a2);
-            a3 = fmaf(u.w, xb[p + 3], a3);
-          }
-        }
-        acc[0] = (a0 + a1) + (a2 + a3);
+      for (int j = 0; j < 4; ++j)
+#pragma unroll
+        for (int q = 0; q < R; ++q) acc[j][q] = T(0);
+      // columns in fours, an equal run of them per warp; forward -32 - 4 .. -32 - nfar
+      const int c0 = nfar / 4 * f / NF * 4, c1 = nfar / 4 * (f + 1) / NF * 4;
+      if (fwd1) {
+        dot_columns<T, R, R>(Lr, yk, -kNB - c1, -kNB - c0, [&](int d) { return d + off >= r; }, acc);
       } else {
-        if (fwd1) {
-          const int pend = off - r - kNB;
-          const T* yb = ys + (size_t)(k1 + r) * R;
-          for (int p = h; p < pend; p += kFarPerRow) {
-            const T l = Lr[p];
-#pragma unroll
-            for (int rr = 0; rr < R; ++rr) acc[rr] += l * yb[(size_t)p * R + rr];
-          }
-        } else {
-          const T* xb = ys + (size_t)(k1 + r + off) * R;
-          for (int p = 2 * kNB - r + h; p < Wp; p += kFarPerRow) {
-            const T u = Lr[p];
-#pragma unroll
-            for (int rr = 0; rr < R; ++rr) acc[rr] += u * xb[(size_t)p * R + rr];
-          }
-        }
+        dot_columns<T, R, R>(Lr, yk, 2 * kNB + c0, 2 * kNB + c1, [&](int d) { return d - r <= off; }, acc);
       }
-      T* fp = farp + (par ^ 1) * kFarBuf;
+      T* fp = farp + (par ^ 1) * kFarBuf + (f * kNB + r) * R;
 #pragma unroll
-      for (int rr = 0; rr < R; ++rr) fp[(h * kNB + r) * R + rr] = acc[rr];
+      for (int q = 0; q < R; ++q) fp[q] = (acc[0][q] + acc[1][q]) + (acc[2][q] + acc[3][q]);
     }
     __syncthreads();
     if (abort_flag) break;
-    if (tid == 0 && s + S < total) {
+    // the last warp issues: the chain warp goes on at once
+    if (tid == kSweepThreads - 1 && s + S < total) {
       fence_proxy_async_smem();
       issue(s + S);
     }
+    slot = slot1;
+    phase = phase1;
   }
   if (abort_flag) {
     if (tid == 0) {
@@ -451,53 +464,62 @@ __global__ void __launch_bounds__(kSweepThreads, 1) k_sweep_pipe(const SweepArgs
     return;
   }
 
-  // ---- epilogue: w_out[e] = 2 x_c - w_in[e]; local solution
+  // ---- epilogue: w_out[e] = 2 x_c - w_in[e]; local solution.  The incoming waves are read again (the
+  // shared memory they would take holds another slab).
+#pragma unroll 4
   for (int q = tid; q < pd.nports; q += kSweepThreads) {
     const int l = a.port_local[pd.port_off + q];
     const int e0 = a.port_end_ptr[pd.port_off + q], e1 = a.port_end_ptr[pd.port_off + q + 1];
-    for (int e = e0; e < e1; ++e)
+    for (int e = e0; e < e1; ++e) {
+      const T* wi = a.wprev + (size_t)a.twin[e] * R;
 #pragma unroll
-      for (int rr = 0; rr < R; ++rr)
-        a.wnext[(size_t)e * R + rr] = (TV)(T(2) * ys[(size_t)(off + l) * R + rr] - win[(e - pd.end_off) * R + rr]);
+      for (int rr = 0; rr < R; ++rr) a.wnext[(size_t)e * R + rr] = T(2) * ys[(size_t)(Wp + l) * R + rr] - wi[rr];
+    }
   }
   if (a.write_x) {
-    TV* xp = a.xc + (size_t)pd.copy_off * R;
-    for (int i = tid; i < pd.n * R; i += kSweepThreads) xp[i] = (TV)ys[(size_t)off * R + i];
+    T* xp = a.xc + (size_t)pd.copy_off * R;
+#pragma unroll 8
+    for (int i = tid; i < pd.n * R; i += kSweepThreads) xp[i] = ys[(size_t)Wp * R + i];
   }
 }
 
-size_t sweep_pipe_smem_bytes(size_t elem, int R, int stages, int slot_elems, int ys_elems, int win_elems) {
-  return 128 + elem * ((size_t)stages * slot_elems + ys_elems + win_elems + (size_t)(2 * kFarPerRow + 1) * kNB * R);
+size_t sweep_pipe_smem_bytes(size_t elem, int R, int stages, int slot_elems, int ys_elems) {
+  // ys: one row more before and five after than the single-block sweep's
+  return 128 + elem * ((size_t)stages * slot_elems + ys_elems + 6 * R +
+                       (size_t)(2 * (kSweepThreads / 32 - kChainWarps[R]) + 1) * kNB * R);
 }
 
-template <typename TF, typename TV>
-cudaError_t sweep_pipe_configure(int R, size_t smem) {
+template <typename T>
+static const void* pipe_kernel(int R) {
   switch (R) {
-    case 1: return cudaFuncSetAttribute(k_sweep_pipe<TF, TV, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    case 2: return cudaFuncSetAttribute(k_sweep_pipe<TF, TV, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    default: return cudaErrorInvalidValue;
+    case 1: return (const void*)k_sweep_pipe<T, 1>;
+    case 2: return (const void*)k_sweep_pipe<T, 2>;
+    case 4: return (const void*)k_sweep_pipe<T, 4>;
+    case 8: return (const void*)k_sweep_pipe<T, 8>;
+    default: return nullptr;
   }
 }
 
-template <typename TF, typename TV>
+template <typename T>
+cudaError_t sweep_pipe_configure(int R) {
+  const void* k = pipe_kernel<T>(R);
+  return k ? cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kPipeSmemMax) : cudaErrorInvalidValue;
+}
+
+template <typename T>
 cudaError_t sweep_pipe_occupancy(int R, size_t smem, int* n) {
-  switch (R) {
-    case 1: return cudaOccupancyMaxActiveBlocksPerMultiprocessor(n, k_sweep_pipe<TF, TV, 1>, kSweepThreads, smem);
-    case 2: return cudaOccupancyMaxActiveBlocksPerMultiprocessor(n, k_sweep_pipe<TF, TV, 2>, kSweepThreads, smem);
-    default: return cudaErrorInvalidValue;
-  }
+  const void* k = pipe_kernel<T>(R);
+  return k ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(n, k, kSweepThreads, smem) : cudaErrorInvalidValue;
 }
 
-template <typename TF, typename TV>
-cudaError_t launch_sweep_pipe(const SweepArgs<TF, TV>& a, int R, int npieces, size_t smem, cudaStream_t st) {
+template <typename T>
+cudaError_t launch_sweep_pipe(const SweepArgs<T, T>& a, int R, int npieces, size_t smem, cudaStream_t st) {
   if (npieces <= 0) return cudaSuccess;
-  dim3 grid(npieces), block(kSweepThreads);
-  switch (R) {
-    case 1: k_sweep_pipe<TF, TV, 1><<<grid, block, smem, st>>>(a); break;
-    case 2: k_sweep_pipe<TF, TV, 2><<<grid, block, smem, st>>>(a); break;
-    default: return cudaErrorInvalidValue;
-  }
-  return cudaGetLastError();
+  const void* k = pipe_kernel<T>(R);
+  if (!k) return cudaErrorInvalidValue;
+  SweepArgs<T, T> args = a;
+  void* av[] = {&args};
+  return cudaLaunchKernel(k, dim3(npieces), dim3(kSweepThreads), av, smem, st);
 }
 
 size_t sweep_smem_bytes(size_t elem, int R, int stages, int slot_elems, int ys_elems, int win_elems) {
@@ -558,12 +580,11 @@ VTM_SWEEP_INST(float, float)
 VTM_SWEEP_INST(double, double)
 VTM_SWEEP_INST(double, float)
 
-#define VTM_PIPE_INST(TF, TV)                                                                      \
-  template cudaError_t sweep_pipe_configure<TF, TV>(int, size_t);                                    \
-  template cudaError_t sweep_pipe_occupancy<TF, TV>(int, size_t, int*);                               \
-  template cudaError_t launch_sweep_pipe<TF, TV>(const SweepArgs<TF, TV>&, int, int, size_t, cudaStream_t);
-VTM_PIPE_INST(float, float)
-VTM_PIPE_INST(double, double)
-VTM_PIPE_INST(double, float)
+#define VTM_PIPE_INST(T)                                  \
+  template cudaError_t sweep_pipe_configure<T>(int);      \
+  template cudaError_t sweep_pipe_occupancy<T>(int, size_t, int*); \
+  template cudaError_t launch_sweep_pipe<T>(const SweepArgs<T, T>&, int, int, size_t, cudaStream_t);
+VTM_PIPE_INST(float)
+VTM_PIPE_INST(double)
 
 }  // namespace vtm

@@ -325,10 +325,11 @@ class Solver:
     z: scalar (uniform), per-line array (order of Partition.lines()), "matched" (§7.1 rule,
        starting from z_init on every line), or an ``MLP`` (learned impedances).
     precision: "fp64" or "fp32".  nrhs: 1, 2, 4, 8, 16 or 32.
-    sweep_variant: "auto" or "single" (one CTA works each block step in turn; the setup-time
-    autotuner picks the staging depth) or "pipelined" (warp 0 finishes block k while the other
-    warps prepare block k+1; nrhs <= 2; opt-in only, it measured slower everywhere) or "simt"
-    (FP32, nrhs 16 / 32: the multi-RHS band sweep without its tensor-core products).
+    sweep_variant (band sweep): "auto" (nrhs <= 8: pipelined for FP32 solvers where it is the faster
+    one, else single) or "single" (one CTA works each block step in turn) or "pipelined" (chain
+    warps finish block k while the other warps prepare block k+1; nrhs <= 2) or "simt" (FP32, nrhs
+    16 / 32: the multi-RHS band sweep without its tensor-core products).  The setup-time autotuner
+    picks the staging depth.
     coupling: coupled lines of §7.2.  None (uncoupled), a number gamma (every candidate pair of
     Partition.line_pairs() gets the conductance gamma |a_ik|), or (pairs (m, 2), y (m,)).
     Right-hand sides / solutions: (nrhs, n) float64 arrays or tensors, host or device.

@@ -55,3 +55,24 @@ def test_divided_sweep(vtmlib, dims, block, nrhs, kind):
                                                ((97, 83), (5, 6), 5)])
 def test_resident_sweep(vtmlib, dims, block, sweeps, nrhs, kind):
     _check(vtmlib, dims, block, nrhs, kind, "native", sweeps, TOL[kind])
+
+
+# the pipelined band sweep with several chain warps: half-bandwidths below 32, around 64 and above,
+# last blocks cut short, one block only, one subgraph without lines
+@pytest.mark.parametrize("nrhs", [1, 2, 4, 8])
+@pytest.mark.parametrize("dims,block", [((21, 19, 18), (8, 8, 8)), ((23, 17), (6, 5)), ((70, 9), (70, 9)),
+                                        ((64, 31), (63, 31)), ((67, 40), (33, 20))])
+def test_pipelined_band_sweep(vtmlib, dims, block, nrhs):
+    A = inputs.grid_poisson(dims, sigma=0.7, seed=8)
+    b = inputs.rhs_uniform(A.n, nrhs, seed=8)
+    part = vtmlib.partition_evs(A, "grid", dims=dims, block=block)
+    osplit = evs.split_grid(A, dims, block)
+    s = vtmlib.Solver(part, z=0.9, precision="fp32", nrhs=nrhs, form="band")
+    assert s.info().sweep_variant == 1
+    s.set_rhs(b)
+    s.reset()
+    s.iterate(4)
+    copies, waves = _oracle_after(osplit, b, 0.9, 4)
+    assert _rel(s.copies(), copies) <= TOL_FP32
+    if len(osplit.vtl):
+        assert _rel(s.get_state(), waves[:, _line_map(part, osplit)]) <= TOL_FP32
