@@ -294,14 +294,13 @@ cudaError_t launch_split(int64_t ncopies, int R, const int64_t* copy_vertex, con
 template <typename T>
 cudaError_t launch_assemble(int64_t n, int R, const int64_t* vc_ptr, const int64_t* vc_copy, const T* xc,
                             const double* xbase, double* xt, int64_t ld, cudaStream_t st);
-// res = b - A x (res may be NULL); norms[r] += ||res_r||^2.
-cudaError_t launch_residual(int64_t n, int R, const int64_t* rowptr, const int32_t* col, const double* val,
-                            const double* b, int64_t ldb, const double* x, int64_t ldx, double* res, int64_t ldr,
-                            double* norms, cudaStream_t st);
-// norms[r] += ||v_r||^2
-cudaError_t launch_sqnorm(int64_t n, int R, const double* v, int64_t ld, double* norms, cudaStream_t st);
-// The same two with fixed-order sums (identical inputs give identical norms): norms[r] = ||res_r||^2
-// (resp. ||v_r||^2), through the scratch part of norm_parts(n) * R doubles.
+// sums_r[q] += ||b_q - A x_q||^2, sums_b[q] += ||b_q||^2 (R <= 8).
+cudaError_t launch_residual_norms(int64_t n, int R, const int64_t* rowptr, const int32_t* col, const double* val,
+                                  const double* b, int64_t ldb, const double* x, int64_t ldx, double* sums_r,
+                                  double* sums_b, cudaStream_t st);
+// res = b - A x (res may be NULL) and squared norms with fixed-order sums (identical inputs give
+// identical norms): norms[r] = ||res_r||^2 (resp. ||v_r||^2), through the scratch part of
+// norm_parts(n) * R doubles.
 int64_t norm_parts(int64_t n);
 cudaError_t launch_residual_det(int64_t n, int R, const int64_t* rowptr, const int32_t* col, const double* val,
                                 const double* b, int64_t ldb, const double* x, int64_t ldx, double* res, int64_t ldr,

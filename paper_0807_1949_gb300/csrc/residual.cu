@@ -1,6 +1,7 @@
 // Vector kernels around the sweeps: source splitting (§4 step 3), assembly of the solution from the
 // copies (mean of the copies; at the fixed point all copies agree, Thm 4.1), and the FP64 residual
 // b - A x with per-right-hand-side squared norms (the convergence test of Table 1 step 6).
+#include <algorithm>
 #include <type_traits>
 
 #include "kernels.h"
@@ -18,24 +19,55 @@ __device__ __forceinline__ double warp_sum(double v) {
   return v;
 }
 
-// Block-wide sum of R values per thread, accumulated into norms[r] with one atomic per block.
-__device__ void block_accumulate(const double* v, int R, double* norms) {
-  __shared__ double red[kBS / 32][kMaxR];
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+// Warp sums of N values per lane (N a power of two up to 32): each step halves the values a lane
+// keeps, N - 1 additions instead of 5 N.  Lane l ends with the sum of value (l >> (5 - log2 N)), the
+// remaining lane bits summed too.
+template <int N>
+__device__ __forceinline__ double warp_scatter_sum(double (&v)[N]) {
+  int o = 16;
 #pragma unroll
-  for (int r = 0; r < kMaxR; ++r) {
-    if (r >= R) break;
-    const double s = warp_sum(v[r]);
-    if (lane == 0) red[warp][r] = s;
+  for (int h = N / 2; h >= 1; h >>= 1) {
+    const bool upper = (threadIdx.x & o) != 0;
+#pragma unroll
+    for (int i = 0; i < h; ++i) {
+      const double send = upper ? v[i] : v[i + h], keep = upper ? v[i + h] : v[i];
+      v[i] = keep + __shfl_xor_sync(0xffffffffu, send, o);
+    }
+    o >>= 1;
   }
-  __syncthreads();
-  if (warp == 0) {
+  double t = v[0];
 #pragma unroll
-    for (int r = 0; r < kMaxR; ++r) {
-      if (r >= R) break;
-      double s = lane < kBS / 32 ? red[lane][r] : 0.0;
-      s = warp_sum(s);
-      if (lane == 0) atomicAdd(&norms[r], s);
+  for (int k = N; k < 32; k <<= 1) {
+    t += __shfl_xor_sync(0xffffffffu, t, o);
+    o >>= 1;
+  }
+  return t;
+}
+
+// ax[q] += (row i of A) x[q] for RG right-hand sides, the row's entries in order (b - A x of a nearly
+// converged x is all rounding: the product is summed before it meets b, as a host check does).  The
+// entries are loaded eight at a time before the products, so that the loads of x for all of them are
+// in flight together.
+template <int RG>
+__device__ __forceinline__ void row_product(int64_t i, const int64_t* __restrict__ rowptr, const int32_t* __restrict__ col,
+                                             const double* __restrict__ val, const double* __restrict__ x, int64_t ldx,
+                                             double (&ax)[RG]) {
+  const int64_t lo = rowptr[i], hi = rowptr[i + 1];
+  for (int64_t k0 = lo; k0 < hi; k0 += 8) {
+    int c[8];
+    double v[8];
+#pragma unroll
+    for (int u = 0; u < 8; ++u) {
+      c[u] = k0 + u < hi ? col[k0 + u] : 0;
+      v[u] = k0 + u < hi ? val[k0 + u] : 0.0;
+    }
+#pragma unroll
+    for (int u = 0; u < 8; ++u) {
+      if (k0 + u < hi) {
+        const double* xk = x + c[u];
+#pragma unroll
+        for (int rr = 0; rr < RG; ++rr) ax[rr] += v[u] * xk[(int64_t)rr * ldx];
+      }
     }
   }
 }
@@ -109,43 +141,58 @@ __global__ void k_assemble(int64_t n, int R, const int64_t* __restrict__ vc_ptr,
   }
 }
 
-template <int RG>
-__global__ void k_residual(int64_t n, int R, const int64_t* __restrict__ rowptr, const int32_t* __restrict__ col,
-                           const double* __restrict__ val, const double* __restrict__ b, int64_t ldb,
-                           const double* __restrict__ x, int64_t ldx, double* __restrict__ res, int64_t ldr,
-                           double* norms) {
-  const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  const int r0 = blockIdx.y * RG;
-  double sq[kMaxR];
+// sums_r[q] += ||b_q - A x_q||^2 and sums_b[q] += ||b_q||^2 in one pass, `rows` rows per thread, two
+// atomics per block and right-hand side.  FP64 arithmetic bounds it (2 FMA per SM and cycle): 7 + 3
+// per row and right-hand side of a 7-point matrix, the warp sums add 2 in 8 rows.  128^3, 8 right-hand
+// sides: 734 us with b's norms in a pass of their own, one row per thread and butterfly sums (40
+// additions per row), 306 us so; the arithmetic alone takes 275.
+template <int RG, int NP>
+__global__ void __launch_bounds__(kBS) k_residual_norms(int64_t n, int rows, const int64_t* __restrict__ rowptr,
+                                                       const int32_t* __restrict__ col, const double* __restrict__ val,
+                                                       const double* __restrict__ b, int64_t ldb,
+                                                       const double* __restrict__ x, int64_t ldx,
+                                                       double* __restrict__ sums_r, double* __restrict__ sums_b) {
+  double sq[2 * NP];  // residuals, then b; NP: RG rounded up to a power of two
 #pragma unroll
-  for (int r = 0; r < kMaxR; ++r) sq[r] = 0.0;
-  if (i < n) {
-    const int64_t lo = rowptr[i], hi = rowptr[i + 1];
-    double ax[RG];
+  for (int q = 0; q < 2 * NP; ++q) sq[q] = 0.0;
+  for (int j = 0; j < rows; ++j) {
+    const int64_t i = (blockIdx.x * (int64_t)rows + j) * kBS + threadIdx.x;
+    if (i < n) {
+      double ax[RG], bi[RG];
 #pragma unroll
-    for (int rr = 0; rr < RG; ++rr) ax[rr] = 0.0;
-    for (int64_t k = lo; k < hi; ++k) {
-      const double v = val[k];
-      const double* xk = x + col[k];
+      for (int q = 0; q < RG; ++q) {
+        bi[q] = b[i + (int64_t)q * ldb];
+        ax[q] = 0.0;
+      }
+      row_product<RG>(i, rowptr, col, val, x, ldx, ax);
 #pragma unroll
-      for (int rr = 0; rr < RG; ++rr) ax[rr] += v * xk[(int64_t)(r0 + rr) * ldx];
-    }
-#pragma unroll
-    for (int rr = 0; rr < RG; ++rr) {
-      const double ri = b[i + (int64_t)(r0 + rr) * ldb] - ax[rr];
-      if (res) res[i + (int64_t)(r0 + rr) * ldr] = ri;
-      sq[rr] = ri * ri;
+      for (int q = 0; q < RG; ++q) {
+        const double r = bi[q] - ax[q];
+        sq[q] = fma(r, r, sq[q]);
+        sq[NP + q] = fma(bi[q], bi[q], sq[NP + q]);
+      }
     }
   }
-  block_accumulate(sq, RG, norms + r0);
+  __shared__ double red[kBS / 32][2 * NP];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  constexpr int kRep = 32 / (2 * NP);  // lanes that hold the same sum
+  const double t = warp_scatter_sum<2 * NP>(sq);
+  if (lane % kRep == 0) red[warp][lane / kRep] = t;
+  __syncthreads();
+  if (threadIdx.x < 2 * NP) {
+    const int q = threadIdx.x % NP;
+    double u = 0.0;
+#pragma unroll
+    for (int w = 0; w < kBS / 32; ++w) u += red[w][threadIdx.x];
+    if (q < RG) atomicAdd((threadIdx.x < NP ? sums_r : sums_b) + q, u);
+  }
 }
 
 // The same residual with fixed-order sums: block (x, y) writes the squared norms of its rows'
 // residuals, column by column, to part[r * gridDim.x + x] (each thread sums kNormRows rows, then the
 // block's warps are summed in warp order), and k_finish_norms adds each column's partials in index
-// order.  The row's entries of A are loaded eight at a time before the products, so that the loads
-// of x for all of them are in flight together.  FP64 arithmetic is the bound on this GPU (a small
-// fraction of the FP32 rate), so every thread covers several rows before the butterfly sums.
+// order.  FP64 arithmetic is the bound on this GPU (a small fraction of the FP32 rate), so every
+// thread covers several rows before the warp sums.
 template <int RG>
 __global__ void __launch_bounds__(kBS) k_residual_part(int64_t n, int R, const int64_t* __restrict__ rowptr,
                                                         const int32_t* __restrict__ col, const double* __restrict__ val,
@@ -159,27 +206,10 @@ __global__ void __launch_bounds__(kBS) k_residual_part(int64_t n, int R, const i
   for (int j = 0; j < kNormRows; ++j) {
     const int64_t i = (blockIdx.x * (int64_t)kNormRows + j) * blockDim.x + threadIdx.x;
     if (i < n) {
-      const int64_t lo = rowptr[i], hi = rowptr[i + 1];
       double ax[RG];
 #pragma unroll
       for (int rr = 0; rr < RG; ++rr) ax[rr] = 0.0;
-      for (int64_t k0 = lo; k0 < hi; k0 += 8) {
-        int c[8];
-        double v[8];
-#pragma unroll
-        for (int u = 0; u < 8; ++u) {
-          c[u] = k0 + u < hi ? col[k0 + u] : 0;
-          v[u] = k0 + u < hi ? val[k0 + u] : 0.0;
-        }
-#pragma unroll
-        for (int u = 0; u < 8; ++u) {
-          if (k0 + u < hi) {
-            const double* xk = x + c[u] + (int64_t)r0 * ldx;
-#pragma unroll
-            for (int rr = 0; rr < RG; ++rr) ax[rr] += v[u] * xk[(int64_t)rr * ldx];
-          }
-        }
-      }
+      row_product<RG>(i, rowptr, col, val, x + (int64_t)r0 * ldx, ldx, ax);
 #pragma unroll
       for (int rr = 0; rr < RG; ++rr) {
         const double ri = b[i + (int64_t)(r0 + rr) * ldb] - ax[rr];
@@ -190,11 +220,8 @@ __global__ void __launch_bounds__(kBS) k_residual_part(int64_t n, int R, const i
   }
   __shared__ double red[kBS / 32][RG];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-#pragma unroll
-  for (int rr = 0; rr < RG; ++rr) {
-    const double t = warp_sum(sq[rr]);
-    if (lane == 0) red[warp][rr] = t;
-  }
+  const double w = warp_scatter_sum<RG>(sq);
+  if (lane % (32 / RG) == 0) red[warp][lane / (32 / RG)] = w;
   __syncthreads();
   if (threadIdx.x < RG) {
     double t = 0.0;
@@ -253,21 +280,6 @@ __global__ void __launch_bounds__(kBS) k_finish_norms(int nparts, const double* 
   }
 }
 
-__global__ void k_sqnorm(int64_t n, int R, const double* __restrict__ v, int64_t ld, double* norms) {
-  const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  double sq[kMaxR];
-#pragma unroll
-  for (int r = 0; r < kMaxR; ++r) sq[r] = 0.0;
-  if (i < n)
-#pragma unroll
-    for (int r = 0; r < kMaxR; ++r) {
-      if (r >= R) break;
-      const double t = v[i + r * ld];
-      sq[r] = t * t;
-    }
-  block_accumulate(sq, R, norms);
-}
-
 __global__ void k_copy2d(int64_t n, int R, const double* __restrict__ src, int64_t lds, double* __restrict__ dst, int64_t ldd) {
   const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (i >= n) return;
@@ -324,16 +336,25 @@ cudaError_t launch_assemble(int64_t n, int R, const int64_t* vc_ptr, const int64
   return cudaGetLastError();
 }
 
-cudaError_t launch_residual(int64_t n, int R, const int64_t* rowptr, const int32_t* col, const double* val,
-                            const double* b, int64_t ldb, const double* x, int64_t ldx, double* res, int64_t ldr,
-                            double* norms, cudaStream_t st) {
-  if (R > kMaxR || R < 1) return cudaErrorInvalidValue;
+cudaError_t launch_residual_norms(int64_t n, int R, const int64_t* rowptr, const int32_t* col, const double* val,
+                                  const double* b, int64_t ldb, const double* x, int64_t ldx, double* sums_r,
+                                  double* sums_b, cudaStream_t st) {
+  if (R < 1 || R > 8) return cudaErrorInvalidValue;
   if (n <= 0) return cudaSuccess;
-  const unsigned bx = nblocks(n);
-  if (R % 8 == 0) k_residual<8><<<dim3(bx, R / 8), kBS, 0, st>>>(n, R, rowptr, col, val, b, ldb, x, ldx, res, ldr, norms);
-  else if (R % 4 == 0) k_residual<4><<<dim3(bx, R / 4), kBS, 0, st>>>(n, R, rowptr, col, val, b, ldb, x, ldx, res, ldr, norms);
-  else if (R % 2 == 0) k_residual<2><<<dim3(bx, R / 2), kBS, 0, st>>>(n, R, rowptr, col, val, b, ldb, x, ldx, res, ldr, norms);
-  else k_residual<1><<<dim3(bx, R), kBS, 0, st>>>(n, R, rowptr, col, val, b, ldb, x, ldx, res, ldr, norms);
+  // several rows per thread only where the GPU stays full (8 blocks per SM): a small matrix waits for
+  // its loads, not for FP64
+  const int rows = (int)std::min<int64_t>(kNormRows, std::max<int64_t>(1, n / ((int64_t)kBS * 8 * 152)));
+  const unsigned bx = (unsigned)((n + (int64_t)kBS * rows - 1) / ((int64_t)kBS * rows));
+  switch (R) {
+    case 1: k_residual_norms<1, 1><<<bx, kBS, 0, st>>>(n, rows, rowptr, col, val, b, ldb, x, ldx, sums_r, sums_b); break;
+    case 2: k_residual_norms<2, 2><<<bx, kBS, 0, st>>>(n, rows, rowptr, col, val, b, ldb, x, ldx, sums_r, sums_b); break;
+    case 3: k_residual_norms<3, 4><<<bx, kBS, 0, st>>>(n, rows, rowptr, col, val, b, ldb, x, ldx, sums_r, sums_b); break;
+    case 4: k_residual_norms<4, 4><<<bx, kBS, 0, st>>>(n, rows, rowptr, col, val, b, ldb, x, ldx, sums_r, sums_b); break;
+    case 5: k_residual_norms<5, 8><<<bx, kBS, 0, st>>>(n, rows, rowptr, col, val, b, ldb, x, ldx, sums_r, sums_b); break;
+    case 6: k_residual_norms<6, 8><<<bx, kBS, 0, st>>>(n, rows, rowptr, col, val, b, ldb, x, ldx, sums_r, sums_b); break;
+    case 7: k_residual_norms<7, 8><<<bx, kBS, 0, st>>>(n, rows, rowptr, col, val, b, ldb, x, ldx, sums_r, sums_b); break;
+    default: k_residual_norms<8, 8><<<bx, kBS, 0, st>>>(n, rows, rowptr, col, val, b, ldb, x, ldx, sums_r, sums_b); break;
+  }
   return cudaGetLastError();
 }
 
@@ -363,12 +384,6 @@ cudaError_t launch_sqnorm_det(int64_t n, int R, const double* v, int64_t ld, dou
   else if (R % 2 == 0) k_sqnorm_part<2><<<dim3(bx, R / 2), kBS, 0, st>>>(n, v, ld, part);
   else k_sqnorm_part<1><<<dim3(bx, R), kBS, 0, st>>>(n, v, ld, part);
   k_finish_norms<<<R, kBS, 0, st>>>((int)bx, part, norms);
-  return cudaGetLastError();
-}
-
-cudaError_t launch_sqnorm(int64_t n, int R, const double* v, int64_t ld, double* norms, cudaStream_t st) {
-  if (R > kMaxR) return cudaErrorInvalidValue;
-  k_sqnorm<<<nblocks(n), kBS, 0, st>>>(n, R, v, ld, norms);
   return cudaGetLastError();
 }
 
