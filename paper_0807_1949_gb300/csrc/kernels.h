@@ -217,9 +217,32 @@ template <typename T>
 cudaError_t launch_port_resident(const ResArgs<T>& a, int R, int grid, size_t smem, size_t xch_bytes, cudaStream_t st);
 
 // Tensor-core port-response sweep for 16 / 32 right-hand sides (port_tc.cu), FP32 solvers.
+constexpr int kTcMaxSplit = 8;        // items that a subgraph is cut into at most
+struct TcItem {
+  int32_t piece;               // index into PortTCArgs::pieces
+  int32_t hi, lo;              // super-rows hi .. lo
+  int64_t part;                // element offset of its share of y (ports x R); -1: the whole subgraph
+};
+struct TcSplit {               // a subgraph of several items
+  int32_t piece, nitems;
+  int32_t hi[kTcMaxSplit];     // first super-row of each item
+  int64_t part;                // the items' shares, one after the other
+};
+struct TcPlan {
+  std::vector<TcItem> items;
+  std::vector<int32_t> cta_item;  // CTA c takes the items cta_item[c] .. cta_item[c + 1] - 1
+  std::vector<TcSplit> splits;
+  int64_t part_elems = 0;
+  int max_split_ports = 0;
+};
+TcPlan tc_plan(const PieceDesc* pieces, int npieces, int R, int ctas);
+
 struct PortTCArgs {
-  const PieceDesc* pieces;     // subgraphs of the launch (largest first); CTA c takes c, c + grid, ...
-  int npieces;
+  const PieceDesc* pieces;     // subgraphs of the launch
+  const TcItem* items;
+  const int32_t* cta_item;
+  const TcSplit* splits;
+  float* part;
   const unsigned char* S16;    // lower block triangle of S_j / sigma_j as fp16 hi / lo panels (h_off)
   const float* sig_s;          // sigma_j per subgraph of the launch
   const float* gscale;         // g_p = sqrt(S_pp) per port (diagonal balance of S_j)
@@ -247,8 +270,10 @@ size_t port_tc_smem_bytes(int R, bool lo);
 cudaError_t launch_port_records(int nports, const int32_t* port_end_ptr, const int32_t* twin, const float* invz,
                                 CoupleRef<float> cpl, int4* rec, cudaStream_t st);
 cudaError_t port_tc_configure(int R);
-// One persistent launch per sweep (grid <= SMs); lo = use the lo half of S_j (FP32-accurate).
-cudaError_t launch_port_sweep_tc(const PortTCArgs& a, int R, bool lo, int grid, cudaStream_t st);
+// One persistent launch per sweep (grid <= SMs), and one for the cut subgraphs' waves if there are
+// any; lo = use the lo half of S_j (FP32-accurate).
+cudaError_t launch_port_sweep_tc(const PortTCArgs& a, int R, bool lo, int grid, int nsplits, int max_split_ports,
+                                 cudaStream_t st);
 cudaError_t launch_gather_port_blocks(const PieceDesc* pieces, int npieces, const int32_t* port_local, int Rs, int b,
                                       const float* xc, float* S32, cudaStream_t st);
 cudaError_t launch_port_blocks_to_f16(const PieceDesc* pieces, int npieces, const float* S32, unsigned char* S16,

@@ -25,7 +25,15 @@
 // fp16 roundings); without it (FP16 storage, half the bytes) S carries fp16 rounding, 2^-11 of
 // sigma_j, and the FP64 defect correction absorbs it as for the FP16 tiles of port.cu.
 //
-// One persistent kernel per sweep, one CTA per SM looping over subgraphs, 448 threads:
+// Work split.  A CTA takes items, each a run of super-rows hi .. lo of one subgraph (tc_plan): whole
+// subgraphs where they are many, cut ones where a subgraph is more than a CTA's share, the items
+// dealt out largest first to the CTA with the least work so far.  An item that is a whole subgraph
+// writes its waves itself; the others leave the rows y_0 .. y_hi they added to as partial sums, and
+// k_port_finish_tc adds a row's partials in the items' order and writes the waves.  (Every CTA
+// taking subgraphs c, c + grid, ... : 64 subgraphs left 88 of 152 SMs idle, 512 uneven ones kept the
+// unluckiest CTA busy 1.3 times the average.)
+//
+// One persistent kernel per sweep, one CTA per SM looping over its items, 448 threads:
 //  * warp 0 streams the blocks (and the s_J tile of off-diagonal blocks) through a ring of 16 KB
 //    shared-memory slots by bulk copies (mbarrier complete_tx).  A block's panels go out one pair
 //    at a time, each as soon as its slots are free, so that the next blocks stream in while the
@@ -42,6 +50,9 @@
 // Every wait is bounded; a CTA that gives up records VTM_ERR_TIMEOUT, lets its copies and MMAs
 // finish, frees its tensor memory and returns.
 #include <cuda_fp16.h>
+
+#include <algorithm>
+#include <cmath>
 
 #include "kernels.h"
 #include "tc.cuh"
@@ -364,7 +375,8 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_port_sweep_tc(const PortTCArg
   const uint32_t row0 = base + P::kRow;
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const int npc = (a.npieces - (int)blockIdx.x + (int)gridDim.x - 1) / (int)gridDim.x;  // subgraphs of this CTA
+  const TcItem* const items = a.items + a.cta_item[blockIdx.x];
+  const int npc = a.cta_item[blockIdx.x + 1] - a.cta_item[blockIdx.x];  // items of this CTA
   const size_t slot_bytes = (size_t)a.n4max * P::kVec;
   unsigned char* scratch = a.scratch + (size_t)blockIdx.x * (2 * slot_bytes + (size_t)a.n4max * kSB * R * 4);
   float* stage32 = reinterpret_cast<float*>(scratch + 2 * slot_bytes);  // FP32 port vectors, ports x R
@@ -424,8 +436,9 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_port_sweep_tc(const PortTCArg
         return true;
       };
       for (int k = 0; k < npc && !abort_flag; ++k) {
-        const PieceDesc pd = a.pieces[blockIdx.x + (size_t)k * gridDim.x];
-        const int Pn = pd.nports, n4 = n_super(Pn);
+        const TcItem it = items[k];
+        const PieceDesc pd = a.pieces[it.piece];
+        const int Pn = pd.nports, n4 = it.hi + 1;
         if (!mbar_wait_bounded(&sready[k & 1], (uint32_t)((k >> 1) & 1), a.wait_limit)) {
           abort_flag = 1;
           break;
@@ -447,7 +460,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_port_sweep_tc(const PortTCArg
           abort_flag = 1;
           break;
         }
-        for (int I = n4 - 1; I >= 0 && !abort_flag; --I) {
+        for (int I = n4 - 1; I >= it.lo && !abort_flag; --I) {
           const int h = sb_rows(Pn, I);
           const uint32_t pbytes = (uint32_t)h * 128;  // one panel
           for (int J = I; J >= 0; --J) {
@@ -484,7 +497,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_port_sweep_tc(const PortTCArg
             ++gblk;
             // the next row's tile goes out a few blocks ahead: by the third block of this row the
             // MMAs have finished the row before it, whose buffer it takes
-            if (ok && I > 0 && J == (I >= 2 ? I - 2 : 0)) ok = issue_row(I - 1);
+            if (ok && I > it.lo && J == (I >= 2 ? I - 2 : 0)) ok = issue_row(I - 1);
             if (!ok) {
               abort_flag = 1;
               break;
@@ -510,9 +523,9 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_port_sweep_tc(const PortTCArg
       int64_t gblk = 0, grow = 0, aslot = 0;
       uint32_t pend = 0, wpar = 0;  // rows handed to the epilogue and not yet waited for; parity of the next wait
       for (int k = 0; k < npc && !abort_flag; ++k) {
-        const PieceDesc pd = a.pieces[blockIdx.x + (size_t)k * gridDim.x];
-        const int Pn = pd.nports, n4 = n_super(Pn);
-        for (int I = n4 - 1; I >= 0 && !abort_flag; --I) {
+        const TcItem it = items[k];
+        const int Pn = a.pieces[it.piece].nports, n4 = it.hi + 1;
+        for (int I = n4 - 1; I >= it.lo && !abort_flag; --I) {
           const int rb = (int)(grow & 1);
           if (!mbar_wait_bounded(&rowfull[rb], (uint32_t)((grow >> 1) & 1), a.wait_limit)) {
             abort_flag = 1;
@@ -546,9 +559,10 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_port_sweep_tc(const PortTCArg
             ++gblk;
           }
           mma_commit(&rowempty[rb]);
-          mma_commit(&rready[I]);  // y_I is final
+          mma_commit(&rready[I]);  // y_I is final (of this item)
           ++grow;
         }
+        for (int J = it.lo - 1; J >= 0; --J) mma_commit(&rready[J]);
         pend |= (n4 >= 32 ? ~0u : (1u << n4) - 1u);
       }
       mma_commit(done);  // arrives once every MMA issued above has completed
@@ -563,9 +577,10 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_port_sweep_tc(const PortTCArg
     uint32_t uses = 0;  // tid 64: parity of the next phase of each row barrier, one bit per super-row
     bool stop = false;
     for (int k = 0; k < npc && !stop; ++k) {
-      const PieceDesc pd = a.pieces[blockIdx.x + (size_t)k * gridDim.x];
-      const int Pn = pd.nports, n4 = n_super(Pn);
-      const float sj = a.sig_s[blockIdx.x + (size_t)k * gridDim.x];
+      const TcItem it = items[k];
+      const PieceDesc pd = a.pieces[it.piece];
+      const int Pn = pd.nports, n4 = it.hi + 1;
+      const float sj = a.sig_s[it.piece];
       if (tid == 64) flags[1] = mbar_wait_bounded(&sready[k & 1], (uint32_t)((k >> 1) & 1), a.wait_limit) ? 0 : 1;
       epi_sync();
       stop = flags[1] != 0;
@@ -587,7 +602,17 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_port_sweep_tc(const PortTCArg
         __syncwarp();
         if (lane == 0) mbar_arrive(&rowread[I]);
         const int p = I * kSB + 32 * q + lane;
-        if (p < Pn) {
+        if (p < Pn && it.part >= 0) {
+          // part of a subgraph: this item's share of y
+          const float gs = sj * a.gscale[pd.port_off + p];
+          float4* o = reinterpret_cast<float4*>(a.part + it.part + (size_t)p * R);
+#pragma unroll
+          for (int k4 = 0; k4 < R / 4; ++k4)
+            o[k4] = make_float4(gs * ssig[k & 1][4 * k4] * __uint_as_float(v[4 * k4]),
+                                gs * ssig[k & 1][4 * k4 + 1] * __uint_as_float(v[4 * k4 + 1]),
+                                gs * ssig[k & 1][4 * k4 + 2] * __uint_as_float(v[4 * k4 + 2]),
+                                gs * ssig[k & 1][4 * k4 + 3] * __uint_as_float(v[4 * k4 + 3]));
+        } else if (p < Pn) {
           const int port = pd.port_off + p;
           const float4* ub = reinterpret_cast<const float4*>(a.ubase + (size_t)port * R);
           const int e0 = a.port_end_ptr[port], e1 = a.port_end_ptr[port + 1];
@@ -642,8 +667,9 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_port_sweep_tc(const PortTCArg
           break;
         }
       }
-      const PieceDesc pd = a.pieces[blockIdx.x + (size_t)k * gridDim.x];
-      const int Pn = pd.nports, np = n_super(Pn) * kSB;
+      const PieceDesc pd = a.pieces[items[k].piece];
+      const int np = (items[k].hi + 1) * kSB;         // rows that the item's products read
+      const int Pn = pd.nports < np ? pd.nports : np;
       // gather: s' = D^-1 s per port into the FP32 staging area; the next port's record is
       // loaded before this port's wave rows
       int4 rec[3];
@@ -738,6 +764,101 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_port_sweep_tc(const PortTCArg
   }
 }
 
+// Waves of the subgraphs whose rows several items added to: u = u_base + the items' shares in their
+// order, w_out[e] = 2u - w_in[e]; thread = (port, four columns).
+template <int R>
+__global__ void __launch_bounds__(256) k_port_finish_tc(const PortTCArgs a) {
+  const TcSplit sp = a.splits[blockIdx.y];
+  const PieceDesc pd = a.pieces[sp.piece];
+  const int i = blockIdx.x * 256 + threadIdx.x;
+  const int p = i / (R / 4), k4 = i % (R / 4);
+  if (p >= pd.nports) return;
+  const int port = pd.port_off + p, I = p / kSB;
+  const int e0 = a.port_end_ptr[port], e1 = a.port_end_ptr[port + 1];
+  float4 u = reinterpret_cast<const float4*>(a.ubase + (size_t)port * R)[k4];
+  float4 y = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+  for (int q = 0; q < kTcMaxSplit; ++q) {
+    if (q < sp.nitems && sp.hi[q] >= I) {
+      const float4 x = reinterpret_cast<const float4*>(a.part + sp.part + ((size_t)q * pd.nports + p) * R)[k4];
+      y.x += x.x, y.y += x.y, y.z += x.z, y.w += x.w;
+    }
+  }
+  u.x += y.x, u.y += y.y, u.z += y.z, u.w += y.w;
+  for (int e = e0; e < e1; ++e) {
+    const float4 w = reinterpret_cast<const float4*>(a.wprev + (size_t)a.twin[e] * R)[k4];
+    reinterpret_cast<float4*>(a.wnext + (size_t)e * R)[k4] =
+        make_float4(2.f * u.x - w.x, 2.f * u.y - w.y, 2.f * u.z - w.z, 2.f * u.w - w.w);
+  }
+}
+
+// Items of the subgraphs for `ctas` CTAs.  A subgraph of more than 1.1 CTA shares (in blocks) is cut
+// between super-rows into up to kTcMaxSplit items of about a share each.
+TcPlan tc_plan(const PieceDesc* pd, int npieces, int R, int ctas) {
+  constexpr double kItemCost = 3.0;  // what an item costs besides its blocks, in blocks
+  TcPlan pl;
+  double total = 0;
+  for (int j = 0; j < npieces; ++j) {
+    const int n4 = n_super(pd[j].nports);
+    total += n4 * (n4 + 1) / 2 + (n4 > 0 ? kItemCost : 0.0);
+  }
+  const double share = total / std::max(1, ctas);
+  std::vector<std::pair<double, TcItem>> items;
+  for (int j = 0; j < npieces; ++j) {
+    const int n4 = n_super(pd[j].nports);
+    if (n4 == 0) continue;
+    const int blocks = n4 * (n4 + 1) / 2;
+    int c = 1;
+    if (blocks + kItemCost > 1.1 * share)
+      c = std::min({kTcMaxSplit, n4, (int)std::ceil(blocks / std::max(1.0, share - kItemCost))});
+    TcSplit sp{};
+    sp.piece = j;
+    sp.part = pl.part_elems;
+    int row = n4 - 1, left = blocks;
+    for (int q = 0; q < c && row >= 0; ++q) {
+      // rows until the item has its share of what is left (the last one takes the rest)
+      const double want = (double)left / (c - q);
+      int lo = row, got = row + 1;
+      while (lo > 0 && (q == c - 1 || got + lo / 2.0 < want)) got += lo--;
+      TcItem it{};
+      it.piece = j;
+      it.hi = row;
+      it.lo = lo;
+      it.part = c > 1 ? sp.part + (int64_t)q * pd[j].nports * R : -1;
+      items.push_back({got + kItemCost, it});
+      sp.hi[q] = row;
+      sp.nitems = q + 1;
+      left -= got;
+      row = lo - 1;
+    }
+    if (sp.nitems == 1) items.back().second.part = -1;
+    if (sp.nitems > 1) {
+      pl.splits.push_back(sp);
+      pl.part_elems += (int64_t)sp.nitems * pd[j].nports * R;
+      pl.max_split_ports = std::max(pl.max_split_ports, (int)pd[j].nports);
+    }
+  }
+  std::stable_sort(items.begin(), items.end(), [](const auto& x, const auto& y) { return x.first > y.first; });
+  const int n = std::max(1, std::min<int>(ctas, (int)items.size()));
+  std::vector<std::vector<TcItem>> of(n);
+  std::vector<std::pair<double, int>> heap;  // least loaded CTA on top
+  for (int c = 0; c < n; ++c) heap.push_back({0.0, c});
+  auto later = [](const std::pair<double, int>& x, const std::pair<double, int>& y) { return x > y; };
+  std::make_heap(heap.begin(), heap.end(), later);
+  for (const auto& it : items) {
+    std::pop_heap(heap.begin(), heap.end(), later);
+    of[heap.back().second].push_back(it.second);
+    heap.back().first += it.first;
+    std::push_heap(heap.begin(), heap.end(), later);
+  }
+  pl.cta_item.push_back(0);
+  for (const auto& v : of) {
+    pl.items.insert(pl.items.end(), v.begin(), v.end());
+    pl.cta_item.push_back((int32_t)pl.items.size());
+  }
+  return pl;
+}
+
 // Gather record of port q: the wave rows and coefficients of its first four entries in the order
 // the sweep adds them (ends e0 .. e1 - 1 with 1 / Z_e, then coupling entries k0 .. k1 - 1 with y;
 // row -1 and coefficient 0 past the last one), and where the remaining entries resume.
@@ -792,8 +913,9 @@ cudaError_t port_tc_configure(int R) {
   return e;
 }
 
-cudaError_t launch_port_sweep_tc(const PortTCArgs& a, int R, bool lo, int grid, cudaStream_t st) {
-  if (a.npieces <= 0 || grid <= 0) return cudaSuccess;
+cudaError_t launch_port_sweep_tc(const PortTCArgs& a, int R, bool lo, int grid, int nsplits, int max_split_ports,
+                                 cudaStream_t st) {
+  if (grid <= 0) return cudaSuccess;
   const size_t smem = port_tc_smem_bytes(R, lo);
   if (R == 16) {
     if (lo) k_port_sweep_tc<16, true><<<grid, kTcThreads, smem, st>>>(a);
@@ -804,6 +926,11 @@ cudaError_t launch_port_sweep_tc(const PortTCArgs& a, int R, bool lo, int grid, 
   } else {
     return cudaErrorInvalidValue;
   }
+  cudaError_t e = cudaGetLastError();
+  if (e != cudaSuccess || nsplits == 0) return e;
+  const dim3 g((max_split_ports * (R / 4) + 255) / 256, nsplits);
+  if (R == 16) k_port_finish_tc<16><<<g, 256, 0, st>>>(a);
+  else k_port_finish_tc<32><<<g, 256, 0, st>>>(a);
   return cudaGetLastError();
 }
 

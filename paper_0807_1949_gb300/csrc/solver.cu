@@ -153,6 +153,8 @@ struct vtm_solver {
   size_t res_smem = 0;
   DevBuf S16, sig16, tc_scratch;     // tensor-core form: fp16 hi / lo blocks, sigma_j, s^T slots
   DevBuf gscale;                     // tensor-core form: sqrt(S_pp) per port (diagonal balance)
+  DevBuf tc_items, tc_cta_item, tc_splits, tc_part;  // division of the subgraphs among CTAs
+  int tc_nsplits = 0, tc_split_ports = 0;
   int tc_grid = 0, tc_n4max = 0, tc_tmem_cols = 0;
   int64_t tc_bytes_hi = 0, tc_bytes_all = 0;  // bytes a sweep streams without / with the lo half
   DevBuf Sh, hscale;                 // FP16 copy of S_j and the scale of each of its tiles
@@ -1040,7 +1042,10 @@ static void launch_port(vtm_solver* s) {
     if (s->port_tc) {
       PortTCArgs t;
       t.pieces = s->pieces_lo.as<PieceDesc>();
-      t.npieces = s->np_lo;
+      t.items = s->tc_items.as<TcItem>();
+      t.cta_item = s->tc_cta_item.as<int32_t>();
+      t.splits = s->tc_splits.as<TcSplit>();
+      t.part = s->tc_part.as<float>();
       t.S16 = s->S16.as<unsigned char>();
       t.sig_s = s->sig16.as<float>();
       t.gscale = s->gscale.as<float>();
@@ -1057,8 +1062,8 @@ static void launch_port(vtm_solver* s) {
       t.prec = s->port_rec.as<int4>();
       t.status = s->status.as<int>();
       t.wait_limit = s->wait_limit;
-      VTM_CUDA(launch_port_sweep_tc(t, s->R, !s->port_half, s->tc_grid, s->stream));
-      s->launches++;
+      VTM_CUDA(launch_port_sweep_tc(t, s->R, !s->port_half, s->tc_grid, s->tc_nsplits, s->tc_split_ports, s->stream));
+      s->launches += s->tc_nsplits > 0 ? 2 : 1;
       return;
     }
   }
@@ -1139,7 +1144,7 @@ static int64_t launches_per_batch(const vtm_solver* s, int k) {
   const int64_t band = (s->np_lo > 0) + (s->np_hi > 0);
   if (!s->port_form || k < 2) return (int64_t)k * band;
   if (s->resident) return 1 + band;
-  const int64_t port = (s->np_lo > 0 ? (s->port_tc ? 1 : 2) : 0) + (s->np_hi > 0);
+  const int64_t port = (s->np_lo > 0 ? (s->port_tc && s->tc_nsplits == 0 ? 1 : 2) : 0) + (s->np_hi > 0);
   return (int64_t)(k - 1) * port + band;
 }
 
@@ -1247,7 +1252,15 @@ static void choose_form(vtm_solver* s, const vtm_setup_opts* o, int64_t s_tiles,
   };
   if (s->resident) {
   } else if (tc) {
-    s->tc_grid = std::min(s->np_lo, nsm);  // one persistent CTA per SM (it holds the SM's tensor memory)
+    const TcPlan pl = tc_plan(lo.data(), (int)lo.size(), s->R, nsm);  // one CTA per SM (it holds its tensor memory)
+    upload(s->tc_items, pl.items, s->stream);
+    upload(s->tc_cta_item, pl.cta_item, s->stream);
+    upload(s->tc_splits, pl.splits, s->stream);
+    s->tc_part.alloc((size_t)pl.part_elems * sizeof(float));
+    VTM_CUDA(cudaStreamSynchronize(s->stream));  // the uploads read pl
+    s->tc_nsplits = (int)pl.splits.size();
+    s->tc_split_ports = pl.max_split_ports;
+    s->tc_grid = pl.items.empty() ? 0 : (int)pl.cta_item.size() - 1;
     s->tc_n4max = n4max;
     s->tc_tmem_cols = tmem_cols;
     s->tc_scratch.alloc((size_t)s->tc_grid * ((size_t)2 * n4max * s->R * 512 + (size_t)n4max * 128 * s->R * 4));
