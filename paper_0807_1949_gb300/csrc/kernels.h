@@ -232,7 +232,8 @@ struct TcPlan {
   std::vector<TcItem> items;
   std::vector<int32_t> cta_item;  // CTA c takes the items cta_item[c] .. cta_item[c + 1] - 1
   std::vector<TcSplit> splits;
-  int64_t part_elems = 0;
+  std::vector<int32_t> tile_off;  // per subgraph, its first operand tile
+  int64_t part_elems = 0, tiles = 0;
   int max_split_ports = 0;
 };
 TcPlan tc_plan(const PieceDesc* pieces, int npieces, int R, int ctas);
@@ -246,8 +247,14 @@ struct PortTCArgs {
   const unsigned char* S16;    // lower block triangle of S_j / sigma_j as fp16 hi / lo panels (h_off)
   const float* sig_s;          // sigma_j per subgraph of the launch
   const float* gscale;         // g_p = sqrt(S_pp) per port (diagonal balance of S_j)
-  unsigned char* scratch;      // per CTA two slots of n4max s^T tiles (R x 512 bytes each)
+  unsigned char* scratch;      // FUSED: per CTA two slots of n4max s^T tiles (R x 512 bytes each)
   int n4max;                   // most 128-port super-rows of a subgraph
+  const int4* prec;            // FUSED: per port 3 x int4: first four entries' wave rows, their coefficients
+                               // (float bits), {next end, e1, next coupling, k1} (launch_port_records)
+  unsigned char* stiles;       // not FUSED: the port vectors' operand tiles (R x 512 bytes per super-row)
+  const int32_t* tile_off;     // per subgraph, its first tile
+  float* ssig;                 // sigma_r per subgraph and column
+  const int32_t* cpl_end;      // per coupling entry, its wave's place among the subgraph's ends
   int tmem_cols;               // tensor-memory columns per CTA (power of two >= n4max R)
   const float* ubase;          // ports x R
   const float* wprev;          // ends x R
@@ -256,8 +263,6 @@ struct PortTCArgs {
   const int32_t* twin;
   const float* invz;
   CoupleRef<float> cpl;        // coupled lines (cpl.ptr == nullptr: none)
-  const int4* prec;            // per port 3 x int4: first four entries' wave rows, their coefficients
-                               // (float bits), {next end, e1, next coupling, k1} (launch_port_records)
   int* status;
   long wait_limit;
 };
@@ -266,14 +271,20 @@ constexpr int kTcMaxSuper = 16;       // 128-port super-rows per subgraph on the
 int64_t port_f16_bytes(int nports);   // fp16 hi / lo blocks of one subgraph (1 KB multiple)
 int64_t port_f32_blocks(int nports);  // 128 x 128 FP32 blocks of the lower triangle (setup)
 size_t port_tc_smem_bytes(int R, bool lo);
-// Per-port gather records of the tensor-core port sweep (3 int4 per port, nports of them).
+// Per-port gather records of the fused sweep (3 int4 per port, nports of them).
 cudaError_t launch_port_records(int nports, const int32_t* port_end_ptr, const int32_t* twin, const float* invz,
                                 CoupleRef<float> cpl, int4* rec, cudaStream_t st);
+// Places of the coupling entries' waves for the separate port vectors.
+cudaError_t launch_coupling_ends(const PieceDesc* pieces, int npieces, const int32_t* twin, CoupleRef<float> cpl,
+                                 int32_t* cpl_end, cudaStream_t st);
+constexpr size_t kVecTcSmemMax = 220 * 1024;
+size_t port_vec_tc_smem_bytes(int max_ends);
 cudaError_t port_tc_configure(int R);
-// One persistent launch per sweep (grid <= SMs), and one for the cut subgraphs' waves if there are
-// any; lo = use the lo half of S_j (FP32-accurate).
-cudaError_t launch_port_sweep_tc(const PortTCArgs& a, int R, bool lo, int grid, int nsplits, int max_split_ports,
-                                 cudaStream_t st);
+// The port vectors (unless fused: a.stiles == nullptr), one persistent launch for the sweep (grid <=
+// SMs), and one for the cut subgraphs' waves if there are any; lo = use the lo half of S_j
+// (FP32-accurate).
+cudaError_t launch_port_sweep_tc(const PortTCArgs& a, int R, bool lo, int npieces, int max_ends, int grid, int nsplits,
+                                 int max_split_ports, cudaStream_t st);
 cudaError_t launch_gather_port_blocks(const PieceDesc* pieces, int npieces, const int32_t* port_local, int Rs, int b,
                                       const float* xc, float* S32, cudaStream_t st);
 cudaError_t launch_port_blocks_to_f16(const PieceDesc* pieces, int npieces, const float* S32, unsigned char* S16,

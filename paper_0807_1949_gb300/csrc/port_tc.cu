@@ -42,11 +42,19 @@
 //  * warp 1 issues the MMAs: y_I at tensor-memory columns I R .. I R + R - 1, lane = port, all
 //    super-rows of a subgraph held at once (n4 R <= 512 columns); tcgen05.commit releases stages
 //    and row buffers and hands each finished y_I to the epilogue;
-//  * warps 2-5 run the epilogue of the current subgraph: tcgen05.ld of each y_I (released at once
-//    for the next subgraph's MMAs), u = u_base + sigma_j sigma_r y, w_out[e] = 2u - w_in[e];
-//  * warps 6-13 compute the next subgraph's s: a gather pass driven by per-port records (FP32
-//    values to a staging area), a coalesced pass over that area for the column maxima, then the
-//    split values written to a per-CTA global scratch slot that stays in L2.
+//  * epilogue warps, four at a time (one per tensor-memory lane quadrant): tcgen05.ld of each y_I
+//    (released at once for the next item's MMAs), u = u_base + sigma_j sigma_r y, w_out[e] = 2u - w_in[e].
+// The port vectors come one of two ways:
+//  * FUSED (many items per CTA): warps 6-13 compute the next item's s: a gather pass driven by per-port
+//    records (FP32 values to a staging area), a coalesced pass over that area for the column maxima,
+//    then the split values written to a per-CTA global scratch slot that stays in L2.  With the next
+//    items' blocks to stream meanwhile the gathers cost nothing (256^3: 27 subgraphs per CTA, 0.955 of
+//    the copy bandwidth).
+//  * else (few items per CTA) in a launch of their own before it (k_port_vec_tc), which has every
+//    subgraph's gathers in flight at once, and warps 6-13 are two more sets of epilogue warps: super-row
+//    I belongs to set I mod 3.  Fused, eight warps waiting for 1.4 MB of scattered rows per subgraph
+//    were what such a sweep waited for.  Measured per sweep, 32 right-hand sides: 64^3 (less than one
+//    item per CTA) 0.193 -> 0.089 ms; at 128^3 (3.4 items per CTA) both take 0.557 ms.
 // Every wait is bounded; a CTA that gives up records VTM_ERR_TIMEOUT, lets its copies and MMAs
 // finish, frees its tensor memory and returns.
 #include <cuda_fp16.h>
@@ -64,12 +72,14 @@ using namespace tc;
 namespace {
 
 constexpr int kSB = 128;                // ports per super-block (MMA M; K extent of a block)
-constexpr int kEpiWarps = 4;            // epilogue: one warp per tensor-memory lane quadrant
-constexpr int kVecWarps = 8;            // port vectors
+constexpr int kEpiWarps = 4;            // a set of epilogue warps: one per tensor-memory lane quadrant
+constexpr int kEpiSets = 3;             // sets, not FUSED
+constexpr int kVecWarps = 8;            // port vectors, FUSED (the place of two sets)
 constexpr int kTcThreads = 32 * (2 + kEpiWarps + kVecWarps);  // warp 0 copies, warp 1 MMA
+static_assert(kEpiSets * kEpiWarps == kEpiWarps + kVecWarps, "warps");
 constexpr int kVecThreads = 32 * kVecWarps;
-constexpr int kVecBar = 1;              // named barrier of the vector warps
-constexpr int kEpiBar = 2;              // named barrier of the epilogue warps
+constexpr int kEpiBar = 1;              // named barriers of the epilogue sets: 1, 2, 3
+constexpr int kVecBar = 4;              // named barrier of the vector warps
 constexpr int kMaxSuper = kTcMaxSuper;  // super-rows per subgraph (and tensor memory: n4 R <= 512)
 
 __host__ __device__ __forceinline__ int n_super(int nports) { return (nports + kSB - 1) / kSB; }
@@ -86,15 +96,17 @@ __host__ __device__ __forceinline__ int64_t blk_off(int nports, int I, int J) {
   return (int64_t)I * (I + 1) / 2 * (kSB * 512) + (int64_t)J * sb_rows(nports, I) * 512;
 }
 
+__device__ __forceinline__ void grid_dep_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void grid_dep_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void vec_sync() { asm volatile("bar.sync %0, %1;" ::"n"(kVecBar), "n"(kVecThreads) : "memory"); }
-__device__ __forceinline__ void epi_sync() {
-  asm volatile("bar.sync %0, %1;" ::"n"(kEpiBar), "n"(32 * kEpiWarps) : "memory");
+__device__ __forceinline__ void epi_sync(int set) {
+  asm volatile("bar.sync %0, %1;" ::"r"(kEpiBar + set), "n"(32 * kEpiWarps) : "memory");
 }
 
 // Header offsets (bytes from the aligned start).
 constexpr uint32_t kOffFull = 0, kOffEmpty = 64, kOffRowFull = 128, kOffRowEmpty = 144, kOffSReady = 160,
                    kOffSlotFree = 176, kOffRReady = 192, kOffRowRead = 320, kOffDone = 448, kOffTslot = 456,
-                   kOffFlags = 464, kOffSsig = 512, kOffOwner = 768, kOffRed = 1024;
+                   kOffFlags = 464, kOffSsig = 512, kOffOwner = 896, kOffRed = 1024;
 static_assert(kOffRReady + 8 * kMaxSuper <= kOffRowRead && kOffRowRead + 8 * kMaxSuper <= kOffDone, "header");
 
 // Shared-memory plan.  The kernel has no static shared memory: up to 1008 bytes to align the start
@@ -113,7 +125,9 @@ struct Plan {
   static constexpr uint32_t kRow = kHead + kSlots * kSlot;  // the two row tiles, from the aligned start
   static constexpr uint32_t kAlloc = 1008 + kRow + 2 * kVec;
   static_assert(kAlloc <= 227 * 1024, "shared-memory plan");
-  static_assert(kOffSsig + 8 * R <= kOffOwner && kOffOwner + 4 * kSlots <= kOffRed, "header");
+  static_assert(kOffSsig + 4 * kEpiSets * R <= kOffOwner && kOffOwner + 4 * kSlots <= kOffRed &&
+                    kOffRed + 4 * kVecWarps * R <= kHead,
+                "header");
 };
 constexpr int kStg = 8;  // stage barriers (full / empty) in use round robin
 
@@ -349,7 +363,138 @@ __global__ void k_port_blocks_to_f16(const PieceDesc* __restrict__ pieces, const
   }
 }
 
-template <int R, bool LO>
+// The port vectors of every subgraph as operand tiles: s = sum_e w_in[e] / Z_e plus the coupling
+// currents, s' = G s, split per subgraph and column as s' / sigma_r = hi + lo (sigma_r the power of two
+// at or above max |s'_r|).  A CTA takes eight columns of a subgraph: their incoming waves go to shared
+// memory once (a row of 32 bytes per end, all ends' loads independent) and the port sums and the
+// coupling currents, which read every wave about five times, are formed from there; the maxima stay
+// inside the CTA.  Bound by L2: the waves, the lists (once per CTA) and the tiles.
+constexpr int kVecTcThreads = 512;
+constexpr int kVecCols = 8;
+
+template <int R>
+__global__ void __launch_bounds__(kVecTcThreads, 2) k_port_vec_tc(const PortTCArgs a) {
+  constexpr int kPorts = kMaxSuper * kSB / kVecTcThreads;  // ports per thread, at most
+  extern __shared__ __align__(16) float win[];              // [ends][kVecCols]
+  __shared__ float red[kVecTcThreads / 32][kVecCols];
+  __shared__ float inv[kVecCols];
+  grid_dep_launch();
+  const int piece = blockIdx.x, q0 = blockIdx.y * kVecCols;
+  const PieceDesc pd = a.pieces[piece];
+  const int Pn = pd.nports, np = n_super(Pn) * kSB;
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  grid_dep_wait();
+#pragma unroll 4
+  for (int i = tid; i < 2 * pd.nends; i += kVecTcThreads) {
+    const int tw = a.twin[pd.end_off + (i >> 1)];
+    reinterpret_cast<float4*>(win)[i] =
+        __ldcg(reinterpret_cast<const float4*>(a.wprev + (size_t)tw * R + q0) + (i & 1));
+  }
+  __syncthreads();
+  // port pairs 2 (i kVecTcThreads + tid), + 1: a thread writes both with one store per column
+  float v[kPorts][kVecCols];
+#pragma unroll
+  for (int i = 0; i < kPorts; i += 2) {
+    const int p = i * kVecTcThreads + 2 * tid;
+    int e0[2], e1[2], k0[2], k1[2];
+    float gp[2];
+#pragma unroll
+    for (int j = 0; j < 2; ++j) {
+      const bool on = p + j < Pn;
+      const int port = pd.port_off + (on ? p + j : 0);
+      e0[j] = a.port_end_ptr[port];
+      e1[j] = on ? a.port_end_ptr[port + 1] : e0[j];
+      k0[j] = a.cpl.ptr ? a.cpl.ptr[port] : 0;
+      k1[j] = on && a.cpl.ptr ? a.cpl.ptr[port + 1] : k0[j];
+      gp[j] = on ? a.gscale[port] : 0.f;
+    }
+#pragma unroll
+    for (int j = 0; j < 2; ++j) {
+      float s[kVecCols], c[kVecCols];
+#pragma unroll
+      for (int q = 0; q < kVecCols; ++q) s[q] = c[q] = 0.f;
+      auto add = [&](int e, float y, float (&sum)[kVecCols]) {
+        const float4 x0 = reinterpret_cast<const float4*>(win)[2 * e], x1 = reinterpret_cast<const float4*>(win)[2 * e + 1];
+        sum[0] += x0.x * y, sum[1] += x0.y * y, sum[2] += x0.z * y, sum[3] += x0.w * y;
+        sum[4] += x1.x * y, sum[5] += x1.y * y, sum[6] += x1.z * y, sum[7] += x1.w * y;
+      };
+      for (int e = e0[j]; e < e1[j]; ++e) add(e - pd.end_off, a.invz[e], s);
+      for (int k = k0[j]; k < k1[j]; k += 4) {  // four entries' loads in flight together
+        int at[4];
+        float y[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+          at[u] = k + u < k1[j] ? a.cpl_end[k + u] : 0;
+          y[u] = k + u < k1[j] ? a.cpl.y[k + u] : 0.f;
+        }
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+          if (k + u < k1[j]) add(at[u], y[u], c);
+      }
+#pragma unroll
+      for (int q = 0; q < kVecCols; ++q) v[i + j][q] = (s[q] + c[q]) * gp[j];
+    }
+  }
+#pragma unroll
+  for (int q = 0; q < kVecCols; ++q) {
+    float m = 0.f;
+#pragma unroll
+    for (int i = 0; i < kPorts; ++i) m = fmaxf(m, fabsf(v[i][q]));
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
+    if (lane == 0) red[warp][q] = m;
+  }
+  __syncthreads();
+  if (tid < kVecCols) {
+    float m = 0.f;
+#pragma unroll
+    for (int w = 0; w < kVecTcThreads / 32; ++w) m = fmaxf(m, red[w][tid]);
+    int e = 0;
+    if (m > 0.f && isfinite(m)) frexpf(m, &e);
+    e = e < -120 ? -120 : e;
+    inv[tid] = ldexpf(1.f, -e);
+    a.ssig[(size_t)piece * R + q0 + tid] = ldexpf(1.f, e);  // power of two >= max |s_r|
+  }
+  __syncthreads();
+  // tile: [hi, ports 0-63][hi, 64-127][lo, 0-63][lo, 64-127] of R rows (columns of s) each
+  unsigned char* const tiles = a.stiles + (size_t)a.tile_off[piece] * ((size_t)R * 512);
+#pragma unroll
+  for (int i = 0; i < kPorts; i += 2) {
+    const int p = i * kVecTcThreads + 2 * tid;
+    if (p >= np) break;
+    unsigned char* const panel = tiles + (size_t)(p / kSB) * R * 512 + (size_t)((p % kSB) / 64) * R * 128;
+#pragma unroll
+    for (int q = 0; q < kVecCols; ++q) {
+      const float x0 = v[i][q] * inv[q], x1 = v[i + 1][q] * inv[q];
+      const __half2 hi = __floats2half2_rn(x0, x1);
+      const uint32_t off = swz16(q0 + q, p % 64);
+      *reinterpret_cast<__half2*>(panel + off) = hi;
+      *reinterpret_cast<__half2*>(panel + 2 * R * 128 + off) =
+          __floats2half2_rn(x0 - __low2float(hi), x1 - __high2float(hi));
+    }
+  }
+}
+
+// Coupling entry k of a port as the place of its wave among the subgraph's ends (the incoming wave of
+// end e' is the twin's, whose own twin is e').
+__global__ void k_coupling_ends(const PieceDesc* __restrict__ pieces, const int32_t* __restrict__ twin,
+                                CoupleRef<float> cpl, int32_t* __restrict__ cpl_end) {
+  const PieceDesc pd = pieces[blockIdx.x];
+  if (pd.nports == 0) return;
+  for (int k = cpl.ptr[pd.port_off] + threadIdx.x; k < cpl.ptr[pd.port_off + pd.nports]; k += blockDim.x)
+    cpl_end[k] = twin[cpl.oth[k]] - pd.end_off;
+}
+
+cudaError_t launch_coupling_ends(const PieceDesc* pieces, int npieces, const int32_t* twin, CoupleRef<float> cpl,
+                                 int32_t* cpl_end, cudaStream_t st) {
+  if (npieces <= 0 || !cpl.ptr) return cudaSuccess;
+  k_coupling_ends<<<npieces, 256, 0, st>>>(pieces, twin, cpl, cpl_end);
+  return cudaGetLastError();
+}
+
+size_t port_vec_tc_smem_bytes(int max_ends) { return (size_t)std::max(1, max_ends) * kVecCols * sizeof(float); }
+
+template <int R, bool LO, bool FUSED>
 __global__ void __launch_bounds__(kTcThreads, 1) k_port_sweep_tc(const PortTCArgs a) {
   using P = Plan<R>;
   constexpr int NS = P::kSlots;
@@ -362,27 +507,27 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_port_sweep_tc(const PortTCArg
   uint64_t* empty = reinterpret_cast<uint64_t*>(sm + kOffEmpty);        // [kStg] MMAs done with the stage
   uint64_t* rowfull = reinterpret_cast<uint64_t*>(sm + kOffRowFull);    // [2] s_I tile landed
   uint64_t* rowempty = reinterpret_cast<uint64_t*>(sm + kOffRowEmpty);  // [2] MMAs done with the s_I tile
-  uint64_t* sready = reinterpret_cast<uint64_t*>(sm + kOffSReady);      // [2] scratch slot written
-  uint64_t* slotfree = reinterpret_cast<uint64_t*>(sm + kOffSlotFree);  // [2] epilogue of the slot's last subgraph done
+  uint64_t* sready = reinterpret_cast<uint64_t*>(sm + kOffSReady);      // FUSED: [2] scratch slot written
+  uint64_t* slotfree = reinterpret_cast<uint64_t*>(sm + kOffSlotFree);  // FUSED: [2] epilogue of the slot's last item done
   uint64_t* rready = reinterpret_cast<uint64_t*>(sm + kOffRReady);      // [kMaxSuper] accumulator y_I complete
   uint64_t* rowread = reinterpret_cast<uint64_t*>(sm + kOffRowRead);    // [kMaxSuper] y_I read by the epilogue
   uint64_t* done = reinterpret_cast<uint64_t*>(sm + kOffDone);
   uint32_t* tslot = reinterpret_cast<uint32_t*>(sm + kOffTslot);
-  volatile int* flags = reinterpret_cast<volatile int*>(sm + kOffFlags);  // abort, epilogue stop, vector stop
-  float (*ssig)[R] = reinterpret_cast<float (*)[R]>(sm + kOffSsig);        // [2][R] sigma_r per scratch slot
-  float (*red)[R] = reinterpret_cast<float (*)[R]>(sm + kOffRed);          // [kVecWarps][R]
+  volatile int* flags = reinterpret_cast<volatile int*>(sm + kOffFlags);  // abort, epilogue stops, vector stop
+  float (*ssig)[R] = reinterpret_cast<float (*)[R]>(sm + kOffSsig);        // sigma_r: [2] per scratch slot (FUSED), or per set
+  float (*red)[R] = reinterpret_cast<float (*)[R]>(sm + kOffRed);          // FUSED: [kVecWarps][R]
   const uint32_t ring = base + P::kHead;
   const uint32_t row0 = base + P::kRow;
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const TcItem* const items = a.items + a.cta_item[blockIdx.x];
   const int npc = a.cta_item[blockIdx.x + 1] - a.cta_item[blockIdx.x];  // items of this CTA
-  const size_t slot_bytes = (size_t)a.n4max * P::kVec;
+  const size_t slot_bytes = (size_t)a.n4max * P::kVec;  // FUSED
   unsigned char* scratch = a.scratch + (size_t)blockIdx.x * (2 * slot_bytes + (size_t)a.n4max * kSB * R * 4);
   float* stage32 = reinterpret_cast<float*>(scratch + 2 * slot_bytes);  // FP32 port vectors, ports x R
 
   if (tid == 0) {
-    flags[0] = flags[1] = flags[2] = 0;
+    for (int i = 0; i < 5; ++i) flags[i] = 0;
     for (int s = 0; s < kStg; ++s) {
       mbar_init(&full[s], 1);
       mbar_init(&empty[s], 1);
@@ -411,6 +556,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_port_sweep_tc(const PortTCArg
   tc_fence_after();
   const uint32_t tmem = *tslot;
   volatile int& abort_flag = flags[0];
+  grid_dep_launch();
 
   if (warp == 0) {
     // ---- copies: super-rows in descending order; per block (I, J), J = I .. 0, its panels and
@@ -426,6 +572,8 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_port_sweep_tc(const PortTCArg
       // the ring leaves small, and this one thread issues every copy
       int* owner = reinterpret_cast<int*>(sm + kOffOwner);
       for (int i = 0; i < NS; ++i) owner[i] = -1;
+      grid_dep_wait();  // the operand tiles
+      asm volatile("fence.proxy.async.global;" ::: "memory");  // written by generic stores, read by bulk copies
       int gblk = 0, rel = -1;  // rel: stages 0 .. rel known released
       int64_t grow = 0, aslot = 0;
       auto release_upto = [&](int j) -> bool {
@@ -439,11 +587,12 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_port_sweep_tc(const PortTCArg
         const TcItem it = items[k];
         const PieceDesc pd = a.pieces[it.piece];
         const int Pn = pd.nports, n4 = it.hi + 1;
-        if (!mbar_wait_bounded(&sready[k & 1], (uint32_t)((k >> 1) & 1), a.wait_limit)) {
+        if (FUSED && !mbar_wait_bounded(&sready[k & 1], (uint32_t)((k >> 1) & 1), a.wait_limit)) {
           abort_flag = 1;
           break;
         }
-        const unsigned char* slot = scratch + (size_t)(k & 1) * slot_bytes;
+        const unsigned char* slot =
+            FUSED ? scratch + (size_t)(k & 1) * slot_bytes : a.stiles + (size_t)a.tile_off[it.piece] * P::kVec;
         const unsigned char* Sp = a.S16 + pd.h_off;
         // s_I tile of super-row I into the row buffer grow & 1, once the MMAs of the row two
         // before it (same buffer) are done
@@ -567,33 +716,43 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_port_sweep_tc(const PortTCArg
       }
       mma_commit(done);  // arrives once every MMA issued above has completed
     }
-  } else if (warp < 2 + kEpiWarps) {
-    // ---- epilogue warps (one per tensor-memory lane quadrant): u = u_base + sigma_j sigma_r y_I,
-    // w_out[e] = 2 u - w_in[e], super-row by super-row as the MMA issuer completes them
-    // (rready[I] completes once per subgraph that has a super-row I, so its phases are counted per
-    // barrier; sready[k & 1] also orders the sigma_r written with subgraph k's port vectors).
-    // Each warp releases y_I (rowread[I]) as soon as its tcgen05.ld has completed.
-    const int q = warp & 3;
-    uint32_t uses = 0;  // tid 64: parity of the next phase of each row barrier, one bit per super-row
+  } else if (!FUSED || warp < 2 + kEpiWarps) {
+    // ---- epilogue warps (a set: one per tensor-memory lane quadrant): u = u_base + sigma_j sigma_r y_I,
+    // w_out[e] = 2 u - w_in[e], super-row by super-row as the MMA issuer completes them, super-row I by
+    // set I mod kSets (a row's loads depend on each other in three steps; other sets' rows go on
+    // meanwhile).  rready[I] completes once per item that has a super-row I, so its phases are counted
+    // per barrier; one set waits for all of them, so none is missed or taken for the next.  A warp releases y_I (rowread[I]) as soon as its tcgen05.ld has completed.
+    constexpr int kSets = FUSED ? 1 : kEpiSets;
+    const int set = FUSED ? 0 : (warp - 2) / kEpiWarps, q = warp & 3;
+    const int lead = 64 + 32 * kEpiWarps * set;  // the set's first thread
+    uint32_t uses = 0;  // lead: parity of the next phase of each row barrier, one bit per super-row
     bool stop = false;
+    grid_dep_wait();  // the waves, sigma_r
     for (int k = 0; k < npc && !stop; ++k) {
       const TcItem it = items[k];
       const PieceDesc pd = a.pieces[it.piece];
       const int Pn = pd.nports, n4 = it.hi + 1;
       const float sj = a.sig_s[it.piece];
-      if (tid == 64) flags[1] = mbar_wait_bounded(&sready[k & 1], (uint32_t)((k >> 1) & 1), a.wait_limit) ? 0 : 1;
-      epi_sync();
-      stop = flags[1] != 0;
-      epi_sync();
-      for (int I = n4 - 1; I >= 0 && !stop; --I) {
-        // the four warps decide together: one lane waits, the named barrier publishes the outcome
-        if (tid == 64) {
-          flags[1] = mbar_wait_bounded(&rready[I], (uses >> I) & 1u, a.wait_limit) ? 0 : 1;
-          uses ^= 1u << I;
-        }
-        epi_sync();
+      float* const sg = ssig[FUSED ? (k & 1) : set];
+      if constexpr (FUSED) {
+        // sready[k & 1] also orders the sigma_r written with the item's port vectors
+        if (tid == lead)
+          flags[1] = mbar_wait_bounded(&sready[k & 1], (uint32_t)((k >> 1) & 1), a.wait_limit) ? 0 : 1;
+        epi_sync(set);
         stop = flags[1] != 0;
-        epi_sync();
+        epi_sync(set);
+      } else {
+        epi_sync(set);  // the set is through with the item before
+        if (tid - lead < R) sg[tid - lead] = __ldcg(a.ssig + (size_t)it.piece * R + tid - lead);
+      }
+      for (int I = n4 - 1; I >= 0 && !stop; --I) {
+        if (I % kSets != set) continue;
+        // the set decides together: one lane waits, the named barrier publishes the outcome
+        if (tid == lead) flags[1 + set] = mbar_wait_bounded(&rready[I], (uses >> I) & 1u, a.wait_limit) ? 0 : 1;
+        uses ^= 1u << I;
+        epi_sync(set);
+        stop = flags[1 + set] != 0;
+        epi_sync(set);
         if (stop) break;
         tc_fence_after();
         uint32_t v[R];
@@ -602,65 +761,64 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_port_sweep_tc(const PortTCArg
         __syncwarp();
         if (lane == 0) mbar_arrive(&rowread[I]);
         const int p = I * kSB + 32 * q + lane;
-        if (p < Pn && it.part >= 0) {
-          // part of a subgraph: this item's share of y
-          const float gs = sj * a.gscale[pd.port_off + p];
-          float4* o = reinterpret_cast<float4*>(a.part + it.part + (size_t)p * R);
-#pragma unroll
-          for (int k4 = 0; k4 < R / 4; ++k4)
-            o[k4] = make_float4(gs * ssig[k & 1][4 * k4] * __uint_as_float(v[4 * k4]),
-                                gs * ssig[k & 1][4 * k4 + 1] * __uint_as_float(v[4 * k4 + 1]),
-                                gs * ssig[k & 1][4 * k4 + 2] * __uint_as_float(v[4 * k4 + 2]),
-                                gs * ssig[k & 1][4 * k4 + 3] * __uint_as_float(v[4 * k4 + 3]));
-        } else if (p < Pn) {
+        if (p < Pn) {
           const int port = pd.port_off + p;
-          const float4* ub = reinterpret_cast<const float4*>(a.ubase + (size_t)port * R);
-          const int e0 = a.port_end_ptr[port], e1 = a.port_end_ptr[port + 1];
           const float gs = sj * a.gscale[port];  // y = D^-1 (sigma_j S'') (sigma_r s'')
 #pragma unroll
-          for (int k4 = 0; k4 < R / 4; ++k4) {
-            const float4 b4 = __ldg(ub + k4);
-            const float u0 = b4.x + gs * ssig[k & 1][4 * k4] * __uint_as_float(v[4 * k4]);
-            const float u1 = b4.y + gs * ssig[k & 1][4 * k4 + 1] * __uint_as_float(v[4 * k4 + 1]);
-            const float u2 = b4.z + gs * ssig[k & 1][4 * k4 + 2] * __uint_as_float(v[4 * k4 + 2]);
-            const float u3 = b4.w + gs * ssig[k & 1][4 * k4 + 3] * __uint_as_float(v[4 * k4 + 3]);
-            v[4 * k4] = __float_as_uint(u0);
-            v[4 * k4 + 1] = __float_as_uint(u1);
-            v[4 * k4 + 2] = __float_as_uint(u2);
-            v[4 * k4 + 3] = __float_as_uint(u3);
-          }
-          for (int e = e0; e < e1; ++e) {
-            const float4* wi = reinterpret_cast<const float4*>(a.wprev + (size_t)a.twin[e] * R);
-            float4* wo = reinterpret_cast<float4*>(a.wnext + (size_t)e * R);
+          for (int c = 0; c < R; ++c) v[c] = __float_as_uint(gs * sg[c] * __uint_as_float(v[c]));
+          if (it.part >= 0) {
+            // part of a subgraph: this item's share of y
+            uint4* o = reinterpret_cast<uint4*>(a.part + it.part + (size_t)p * R);
+#pragma unroll
+            for (int k4 = 0; k4 < R / 4; ++k4) o[k4] = make_uint4(v[4 * k4], v[4 * k4 + 1], v[4 * k4 + 2], v[4 * k4 + 3]);
+          } else {
+            const float4* ub = reinterpret_cast<const float4*>(a.ubase + (size_t)port * R);
+            const int e0 = a.port_end_ptr[port], e1 = a.port_end_ptr[port + 1];
 #pragma unroll
             for (int k4 = 0; k4 < R / 4; ++k4) {
-              const float4 w = __ldg(wi + k4);
-              wo[k4] = make_float4(2.f * __uint_as_float(v[4 * k4]) - w.x, 2.f * __uint_as_float(v[4 * k4 + 1]) - w.y,
-                                   2.f * __uint_as_float(v[4 * k4 + 2]) - w.z,
-                                   2.f * __uint_as_float(v[4 * k4 + 3]) - w.w);
+              const float4 b4 = __ldg(ub + k4);
+              v[4 * k4] = __float_as_uint(b4.x + __uint_as_float(v[4 * k4]));
+              v[4 * k4 + 1] = __float_as_uint(b4.y + __uint_as_float(v[4 * k4 + 1]));
+              v[4 * k4 + 2] = __float_as_uint(b4.z + __uint_as_float(v[4 * k4 + 2]));
+              v[4 * k4 + 3] = __float_as_uint(b4.w + __uint_as_float(v[4 * k4 + 3]));
+            }
+            for (int e = e0; e < e1; ++e) {
+              const float4* wi = reinterpret_cast<const float4*>(a.wprev + (size_t)a.twin[e] * R);
+              float4* wo = reinterpret_cast<float4*>(a.wnext + (size_t)e * R);
+#pragma unroll
+              for (int k4 = 0; k4 < R / 4; ++k4) {
+                const float4 w = __ldg(wi + k4);
+                wo[k4] = make_float4(2.f * __uint_as_float(v[4 * k4]) - w.x, 2.f * __uint_as_float(v[4 * k4 + 1]) - w.y,
+                                     2.f * __uint_as_float(v[4 * k4 + 2]) - w.z,
+                                     2.f * __uint_as_float(v[4 * k4 + 3]) - w.w);
+              }
             }
           }
         }
+        __syncwarp();
       }
       if (stop) {
-        if (tid == 64) abort_flag = 1;
+        if (tid == lead) abort_flag = 1;
         break;
       }
-      epi_sync();
-      if (tid == 64) mbar_arrive(&slotfree[k & 1]);
+      if constexpr (FUSED) {
+        epi_sync(set);
+        if (tid == lead) mbar_arrive(&slotfree[k & 1]);
+      }
     }
-  } else {
+  } else if constexpr (FUSED) {
     // ---- vector warps: the port vectors s of subgraph k, one gather pass (FP32 values to a
     // staging area and the column maxima), then the fp16 split into the scratch slot k & 1.  Slot
     // and sigma_r of subgraph k are free again once the epilogue of subgraph k - 2 is done
     // (slotfree[k & 1] completes once per subgraph of that slot).
     const int vt = tid - 32 * (2 + kEpiWarps);
     const int vw = vt >> 5;
+    grid_dep_wait();  // the waves
     for (int k = 0; k < npc; ++k) {
       if (k >= 2) {
-        if (vt == 0) flags[2] = mbar_wait_bounded(&slotfree[k & 1], (uint32_t)(((k >> 1) - 1) & 1), a.wait_limit) ? 0 : 1;
+        if (vt == 0) flags[4] = mbar_wait_bounded(&slotfree[k & 1], (uint32_t)(((k >> 1) - 1) & 1), a.wait_limit) ? 0 : 1;
         vec_sync();
-        const bool stop = flags[2] != 0;
+        const bool stop = flags[4] != 0;
         vec_sync();
         if (stop) {
           if (vt == 0) abort_flag = 1;
@@ -768,25 +926,27 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_port_sweep_tc(const PortTCArg
 // order, w_out[e] = 2u - w_in[e]; thread = (port, four columns).
 template <int R>
 __global__ void __launch_bounds__(256) k_port_finish_tc(const PortTCArgs a) {
+  grid_dep_launch();
   const TcSplit sp = a.splits[blockIdx.y];
   const PieceDesc pd = a.pieces[sp.piece];
+  grid_dep_wait();
   const int i = blockIdx.x * 256 + threadIdx.x;
   const int p = i / (R / 4), k4 = i % (R / 4);
   if (p >= pd.nports) return;
   const int port = pd.port_off + p, I = p / kSB;
   const int e0 = a.port_end_ptr[port], e1 = a.port_end_ptr[port + 1];
-  float4 u = reinterpret_cast<const float4*>(a.ubase + (size_t)port * R)[k4];
+  float4 u = __ldcg(reinterpret_cast<const float4*>(a.ubase + (size_t)port * R) + k4);
   float4 y = make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
   for (int q = 0; q < kTcMaxSplit; ++q) {
     if (q < sp.nitems && sp.hi[q] >= I) {
-      const float4 x = reinterpret_cast<const float4*>(a.part + sp.part + ((size_t)q * pd.nports + p) * R)[k4];
+      const float4 x = __ldcg(reinterpret_cast<const float4*>(a.part + sp.part + ((size_t)q * pd.nports + p) * R) + k4);
       y.x += x.x, y.y += x.y, y.z += x.z, y.w += x.w;
     }
   }
   u.x += y.x, u.y += y.y, u.z += y.z, u.w += y.w;
   for (int e = e0; e < e1; ++e) {
-    const float4 w = reinterpret_cast<const float4*>(a.wprev + (size_t)a.twin[e] * R)[k4];
+    const float4 w = __ldcg(reinterpret_cast<const float4*>(a.wprev + (size_t)a.twin[e] * R) + k4);
     reinterpret_cast<float4*>(a.wnext + (size_t)e * R)[k4] =
         make_float4(2.f * u.x - w.x, 2.f * u.y - w.y, 2.f * u.z - w.z, 2.f * u.w - w.w);
   }
@@ -801,6 +961,10 @@ TcPlan tc_plan(const PieceDesc* pd, int npieces, int R, int ctas) {
   for (int j = 0; j < npieces; ++j) {
     const int n4 = n_super(pd[j].nports);
     total += n4 * (n4 + 1) / 2 + (n4 > 0 ? kItemCost : 0.0);
+  }
+  for (int j = 0; j < npieces; ++j) {
+    pl.tile_off.push_back((int32_t)pl.tiles);
+    pl.tiles += n_super(pd[j].nports);
   }
   const double share = total / std::max(1, ctas);
   std::vector<std::pair<double, TcItem>> items;
@@ -891,47 +1055,58 @@ cudaError_t launch_port_records(int nports, const int32_t* port_end_ptr, const i
   return cudaGetLastError();
 }
 
+template <int R>
+static const void* tc_kernel(bool lo, bool fused) {
+  return lo ? (fused ? (const void*)k_port_sweep_tc<R, true, true> : (const void*)k_port_sweep_tc<R, true, false>)
+            : (fused ? (const void*)k_port_sweep_tc<R, false, true> : (const void*)k_port_sweep_tc<R, false, false>);
+}
+
 cudaError_t port_tc_configure(int R) {
-  cudaError_t e = cudaErrorInvalidValue;
-  switch (R) {
-    case 16:
-      e = cudaFuncSetAttribute(k_port_sweep_tc<16, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                               (int)port_tc_smem_bytes(16, true));
-      if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(k_port_sweep_tc<16, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)port_tc_smem_bytes(16, false));
-      break;
-    case 32:
-      e = cudaFuncSetAttribute(k_port_sweep_tc<32, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                               (int)port_tc_smem_bytes(32, true));
-      if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(k_port_sweep_tc<32, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)port_tc_smem_bytes(32, false));
-      break;
-    default: break;
+  if (R != 16 && R != 32) return cudaErrorInvalidValue;
+  cudaError_t e = cudaSuccess;
+  for (int i = 0; i < 4 && e == cudaSuccess; ++i) {
+    const void* k = R == 16 ? tc_kernel<16>(i & 1, i & 2) : tc_kernel<32>(i & 1, i & 2);
+    e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)port_tc_smem_bytes(R, true));
   }
+  if (e == cudaSuccess)
+    e = cudaFuncSetAttribute(R == 16 ? (const void*)k_port_vec_tc<16> : (const void*)k_port_vec_tc<32>,
+                             cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kVecTcSmemMax);
   return e;
 }
 
-cudaError_t launch_port_sweep_tc(const PortTCArgs& a, int R, bool lo, int grid, int nsplits, int max_split_ports,
-                                 cudaStream_t st) {
+cudaError_t launch_port_sweep_tc(const PortTCArgs& a, int R, bool lo, int npieces, int max_ends, int grid, int nsplits,
+                                 int max_split_ports, cudaStream_t st) {
   if (grid <= 0) return cudaSuccess;
-  const size_t smem = port_tc_smem_bytes(R, lo);
-  if (R == 16) {
-    if (lo) k_port_sweep_tc<16, true><<<grid, kTcThreads, smem, st>>>(a);
-    else k_port_sweep_tc<16, false><<<grid, kTcThreads, smem, st>>>(a);
-  } else if (R == 32) {
-    if (lo) k_port_sweep_tc<32, true><<<grid, kTcThreads, smem, st>>>(a);
-    else k_port_sweep_tc<32, false><<<grid, kTcThreads, smem, st>>>(a);
-  } else {
-    return cudaErrorInvalidValue;
-  }
-  cudaError_t e = cudaGetLastError();
+  if (R != 16 && R != 32) return cudaErrorInvalidValue;
+  PortTCArgs args = a;
+  void* av[] = {&args};
+  const bool fused = a.stiles == nullptr;
+  // early: the kernel's CTAs may start while the launch before still runs; they wait for its results
+  // themselves, and read them past the L1 cache.  Not the sweep proper: its epilogue reads a row of
+  // waves per lane, in 16-byte pieces that need the L1 cache.
+  auto launch = [&](const void* k, dim3 g, int threads, size_t smem, bool early) {
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = g;
+    cfg.blockDim = dim3(threads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cfg.attrs = at;
+    cfg.numAttrs = early ? 1 : 0;
+    return cudaLaunchKernelExC(&cfg, k, av);
+  };
+  cudaError_t e = cudaSuccess;
+  if (!fused)
+    e = launch(R == 16 ? (const void*)k_port_vec_tc<16> : (const void*)k_port_vec_tc<32>, dim3(npieces, R / kVecCols),
+               kVecTcThreads, port_vec_tc_smem_bytes(max_ends), true);
+  if (e != cudaSuccess) return e;
+  const void* k = R == 16 ? tc_kernel<16>(lo, fused) : tc_kernel<32>(lo, fused);
+  e = launch(k, dim3(grid), kTcThreads, port_tc_smem_bytes(R, lo), false);
   if (e != cudaSuccess || nsplits == 0) return e;
-  const dim3 g((max_split_ports * (R / 4) + 255) / 256, nsplits);
-  if (R == 16) k_port_finish_tc<16><<<g, 256, 0, st>>>(a);
-  else k_port_finish_tc<32><<<g, 256, 0, st>>>(a);
-  return cudaGetLastError();
+  return launch(R == 16 ? (const void*)k_port_finish_tc<16> : (const void*)k_port_finish_tc<32>,
+                dim3((max_split_ports * (R / 4) + 255) / 256, nsplits), 256, 0, true);
 }
 
 cudaError_t launch_gather_port_blocks(const PieceDesc* pieces, int npieces, const int32_t* port_local, int Rs, int b,

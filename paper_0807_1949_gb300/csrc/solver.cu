@@ -90,7 +90,7 @@ struct vtm_solver {
   int32_t npieces = 0, nports = 0;
   size_t elem = 8;
 
-  DevBuf pieces, factor, factor_u, bt, xc, w[2], port_local, port_end_ptr, twin, invz_t, status, port_rec;
+  DevBuf pieces, factor, factor_u, bt, xc, w[2], port_local, port_end_ptr, twin, invz_t, status;
   DevBuf a_rowptr, a_col, a_val, vc_ptr, vc_copy, copy_vertex, share;
   DevBuf vb, vx, vxt, vr, vrt, norms, nparts;  // nparts: per-block partial sums of the residual norms
   double* h_norms = nullptr;  // pinned: [R] residual^2, [R] b^2 ... plus status
@@ -151,11 +151,14 @@ struct vtm_solver {
   DevBuf res_ctas, res_units, res_ports, res_ps, res_xch;
   int res_grid = 0, res_pieces = 0;
   size_t res_smem = 0;
-  DevBuf S16, sig16, tc_scratch;     // tensor-core form: fp16 hi / lo blocks, sigma_j, s^T slots
+  DevBuf S16, sig16;                 // tensor-core form: fp16 hi / lo blocks, sigma_j
+  DevBuf tc_stiles, tc_tile_off, tc_ssig, tc_cpl_end;  // separate port vectors: operand tiles, their places, sigma_r
+  DevBuf tc_scratch, port_rec;       // fused port vectors: s^T slots, gather records
+  int tc_n4max = 0, tc_max_ends = 0;
   DevBuf gscale;                     // tensor-core form: sqrt(S_pp) per port (diagonal balance)
   DevBuf tc_items, tc_cta_item, tc_splits, tc_part;  // division of the subgraphs among CTAs
   int tc_nsplits = 0, tc_split_ports = 0;
-  int tc_grid = 0, tc_n4max = 0, tc_tmem_cols = 0;
+  int tc_grid = 0, tc_tmem_cols = 0;
   int64_t tc_bytes_hi = 0, tc_bytes_all = 0;  // bytes a sweep streams without / with the lo half
   DevBuf Sh, hscale;                 // FP16 copy of S_j and the scale of each of its tiles
   bool port_half = false;            // the port sweep reads the FP16 copy (tensor cores: hi half only)
@@ -1051,6 +1054,11 @@ static void launch_port(vtm_solver* s) {
       t.gscale = s->gscale.as<float>();
       t.scratch = s->tc_scratch.as<unsigned char>();
       t.n4max = s->tc_n4max;
+      t.prec = s->port_rec.as<int4>();
+      t.cpl_end = s->tc_cpl_end.as<int32_t>();
+      t.stiles = s->tc_stiles.as<unsigned char>();  // null: fused
+      t.tile_off = s->tc_tile_off.as<int32_t>();
+      t.ssig = s->tc_ssig.as<float>();
       t.tmem_cols = s->tc_tmem_cols;
       t.ubase = s->ubase.as<float>();
       t.wprev = s->w[s->cur].as<float>();
@@ -1059,11 +1067,11 @@ static void launch_port(vtm_solver* s) {
       t.twin = s->twin.as<int32_t>();
       t.invz = s->invz_t.as<float>();
       t.cpl = couple_ref<float>(s);
-      t.prec = s->port_rec.as<int4>();
       t.status = s->status.as<int>();
       t.wait_limit = s->wait_limit;
-      VTM_CUDA(launch_port_sweep_tc(t, s->R, !s->port_half, s->tc_grid, s->tc_nsplits, s->tc_split_ports, s->stream));
-      s->launches += s->tc_nsplits > 0 ? 2 : 1;
+      VTM_CUDA(launch_port_sweep_tc(t, s->R, !s->port_half, s->np_lo, s->tc_max_ends, s->tc_grid, s->tc_nsplits,
+                                    s->tc_split_ports, s->stream));
+      s->launches += 1 + (s->tc_stiles.p ? 1 : 0) + (s->tc_nsplits > 0 ? 1 : 0);
       return;
     }
   }
@@ -1144,7 +1152,7 @@ static int64_t launches_per_batch(const vtm_solver* s, int k) {
   const int64_t band = (s->np_lo > 0) + (s->np_hi > 0);
   if (!s->port_form || k < 2) return (int64_t)k * band;
   if (s->resident) return 1 + band;
-  const int64_t port = (s->np_lo > 0 ? (s->port_tc && s->tc_nsplits == 0 ? 1 : 2) : 0) + (s->np_hi > 0);
+  const int64_t port = (s->np_lo > 0 ? (s->port_tc ? 1 + (s->tc_stiles.p ? 1 : 0) + (s->tc_nsplits > 0 ? 1 : 0) : 2) : 0) + (s->np_hi > 0);
   return (int64_t)(k - 1) * port + band;
 }
 
@@ -1261,18 +1269,38 @@ static void choose_form(vtm_solver* s, const vtm_setup_opts* o, int64_t s_tiles,
     s->tc_nsplits = (int)pl.splits.size();
     s->tc_split_ports = pl.max_split_ports;
     s->tc_grid = pl.items.empty() ? 0 : (int)pl.cta_item.size() - 1;
-    s->tc_n4max = n4max;
     s->tc_tmem_cols = tmem_cols;
-    s->tc_scratch.alloc((size_t)s->tc_grid * ((size_t)2 * n4max * s->R * 512 + (size_t)n4max * 128 * s->R * 4));
+    s->tc_n4max = n4max;
+    for (const PieceDesc& d : lo) s->tc_max_ends = std::max(s->tc_max_ends, d.nends);
+    // The port vectors: a launch of their own up to kTcSeparate items per CTA, fused beyond (there the
+    // gathers hide behind the next items' blocks, and the operand tiles would pass through HBM).
+    // 64^3 with 32 right-hand sides (1.2 items per CTA) 0.089 ms separate, 0.193 fused; 128^3 (3.4)
+    // 0.557 either way; 256^3 (27) 3.86 fused.
+    constexpr double kTcSeparate = 2.0;
+    const bool separate = (double)pl.items.size() <= kTcSeparate * nsm &&
+                          port_vec_tc_smem_bytes(s->tc_max_ends) <= kVecTcSmemMax;
+    if (separate) {
+      upload(s->tc_tile_off, pl.tile_off, s->stream);
+      VTM_CUDA(cudaStreamSynchronize(s->stream));
+      s->tc_stiles.alloc((size_t)std::max<int64_t>(1, pl.tiles) * s->R * 512);
+      s->tc_ssig.alloc((size_t)s->np_lo * s->R * sizeof(float));
+      if (s->coupled) {
+        s->tc_cpl_end.alloc(s->cp_oth.bytes);
+        VTM_CUDA(launch_coupling_ends(s->pieces_lo.as<PieceDesc>(), s->np_lo, s->twin.as<int32_t>(), couple_ref<float>(s),
+                                      s->tc_cpl_end.as<int32_t>(), s->stream));
+      }
+    } else {
+      s->tc_scratch.alloc((size_t)s->tc_grid * ((size_t)2 * n4max * s->R * 512 + (size_t)n4max * 128 * s->R * 4));
+      s->port_rec.alloc((size_t)std::max(1, s->nports) * 3 * sizeof(int4));
+      VTM_CUDA(launch_port_records(s->nports, s->port_end_ptr.as<int32_t>(), s->twin.as<int32_t>(),
+                                   s->invz_t.as<float>(), couple_ref<float>(s), s->port_rec.as<int4>(), s->stream));
+    }
     s->S16.alloc((size_t)std::max<int64_t>(1024, h_bytes));
     s->sig16.alloc((size_t)std::max(1, s->np_lo) * sizeof(float));
     s->gscale.alloc((size_t)std::max(1, s->nports) * sizeof(float));
     VTM_CUDA(cudaMemsetAsync(s->gscale.p, 0, s->gscale.bytes, s->stream));
     s->tc_bytes_all = h_bytes;
     s->tc_bytes_hi = h_bytes / 2;
-    s->port_rec.alloc((size_t)std::max(1, s->nports) * 3 * sizeof(int4));
-    VTM_CUDA(launch_port_records(s->nports, s->port_end_ptr.as<int32_t>(), s->twin.as<int32_t>(),
-                                 s->invz_t.as<float>(), couple_ref<float>(s), s->port_rec.as<int4>(), s->stream));
     VTM_CUDA(port_tc_configure(s->R));
   } else {
     s->port_s.alloc((size_t)std::max(1, s->nports) * s->R * sizeof(T));

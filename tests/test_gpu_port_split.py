@@ -76,3 +76,13 @@ def test_pipelined_band_sweep(vtmlib, dims, block, nrhs):
     assert _rel(s.copies(), copies) <= TOL_FP32
     if len(osplit.vtl):
         assert _rel(s.get_state(), waves[:, _line_map(part, osplit)]) <= TOL_FP32
+
+
+# tensor-core port sweep, port vectors in a launch of their own: 75 subgraphs of up to four super-rows cut
+# in two, 8 of six cut into more (FP16; their FP32 responses stay resident); fused: 504 of one to three
+@pytest.mark.parametrize("nrhs", [16, 32])
+@pytest.mark.parametrize("kind", ["fp32", "fp16"])
+@pytest.mark.parametrize("dims,block", [((40, 37, 21), (8, 8, 8)), ((26, 26, 26), (13, 13, 13)),
+                                        ((52, 47, 41), (6, 6, 6))])
+def test_tensor_core_sweep(vtmlib, dims, block, nrhs, kind):
+    _check(vtmlib, dims, block, nrhs, "fp32", "fp16" if kind == "fp16" else "native", 6, TOL[kind])
