@@ -41,6 +41,13 @@ struct SweepArgs {
                                // piece at row_off (nullptr: y goes through xc, TF == TV)
   CoupleRef<TV> cpl;           // coupled lines: per-port coupling lists (cpl.ptr == nullptr: none)
   const unsigned char* wt;     // tensor-core factor of sweep_wide_tc.cu (nullptr: not built)
+  // Wide kernels, unit sources at the ports instead of b̃ and waves (the columns of S_j): CTA (j, y)
+  // solves for the R ports from (unit_b0 + y) R on, for the rows from port
+  // floor((unit_b0 + y) R / unit_gran) unit_gran on, into xc + y unit_stride; no waves are read or written.
+  int unit = 0;
+  int unit_b0 = 0;
+  int unit_gran = 1;
+  int64_t unit_stride = 0;
 };
 
 size_t sweep_smem_bytes(size_t elem, int R, int stages, int slot_elems, int ys_elems, int win_elems);
@@ -73,14 +80,16 @@ size_t wide_tc_smem_bytes(int R);
 cudaError_t wide_tc_configure(int R);
 cudaError_t launch_wide_tc_factor(const PieceDesc* pieces, int npieces, int max_groups, const float* band,
                                   unsigned char* wt, cudaStream_t st);
-cudaError_t launch_sweep_wide_tc(const SweepArgs<float, float>& a, int R, int npieces, cudaStream_t st);
+cudaError_t launch_sweep_wide_tc(const SweepArgs<float, float>& a, int R, int npieces, cudaStream_t st,
+                                 int batches = 1);
 
 // Wide variant (R = 16, 32): vectors spill to xc, a circular window of 512 rows stays in shared memory.
 size_t sweep_wide_smem_bytes(size_t elem, int R, int stages, int slot_elems, int cap);
 template <typename TF, typename TV>
 cudaError_t sweep_wide_configure(int R, size_t smem);
 template <typename TF, typename TV>
-cudaError_t launch_sweep_wide(const SweepArgs<TF, TV>& a, int R, int npieces, size_t smem, cudaStream_t st);
+cudaError_t launch_sweep_wide(const SweepArgs<TF, TV>& a, int R, int npieces, size_t smem, cudaStream_t st,
+                              int batches = 1);
 // One segment of a port sweep (port.cu): the tiles (I0, J0) .. (I1, J1) of a subgraph's lower block
 // triangle, row by row.
 struct PortSeg {
@@ -147,7 +156,8 @@ template <typename T>
 cudaError_t launch_port_sweep(const PortArgs<T>& a, int R, int nports, int grid, size_t smem, cudaStream_t st);
 template <typename T>
 cudaError_t launch_gather_port_response(const PieceDesc* pieces, int npieces, const int32_t* port_local, int Rs, int b,
-                                        const T* xc, T* S, int layout, cudaStream_t st);
+                                        const T* xc, T* S, int layout, cudaStream_t st, int batches = 1,
+                                        int64_t stride = 0);
 template <typename T>
 cudaError_t launch_gather_ports(const PieceDesc* pieces, int npieces, const int32_t* port_local, int R, const T* xc,
                                 T* ubase, cudaStream_t st);
@@ -209,7 +219,8 @@ ResPlan res_plan(const PieceDesc* pd, int npieces, size_t elem, int R, int nsm);
 void res_plan_ends(ResPlan& pl, const int32_t* port_end_ptr);  // host copy of the end lists
 template <typename T>
 cudaError_t launch_gather_port_dense(const ResPieceS* ps, int n, const PieceDesc* pieces, const int32_t* port_local,
-                                     int Rs, int b, const T* xc, T* S, cudaStream_t st);
+                                     int Rs, int b, const T* xc, T* S, cudaStream_t st, int batches = 1,
+                                     int64_t stride = 0);
 template <typename T>
 cudaError_t port_resident_configure(int R, size_t smem, int* ctas_per_sm);
 // a.sweeps sweeps in one cooperative launch (after clearing the exchange buffers, xch_bytes in all).
@@ -286,7 +297,8 @@ cudaError_t port_tc_configure(int R);
 cudaError_t launch_port_sweep_tc(const PortTCArgs& a, int R, bool lo, int npieces, int max_ends, int grid, int nsplits,
                                  int max_split_ports, cudaStream_t st);
 cudaError_t launch_gather_port_blocks(const PieceDesc* pieces, int npieces, const int32_t* port_local, int Rs, int b,
-                                      const float* xc, float* S32, cudaStream_t st);
+                                      const float* xc, float* S32, cudaStream_t st, int batches = 1,
+                                      int64_t stride = 0);
 cudaError_t launch_port_blocks_to_f16(const PieceDesc* pieces, int npieces, const float* S32, unsigned char* S16,
                                       float* sig, float* gscale, cudaStream_t st);
 

@@ -150,13 +150,16 @@ __host__ __device__ int64_t port_tiles(int nports) {
 }
 
 // S_j columns from unit-source solves: column cc = b * Rs + r of S_j is x at the ports for the
-// unit source at port cc (xc holds copies x Rs).  Only tiles with I >= J are written.
+// unit source at port cc (x0 holds copies x Rs per batch, blockIdx.y: batch b0 + y).  Only tiles with I >= J are written.
 template <typename T>
 __global__ void k_gather_port_response(const PieceDesc* __restrict__ pieces, const int32_t* __restrict__ port_local,
-                                       int Rs, int b, const T* __restrict__ xc, T* __restrict__ S, int layout) {
+                                       int Rs, int b0, const T* __restrict__ x0, int64_t stride, T* __restrict__ S,
+                                       int layout) {
   const PieceDesc pd = pieces[blockIdx.x];
+  const int b = b0 + (int)blockIdx.y;
+  const T* xc = x0 + (size_t)blockIdx.y * stride;
   constexpr int V = Vec16<T>::V;
-  for (int i = threadIdx.x; i < pd.nports * Rs; i += blockDim.x) {
+  for (int i = b * Rs / kNB * kNB * Rs + threadIdx.x; i < pd.nports * Rs; i += blockDim.x) {
     const int q = i / Rs, r = i % Rs;
     const int cc = b * Rs + r;
     if (cc >= pd.nports) continue;
@@ -1222,9 +1225,9 @@ cudaError_t launch_port_to_half(const PieceDesc* pieces, int npieces, const floa
 
 template <typename T>
 cudaError_t launch_gather_port_response(const PieceDesc* pieces, int npieces, const int32_t* port_local, int Rs, int b,
-                                        const T* xc, T* S, int layout, cudaStream_t st) {
+                                        const T* xc, T* S, int layout, cudaStream_t st, int batches, int64_t stride) {
   if (npieces <= 0) return cudaSuccess;
-  k_gather_port_response<T><<<npieces, 256, 0, st>>>(pieces, port_local, Rs, b, xc, S, layout);
+  k_gather_port_response<T><<<dim3(npieces, batches), 256, 0, st>>>(pieces, port_local, Rs, b, xc, stride, S, layout);
   return cudaGetLastError();
 }
 
@@ -1240,7 +1243,7 @@ cudaError_t launch_gather_ports(const PieceDesc* pieces, int npieces, const int3
   template cudaError_t port_sweep_configure<T>(int, const PortShape&, bool, int*);                             \
   template cudaError_t launch_port_sweep<T>(const PortArgs<T>&, int, int, int, size_t, cudaStream_t);          \
   template cudaError_t launch_gather_port_response<T>(const PieceDesc*, int, const int32_t*, int, int, const T*, \
-                                                      T*, int, cudaStream_t);                                      \
+                                                      T*, int, cudaStream_t, int, int64_t);                        \
   template cudaError_t launch_gather_ports<T>(const PieceDesc*, int, const int32_t*, int, const T*, T*, cudaStream_t);
 VTM_PORT_INST(float)
 VTM_PORT_INST(double)

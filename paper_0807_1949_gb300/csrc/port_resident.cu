@@ -391,11 +391,13 @@ void res_plan_ends(ResPlan& pl, const int32_t* port_end_ptr) {
 // (i, c) and (c, i): S_j is symmetric up to the rounding of those solves.
 template <typename T>
 __global__ void k_gather_port_dense(const ResPieceS* __restrict__ ps, const PieceDesc* __restrict__ pieces,
-                                    const int32_t* __restrict__ port_local, int Rs, int b, const T* __restrict__ xc,
-                                    T* __restrict__ S) {
+                                    const int32_t* __restrict__ port_local, int Rs, int b0, const T* __restrict__ x0,
+                                    int64_t stride, T* __restrict__ S) {
   const ResPieceS p = ps[blockIdx.x];
+  const int b = b0 + (int)blockIdx.y;
+  const T* xc = x0 + (size_t)blockIdx.y * stride;
   const int64_t copy0 = pieces[p.piece].copy_off;
-  for (int i = threadIdx.x; i < p.n * Rs; i += blockDim.x) {
+  for (int i = b * Rs / kNB * kNB * Rs + threadIdx.x; i < p.n * Rs; i += blockDim.x) {
     const int q = i / Rs, r = i % Rs;
     const int cc = b * Rs + r;
     if (cc >= p.n || q / kNB < cc / kNB) continue;
@@ -407,9 +409,9 @@ __global__ void k_gather_port_dense(const ResPieceS* __restrict__ ps, const Piec
 
 template <typename T>
 cudaError_t launch_gather_port_dense(const ResPieceS* ps, int n, const PieceDesc* pieces, const int32_t* port_local,
-                                     int Rs, int b, const T* xc, T* S, cudaStream_t st) {
+                                     int Rs, int b, const T* xc, T* S, cudaStream_t st, int batches, int64_t stride) {
   if (n <= 0) return cudaSuccess;
-  k_gather_port_dense<T><<<n, 256, 0, st>>>(ps, pieces, port_local, Rs, b, xc, S);
+  k_gather_port_dense<T><<<dim3(n, batches), 256, 0, st>>>(ps, pieces, port_local, Rs, b, xc, stride, S);
   return cudaGetLastError();
 }
 
@@ -451,7 +453,7 @@ cudaError_t launch_port_resident(const ResArgs<T>& a, int R, int grid, size_t sm
 
 #define VTM_RES_INST(T)                                                                                           \
   template cudaError_t launch_gather_port_dense<T>(const ResPieceS*, int, const PieceDesc*, const int32_t*, int, int, \
-                                                   const T*, T*, cudaStream_t);                                   \
+                                                   const T*, T*, cudaStream_t, int, int64_t);                     \
   template cudaError_t port_resident_configure<T>(int, size_t, int*);                                             \
   template cudaError_t launch_port_resident<T>(const ResArgs<T>&, int, int, size_t, size_t, cudaStream_t);
 VTM_RES_INST(float)

@@ -281,9 +281,12 @@ size_t port_tc_smem_bytes(int R, bool) { return R == 16 ? Plan<16>::kAlloc : Pla
 // S_j columns cc = b * Rs + r from unit-source solves into FP32 128 x 128 row-major blocks of the
 // lower block triangle (block (I, J) at s_off + I (I + 1) / 2 + J; diagonal blocks whole).
 __global__ void k_gather_port_blocks(const PieceDesc* __restrict__ pieces, const int32_t* __restrict__ port_local,
-                                     int Rs, int b, const float* __restrict__ xc, float* __restrict__ S32) {
+                                     int Rs, int b0, const float* __restrict__ x0, int64_t stride,
+                                     float* __restrict__ S32) {
   const PieceDesc pd = pieces[blockIdx.x];
-  for (int i = threadIdx.x; i < pd.nports * Rs; i += blockDim.x) {
+  const int b = b0 + (int)blockIdx.y;
+  const float* xc = x0 + (size_t)blockIdx.y * stride;
+  for (int i = b * Rs / kSB * kSB * Rs + threadIdx.x; i < pd.nports * Rs; i += blockDim.x) {
     const int q = i / Rs, r = i % Rs;
     const int cc = b * Rs + r;
     if (cc >= pd.nports) continue;
@@ -1110,9 +1113,9 @@ cudaError_t launch_port_sweep_tc(const PortTCArgs& a, int R, bool lo, int npiece
 }
 
 cudaError_t launch_gather_port_blocks(const PieceDesc* pieces, int npieces, const int32_t* port_local, int Rs, int b,
-                                      const float* xc, float* S32, cudaStream_t st) {
+                                      const float* xc, float* S32, cudaStream_t st, int batches, int64_t stride) {
   if (npieces <= 0) return cudaSuccess;
-  k_gather_port_blocks<<<npieces, 256, 0, st>>>(pieces, port_local, Rs, b, xc, S32);
+  k_gather_port_blocks<<<dim3(npieces, batches), 256, 0, st>>>(pieces, port_local, Rs, b, xc, stride, S32);
   return cudaGetLastError();
 }
 

@@ -895,11 +895,16 @@ static void autotune_sweep(vtm_solver* s) {
 
 // ---------------------------------------------------------------- port-response form (port.cu)
 
-// S_j = P^T K_j^{-1} P from unit sources at the ports with zero incident waves: 32 port columns
-// per launch of the multi-RHS band sweep where it fits in shared memory, else the solver's own
-// sweep with its R columns.  Only the subgraphs of the main launch get an S_j: subgraphs flagged
-// ill-conditioned keep their FP64 band sweep every sweep (S_j in FP32 would carry the same
-// cancellation that made their FP32 factor fail).
+// S_j = P^T K_j^{-1} P from unit sources at the ports with zero incident waves: the multi-RHS band
+// sweep with 32 port columns (16 with 16 right-hand sides) per subgraph and batch where it fits in shared
+// memory, else the solver's own sweep with its R columns.  Of a batch only the rows from its first port
+// on are solved for: the solution of the forward pass is zero above them, and of S_j, which is
+// symmetric, only the blocks on and below the diagonal are kept, so the backward pass ends there too
+// (about half the work).  A launch takes several batches, eight CTAs per SM in all: with a launch per
+// batch 64 subgraphs left 88 of 152 SMs idle, and 512 took four waves of CTAs for 3.4.  FP32, 16^3
+// blocks: 64^3 29 -> 4.5 ms, 128^3 114 -> 39 ms.  Only the subgraphs of the main launch get an S_j:
+// subgraphs flagged ill-conditioned keep their FP64 band sweep every sweep (S_j in FP32 would carry the
+// same cancellation that made their FP32 factor fail).
 template <typename T>
 static void compute_port_response(vtm_solver* s, int64_t s_tiles) {
   cudaStream_t st = s->stream;
@@ -907,67 +912,86 @@ static void compute_port_response(vtm_solver* s, int64_t s_tiles) {
   if (!s->resident) s->S.alloc((size_t)s_tiles * kNB * kNB * sizeof(T));
   VTM_CUDA(cudaMemsetAsync(s->S.p, 0, s->S.bytes, st));
   const size_t kSmemMax = 227 * 1024;
-  int st_lo = 0;
-  size_t sm_lo = 0;
+  int st_lo = s->wide ? s->stages : 0;
+  size_t sm_lo = s->wide ? s->sweep_smem : 0;
   if (!s->wide && s->cap <= kWideWindow)
     for (int k : {8, 6, 4, 3, 2}) {
       const size_t b = sweep_wide_smem_bytes(sizeof(T), 32, k, s->slot_elems, s->cap);
       if (!st_lo && b <= kSmemMax) st_lo = k, sm_lo = b;
     }
+  auto gather = [&](int Rs, int b, const T* xc, int batches, int64_t stride) {
+    const PieceDesc* pieces = s->pieces_lo.as<PieceDesc>();
+    const int32_t* local = s->port_local.as<int32_t>();
+    if (s->resident) {
+      VTM_CUDA(launch_gather_port_dense<T>(s->res_ps.as<ResPieceS>(), s->res_pieces, pieces, local, Rs, b, xc,
+                                           s->S.as<T>(), st, batches, stride));
+      return;
+    }
+    if constexpr (sizeof(T) == 4) {
+      if (s->port_tc) {
+        VTM_CUDA(launch_gather_port_blocks(pieces, s->np_lo, local, Rs, b, xc, s->S.as<float>(), st, batches, stride));
+        return;
+      }
+    }
+    VTM_CUDA(launch_gather_port_response<T>(pieces, s->np_lo, local, Rs, b, xc, s->S.as<T>(),
+                                            s->port_div[0].sh.layout, st, batches, stride));
+  };
   cudaEvent_t e0, e1;
   VTM_CUDA(cudaEventCreate(&e0));
   VTM_CUDA(cudaEventCreate(&e1));
   VTM_CUDA(cudaEventRecord(e0, st));
-  if (st_lo) {
-    constexpr int Rs = 32;
-    DevBuf bt32, xc32, w0, wsc;
-    bt32.alloc((size_t)s->C * Rs * sizeof(T));
-    xc32.alloc((size_t)s->C * Rs * sizeof(T));
-    w0.alloc((size_t)std::max<int64_t>(1, s->E) * Rs * sizeof(T));
-    wsc.alloc(w0.bytes);
-    VTM_CUDA(cudaMemsetAsync(w0.p, 0, w0.bytes, st));
-    VTM_CUDA((sweep_wide_configure<T, T>(Rs, sm_lo)));
-    // the tensor-core form of the multi-RHS sweep where it applies (FP32 band factor, half-bandwidths
-    // <= 384), its factor kept only for these solves
-    DevBuf wt_tmp;
-    if constexpr (sizeof(T) == 4) {
-      size_t fb = 0, tb = 0;
-      VTM_CUDA(cudaMemGetInfo(&fb, &tb));
-      if (s->wt_ok && s->np_lo > 0 && (double)s->wt_bytes < 0.4 * (double)fb) {
-        wt_tmp.alloc((size_t)s->wt_bytes);
-        VTM_CUDA(cudaMemsetAsync(wt_tmp.p, 0, (size_t)wide_tc_zero_bytes(), st));
-        VTM_CUDA(wide_tc_configure(Rs));
-        VTM_CUDA(launch_wide_tc_factor(s->pieces_lo.as<PieceDesc>(), s->np_lo, s->wt_max_groups, s->factor.as<float>(),
-                                       wt_tmp.as<unsigned char>(), st));
-      }
-    }
+  if (st_lo && s->np_lo > 0) {
+    const int Rs = s->wide ? s->R : 32;
     const int nb = (s->max_ports + Rs - 1) / Rs;
-    for (int b = 0; b < nb; ++b) {
-      VTM_CUDA(launch_unit_rhs<T>(s->pieces.as<PieceDesc>(), np, s->port_local.as<int32_t>(), Rs, b, bt32.as<T>(), st));
-      if (s->np_lo > 0) {
-        SweepArgs<T, T> a = sweep_args<T, T>(s, 1, false);
-        a.bt = bt32.as<T>();
-        a.xc = xc32.as<T>();
-        a.wprev = w0.as<T>();
-        a.wnext = wsc.as<T>();
-        a.stages = st_lo;
-        a.withhold = -1;
-        a.yspill = nullptr;
-        a.cpl.ptr = nullptr;  // unit sources, zero waves: no coupling current
-        a.wt = wt_tmp.as<unsigned char>();
-        if constexpr (sizeof(T) == 4) {
-          if (a.wt) VTM_CUDA(launch_sweep_wide_tc(a, Rs, s->np_lo, st));
-          else VTM_CUDA((launch_sweep_wide<T, T>(a, Rs, s->np_lo, sm_lo, st)));
-        } else {
-          VTM_CUDA((launch_sweep_wide<T, T>(a, Rs, s->np_lo, sm_lo, st)));
+    SweepArgs<T, T> a = sweep_args<T, T>(s, 1, false);
+    a.stages = st_lo;
+    a.withhold = -1;
+    a.yspill = nullptr;
+    a.unit = 1;
+    a.unit_gran = s->port_tc ? 128 : kNB;
+    a.unit_stride = s->C * Rs;
+    // the tensor-core form of the multi-RHS sweep where it applies (FP32 band factor, half-bandwidths
+    // <= 384), its factor kept only for these solves where the solver's own sweep is another one
+    DevBuf wt_tmp, xcs;
+    size_t fb = 0, tb = 0;
+    VTM_CUDA(cudaMemGetInfo(&fb, &tb));
+    if (!s->wide) {
+      VTM_CUDA((sweep_wide_configure<T, T>(Rs, sm_lo)));
+      if constexpr (sizeof(T) == 4) {
+        if (s->wt_ok && (double)s->wt_bytes < 0.4 * (double)fb) {
+          wt_tmp.alloc((size_t)s->wt_bytes);
+          VTM_CUDA(cudaMemsetAsync(wt_tmp.p, 0, (size_t)wide_tc_zero_bytes(), st));
+          VTM_CUDA(wide_tc_configure(Rs));
+          VTM_CUDA(launch_wide_tc_factor(s->pieces_lo.as<PieceDesc>(), s->np_lo, s->wt_max_groups, s->factor.as<float>(),
+                                         wt_tmp.as<unsigned char>(), st));
+          fb -= std::min(fb, (size_t)s->wt_bytes);
         }
       }
-      if (s->resident)
-        VTM_CUDA(launch_gather_port_dense<T>(s->res_ps.as<ResPieceS>(), s->res_pieces, s->pieces_lo.as<PieceDesc>(),
-                                             s->port_local.as<int32_t>(), Rs, b, xc32.as<T>(), s->S.as<T>(), st));
-      else
-        VTM_CUDA(launch_gather_port_response<T>(s->pieces_lo.as<PieceDesc>(), s->np_lo, s->port_local.as<int32_t>(),
-                                                Rs, b, xc32.as<T>(), s->S.as<T>(), s->port_div[0].sh.layout, st));
+      a.wt = wt_tmp.as<unsigned char>();
+    }
+    int dev = 0, nsm = 1;
+    VTM_CUDA(cudaGetDevice(&dev));
+    VTM_CUDA(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
+    const size_t one = (size_t)std::max<int64_t>(1, a.unit_stride) * sizeof(T);  // solutions of a batch
+    const int per = std::max(1, std::min({nb, (8 * nsm + s->np_lo - 1) / s->np_lo, (int)std::min<size_t>(nb, fb / 10 / one)}));
+    if (per == 1 && Rs == s->R) {
+      a.xc = s->xc.as<T>();
+    } else {
+      xcs.alloc(one * per);
+      a.xc = xcs.as<T>();
+    }
+    for (int b = 0; b < nb; b += per) {
+      const int m = std::min(per, nb - b);
+      a.unit_b0 = b;
+      bool done = false;
+      if constexpr (sizeof(T) == 4) {
+        if (a.wt) {
+          VTM_CUDA(launch_sweep_wide_tc(a, Rs, s->np_lo, st, m));
+          done = true;
+        }
+      }
+      if (!done) VTM_CUDA((launch_sweep_wide<T, T>(a, Rs, s->np_lo, sm_lo, st, m)));
+      gather(Rs, b, a.xc, m, a.unit_stride);
     }
     VTM_CUDA(cudaStreamSynchronize(st));
   } else {
@@ -977,20 +1001,7 @@ static void compute_port_response(vtm_solver* s, int64_t s_tiles) {
       VTM_CUDA(launch_unit_rhs<T>(s->pieces.as<PieceDesc>(), np, s->port_local.as<int32_t>(), R, b, s->bt.as<T>(), st));
       reset_waves(s);
       sweeps_typed<T>(s, 1);
-      if (s->resident) {
-        VTM_CUDA(launch_gather_port_dense<T>(s->res_ps.as<ResPieceS>(), s->res_pieces, s->pieces_lo.as<PieceDesc>(),
-                                             s->port_local.as<int32_t>(), R, b, s->xc.as<T>(), s->S.as<T>(), st));
-        continue;
-      }
-      if constexpr (sizeof(T) == 4) {
-        if (s->port_tc) {
-          VTM_CUDA(launch_gather_port_blocks(s->pieces_lo.as<PieceDesc>(), s->np_lo, s->port_local.as<int32_t>(), R, b,
-                                             s->xc.as<float>(), s->S.as<float>(), st));
-          continue;
-        }
-      }
-      VTM_CUDA(launch_gather_port_response<T>(s->pieces_lo.as<PieceDesc>(), s->np_lo, s->port_local.as<int32_t>(),
-                                              R, b, s->xc.as<T>(), s->S.as<T>(), s->port_div[0].sh.layout, st));
+      gather(R, b, s->xc.as<T>(), 1, 0);
     }
     VTM_CUDA(cudaMemsetAsync(s->bt.p, 0, s->bt.bytes, st));
     reset_waves(s);

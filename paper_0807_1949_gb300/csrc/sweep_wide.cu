@@ -67,10 +67,16 @@ __global__ void __launch_bounds__(kWideThreads, 1) k_sweep_wide(const SweepArgs<
   const int Wp = pd.Wp;
   const int off = Wp - 1;
   const int nblk = pd.n_pad / kNB;
-  const int total = 2 * nblk;
+  // unit sources: batch blockIdx.y's columns, rows from the first one that S_j is wanted at
+  const int ub = (a.unit_b0 + (int)blockIdx.y) * R;  // first port of the batch
+  if (a.unit && ub >= pd.nports) return;
+  const int blk0 = a.unit ? a.port_local[pd.port_off + ub / a.unit_gran * a.unit_gran] / kNB : 0;  // first block
+  const int row0 = blk0 * kNB;
+  const int nfwd = nblk - blk0;
+  const int total = 2 * nfwd;
   const uint32_t slab_bytes = (uint32_t)(kNB * Wp * sizeof(T));
   const T* fbase = a.factor + pd.factor_off;
-  TV* xg = a.xc + (size_t)pd.copy_off * R;        // y, then x, of this subgraph (n rows x R)
+  TV* xg = a.xc + (size_t)blockIdx.y * a.unit_stride + (size_t)pd.copy_off * R;        // y, then x, of this subgraph (n rows x R)
   T* yg = a.yspill ? a.yspill + (size_t)pd.row_off * R : nullptr;  // y in factor precision
   const TV* bg = a.bt + (size_t)pd.copy_off * R;
 
@@ -83,7 +89,7 @@ __global__ void __launch_bounds__(kWideThreads, 1) k_sweep_wide(const SweepArgs<
   __syncthreads();
   auto issue = [&](int s) {
     if (s == a.withhold) return;  // testing hook: this slab's wait can only run out
-    const int kb = s < nblk ? s : total - 1 - s;
+    const int kb = blk0 + (s < nfwd ? s : total - 1 - s);
     const int slot = s % S;
     mbar_arrive_expect_tx(&bars[slot], slab_bytes);
     bulk_copy_g2s(ring + (size_t)slot * a.slot_elems, fbase + (size_t)kb * kNB * Wp, slab_bytes, &bars[slot]);
@@ -101,13 +107,17 @@ __global__ void __launch_bounds__(kWideThreads, 1) k_sweep_wide(const SweepArgs<
   // r = b̃ + P (Y w_in) for every row of the subgraph first (the port currents gathered from the
   // twins' waves by all threads at once), into the y storage, which the forward pass then reads
   // row block by row block and overwrites with y.
-  if (yg) {
+  if (a.unit) {
+    for (int i = row0 * R + tid; i < pd.n * R; i += kWideThreads) xg[i] = TV(0);
+  } else if (yg) {
     for (int i = tid; i < pd.n * R; i += kWideThreads) yg[i] = (T)bg[i];
   } else {
     for (int i = tid; i < pd.n * R; i += kWideThreads) xg[i] = bg[i];
   }
   __syncthreads();
-  for (int i = tid; i < pd.nports * R; i += kWideThreads) {
+  if (a.unit) {
+    if (tid < R && ub + tid < pd.nports) xg[(size_t)a.port_local[pd.port_off + ub + tid] * R + tid] = TV(1);
+  } else for (int i = tid; i < pd.nports * R; i += kWideThreads) {
     const int q = i / R, c = i % R;
     T acc = T(0);
     for (int e = a.port_end_ptr[pd.port_off + q]; e < a.port_end_ptr[pd.port_off + q + 1]; ++e)
@@ -127,8 +137,8 @@ __global__ void __launch_bounds__(kWideThreads, 1) k_sweep_wide(const SweepArgs<
   T in_v[kPer];
   auto prefetch = [&](int s2) {
     if (s2 >= total) return;
-    const bool f2 = s2 < nblk;
-    const int k2 = (f2 ? s2 : total - 1 - s2) * kNB;
+    const bool f2 = s2 < nfwd;
+    const int k2 = row0 + (f2 ? s2 : total - 1 - s2) * kNB;
     if (f2) {
 #pragma unroll
       for (int j = 0; j < kPer; ++j) {
@@ -136,12 +146,12 @@ __global__ void __launch_bounds__(kWideThreads, 1) k_sweep_wide(const SweepArgs<
         const int row = k2 + i / R;
         in_v[j] = row < pd.n ? (yg ? yg[(size_t)row * R + i % R] : (T)xg[(size_t)row * R + i % R]) : T(0);
       }
-    } else if (s2 > nblk) {
+    } else if (s2 > nfwd) {
 #pragma unroll
       for (int j = 0; j < kPer; ++j) {
         const int i = tid + j * kWideThreads;
         const int row = k2 - off + i / R, c = i % R;
-        in_v[j] = row >= 0 ? (yg ? yg[(size_t)row * R + c] : (T)xg[(size_t)row * R + c]) : T(0);
+        in_v[j] = row >= row0 ? (yg ? yg[(size_t)row * R + c] : (T)xg[(size_t)row * R + c]) : T(0);
       }
     }
   };
@@ -149,8 +159,8 @@ __global__ void __launch_bounds__(kWideThreads, 1) k_sweep_wide(const SweepArgs<
 
   int s = 0;
   for (; s < total; ++s) {
-    const bool fwd = s < nblk;
-    const int k0 = (fwd ? s : total - 1 - s) * kNB;
+    const bool fwd = s < nfwd;
+    const int k0 = row0 + (fwd ? s : total - 1 - s) * kNB;
     if (fwd) {
       // rows k0..k0+31 of r enter the window
 #pragma unroll
@@ -158,13 +168,13 @@ __global__ void __launch_bounds__(kWideThreads, 1) k_sweep_wide(const SweepArgs<
         const int i = tid + j * kWideThreads;
         Yw[(size_t)((k0 + i / R) & kMask) * R + i % R] = in_v[j];
       }
-    } else if (s > nblk) {
+    } else if (s > nfwd) {
       // backward: rows k0 - off .. k0 - off + 31 enter the window from the stored y
 #pragma unroll
       for (int j = 0; j < kPer; ++j) {
         const int i = tid + j * kWideThreads;
         const int row = k0 - off + i / R;
-        if (row >= 0) Yw[(size_t)(row & kMask) * R + i % R] = in_v[j];
+        if (row >= row0) Yw[(size_t)(row & kMask) * R + i % R] = in_v[j];
       }
     }
     prefetch(s + 1);
@@ -265,6 +275,7 @@ __global__ void __launch_bounds__(kWideThreads, 1) k_sweep_wide(const SweepArgs<
       const int nq = (off + kQT - 1) / kQT;
       for (int tile = tid; tile < nq * LY::kCG; tile += kWideThreads) {
         const int qb = (tile / LY::kCG) * kQT, cc = (tile % LY::kCG) * 4;
+        if (k0 - off + qb + kQT <= row0) continue;  // rows above the first one
         T acc[kQT][4];
 #pragma unroll
         for (int i = 0; i < kQT; ++i)
@@ -300,7 +311,7 @@ __global__ void __launch_bounds__(kWideThreads, 1) k_sweep_wide(const SweepArgs<
 #pragma unroll
         for (int i = 0; i < kQT; ++i) {
           const int q = qb + i;
-          if (q < off && k0 - off + q >= 0)
+          if (q < off && k0 - off + q >= row0)
 #pragma unroll
             for (int j = 0; j < 4; ++j) Yw[(size_t)((k0 - off + q) & kMask) * R + cc + j] -= acc[i][j];
         }
@@ -320,6 +331,7 @@ __global__ void __launch_bounds__(kWideThreads, 1) k_sweep_wide(const SweepArgs<
     }
     return;
   }
+  if (a.unit) return;
   __syncthreads();
   // w_out[e] = 2 x_c - w_in[e]
   for (int i = tid; i < pd.nports * R; i += kWideThreads) {
@@ -346,9 +358,10 @@ cudaError_t sweep_wide_configure(int R, size_t smem) {
 }
 
 template <typename TF, typename TV>
-cudaError_t launch_sweep_wide(const SweepArgs<TF, TV>& a, int R, int npieces, size_t smem, cudaStream_t st) {
+cudaError_t launch_sweep_wide(const SweepArgs<TF, TV>& a, int R, int npieces, size_t smem, cudaStream_t st,
+                              int batches) {
   if (npieces <= 0) return cudaSuccess;
-  dim3 grid(npieces), block(kWideThreads);
+  dim3 grid(npieces, batches), block(kWideThreads);
   switch (R) {
     case 16: k_sweep_wide<TF, TV, 16><<<grid, block, smem, st>>>(a); break;
     case 32: k_sweep_wide<TF, TV, 32><<<grid, block, smem, st>>>(a); break;
@@ -359,7 +372,7 @@ cudaError_t launch_sweep_wide(const SweepArgs<TF, TV>& a, int R, int npieces, si
 
 #define VTM_WIDE_INST(TF, TV)                                  \
   template cudaError_t sweep_wide_configure<TF, TV>(int, size_t); \
-  template cudaError_t launch_sweep_wide<TF, TV>(const SweepArgs<TF, TV>&, int, int, size_t, cudaStream_t);
+  template cudaError_t launch_sweep_wide<TF, TV>(const SweepArgs<TF, TV>&, int, int, size_t, cudaStream_t, int);
 VTM_WIDE_INST(float, float)
 VTM_WIDE_INST(double, double)
 VTM_WIDE_INST(double, float)

@@ -278,7 +278,12 @@ __global__ void __launch_bounds__(kWtThreads, 1) k_sweep_wide_tc(const SweepArgs
   const int64_t GB = wt_group_bytes(pd.w);
   const unsigned char* gb0 = a.wt + pd.wt_off;
   const unsigned char* zero_panel = a.wt;  // the factor buffer starts with a zero panel
-  float* xg = a.xc + (size_t)pd.copy_off * R;
+  // unit sources: batch blockIdx.y's columns, rows from the first one that S_j is wanted at
+  const int ub = (a.unit_b0 + (int)blockIdx.y) * R;  // first port of the batch
+  if (a.unit && ub >= pd.nports) return;
+  const int g0 = a.unit ? a.port_local[pd.port_off + ub / a.unit_gran * a.unit_gran] / kG : 0;  // first group
+  const int m = ng - g0;                                                                        // groups solved
+  float* xg = a.xc + (size_t)blockIdx.y * a.unit_stride + (size_t)pd.copy_off * R;
   const float* bg = a.bt + (size_t)pd.copy_off * R;
   auto dval = [&](int row) -> float {
     return *reinterpret_cast<const float*>(gb0 + (int64_t)(row / kG) * GB + (size_t)(2 * nl + 4) * kChunk +
@@ -306,7 +311,20 @@ __global__ void __launch_bounds__(kWtThreads, 1) k_sweep_wide_tc(const SweepArgs
   // ---- r~ = D^-1/2 (b~ + P (Y w_in)) (port currents from the twins' waves) into xc, and the column
   // maxima of r~ (a port row also counts with its value before the currents: sigma only has to be
   // at or above max |r~|)
-  {
+  if (a.unit) {
+    float4* x4 = reinterpret_cast<float4*>(xg);
+    for (int i = g0 * kG * (R / 4) + tid; i < n * (R / 4); i += kWtThreads) x4[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+    __syncthreads();
+    if (tid < R) {
+      float dv = 0.f;
+      if (ub + tid < pd.nports) {
+        const int row = a.port_local[pd.port_off + ub + tid];
+        dv = dval(row);
+        xg[(size_t)row * R + tid] = dv;
+      }
+      sigf[tid] = pow2_at_or_above(dv);
+    }
+  } else {
     float mx[4] = {0.f, 0.f, 0.f, 0.f};  // columns 4 (tid % (R / 4)) .. + 3 (kWtThreads is a multiple of R / 4)
     const float4* b4 = reinterpret_cast<const float4*>(bg);
     float4* x4 = reinterpret_cast<float4*>(xg);
@@ -386,8 +404,10 @@ __global__ void __launch_bounds__(kWtThreads, 1) k_sweep_wide_tc(const SweepArgs
       for (int t = 0; t < kWtThreads; ++t) m = fmaxf(m, red[4 * kWtThreads + tid * kWtThreads + t]);
       sigf[tid] = pow2_at_or_above(m);
     }
-    __syncthreads();
-    // the forward window starts as zeros (the columns left of row 0)
+  }
+  __syncthreads();
+  {
+    // the forward window starts as zeros (the columns left of the first row)
     uint4* win = reinterpret_cast<uint4*>(pA + LY::kWin);
     for (int i = tid; i < (int)(kNWC * LY::kWinChunk / 16); i += kWtThreads) win[i] = make_uint4(0, 0, 0, 0);
     fence_proxy_async_smem();
@@ -435,21 +455,21 @@ __global__ void __launch_bounds__(kWtThreads, 1) k_sweep_wide_tc(const SweepArgs
         const unsigned char* src = gb0 + (int64_t)g * GB + (size_t)(2 * nl) * kChunk;
         for (int i = 0; i < 4; ++i) next(src + (size_t)i * kChunk);
       };
-      left(0, 0, 2 * T);
-      for (int g = 0; g < ng && ok && !flags[0]; ++g) {
+      left(g0, 0, 2 * T);
+      for (int g = g0; g < ng && ok && !flags[0]; ++g) {
         if (g + 1 < ng) left(g + 1, 0, nearly);
         gpanels(g);
         if (g + 1 < ng) left(g + 1, nearly, 2 * T);
       }
-      for (int k = 0; k < ng && ok && !flags[0]; ++k) {
+      for (int k = 0; k < m && ok && !flags[0]; ++k) {
         const int g = ng - 1 - k;
         gpanels(g);
-        for (int m = T - 1; m >= 0 && ok; --m) {
-          if (g - T + m < 0) continue;
-          next(left_panel(g, 2 * m, 0));
-          next(left_panel(g, 2 * m + 1, 0));
-          next(left_panel(g, 2 * m, 1));
-          next(left_panel(g, 2 * m + 1, 1));
+        for (int t = T - 1; t >= 0 && ok; --t) {
+          if (g - T + t < g0) continue;
+          next(left_panel(g, 2 * t, 0));
+          next(left_panel(g, 2 * t + 1, 0));
+          next(left_panel(g, 2 * t, 1));
+          next(left_panel(g, 2 * t + 1, 1));
         }
       }
       if (!ok) flags[0] = 1;
@@ -534,34 +554,34 @@ __global__ void __launch_bounds__(kWtThreads, 1) k_sweep_wide_tc(const SweepArgs
         mma_commit(yready);
       };
       // forward
-      left_product(0, 0, 2 * T, tmem, true);
+      left_product(g0, 0, 2 * T, tmem + (uint32_t)((g0 & 1) * 2 * kSet), true);
       if (ok) mma_commit(accfull);
-      for (int g = 0; g < ng && ok; ++g) {
+      for (int g = g0; g < ng && ok; ++g) {
         const uint32_t dn = tmem + (uint32_t)(((g + 1) & 1) * 2 * kSet);
         if (g + 1 < ng) left_product(g + 1, 0, nearly, dn, true);
         if (!ok) break;
-        if (!(ok = wait_or_abort(tready, (uint32_t)(g & 1), a.wait_limit, flags))) break;
+        if (!(ok = wait_or_abort(tready, (uint32_t)((g - g0) & 1), a.wait_limit, flags))) break;
         tc_fence_after();
         g_product(false, dGf);
         if (!ok || g + 1 >= ng) break;
-        if (!(ok = wait_or_abort(bready, (uint32_t)(g & 1), a.wait_limit, flags))) break;
+        if (!(ok = wait_or_abort(bready, (uint32_t)((g - g0) & 1), a.wait_limit, flags))) break;
         tc_fence_after();
         left_product(g + 1, nearly, 2 * T, dn, nearly <= z);
         if (ok) mma_commit(accfull);
       }
       // backward: x~_g = G_g^T t, then group g adds L~_(g, left)^T x~_g to the accumulators of
       // groups g - T .. g - 1 (tile T - 1 first: group g - 1 reads its accumulator next)
-      for (int k = 0; k < ng && ok; ++k) {
+      for (int k = 0; k < m && ok; ++k) {
         const int g = ng - 1 - k;
-        if (!(ok = wait_or_abort(tready, (uint32_t)((ng + k) & 1), a.wait_limit, flags))) break;
+        if (!(ok = wait_or_abort(tready, (uint32_t)((m + k) & 1), a.wait_limit, flags))) break;
         tc_fence_after();
         g_product(true, dGb);
         if (!ok) break;
         if (!(ok = wait_or_abort(xready, (uint32_t)(k & 1), a.wait_limit, flags))) break;
         tc_fence_after();
-        for (int m = T - 1; m >= 0 && ok; --m) {
-          const int h = g - T + m;
-          if (h < 0) continue;
+        for (int t = T - 1; t >= 0 && ok; --t) {
+          const int h = g - T + t;
+          if (h < g0) continue;
           const uint32_t d = tmem + (uint32_t)((h % 3) * 2 * kSet);
           const bool first = (g == min(h + T, ng - 1));
           const uint32_t s0 = take();
@@ -583,7 +603,7 @@ __global__ void __launch_bounds__(kWtThreads, 1) k_sweep_wide_tc(const SweepArgs
             mma_f16_acc(ds + R, aTl + (uint64_t)(kk * 128), bH, idT);
           }
           give(4);
-          if (m == T - 1) mma_commit(baccready);
+          if (t == T - 1) mma_commit(baccready);
         }
         if (ok) mma_commit(xfree);
       }
@@ -651,10 +671,10 @@ __global__ void __launch_bounds__(kWtThreads, 1) k_sweep_wide_tc(const SweepArgs
     }
     bool ok = true;
     float rv[kHalf];
-    load_rows(0, rv);
+    load_rows(g0, rv);
     // forward
-    for (int g = 0; g < ng && ok; ++g) {
-      if (!(ok = decide(accfull, (uint32_t)(g & 1)))) break;
+    for (int g = g0; g < ng && ok; ++g) {
+      if (!(ok = decide(accfull, (uint32_t)((g - g0) & 1)))) break;
       tc_fence_after();
       float t[kHalf];
       tmem_pair((uint32_t)((g & 1) * 2 * kSet), t);
@@ -666,7 +686,7 @@ __global__ void __launch_bounds__(kWtThreads, 1) k_sweep_wide_tc(const SweepArgs
       simt_sync();
       if (st == 0) mbar_arrive(tready);
       load_rows(g + 1 < ng ? g + 1 : -1, rv);
-      if (!(ok = decide(yready, (uint32_t)(g & 1)))) break;
+      if (!(ok = decide(yready, (uint32_t)((g - g0) & 1)))) break;
       tc_fence_after();
       float y[kHalf];
       tmem_pair(8 * R, y);
@@ -717,7 +737,7 @@ __global__ void __launch_bounds__(kWtThreads, 1) k_sweep_wide_tc(const SweepArgs
     }
     // backward
     if (ok) load_rows(ng - 1, rv);
-    for (int k = 0; k < ng && ok; ++k) {
+    for (int k = 0; k < m && ok; ++k) {
       const int g = ng - 1 - k;
       float t[kHalf];
       if (g + 1 <= ng - 1) {
@@ -737,8 +757,8 @@ __global__ void __launch_bounds__(kWtThreads, 1) k_sweep_wide_tc(const SweepArgs
       if (st == 0) mbar_arrive(tready);
       const int row = g * kG + rq;
       const float drow = row < n ? dval(row) : 0.f;
-      load_rows(g - 1, rv);
-      if (!(ok = decide(yready, (uint32_t)((ng + k) & 1)))) break;
+      load_rows(g > g0 ? g - 1 : -1, rv);
+      if (!(ok = decide(yready, (uint32_t)((m + k) & 1)))) break;
       tc_fence_after();
       float x[kHalf];
       tmem_pair(12 * R, x);
@@ -763,7 +783,7 @@ __global__ void __launch_bounds__(kWtThreads, 1) k_sweep_wide_tc(const SweepArgs
   __syncthreads();
   const bool ok = mbar_wait_bounded(done, 0, kDrainPolls) && !flags[0];
   if (!ok && tid == 0) atomicExch(a.status, kStatusTimeout);
-  if (ok) {
+  if (ok && !a.unit) {
     // w_out[e] = 2 x_c - w_in[e], one port per thread, 16-byte rows
     for (int q = tid; q < pd.nports; q += kWtThreads) {
       const int port = pd.port_off + q;
@@ -809,11 +829,13 @@ cudaError_t launch_wide_tc_factor(const PieceDesc* pieces, int npieces, int max_
   return cudaGetLastError();
 }
 
-cudaError_t launch_sweep_wide_tc(const SweepArgs<float, float>& a, int R, int npieces, cudaStream_t st) {
+cudaError_t launch_sweep_wide_tc(const SweepArgs<float, float>& a, int R, int npieces, cudaStream_t st,
+                                 int batches) {
   if (npieces <= 0) return cudaSuccess;
   if (!a.wt) return cudaErrorInvalidValue;
-  if (R == 16) k_sweep_wide_tc<16><<<npieces, kWtThreads, WtLayout<16>::kBytes, st>>>(a);
-  else if (R == 32) k_sweep_wide_tc<32><<<npieces, kWtThreads, WtLayout<32>::kBytes, st>>>(a);
+  const dim3 grid(npieces, batches);
+  if (R == 16) k_sweep_wide_tc<16><<<grid, kWtThreads, WtLayout<16>::kBytes, st>>>(a);
+  else if (R == 32) k_sweep_wide_tc<32><<<grid, kWtThreads, WtLayout<32>::kBytes, st>>>(a);
   else return cudaErrorInvalidValue;
   return cudaGetLastError();
 }

@@ -86,3 +86,14 @@ def test_pipelined_band_sweep(vtmlib, dims, block, nrhs):
                                         ((52, 47, 41), (6, 6, 6))])
 def test_tensor_core_sweep(vtmlib, dims, block, nrhs, kind):
     _check(vtmlib, dims, block, nrhs, "fp32", "fp16" if kind == "fp16" else "native", 6, TOL[kind])
+
+
+# port responses from the band kernels without the tensor cores (half-bandwidth above 384) and with them
+# (385 > w): the batches start at the first row they need, here deep inside the subgraph
+@pytest.mark.parametrize("dims,block,nrhs,kind", [((41, 20, 21), (20, 20, 21), 1, "fp32"),
+                                                  ((41, 20, 21), (20, 20, 21), 16, "fp32"),
+                                                  ((37, 19, 18), (18, 19, 18), 1, "fp32"),
+                                                  ((37, 19, 18), (18, 19, 18), 16, "fp32"),
+                                                  ((27, 13, 12), (13, 13, 12), 1, "fp64")])
+def test_port_response(vtmlib, dims, block, nrhs, kind):
+    _check(vtmlib, dims, block, nrhs, kind, "native", 4, TOL[kind])
