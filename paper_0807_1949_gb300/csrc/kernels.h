@@ -110,7 +110,7 @@ struct PortShape {
   int pad;         // unused entries after every four ports
   int op_stride;   // tensor cores: 16-bit entries of a row of the vector operand
   int layout;      // of S_j's tiles (kPort...)
-  int mma;         // 1: products on the tensor cores
+  int mma;         // warps of a CTA with its products on the tensor cores (0: SIMT products)
   int priv;        // 1: an accumulator per warp (R <= 2), 0: one for all
   int ring;        // 1: shared-memory slots for the tiles in flight (0: no room)
   int sb;          // strips whose row sums the warps keep between barriers (0: no room)
@@ -148,7 +148,8 @@ struct PortArgs {
 
 __host__ __device__ int64_t port_tiles(int nports);
 PortShape port_shape(size_t elem, size_t stored, int R, int max_ports);
-PortPlan port_plan(const PieceDesc* pieces, int npieces, size_t elem, size_t stored, int R, int ctas);
+PortPlan port_plan(const PieceDesc* pieces, int npieces, size_t elem, size_t stored, int R, int ctas,
+                   int mma);
 template <typename T>
 cudaError_t port_sweep_configure(int R, const PortShape& sh, bool half, int* ctas_per_sm);
 // Two launches: the port vectors of all nports ports, then the sweep proper.

@@ -289,7 +289,7 @@ __device__ __forceinline__ void reduce_scatter(T (&v)[N][RC], int pos) {
 // order.  Nothing waits, and the order of arrival does not enter the sums: identical runs agree bit
 // for bit.  The waves, w_out[e] = 2 (u_base + y)_q - w_in[e], take kU entries per thread at a time,
 // their partials, end ranges, twins and incoming waves loaded in three independent rounds.
-template <typename T, int R, typename Y>
+template <typename T, int R, int TH, typename Y>
 __device__ __forceinline__ void finish_segment(const PortArgs<T>& a, const PortSeg& sg, int si, const PieceDesc& pd,
                                                int rows, int* flag, Y y) {
   constexpr int RV = vec_cols<T, R>();
@@ -298,7 +298,7 @@ __device__ __forceinline__ void finish_segment(const PortArgs<T>& a, const PortS
   const int npad = (np + kNB - 1) / kNB * kNB;
   T* const part = a.part + sg.part;  // [nseg][npad * R]
   if (sg.nseg > 1) {
-    for (int i = tid; i < npad * (R / RV); i += kSweepThreads) {
+    for (int i = tid; i < npad * (R / RV); i += TH) {
       T v[RV] = {};
       const int q = i / (R / RV), r = i % (R / RV) * RV;
       if (q < rows) y(q, r, v);
@@ -318,12 +318,12 @@ __device__ __forceinline__ void finish_segment(const PortArgs<T>& a, const PortS
     __threadfence();
   }
   const int nv = np * (R / RV);
-  for (int i0 = tid; i0 < nv; i0 += kSweepThreads * kU) {
+  for (int i0 = tid; i0 < nv; i0 += TH * kU) {
     int e0[kU], e1[kU], tw[kU];
     T uu[kU][RV], ub[kU][RV];
 #pragma unroll
     for (int u = 0; u < kU; ++u) {
-      const int i = i0 + u * kSweepThreads;
+      const int i = i0 + u * TH;
       e0[u] = e1[u] = 0;
 #pragma unroll
       for (int c = 0; c < RV; ++c) uu[u][c] = T(0);
@@ -343,7 +343,7 @@ __device__ __forceinline__ void finish_segment(const PortArgs<T>& a, const PortS
         for (int u = 0; u < kU; ++u)
 #pragma unroll
           for (int k = 0; k < kP; ++k) {
-            const int i = i0 + u * kSweepThreads;
+            const int i = i0 + u * TH;
 #pragma unroll
             for (int c = 0; c < RV; ++c) v[u][k][c] = T(0);
             if (i < nv && k0 + k < sg.nseg) load_cg<T, RV>(part + (size_t)(k0 + k) * npad * R + (size_t)i * RV, v[u][k]);
@@ -363,7 +363,7 @@ __device__ __forceinline__ void finish_segment(const PortArgs<T>& a, const PortS
     for (int u = 0; u < kU; ++u) tw[u] = (e1[u] > e0[u]) ? a.twin[e0[u]] : 0;
 #pragma unroll
     for (int u = 0; u < kU; ++u) {
-      const int i = i0 + u * kSweepThreads;
+      const int i = i0 + u * TH;
       if (i >= nv) break;
       const int r = i % (R / RV) * RV;
       T w[RV], o[RV];
@@ -440,6 +440,9 @@ __host__ __device__ constexpr int operand_rows() {
   return sizeof(TS) == 2 ? 2 * R : 3 * R;
 }
 
+// Threads of a CTA: MMA = its warps when the products run on the tensor cores, 0 when they do not.
+__host__ __device__ constexpr int sweep_threads(int mma) { return mma ? 32 * mma : kSweepThreads; }
+
 // One sweep in port-response form, R right-hand sides.
 //
 // Work split.  A CTA works through segments, runs of consecutive 32 x 32 tiles of one subgraph's
@@ -466,18 +469,19 @@ __host__ __device__ constexpr int operand_rows() {
 // lane (32 conversions, 64 FMAs, shuffles), of an FP32 tile at R = 8 about 980: the issue rate, not
 // the memory, bound those sweeps.
 //
-// What bounds it (GB300): HBM at R = 1, 2 and with FP16 tiles, FP64 arithmetic in FP64 (0.84 of its
-// pipe).  Measured per sweep against one CTA per subgraph with shared-memory atomics (R > 1, FP64) or
-// an accumulator per warp (FP32 / FP16, R = 1): 64^3 in 64 subgraphs 0.116 -> 0.044 ms (FP32, R = 1,
-// 188 MB) and 0.82 -> 0.21 ms (FP64, 376 MB); 101 x 67 x 83 in 288 ragged subgraphs, R = 8, 439 MB:
-// 0.54 -> 0.22 ms; 128^3 in 512 subgraphs, FP16, 1.01 GB: 0.199 -> 0.185 ms (0.80 of the copy
-// bandwidth with the port vectors' own launch; the tiles are read with an evict-first hint, without
-// it 0.198 ms).
-template <typename T, typename TS, int R, bool PRIV, bool MMA>
-__global__ void __launch_bounds__(kSweepThreads, sizeof(T) == 8 ? 1 : 2)
+// What bounds it (GB300): HBM at R = 1, 2 and with FP16 tiles, FP64 arithmetic in FP64 (0.9 of its
+// pipe), with three-term FP32 tiles the issue rate and the segments' latency.  Measured per sweep
+// against one CTA per subgraph with shared-memory atomics (R > 1, FP64) or an accumulator per warp
+// (FP32 / FP16, R = 1): 64^3 in 64 subgraphs 0.116 -> 0.042 ms (FP32, R = 1, 188 MB) and 0.82 -> 0.19 ms
+// (FP64, 376 MB); 101 x 67 x 83 in 288 ragged subgraphs, R = 8, 439 MB: 0.54 -> 0.16 ms (0.22 with shares
+// that counted a segment as 20 tiles, and 8 warps); 128^3 in 512 subgraphs, FP16, 1.01 GB: 0.199 ->
+// 0.183 ms (0.81 of the copy bandwidth with the port vectors' own launch; the tiles are read with an
+// evict-first hint, without it 0.198 ms).
+template <typename T, typename TS, int R, bool PRIV, int MMA>
+__global__ void __launch_bounds__(sweep_threads(MMA), sizeof(T) == 8 || MMA > 8 ? 1 : 2)
     k_port_sweep(const PortArgs<T> a) {
   extern __shared__ __align__(128) unsigned char smem[];
-  constexpr int kWarps = kSweepThreads / 32;
+  constexpr int TH = sweep_threads(MMA), kWarps = TH / 32;
   constexpr int RC = R >= 2 ? 2 : 1;         // columns per pass
   constexpr int PR = patch_rows(R), PC = kNB / PR;  // a lane's patch
   constexpr int RV = vec_cols<T, R>();
@@ -589,7 +593,7 @@ __global__ void __launch_bounds__(kSweepThreads, sizeof(T) == 8 ? 1 : 2)
       float m[RV] = {};
       if (HALF && tid < R) smax[tid] = 0;
 #pragma unroll 4
-      for (int i = tid; i < rows * (R / RV); i += kSweepThreads) {
+      for (int i = tid; i < rows * (R / RV); i += TH) {
         T v[RV] = {};
         if (i / (R / RV) < np) load_cg<T, RV>(sp + (size_t)i * RV, v);
         store_vec<T, RV>(yv + i * RV, v);
@@ -614,7 +618,7 @@ __global__ void __launch_bounds__(kSweepThreads, sizeof(T) == 8 ? 1 : 2)
           sigma[c] = ldexpf(1.f, max(-120, e));
         }
       }
-      for (int i = tid; i < rows * (R / RV); i += kSweepThreads) {
+      for (int i = tid; i < rows * (R / RV); i += TH) {
         const int q = i / (R / RV);
         uint16_t* o = sop + (q & ~(kNB - 1)) + operand_pos(q & (kNB - 1));
         T v[RV];
@@ -640,14 +644,14 @@ __global__ void __launch_bounds__(kSweepThreads, sizeof(T) == 8 ? 1 : 2)
       if constexpr (PRIV) {
         for (int i = lane; i < rows * R / W; i += 32) store_vec<T, W>(yw + i * W, z4);
       } else {
-        for (int i = tid; i < rows * R / W; i += kSweepThreads) store_vec<T, W>(yv + i * W, z4);
+        for (int i = tid; i < rows * R / W; i += TH) store_vec<T, W>(yv + i * W, z4);
       }
     } else {
       // s and y = 0, RV columns at a time; padding ports are zero
       const T* sp = a.s + (size_t)pd.port_off * R;
       const T zero[RV] = {};
 #pragma unroll 4
-      for (int i = tid; i < rows * (R / RV); i += kSweepThreads) {
+      for (int i = tid; i < rows * (R / RV); i += TH) {
         const int q = i / (R / RV), r = i % (R / RV) * RV;
         T v[RV] = {};
         if (q < np) load_cg<T, RV>(sp + (size_t)q * R + r, v);
@@ -878,7 +882,7 @@ __global__ void __launch_bounds__(kSweepThreads, sizeof(T) == 8 ? 1 : 2)
         __syncwarp();
       }
       __syncthreads();
-      finish_segment<T, R>(a, sg, si, pd, rows, reinterpret_cast<int*>(sv), [&](int q, int r, T(&v)[RV]) {
+      finish_segment<T, R, TH>(a, sg, si, pd, rows, reinterpret_cast<int*>(sv), [&](int q, int r, T(&v)[RV]) {
 #pragma unroll
         for (int w = 0; w < kWarps; ++w) {
           T x[RV];
@@ -943,7 +947,7 @@ __global__ void __launch_bounds__(kSweepThreads, sizeof(T) == 8 ? 1 : 2)
         }
         if (sb > 0) {
           __syncthreads();
-          for (int i = tid; i < (Ie - Ib) * kNB * R; i += kSweepThreads) {
+          for (int i = tid; i < (Ie - Ib) * kNB * R; i += TH) {
             T v = T(0);
 #pragma unroll
             for (int w = 0; w < kWarps; ++w) v += buf[(size_t)w * sb * kNB * R + i];
@@ -952,7 +956,7 @@ __global__ void __launch_bounds__(kSweepThreads, sizeof(T) == 8 ? 1 : 2)
           __syncthreads();
         }
       }
-      finish_segment<T, R>(a, sg, si, pd, rows, reinterpret_cast<int*>(sv),
+      finish_segment<T, R, TH>(a, sg, si, pd, rows, reinterpret_cast<int*>(sv),
                            [&](int q, int r, T(&v)[RV]) {
                              load_vec<T, RV>(yv + vidx<R>(q, pad) + r, v);
                              if constexpr (MMA && HALF)
@@ -1021,16 +1025,15 @@ __global__ void __launch_bounds__(256) k_port_vec(const PortArgs<T> a, int nport
 // the gaps, the slots and the row sums.
 PortShape port_shape(size_t elem, size_t stored, int R, int max_ports) {
   const size_t npad = (size_t)((max_ports + kNB - 1) / kNB) * kNB;
-  constexpr int kWarps = kSweepThreads / 32;
-  const size_t sum = (size_t)kWarps * kNB * R * elem;  // one strip's row sums
-  const size_t slot =
-      (size_t)kWarps * (stored == 2 ? slot_bytes<__half>() : stored == 4 ? slot_bytes<float>() : slot_bytes<double>());
+  const size_t sum1 = (size_t)kNB * R * elem;  // a warp's row sums of one strip
+  const size_t slot1 = (stored == 2 ? slot_bytes<__half>() : stored == 4 ? slot_bytes<float>() : slot_bytes<double>());
   const size_t kSmemMax = 226 * 1024;  // the tensor-core kernels have a static part
   const int per_sm = elem == 8 ? 1 : 2;
   const size_t all = (228 * 1024) / per_sm - 1024;  // an SM's shared memory, 1 KB per CTA reserved
   const size_t share = all < kSmemMax ? all : kSmemMax;
   PortShape p{};
-  auto fit = [&](bool mma, bool priv, int pad, bool ring, int sb, size_t most) {
+  auto fit = [&](int mma, bool priv, int pad, bool ring, int sb, size_t most) {
+    const int warps = sweep_threads(mma) / 32;
     p.mma = mma;
     p.priv = priv;
     p.pad = pad;
@@ -1041,96 +1044,146 @@ PortShape port_shape(size_t elem, size_t stored, int R, int max_ports) {
     p.op_stride = (int)(npad / kNB % 2 ? npad : npad + kNB);
     const size_t op = (size_t)(stored == 2 ? operand_rows<__half, 1>() : operand_rows<float, 1>()) * R * p.op_stride * 2;
     const size_t depth = stored == 2 && mma && priv ? port_depth<__half, true>() : 1;
-    p.smem = (ring ? slot * depth : 0) + (mma ? op : p.vec_elems * elem) + (size_t)p.vec_elems * elem * (priv ? kWarps : 1) +
-             sb * sum;
+    p.smem = (ring ? warps * slot1 * depth : 0) + (mma ? op : p.vec_elems * elem) + (size_t)p.vec_elems * elem * (priv ? warps : 1) +
+             sb * warps * sum1;
     p.layout = mma && stored == 4 ? kPortFragments : R <= 2 ? kPortPatch8x4 : kPortPatch4x8;
     return p.smem <= most;
   };
   const bool mma = stored == 2 || (stored == 4 && R >= 4);
-  if (R <= 2 && fit(mma, true, 0, true, 0, share)) return p;
+  if (R <= 2 && fit(mma ? 8 : 0, true, 0, true, 0, share)) return p;
+  // tensor cores: two CTAs of 8 warps per SM where they fit, else FP32 one of 16 warps (R = 8, 439 MB,
+  // one CTA per SM: 260 k cycles with 16 warps, 283 k with 8; R = 4, where two fit: two of 8 warps
+  // 191 k, one of 16 242 k), else one of 8
   if (mma)
-    for (size_t most : {share, kSmemMax})
-      for (int sb : {8, 4, 2, 1})
-        if (fit(true, false, 0, true, sb, most)) return p;
+    for (int sb : {8, 4, 2, 1})
+      if (fit(8, false, 0, true, sb, share)) return p;
+  if (mma && stored == 4)
+    for (int sb : {8, 4, 2, 1})
+      if (fit(16, false, 0, true, sb, kSmemMax)) return p;
+  if (mma)
+    for (int sb : {8, 4, 2, 1})
+      if (fit(8, false, 0, true, sb, kSmemMax)) return p;
   const int pad = (elem == 4 && R >= 4) ? 4 : 0;
   for (size_t most : {share, kSmemMax})
     for (int sb : {8, 4, 2, 1})
-      if (fit(false, false, pad, true, sb, most)) return p;
+      if (fit(0, false, pad, true, sb, most)) return p;
   const size_t all_smem = 227 * 1024;
-  if (fit(false, false, 0, true, 1, all_smem) || fit(false, false, 0, false, 1, all_smem)) return p;
-  fit(false, false, 0, false, 0, all_smem);
+  if (fit(0, false, 0, true, 1, all_smem) || fit(0, false, 0, false, 1, all_smem)) return p;
+  fit(0, false, 0, false, 0, all_smem);
   return p;
 }
 
-// Cuts the tiles of all subgraphs, in order, into equal shares for `ctas` CTAs (cut points at whole
-// tiles; a cut that would leave a piece of a subgraph with fewer than kMinSeg tiles moves to the
-// subgraph's end).  Besides its tiles a segment costs about 7 us of latency (its vectors, its
-// partial sums, its waves), which counts as the tiles that one CTA gets through in that time.
-PortPlan port_plan(const PieceDesc* pd, int npieces, size_t elem, size_t stored, int R, int ctas) {
+// Cuts the tiles of all subgraphs, in order, into shares for `ctas` CTAs, as equal as whole tiles and
+// pieces of at least kMinSeg tiles allow: the smallest share for which the last CTA has no more than the
+// others, by bisection.  Besides its tiles a segment costs the latency of its vectors, its partial sums
+// and its waves, and a little per strip of them.  In tiles of the same kernel, from the cycles of every
+// CTA of a sweep over 288 ragged subgraphs of 1 to 33 strips (least squares):
+//   FP64 8 + 0.3 per strip (R = 1), 5 + 0.3 (R = 2); FP32 27 + 0.6 (R = 1, 2); FP16 41 + 1.2 (R = 1);
+//   tensor cores, 8 warps: FP32 44 + 0.7 (R = 4), 48 + 1.0 (R = 8), FP16 54 + 1.9 and 67 + 2.6;
+//   16 warps: FP32 71 + 0.1.
+// (With 20 for R >= 4 the CTAs of many small subgraphs took 1.4 times the average.)
+PortPlan port_plan(const PieceDesc* pd, int npieces, size_t elem, size_t stored, int R, int ctas, int mma) {
   constexpr int kMinSeg = 32;
-  const double kSegCost = elem == 8 ? 10.0 : R >= 4 ? 20.0 : 35.0;
-  PortPlan pl;
-  double total = 0;
+  double seg = 20, strip = 0;  // SIMT products, R >= 4
+  if (elem == 8) seg = 7, strip = 0.3;
+  else if (R <= 2) seg = stored == 2 ? 41 : 27, strip = stored == 2 ? 1.2 : 0.6;
+  else if (mma == 16) seg = 71, strip = 0.1;
+  else if (mma) seg = stored == 2 ? 60 : 46, strip = stored == 2 ? 2.3 : 0.9;
+  auto strips = [](int t) {  // of the rows up to tile t's
+    int I, J;
+    tile_of(t, I, J);
+    return I + 1;
+  };
+  // shares of `share` each, the last CTA takes the rest; returns what it has got
+  auto cut = [&](double share, PortPlan* pl) {
+    int cta = 0, nseg_all = 0;
+    double load = 0;
+    auto close = [&]() {
+      ++cta;
+      load = 0;
+      if (pl) pl->cta_seg.push_back(nseg_all);
+    };
+    if (pl) pl->cta_seg.push_back(0);
+    for (int j = 0; j < npieces; ++j) {
+      if (pd[j].nports <= 0) continue;
+      const int n = (int)port_tiles(pd[j].nports), first = nseg_all;
+      int t = 0;
+      while (t < n) {
+        int take = n - t;
+        const double room = share - load - seg;
+        if (cta + 1 < ctas && take + strip * strips(n - 1) > room) {
+          take = (int)room;
+          if (take > 0) take = (int)(room - strip * strips(std::min(n, t + take) - 1));
+          if (n - t - take < kMinSeg) take = n - t - kMinSeg;
+          if (take < kMinSeg) {
+            if (load > 0) {
+              close();
+              continue;
+            }
+            take = n - t < 2 * kMinSeg ? n - t : kMinSeg;
+          }
+        }
+        if (pl) {
+          PortSeg sg{};
+          sg.piece = j;
+          sg.s_off = pd[j].s_off;
+          tile_of(t, sg.I0, sg.J0);
+          tile_of(t + take - 1, sg.I1, sg.J1);
+          sg.first = first;
+          pl->segs.push_back(sg);
+        }
+        ++nseg_all;
+        load += seg + take + strip * strips(t + take - 1);
+        t += take;
+        if (t < n && cta + 1 < ctas) close();
+      }
+      if (!pl) continue;
+      const int nseg = nseg_all - first;
+      for (int k = first; k < nseg_all; ++k) {
+        pl->segs[k].nseg = nseg;
+        pl->segs[k].part = pl->part_elems;
+      }
+      if (nseg > 1) pl->part_elems += (int64_t)nseg * ((pd[j].nports + kNB - 1) / kNB) * kNB * R;
+    }
+    if (pl && pl->cta_seg.back() != nseg_all) pl->cta_seg.push_back(nseg_all);
+    return load;
+  };
+  double lo = 0, hi = 1;
   for (int j = 0; j < npieces; ++j)
-    if (pd[j].nports > 0) total += (double)port_tiles(pd[j].nports) + kSegCost;
-  // about one segment per cut more than subgraphs
-  const double share = std::max(1.0, (total + kSegCost * ctas) / std::max(1, ctas));
-  double pos = 0;  // cost placed so far
-  int cta = 0;
-  pl.cta_seg.push_back(0);
-  for (int j = 0; j < npieces; ++j) {
-    if (pd[j].nports <= 0) continue;
-    const int n = (int)port_tiles(pd[j].nports);
-    const int first = (int)pl.segs.size();
-    int t = 0;
-    while (t < n) {
-      pos += kSegCost;
-      const double room = (cta + 1) * share - pos;
-      int take = n - t;
-      if (room < take) {
-        take = std::max(kMinSeg, (int)std::ceil(room));
-        if (n - t - take < kMinSeg) take = n - t;
-      }
-      PortSeg sg{};
-      sg.piece = j;
-      sg.s_off = pd[j].s_off;
-      tile_of(t, sg.I0, sg.J0);
-      tile_of(t + take - 1, sg.I1, sg.J1);
-      sg.first = first;
-      pl.segs.push_back(sg);
-      t += take;
-      pos += take;
-      while (cta + 1 < ctas && pos >= (cta + 1) * share - 1e-9) {
-        ++cta;
-        if (pl.cta_seg.back() != (int)pl.segs.size()) pl.cta_seg.push_back((int)pl.segs.size());
-      }
+    if (pd[j].nports > 0) {
+      const int n = (int)port_tiles(pd[j].nports);
+      lo += n + seg + strip * strips(n - 1);
     }
-    const int nseg = (int)pl.segs.size() - first;
-    for (int k = first; k < first + nseg; ++k) {
-      pl.segs[k].nseg = nseg;
-      pl.segs[k].part = pl.part_elems;
-    }
-    if (nseg > 1) pl.part_elems += (int64_t)nseg * ((pd[j].nports + kNB - 1) / kNB) * kNB * R;
+  lo = std::max(1.0, lo / std::max(1, ctas));
+  hi = 2 * lo + seg + 2 * kMinSeg;
+  while (cut(hi, nullptr) > hi) hi *= 2;
+  for (int k = 0; k < 12; ++k) {
+    const double mid = (lo + hi) / 2;
+    (cut(mid, nullptr) > mid ? lo : hi) = mid;
   }
-  if (pl.cta_seg.back() != (int)pl.segs.size()) pl.cta_seg.push_back((int)pl.segs.size());
+  PortPlan pl;
+  cut(hi, &pl);
   return pl;
 }
 
 template <typename T, typename TS, int R>
-static const void* port_kernel_r(bool priv, bool mma) {
+static const void* port_kernel_r(bool priv, int mma) {
   constexpr bool can_mma = sizeof(TS) == 2 || (sizeof(TS) == 4 && R >= 4);
   if constexpr (can_mma) {
-    if constexpr (R <= 2)
-      if (mma && priv) return (const void*)k_port_sweep<T, TS, R, true, true>;
-    if (mma) return (const void*)k_port_sweep<T, TS, R, false, true>;
+    if constexpr (R <= 2) {
+      if (mma && priv) return (const void*)k_port_sweep<T, TS, R, true, 8>;
+    } else if constexpr (sizeof(TS) == 4) {
+      if (mma == 16) return (const void*)k_port_sweep<T, TS, R, false, 16>;
+    }
+    if (mma) return (const void*)k_port_sweep<T, TS, R, false, 8>;
   } else if constexpr (R <= 2) {
-    if (priv) return (const void*)k_port_sweep<T, TS, R, true, false>;
+    if (priv) return (const void*)k_port_sweep<T, TS, R, true, 0>;
   }
-  return (const void*)k_port_sweep<T, TS, R, false, false>;
+  return (const void*)k_port_sweep<T, TS, R, false, 0>;
 }
 
 template <typename T, typename TS>
-static const void* port_kernel(int R, bool priv, bool mma) {
+static const void* port_kernel(int R, bool priv, int mma) {
   switch (R) {
     case 1: return port_kernel_r<T, TS, 1>(priv, mma);
     case 2: return port_kernel_r<T, TS, 2>(priv, mma);
@@ -1141,7 +1194,7 @@ static const void* port_kernel(int R, bool priv, bool mma) {
 }
 
 template <typename T>
-static const void* port_kernel_of(int R, bool priv, bool mma, bool half) {
+static const void* port_kernel_of(int R, bool priv, int mma, bool half) {
   if constexpr (sizeof(T) == 4)
     if (half) return port_kernel<T, __half>(R, priv, mma);
   return port_kernel<T, T>(R, priv, mma);
@@ -1154,7 +1207,7 @@ cudaError_t port_sweep_configure(int R, const PortShape& sh, bool half, int* cta
   // the limit is the kernel's, not the solver's: the device maximum, whatever solver came last
   cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        (sh.mma ? 226 : 227) * 1024);
-  if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(ctas_per_sm, k, kSweepThreads, sh.smem);
+  if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(ctas_per_sm, k, sweep_threads(sh.mma), sh.smem);
   return e;
 }
 
@@ -1178,7 +1231,7 @@ static cudaError_t launch_dependent(const void* k, int grid, int block, size_t s
 template <typename T>
 cudaError_t launch_port_sweep(const PortArgs<T>& a, int R, int nports, int grid, size_t smem, cudaStream_t st) {
   if (grid <= 0 || nports <= 0) return cudaSuccess;
-  const void* k = port_kernel_of<T>(R, a.priv != 0, a.mma != 0, sizeof(T) == 4 && a.Sh);
+  const void* k = port_kernel_of<T>(R, a.priv != 0, a.mma, sizeof(T) == 4 && a.Sh);
   const void* v = R == 1   ? (const void*)k_port_vec<T, 1>
                   : R == 2 ? (const void*)k_port_vec<T, 2>
                   : R == 4 ? (const void*)k_port_vec<T, 4>
@@ -1189,7 +1242,7 @@ cudaError_t launch_port_sweep(const PortArgs<T>& a, int R, int nports, int grid,
   void* av[] = {&args, &nports};
   cudaError_t e = launch_dependent<T>(v, (n + 255) / 256, 256, 0, av, st);
   if (e != cudaSuccess) return e;
-  return launch_dependent<T>(k, grid, kSweepThreads, smem, av, st);
+  return launch_dependent<T>(k, grid, sweep_threads(a.mma), smem, av, st);
 }
 
 // FP16 copy of the FP32 tiles of one subgraph per CTA, one warp per tile: each tile is divided by

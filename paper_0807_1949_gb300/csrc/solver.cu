@@ -1260,7 +1260,7 @@ static void choose_form(vtm_solver* s, const vtm_setup_opts* o, int64_t s_tiles,
     d.sh = port_shape(sizeof(T), half ? sizeof(__half) : sizeof(T), s->R, max_ports_lo);
     VTM_CUDA(port_sweep_configure<T>(s->R, d.sh, half, &per_sm));
     const PortPlan pl = port_plan(lo.data(), (int)lo.size(), sizeof(T), half ? sizeof(__half) : sizeof(T), s->R,
-                                  std::max(1, per_sm) * nsm);
+                                  std::max(1, per_sm) * nsm, d.sh.mma);
     upload(d.segs, pl.segs, s->stream);
     upload(d.cta_seg, pl.cta_seg, s->stream);
     d.part.alloc((size_t)pl.part_elems * sizeof(T));

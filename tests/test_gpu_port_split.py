@@ -47,6 +47,11 @@ def test_divided_sweep(vtmlib, dims, block, nrhs, kind):
            TOL[kind])
 
 
+# subgraphs of up to 1000 ports with eight right-hand sides: one CTA of 16 warps per SM
+def test_divided_sweep_large(vtmlib):
+    _check(vtmlib, (40, 34, 47), (13, 11, 16), 8, "fp32", "native", 4, TOL["fp32"])
+
+
 # one CTA per subgraph and several subgraphs per CTA, every number of right-hand sides; two sweeps
 # (one resident sweep), three, and enough for both exchange buffers to be used again
 @pytest.mark.parametrize("nrhs,kind", [(1, "fp64"), (2, "fp64"), (4, "fp64"), (8, "fp64"), (1, "fp32"), (2, "fp32"),
