@@ -266,7 +266,8 @@ struct PortTCArgs {
   unsigned char* stiles;       // not FUSED: the port vectors' operand tiles (R x 512 bytes per super-row)
   const int32_t* tile_off;     // per subgraph, its first tile
   float* ssig;                 // sigma_r per subgraph and column
-  const int32_t* cpl_end;      // per coupling entry, its wave's place among the subgraph's ends
+  const int32_t* ent_ptr;      // not FUSED: per port, first entry of its sum's terms
+  const int2* ent;             // (the wave's place among the subgraph's ends, coefficient)
   int tmem_cols;               // tensor-memory columns per CTA (power of two >= n4max R)
   const float* ubase;          // ports x R
   const float* wprev;          // ends x R
@@ -287,8 +288,8 @@ size_t port_tc_smem_bytes(int R, bool lo);
 cudaError_t launch_port_records(int nports, const int32_t* port_end_ptr, const int32_t* twin, const float* invz,
                                 CoupleRef<float> cpl, int4* rec, cudaStream_t st);
 // Places of the coupling entries' waves for the separate port vectors.
-cudaError_t launch_coupling_ends(const PieceDesc* pieces, int npieces, const int32_t* twin, CoupleRef<float> cpl,
-                                 int32_t* cpl_end, cudaStream_t st);
+cudaError_t launch_port_entries(const PieceDesc* pieces, int npieces, const int32_t* port_end_ptr, const int32_t* twin,
+                                const float* invz, CoupleRef<float> cpl, int32_t* ent_ptr, int2* ent, cudaStream_t st);
 constexpr size_t kVecTcSmemMax = 220 * 1024;
 size_t port_vec_tc_smem_bytes(int max_ends);
 cudaError_t port_tc_configure(int R);

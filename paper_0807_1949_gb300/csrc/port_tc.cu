@@ -53,8 +53,8 @@
 //  * else (few items per CTA) in a launch of their own before it (k_port_vec_tc), which has every
 //    subgraph's gathers in flight at once, and warps 6-13 are two more sets of epilogue warps: super-row
 //    I belongs to set I mod 3.  Fused, eight warps waiting for 1.4 MB of scattered rows per subgraph
-//    were what such a sweep waited for.  Measured per sweep, 32 right-hand sides: 64^3 (less than one
-//    item per CTA) 0.193 -> 0.089 ms; at 128^3 (3.4 items per CTA) both take 0.557 ms.
+//    were what such a sweep waited for.  Measured per sweep, 32 right-hand sides: 64^3 (1.2 items per
+//    CTA) 0.193 -> 0.083 ms, 128^3 (3.4) 0.557 -> 0.521 ms.
 // Every wait is bounded; a CTA that gives up records VTM_ERR_TIMEOUT, lets its copies and MMAs
 // finish, frees its tensor memory and returns.
 #include <cuda_fp16.h>
@@ -368,109 +368,123 @@ __global__ void k_port_blocks_to_f16(const PieceDesc* __restrict__ pieces, const
 
 // The port vectors of every subgraph as operand tiles: s = sum_e w_in[e] / Z_e plus the coupling
 // currents, s' = G s, split per subgraph and column as s' / sigma_r = hi + lo (sigma_r the power of two
-// at or above max |s'_r|).  A CTA takes eight columns of a subgraph: their incoming waves go to shared
-// memory once (a row of 32 bytes per end, all ends' loads independent) and the port sums and the
-// coupling currents, which read every wave about five times, are formed from there; the maxima stay
-// inside the CTA.  Bound by L2: the waves, the lists (once per CTA) and the tiles.
-constexpr int kVecTcThreads = 512;
-constexpr int kVecCols = 8;
+// at or above max |s'_r|).  A CTA takes sixteen columns of a subgraph: their incoming waves go to shared
+// memory once (a row of 64 bytes per end, all ends' loads independent) and the sums, which read every
+// wave about five times, are formed from there, a port's terms from one list (launch_port_entries); the
+// maxima stay inside the CTA.  Four lanes share a port, each with four columns: a row's four 16-byte
+// pieces come from four lanes of one load, so two ports' rows meet in a bank half the time (a port per
+// lane: eight lanes, four bank groups).  Bound by the latency of its phases and the issue rate of the sums,
+// one CTA of 32 warps per SM: 64^3 with 32 right-hand sides 19 us, 128^3 115 us (22 and 150 with a port
+// per lane and its lists read from global memory).
+constexpr int kVecTcThreads = 1024;
+constexpr int kVecCols = 16;
 
 template <int R>
-__global__ void __launch_bounds__(kVecTcThreads, 2) k_port_vec_tc(const PortTCArgs a) {
-  constexpr int kPorts = kMaxSuper * kSB / kVecTcThreads;  // ports per thread, at most
-  extern __shared__ __align__(16) float win[];              // [ends][kVecCols]
+__global__ void __launch_bounds__(kVecTcThreads, 1) k_port_vec_tc(const PortTCArgs a) {
+  constexpr int kStep = kVecTcThreads / 4;                // ports per pass
+  constexpr int kPass = kMaxSuper * kSB / kStep;          // passes, at most
+  extern __shared__ __align__(16) float win[];            // [ends][kVecCols]
   __shared__ float red[kVecTcThreads / 32][kVecCols];
   __shared__ float inv[kVecCols];
   grid_dep_launch();
   const int piece = blockIdx.x, q0 = blockIdx.y * kVecCols;
   const PieceDesc pd = a.pieces[piece];
   const int Pn = pd.nports, np = n_super(Pn) * kSB;
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, c4 = tid & 3, p0 = tid >> 2;
+  // before the wait, what no sweep changes: the lists into the shared memory that the waves leave (read
+  // in place where they do not fit), their bounds and the first twins into registers
+  const int first = Pn > 0 ? a.ent_ptr[pd.port_off] : 0, nent = Pn > 0 ? a.ent_ptr[pd.port_off + Pn] - first : 0;
+  int2* const list = reinterpret_cast<int2*>(win + (size_t)pd.nends * kVecCols);
+  const bool staged = ((size_t)pd.nends * kVecCols + 2 * (size_t)nent) * sizeof(float) <= kVecTcSmemMax;
+  if (staged)
+    for (int k = tid; k < nent; k += kVecTcThreads)
+      asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(smem_u32(list + k)), "l"(a.ent + first + k));
+  const int2* const ent = staged ? list : a.ent + first;
+  int k0[kPass], k1[kPass];
+#pragma unroll
+  for (int i = 0; i < kPass; ++i) {
+    const int p = i * kStep + p0;
+    k0[i] = k1[i] = 0;
+    if (p < Pn) {
+      k0[i] = a.ent_ptr[pd.port_off + p] - first;
+      k1[i] = a.ent_ptr[pd.port_off + p + 1] - first;
+    }
+  }
+  constexpr int kTwins = 8;
+  int tw[kTwins];
+#pragma unroll
+  for (int u = 0; u < kTwins; ++u) {
+    const int i = tid + u * kVecTcThreads;
+    tw[u] = i < 4 * pd.nends ? a.twin[pd.end_off + (i >> 2)] : 0;
+  }
   grid_dep_wait();
+  auto wave = [&](int i, int t) {  // 16 bytes of the incoming wave of end i / 4
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_u32(win + 4 * i)),
+                 "l"(a.wprev + (size_t)t * R + q0 + 4 * c4));
+  };
+#pragma unroll
+  for (int u = 0; u < kTwins; ++u)
+    if (tid + u * kVecTcThreads < 4 * pd.nends) wave(tid + u * kVecTcThreads, tw[u]);
+  for (int i = tid + kTwins * kVecTcThreads; i < 4 * pd.nends; i += kVecTcThreads)
+    wave(i, a.twin[pd.end_off + (i >> 2)]);
+  asm volatile("cp.async.wait_all;" ::: "memory");
+  __syncthreads();
+  float v[kPass][4];
+#pragma unroll
+  for (int i = 0; i < kPass; ++i) {
+    float s[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll 4
-  for (int i = tid; i < 2 * pd.nends; i += kVecTcThreads) {
-    const int tw = a.twin[pd.end_off + (i >> 1)];
-    reinterpret_cast<float4*>(win)[i] =
-        __ldcg(reinterpret_cast<const float4*>(a.wprev + (size_t)tw * R + q0) + (i & 1));
-  }
-  __syncthreads();
-  // port pairs 2 (i kVecTcThreads + tid), + 1: a thread writes both with one store per column
-  float v[kPorts][kVecCols];
-#pragma unroll
-  for (int i = 0; i < kPorts; i += 2) {
-    const int p = i * kVecTcThreads + 2 * tid;
-    int e0[2], e1[2], k0[2], k1[2];
-    float gp[2];
-#pragma unroll
-    for (int j = 0; j < 2; ++j) {
-      const bool on = p + j < Pn;
-      const int port = pd.port_off + (on ? p + j : 0);
-      e0[j] = a.port_end_ptr[port];
-      e1[j] = on ? a.port_end_ptr[port + 1] : e0[j];
-      k0[j] = a.cpl.ptr ? a.cpl.ptr[port] : 0;
-      k1[j] = on && a.cpl.ptr ? a.cpl.ptr[port + 1] : k0[j];
-      gp[j] = on ? a.gscale[port] : 0.f;
+    for (int k = k0[i]; k < k1[i]; ++k) {
+      const int2 en = ent[k];
+      const float4 x = reinterpret_cast<const float4*>(win)[4 * en.x + c4];
+      const float y = __int_as_float(en.y);
+      s[0] += x.x * y, s[1] += x.y * y, s[2] += x.z * y, s[3] += x.w * y;
     }
+    const int p = i * kStep + p0;
+    const float gp = p < Pn ? a.gscale[pd.port_off + p] : 0.f;
 #pragma unroll
-    for (int j = 0; j < 2; ++j) {
-      float s[kVecCols], c[kVecCols];
-#pragma unroll
-      for (int q = 0; q < kVecCols; ++q) s[q] = c[q] = 0.f;
-      auto add = [&](int e, float y, float (&sum)[kVecCols]) {
-        const float4 x0 = reinterpret_cast<const float4*>(win)[2 * e], x1 = reinterpret_cast<const float4*>(win)[2 * e + 1];
-        sum[0] += x0.x * y, sum[1] += x0.y * y, sum[2] += x0.z * y, sum[3] += x0.w * y;
-        sum[4] += x1.x * y, sum[5] += x1.y * y, sum[6] += x1.z * y, sum[7] += x1.w * y;
-      };
-      for (int e = e0[j]; e < e1[j]; ++e) add(e - pd.end_off, a.invz[e], s);
-      for (int k = k0[j]; k < k1[j]; k += 4) {  // four entries' loads in flight together
-        int at[4];
-        float y[4];
-#pragma unroll
-        for (int u = 0; u < 4; ++u) {
-          at[u] = k + u < k1[j] ? a.cpl_end[k + u] : 0;
-          y[u] = k + u < k1[j] ? a.cpl.y[k + u] : 0.f;
-        }
-#pragma unroll
-        for (int u = 0; u < 4; ++u)
-          if (k + u < k1[j]) add(at[u], y[u], c);
-      }
-#pragma unroll
-      for (int q = 0; q < kVecCols; ++q) v[i + j][q] = (s[q] + c[q]) * gp[j];
-    }
+    for (int q = 0; q < 4; ++q) v[i][q] = s[q] * gp;
   }
 #pragma unroll
-  for (int q = 0; q < kVecCols; ++q) {
+  for (int q = 0; q < 4; ++q) {
     float m = 0.f;
 #pragma unroll
-    for (int i = 0; i < kPorts; ++i) m = fmaxf(m, fabsf(v[i][q]));
+    for (int i = 0; i < kPass; ++i) m = fmaxf(m, fabsf(v[i][q]));
 #pragma unroll
-    for (int o = 1; o < 32; o <<= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
-    if (lane == 0) red[warp][q] = m;
+    for (int o = 4; o < 32; o <<= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
+    if (lane < 4) red[warp][4 * lane + q] = m;
   }
   __syncthreads();
-  if (tid < kVecCols) {
-    float m = 0.f;
+  if (warp < kVecCols / 2) {  // two columns per warp, sixteen lanes each
+    const int c = 2 * warp + (lane >> 4);
+    float m = fmaxf(red[lane & 15][c], red[16 + (lane & 15)][c]);
 #pragma unroll
-    for (int w = 0; w < kVecTcThreads / 32; ++w) m = fmaxf(m, red[w][tid]);
-    int e = 0;
-    if (m > 0.f && isfinite(m)) frexpf(m, &e);
-    e = e < -120 ? -120 : e;
-    inv[tid] = ldexpf(1.f, -e);
-    a.ssig[(size_t)piece * R + q0 + tid] = ldexpf(1.f, e);  // power of two >= max |s_r|
+    for (int o = 1; o < 16; o <<= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
+    if ((lane & 15) == 0) {
+      int e = 0;
+      if (m > 0.f && isfinite(m)) frexpf(m, &e);
+      e = e < -120 ? -120 : e;
+      inv[c] = ldexpf(1.f, -e);
+      a.ssig[(size_t)piece * R + q0 + c] = ldexpf(1.f, e);  // power of two >= max |s_r|
+    }
   }
   __syncthreads();
-  // tile: [hi, ports 0-63][hi, 64-127][lo, 0-63][lo, 64-127] of R rows (columns of s) each
+  // tile: [hi, ports 0-63][hi, 64-127][lo, 0-63][lo, 64-127] of R rows (columns of s) each.  The lanes of
+  // ports p and p + 1 exchange half their columns, so that each writes both ports of two columns at once.
   unsigned char* const tiles = a.stiles + (size_t)a.tile_off[piece] * ((size_t)R * 512);
+  const bool odd = lane & 4;
 #pragma unroll
-  for (int i = 0; i < kPorts; i += 2) {
-    const int p = i * kVecTcThreads + 2 * tid;
-    if (p >= np) break;
+  for (int i = 0; i < kPass; ++i) {
+    const int p = (i * kStep + p0) & ~1;
+    if (p >= np) continue;  // the same for both lanes of a pair: np is a multiple of 128, and for the warp
     unsigned char* const panel = tiles + (size_t)(p / kSB) * R * 512 + (size_t)((p % kSB) / 64) * R * 128;
 #pragma unroll
-    for (int q = 0; q < kVecCols; ++q) {
-      const float x0 = v[i][q] * inv[q], x1 = v[i + 1][q] * inv[q];
+    for (int h = 0; h < 2; ++h) {
+      const float got = __shfl_xor_sync(0xffffffffu, odd ? v[i][h] : v[i][2 + h], 4);
+      const int c = 4 * c4 + (odd ? 2 : 0) + h;
+      const float x0 = (odd ? got : v[i][h]) * inv[c], x1 = (odd ? v[i][2 + h] : got) * inv[c];
       const __half2 hi = __floats2half2_rn(x0, x1);
-      const uint32_t off = swz16(q0 + q, p % 64);
+      const uint32_t off = swz16(q0 + c, p % 64);
       *reinterpret_cast<__half2*>(panel + off) = hi;
       *reinterpret_cast<__half2*>(panel + 2 * R * 128 + off) =
           __floats2half2_rn(x0 - __low2float(hi), x1 - __high2float(hi));
@@ -478,20 +492,28 @@ __global__ void __launch_bounds__(kVecTcThreads, 2) k_port_vec_tc(const PortTCAr
   }
 }
 
-// Coupling entry k of a port as the place of its wave among the subgraph's ends (the incoming wave of
-// end e' is the twin's, whose own twin is e').
-__global__ void k_coupling_ends(const PieceDesc* __restrict__ pieces, const int32_t* __restrict__ twin,
-                                CoupleRef<float> cpl, int32_t* __restrict__ cpl_end) {
+// The terms of a port's sum as one list, (place of the wave among the subgraph's ends, coefficient): its
+// ends with 1 / Z_e, then its coupling entries (the incoming wave of end e' is the twin's, whose own twin
+// is e').  The lists of the ports follow each other in port order.
+__global__ void k_port_entries(const PieceDesc* __restrict__ pieces, const int32_t* __restrict__ port_end_ptr,
+                               const int32_t* __restrict__ twin, const float* __restrict__ invz, CoupleRef<float> cpl,
+                               int32_t* __restrict__ ent_ptr, int2* __restrict__ ent) {
   const PieceDesc pd = pieces[blockIdx.x];
-  if (pd.nports == 0) return;
-  for (int k = cpl.ptr[pd.port_off] + threadIdx.x; k < cpl.ptr[pd.port_off + pd.nports]; k += blockDim.x)
-    cpl_end[k] = twin[cpl.oth[k]] - pd.end_off;
+  for (int q = pd.port_off + threadIdx.x; q < pd.port_off + pd.nports; q += blockDim.x) {
+    const int e0 = port_end_ptr[q], e1 = port_end_ptr[q + 1];
+    const int k0 = cpl.ptr ? cpl.ptr[q] : 0, k1 = cpl.ptr ? cpl.ptr[q + 1] : 0;
+    int at = e0 + k0;
+    ent_ptr[q] = at;
+    ent_ptr[q + 1] = e1 + k1;  // the next port's thread writes the same
+    for (int e = e0; e < e1; ++e) ent[at++] = make_int2(e - pd.end_off, __float_as_int(invz[e]));
+    for (int k = k0; k < k1; ++k) ent[at++] = make_int2(twin[cpl.oth[k]] - pd.end_off, __float_as_int(cpl.y[k]));
+  }
 }
 
-cudaError_t launch_coupling_ends(const PieceDesc* pieces, int npieces, const int32_t* twin, CoupleRef<float> cpl,
-                                 int32_t* cpl_end, cudaStream_t st) {
-  if (npieces <= 0 || !cpl.ptr) return cudaSuccess;
-  k_coupling_ends<<<npieces, 256, 0, st>>>(pieces, twin, cpl, cpl_end);
+cudaError_t launch_port_entries(const PieceDesc* pieces, int npieces, const int32_t* port_end_ptr, const int32_t* twin,
+                                const float* invz, CoupleRef<float> cpl, int32_t* ent_ptr, int2* ent, cudaStream_t st) {
+  if (npieces <= 0) return cudaSuccess;
+  k_port_entries<<<npieces, 256, 0, st>>>(pieces, port_end_ptr, twin, invz, cpl, ent_ptr, ent);
   return cudaGetLastError();
 }
 
@@ -1103,7 +1125,7 @@ cudaError_t launch_port_sweep_tc(const PortTCArgs& a, int R, bool lo, int npiece
   cudaError_t e = cudaSuccess;
   if (!fused)
     e = launch(R == 16 ? (const void*)k_port_vec_tc<16> : (const void*)k_port_vec_tc<32>, dim3(npieces, R / kVecCols),
-               kVecTcThreads, port_vec_tc_smem_bytes(max_ends), true);
+               kVecTcThreads, kVecTcSmemMax, true);
   if (e != cudaSuccess) return e;
   const void* k = R == 16 ? tc_kernel<16>(lo, fused) : tc_kernel<32>(lo, fused);
   e = launch(k, dim3(grid), kTcThreads, port_tc_smem_bytes(R, lo), false);

@@ -152,7 +152,7 @@ struct vtm_solver {
   int res_grid = 0, res_pieces = 0;
   size_t res_smem = 0;
   DevBuf S16, sig16;                 // tensor-core form: fp16 hi / lo blocks, sigma_j
-  DevBuf tc_stiles, tc_tile_off, tc_ssig, tc_cpl_end;  // separate port vectors: operand tiles, their places, sigma_r
+  DevBuf tc_stiles, tc_tile_off, tc_ssig, tc_ent, tc_ent_ptr;  // separate port vectors: operand tiles, their places, sigma_r, terms
   DevBuf tc_scratch, port_rec;       // fused port vectors: s^T slots, gather records
   int tc_n4max = 0, tc_max_ends = 0;
   DevBuf gscale;                     // tensor-core form: sqrt(S_pp) per port (diagonal balance)
@@ -1066,7 +1066,8 @@ static void launch_port(vtm_solver* s) {
       t.scratch = s->tc_scratch.as<unsigned char>();
       t.n4max = s->tc_n4max;
       t.prec = s->port_rec.as<int4>();
-      t.cpl_end = s->tc_cpl_end.as<int32_t>();
+      t.ent_ptr = s->tc_ent_ptr.as<int32_t>();
+      t.ent = s->tc_ent.as<int2>();
       t.stiles = s->tc_stiles.as<unsigned char>();  // null: fused
       t.tile_off = s->tc_tile_off.as<int32_t>();
       t.ssig = s->tc_ssig.as<float>();
@@ -1285,9 +1286,10 @@ static void choose_form(vtm_solver* s, const vtm_setup_opts* o, int64_t s_tiles,
     for (const PieceDesc& d : lo) s->tc_max_ends = std::max(s->tc_max_ends, d.nends);
     // The port vectors: a launch of their own up to kTcSeparate items per CTA, fused beyond (there the
     // gathers hide behind the next items' blocks, and the operand tiles would pass through HBM).
-    // 64^3 with 32 right-hand sides (1.2 items per CTA) 0.089 ms separate, 0.193 fused; 128^3 (3.4)
-    // 0.557 either way; 256^3 (27) 3.86 fused.
-    constexpr double kTcSeparate = 2.0;
+    // 64^3 with 32 right-hand sides (1.2 items per CTA) 0.083 ms separate, 0.193 fused; 128^3 (3.4)
+    // 0.521 and 0.557; 256^3 (27) 3.86 fused, where the tiles and a second pass over the waves would
+    // add 2.3 GB to 25.
+    constexpr double kTcSeparate = 5.0;
     const bool separate = (double)pl.items.size() <= kTcSeparate * nsm &&
                           port_vec_tc_smem_bytes(s->tc_max_ends) <= kVecTcSmemMax;
     if (separate) {
@@ -1295,11 +1297,11 @@ static void choose_form(vtm_solver* s, const vtm_setup_opts* o, int64_t s_tiles,
       VTM_CUDA(cudaStreamSynchronize(s->stream));
       s->tc_stiles.alloc((size_t)std::max<int64_t>(1, pl.tiles) * s->R * 512);
       s->tc_ssig.alloc((size_t)s->np_lo * s->R * sizeof(float));
-      if (s->coupled) {
-        s->tc_cpl_end.alloc(s->cp_oth.bytes);
-        VTM_CUDA(launch_coupling_ends(s->pieces_lo.as<PieceDesc>(), s->np_lo, s->twin.as<int32_t>(), couple_ref<float>(s),
-                                      s->tc_cpl_end.as<int32_t>(), s->stream));
-      }
+      s->tc_ent_ptr.alloc((size_t)(s->nports + 1) * sizeof(int32_t));
+      s->tc_ent.alloc(((size_t)std::max<int64_t>(1, s->E) + (s->coupled ? s->cp_oth.bytes / sizeof(int32_t) : 0)) * sizeof(int2));
+      VTM_CUDA(launch_port_entries(s->pieces_lo.as<PieceDesc>(), s->np_lo, s->port_end_ptr.as<int32_t>(),
+                                   s->twin.as<int32_t>(), s->invz_t.as<float>(), couple_ref<float>(s),
+                                   s->tc_ent_ptr.as<int32_t>(), s->tc_ent.as<int2>(), s->stream));
     } else {
       s->tc_scratch.alloc((size_t)s->tc_grid * ((size_t)2 * n4max * s->R * 512 + (size_t)n4max * 128 * s->R * 4));
       s->port_rec.alloc((size_t)std::max(1, s->nports) * 3 * sizeof(int4));
