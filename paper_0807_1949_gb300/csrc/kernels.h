@@ -41,7 +41,7 @@ struct SweepArgs {
                                // piece at row_off (nullptr: y goes through xc, TF == TV)
   CoupleRef<TV> cpl;           // coupled lines: per-port coupling lists (cpl.ptr == nullptr: none)
   const unsigned char* wt;     // tensor-core factor of sweep_wide_tc.cu (nullptr: not built)
-  // Wide kernels, unit sources at the ports instead of b̃ and waves (the columns of S_j): CTA (j, y)
+  // Unit sources (all kernels but the pipelined one) at the ports instead of b̃ and waves (the columns of S_j): CTA (j, y)
   // solves for the R ports from (unit_b0 + y) R on, for the rows from port
   // floor((unit_b0 + y) R / unit_gran) unit_gran on, into xc + y unit_stride; no waves are read or written.
   int unit = 0;
@@ -56,7 +56,7 @@ cudaError_t sweep_configure(int R, size_t smem);
 template <typename TF, typename TV>
 cudaError_t sweep_occupancy(int R, size_t smem, int* ctas_per_sm);
 template <typename TF, typename TV>
-cudaError_t launch_sweep(const SweepArgs<TF, TV>& a, int R, int npieces, size_t smem, cudaStream_t st);
+cudaError_t launch_sweep(const SweepArgs<TF, TV>& a, int R, int npieces, size_t smem, cudaStream_t st, int batches = 1);
 
 // Pipelined variant: chain warps finish block k while the others prepare block k+1.
 constexpr size_t kPipeSmemMax = 226 * 1024;  // dynamic shared memory the kernel may take

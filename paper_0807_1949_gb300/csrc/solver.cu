@@ -901,12 +901,12 @@ static void autotune_sweep(vtm_solver* s) {
 
 // S_j = P^T K_j^{-1} P from unit sources at the ports with zero incident waves: the multi-RHS band
 // sweep with 32 port columns (16 with 16 right-hand sides) per subgraph and batch where it fits in shared
-// memory, else the solver's own sweep with its R columns.  Of a batch only the rows from its first port
+// memory, else the solver's own sweep with its R columns (FP64 with half-bandwidths above 160).  Of a batch only the rows from its first port
 // on are solved for: the solution of the forward pass is zero above them, and of S_j, which is
 // symmetric, only the blocks on and below the diagonal are kept, so the backward pass ends there too
 // (about half the work).  A launch takes several batches, eight CTAs per SM in all: with a launch per
 // batch 64 subgraphs left 88 of 152 SMs idle, and 512 took four waves of CTAs for 3.4.  FP32, 16^3
-// blocks: 64^3 29 -> 4.5 ms, 128^3 114 -> 39 ms.  Only the subgraphs of the main launch get an S_j:
+// blocks: 64^3 29 -> 4.5 ms, 128^3 114 -> 39 ms; FP64 64^3 (own sweep) 1790 -> 290 ms.  Only the subgraphs of the main launch get an S_j:
 // subgraphs flagged ill-conditioned keep their FP64 band sweep every sweep (S_j in FP32 would carry the
 // same cancellation that made their FP32 factor fail).
 template <typename T>
@@ -944,11 +944,12 @@ static void compute_port_response(vtm_solver* s, int64_t s_tiles) {
   VTM_CUDA(cudaEventCreate(&e0));
   VTM_CUDA(cudaEventCreate(&e1));
   VTM_CUDA(cudaEventRecord(e0, st));
-  if (st_lo && s->np_lo > 0) {
-    const int Rs = s->wide ? s->R : 32;
+  const bool own = !st_lo && !s->pipe;  // the solver's own single-block sweep
+  if ((st_lo || own) && s->np_lo > 0) {
+    const int Rs = s->wide || own ? s->R : 32;
     const int nb = (s->max_ports + Rs - 1) / Rs;
     SweepArgs<T, T> a = sweep_args<T, T>(s, 1, false);
-    a.stages = st_lo;
+    if (!own) a.stages = st_lo;
     a.withhold = -1;
     a.yspill = nullptr;
     a.unit = 1;
@@ -959,7 +960,7 @@ static void compute_port_response(vtm_solver* s, int64_t s_tiles) {
     DevBuf wt_tmp, xcs;
     size_t fb = 0, tb = 0;
     VTM_CUDA(cudaMemGetInfo(&fb, &tb));
-    if (!s->wide) {
+    if (!s->wide && !own) {
       VTM_CUDA((sweep_wide_configure<T, T>(Rs, sm_lo)));
       if constexpr (sizeof(T) == 4) {
         if (s->wt_ok && (double)s->wt_bytes < 0.4 * (double)fb) {
@@ -994,7 +995,8 @@ static void compute_port_response(vtm_solver* s, int64_t s_tiles) {
           done = true;
         }
       }
-      if (!done) VTM_CUDA((launch_sweep_wide<T, T>(a, Rs, s->np_lo, sm_lo, st, m)));
+      if (own) VTM_CUDA((launch_sweep<T, T>(a, Rs, s->np_lo, s->sweep_smem, st, m)));
+      else if (!done) VTM_CUDA((launch_sweep_wide<T, T>(a, Rs, s->np_lo, sm_lo, st, m)));
       gather(Rs, b, a.xc, m, a.unit_stride);
     }
     VTM_CUDA(cudaStreamSynchronize(st));

@@ -32,7 +32,13 @@ __global__ void __launch_bounds__(kSweepThreads, 2) k_sweep(const SweepArgs<T, T
   const int Wp = pd.Wp;
   const int off = Wp - 1;  // ys row of column 0
   const int nblk = pd.n_pad / kNB;
-  const int total = 2 * nblk;
+  // unit sources: batch blockIdx.y's columns, rows from the first one that S_j is wanted at
+  const int ub = (a.unit_b0 + (int)blockIdx.y) * R;  // first port of the batch
+  if (a.unit && ub >= pd.nports) return;
+  const int blk0 = a.unit ? a.port_local[pd.port_off + ub / a.unit_gran * a.unit_gran] / kNB : 0;  // first block
+  const int row0 = blk0 * kNB;
+  const int nfwd = nblk - blk0;
+  const int total = 2 * nfwd;
   const uint32_t slab_bytes = (uint32_t)(kNB * Wp * sizeof(T));
   const T* fbase = a.factor + pd.factor_off;
   const T* ubase = a.factor_u + pd.factor_off;
@@ -46,10 +52,10 @@ __global__ void __launch_bounds__(kSweepThreads, 2) k_sweep(const SweepArgs<T, T
   __syncthreads();
   auto issue = [&](int s) {
     if (s == a.withhold) return;  // testing hook: this slab's wait can only run out
-    const int kb = s < nblk ? s : total - 1 - s;
+    const int kb = blk0 + (s < nfwd ? s : total - 1 - s);
     const int slot = s % S;
     mbar_arrive_expect_tx(&bars[slot], slab_bytes);
-    bulk_copy_g2s(ring + (size_t)slot * a.slot_elems, (s < nblk ? fbase : ubase) + (size_t)kb * kNB * Wp, slab_bytes,
+    bulk_copy_g2s(ring + (size_t)slot * a.slot_elems, (s < nfwd ? fbase : ubase) + (size_t)kb * kNB * Wp, slab_bytes,
                   &bars[slot]);
   };
   if (tid == 0)
@@ -61,9 +67,15 @@ __global__ void __launch_bounds__(kSweepThreads, 2) k_sweep(const SweepArgs<T, T
     ys[(size_t)(off + pd.n_pad) * R + i] = T(0);
   }
   const TV* btp = a.bt + (size_t)pd.copy_off * R;
-  for (int i = tid; i < pd.n_pad * R; i += kSweepThreads) ys[(size_t)off * R + i] = (i < pd.n * R) ? (T)btp[i] : T(0);
+  if (a.unit) {
+    // the rows read: from off above row0 (zero: the forward solution starts there)
+    for (int i = row0 * R + tid; i < (off + pd.n_pad) * R; i += kSweepThreads) ys[i] = T(0);
+  } else {
+    for (int i = tid; i < pd.n_pad * R; i += kSweepThreads) ys[(size_t)off * R + i] = (i < pd.n * R) ? (T)btp[i] : T(0);
+  }
   __syncthreads();
-  for (int q = tid; q < pd.nports; q += kSweepThreads) {
+  if (a.unit && tid < R && ub + tid < pd.nports) ys[(size_t)(off + a.port_local[pd.port_off + ub + tid]) * R + tid] = T(1);
+  for (int q = tid; q < pd.nports && !a.unit; q += kSweepThreads) {
     const int l = a.port_local[pd.port_off + q];
     const int e0 = a.port_end_ptr[pd.port_off + q], e1 = a.port_end_ptr[pd.port_off + q + 1];
     T acc[R];
@@ -87,7 +99,7 @@ __global__ void __launch_bounds__(kSweepThreads, 2) k_sweep(const SweepArgs<T, T
   }
   __syncthreads();
 
-  // ---- forward (s < nblk) then backward (s >= nblk) over the staged slabs
+  // ---- forward (s < nfwd) then backward (s >= nfwd) over the staged slabs
   const int rg = tid >> 3, g = tid & 7;
   int s = 0;
   for (; s < total; ++s) {
@@ -96,8 +108,8 @@ __global__ void __launch_bounds__(kSweepThreads, 2) k_sweep(const SweepArgs<T, T
     __syncthreads();
     if (abort_flag) break;
     const T* L = ring + (size_t)slot * a.slot_elems;
-    if (s < nblk) {
-      const int k0 = s * kNB;
+    if (s < nfwd) {
+      const int k0 = row0 + s * kNB;
       // t_r = r_r - sum_{col < k0} L[r][col] y_col   (positions p < off - r of row r)
       const T* Lr = L + rg * Wp;
       const int pend = off - rg;
@@ -148,7 +160,7 @@ __global__ void __launch_bounds__(kSweepThreads, 2) k_sweep(const SweepArgs<T, T
 #pragma unroll
         for (int rr = 0; rr < R; ++rr) ys[(size_t)(k0 + rg + off) * R + rr] = acc2[rr];
     } else {
-      const int k0 = (total - 1 - s) * kNB;
+      const int k0 = row0 + (total - 1 - s) * kNB;
       // rows of U = L^T: t_r = y_r - sum_{col > k0+31} U[r][col] x_col  (positions p >= 32 - r)
       const T* Ur = L + rg * Wp;
       const int pbeg = kNB - rg;
@@ -215,7 +227,7 @@ __global__ void __launch_bounds__(kSweepThreads, 2) k_sweep(const SweepArgs<T, T
   }
 
   // ---- epilogue: w_out[e] = 2 x_c - w_in[e]; local solution
-  for (int q = tid; q < pd.nports; q += kSweepThreads) {
+  for (int q = tid; q < pd.nports && !a.unit; q += kSweepThreads) {
     const int l = a.port_local[pd.port_off + q];
     const int e0 = a.port_end_ptr[pd.port_off + q], e1 = a.port_end_ptr[pd.port_off + q + 1];
     for (int e = e0; e < e1; ++e)
@@ -224,8 +236,8 @@ __global__ void __launch_bounds__(kSweepThreads, 2) k_sweep(const SweepArgs<T, T
         a.wnext[(size_t)e * R + rr] = (TV)(T(2) * ys[(size_t)(off + l) * R + rr] - win[(e - pd.end_off) * R + rr]);
   }
   if (a.write_x) {
-    TV* xp = a.xc + (size_t)pd.copy_off * R;
-    for (int i = tid; i < pd.n * R; i += kSweepThreads) xp[i] = (TV)ys[(size_t)off * R + i];
+    TV* xp = a.xc + (size_t)blockIdx.y * a.unit_stride + (size_t)pd.copy_off * R;
+    for (int i = row0 * R + tid; i < pd.n * R; i += kSweepThreads) xp[i] = (TV)ys[(size_t)off * R + i];
   }
 }
 
@@ -559,9 +571,10 @@ cudaError_t sweep_occupancy(int R, size_t smem, int* n) {
 }
 
 template <typename TF, typename TV>
-cudaError_t launch_sweep(const SweepArgs<TF, TV>& a, int R, int npieces, size_t smem, cudaStream_t st) {
+cudaError_t launch_sweep(const SweepArgs<TF, TV>& a, int R, int npieces, size_t smem, cudaStream_t st,
+                         int batches) {
   if (npieces <= 0) return cudaSuccess;
-  dim3 grid(npieces), block(kSweepThreads);
+  dim3 grid(npieces, batches), block(kSweepThreads);
   switch (R) {
     case 1: k_sweep<TF, TV, 1><<<grid, block, smem, st>>>(a); break;
     case 2: k_sweep<TF, TV, 2><<<grid, block, smem, st>>>(a); break;
@@ -575,7 +588,7 @@ cudaError_t launch_sweep(const SweepArgs<TF, TV>& a, int R, int npieces, size_t 
 #define VTM_SWEEP_INST(TF, TV)                                                                    \
   template cudaError_t sweep_configure<TF, TV>(int, size_t);                                       \
   template cudaError_t sweep_occupancy<TF, TV>(int, size_t, int*);                                 \
-  template cudaError_t launch_sweep<TF, TV>(const SweepArgs<TF, TV>&, int, int, size_t, cudaStream_t);
+  template cudaError_t launch_sweep<TF, TV>(const SweepArgs<TF, TV>&, int, int, size_t, cudaStream_t, int);
 VTM_SWEEP_INST(float, float)
 VTM_SWEEP_INST(double, double)
 VTM_SWEEP_INST(double, float)
