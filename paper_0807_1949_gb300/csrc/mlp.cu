@@ -510,7 +510,7 @@ struct vtm_mlp {
   float* v = nullptr;       // Adam second moment
   float* g = nullptr;       // gradient
   float* loss = nullptr;    // device scalar
-  float* part = nullptr;    // the gradient kernel's partials, made by the first loss_grad
+  float* part = nullptr;    // the gradient kernel's partials
   int part_ctas = 0;
   float* h_loss = nullptr;  // pinned
   __nv_bfloat16* wb = nullptr;  // BF16 weights used by the kernels
@@ -554,6 +554,15 @@ vtm_mlp* mlp_create(uint64_t seed) {
   MLP_CUDA(cudaMalloc(&m->g, pb));
   MLP_CUDA(cudaMalloc(&m->loss, sizeof(float)));
   MLP_CUDA(cudaMalloc(&m->wb, kParams * sizeof(__nv_bfloat16)));
+  // the gradient's workspace (5.8 MB), here so that the first gradient costs what the others do
+  int dev = 0, nsm = 1;
+  MLP_CUDA(cudaGetDevice(&dev));
+  MLP_CUDA(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
+  m->part_ctas = 2 * nsm;  // as many CTAs as run at a time
+  MLP_CUDA(cudaMalloc(&m->part, (size_t)m->part_ctas * kPart * sizeof(float)));
+  MLP_CUDA(cudaMallocHost(&m->h_loss, sizeof(float)));
+  for (const void* k : {(const void*)k_mlp_grad<true>, (const void*)k_mlp_grad<false>})
+    MLP_CUDA(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(GradSmem)));
   // He-uniform weights, zero biases
   std::vector<float> h(kParams, 0.f);
   auto fill = [&](int off, int rows, int cols) {
@@ -606,16 +615,6 @@ void mlp_forward(const vtm_mlp* m, const float* X, float* y, int64_t n, cudaStre
 
 float mlp_loss_grad(vtm_mlp* m, const float* X, const float* t, int64_t n, cudaStream_t st) {
   if (n <= 0) fail(VTM_ERR_INVALID, "empty batch");
-  if (!m->part) {
-    int dev = 0, nsm = 1;
-    MLP_CUDA(cudaGetDevice(&dev));
-    MLP_CUDA(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
-    if (!m->h_loss) MLP_CUDA(cudaMallocHost(&m->h_loss, sizeof(float)));
-    MLP_CUDA(cudaMalloc(&m->part, (size_t)2 * nsm * kPart * sizeof(float)));
-    m->part_ctas = 2 * nsm;  // as many CTAs as run at a time
-    for (const void* k : {(const void*)k_mlp_grad<true>, (const void*)k_mlp_grad<false>})
-      MLP_CUDA(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(GradSmem)));
-  }
   const int grid = (int)std::min<int64_t>((n + kTile - 1) / kTile, m->part_ctas);
   const float inv_n = 1.f / (float)n;
   if (reinterpret_cast<uintptr_t>(X) % 8 == 0)
