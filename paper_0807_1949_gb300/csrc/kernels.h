@@ -296,7 +296,7 @@ cudaError_t port_tc_configure(int R);
 // The port vectors (unless fused: a.stiles == nullptr), one persistent launch for the sweep (grid <=
 // SMs), and one for the cut subgraphs' waves if there are any; lo = use the lo half of S_j
 // (FP32-accurate).
-cudaError_t launch_port_sweep_tc(const PortTCArgs& a, int R, bool lo, int npieces, int max_ends, int grid, int nsplits,
+cudaError_t launch_port_sweep_tc(const PortTCArgs& a, int R, bool lo, int npieces, int grid, int nsplits,
                                  int max_split_ports, cudaStream_t st);
 cudaError_t launch_gather_port_blocks(const PieceDesc* pieces, int npieces, const int32_t* port_local, int Rs, int b,
                                       const float* xc, float* S32, cudaStream_t st, int batches = 1,

@@ -1099,7 +1099,7 @@ cudaError_t port_tc_configure(int R) {
   return e;
 }
 
-cudaError_t launch_port_sweep_tc(const PortTCArgs& a, int R, bool lo, int npieces, int max_ends, int grid, int nsplits,
+cudaError_t launch_port_sweep_tc(const PortTCArgs& a, int R, bool lo, int npieces, int grid, int nsplits,
                                  int max_split_ports, cudaStream_t st) {
   if (grid <= 0) return cudaSuccess;
   if (R != 16 && R != 32) return cudaErrorInvalidValue;

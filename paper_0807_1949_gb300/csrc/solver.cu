@@ -1087,7 +1087,7 @@ static void launch_port(vtm_solver* s) {
       t.cpl = couple_ref<float>(s);
       t.status = s->status.as<int>();
       t.wait_limit = s->wait_limit;
-      VTM_CUDA(launch_port_sweep_tc(t, s->R, !s->port_half, s->np_lo, s->tc_max_ends, s->tc_grid, s->tc_nsplits,
+      VTM_CUDA(launch_port_sweep_tc(t, s->R, !s->port_half, s->np_lo, s->tc_grid, s->tc_nsplits,
                                     s->tc_split_ports, s->stream));
       s->launches += 1 + (s->tc_stiles.p ? 1 : 0) + (s->tc_nsplits > 0 ? 1 : 0);
       return;
