@@ -57,6 +57,24 @@ __device__ __forceinline__ void split3(float x, float y, uint32_t (&p)[3]) {
   }
 }
 
+// The same with the first two terms rounded to nearest: their remainders are at most 2^-8 and 2^-17 of the
+// power of two below |x|, of either sign, and the third term is exact.  For products of two split
+// operands, where the terms' own products that are left out count: with cut-off terms the remainders all
+// have x's sign and are up to twice as large, and leaving out mid lo + lo mid (and lo lo) lost up to 2^-21
+// of a product, always towards zero; rounded ones lose 2^-24 at most and nothing on average.
+__device__ __forceinline__ void split3_nearest(float x, float y, uint32_t (&p)[3]) {
+#pragma unroll
+  for (int i = 0; i < 3; ++i) {
+    asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(p[i]) : "f"(y), "f"(x));
+    x -= __uint_as_float(p[i] << 16);
+    y -= __uint_as_float(p[i] & 0xFFFF0000u);
+    if (i == 0) {  // an infinity (or a value that rounds to one) or NaN is the first term alone
+      x = fabsf(x) < INFINITY ? x : 0.f;
+      y = fabsf(y) < INFINITY ? y : 0.f;
+    }
+  }
+}
+
 // Entries 2 t, 2 t + 1 of sample i; VEC: X is 8-byte aligned.
 template <bool VEC>
 __device__ __forceinline__ float2 load_pair(const float* __restrict__ X, int64_t i, int64_t n, int t) {
@@ -168,9 +186,11 @@ __global__ void __launch_bounds__(kFwdThreads, 3) k_mlp_forward(const __nv_bfloa
 // tiles of 64 samples, 16 per warp.  Forward as in k_mlp_forward; the layers' deltas and activations
 // (FP32 values as three exact bf16 terms) go to shared memory, where ldmatrix.trans turns them into
 // the operands of the sums over samples: warp m computes rows 16 m .. 16 m + 15 of dW2 = D2^T H1 and
-// of dW1 = D1^T X, and db2, db1 as products with a column of ones.  Of the nine products of terms the
-// six above 2^-24 count; those of the two first terms accumulate apart from the rest, and every
-// tile's sums are added in FP32.  Each CTA writes its partial gradient and loss; k_mlp_reduce adds
+// of dW1 = D1^T X, and db2, db1 as products with a column of ones.  Of the nine products of terms (split3_nearest)
+// six count, the other three are at most 2^-24 of the whole; those of the two first terms accumulate apart from the rest, and every
+// tile's sums are added in FP32, the bias sums' after every 16 samples and first terms apart (through one
+// accumulator for all terms of a tile the tensor core cut off twelve times: 64 equal samples gave biases
+// up to 6e-7 away from one sample's, now the same bits).  Each CTA writes its partial gradient and loss; k_mlp_reduce adds
 // the CTAs' partials in their order, so the gradient is the same bit for bit from run to run.
 //
 // What bounds it: latency at the training loop's 16,384 samples (one or two tiles per CTA).  There
@@ -261,16 +281,11 @@ __global__ void __launch_bounds__(kGradThreads, 2) k_mlp_grad(const __nv_bfloat1
     for (int e = 0; e < 4; ++e) v[e] = ((hi[0][e] + hi[1][e]) + (hi[2][e] + hi[3][e])) + lo[e];
   };
   // a pair of rows' values of columns 8 nb + 2 t, + 1 as terms: into operand registers and shared memory
-  auto keep = [&](float v0, float v1, float v2, float v3, int nb, bool pos, uint32_t (*a)[4][4],
+  auto keep = [&](float v0, float v1, float v2, float v3, int nb, uint32_t (*a)[4][4],
                   __nv_bfloat16 (&dst)[3][kTile][kRow]) {
     uint32_t p[3], q[3];
-    if (pos) {
-      split3<true>(v0, v1, p);
-      split3<true>(v2, v3, q);
-    } else {
-      split3<false>(v0, v1, p);
-      split3<false>(v2, v3, q);
-    }
+    split3_nearest(v0, v1, p);
+    split3_nearest(v2, v3, q);
 #pragma unroll
     for (int k = 0; k < 3; ++k) {
       if (a) {
@@ -287,8 +302,8 @@ __global__ void __launch_bounds__(kGradThreads, 2) k_mlp_grad(const __nv_bfloat1
     const float2 x0 = load_pair<VEC>(X, i0, n, t), x1 = load_pair<VEC>(X, i1, n, t);
     const float t0 = i0 < n ? tg[i0] : 0.f, t1 = i1 < n ? tg[i1] : 0.f;
     uint32_t xa[3], xb[3];
-    split3<false>(x0.x, x0.y, xa);
-    split3<false>(x1.x, x1.y, xb);
+    split3_nearest(x0.x, x0.y, xa);
+    split3_nearest(x1.x, x1.y, xb);
 #pragma unroll
     for (int k = 0; k < 3; ++k) {
       *reinterpret_cast<uint32_t*>(&sm.xs[k][16 * warp + g][2 * t]) = xa[k];
@@ -309,7 +324,7 @@ __global__ void __launch_bounds__(kGradThreads, 2) k_mlp_grad(const __nv_bfloat1
         v[e] = fmaxf((hi[e] + ((e & 1) ? b.y : b.x)) + lo[e], 0.f);
         live1 |= (v[e] > 0.f ? 1u : 0u) << (4 * nb + e);
       }
-      keep(v[0], v[1], v[2], v[3], nb, true, op, sm.h1);
+      keep(v[0], v[1], v[2], v[3], nb, op, sm.h1);
     }
     float h2[8][4], o0 = 0.f, o1 = 0.f;
 #pragma unroll
@@ -337,7 +352,7 @@ __global__ void __launch_bounds__(kGradThreads, 2) k_mlp_grad(const __nv_bfloat1
       aw3[nb][0] += dy0 * h2[nb][0] + dy1 * h2[nb][2];
       aw3[nb][1] += dy0 * h2[nb][1] + dy1 * h2[nb][3];
       keep(h2[nb][0] > 0.f ? dy0 * w3.x : 0.f, h2[nb][1] > 0.f ? dy0 * w3.y : 0.f,
-           h2[nb][2] > 0.f ? dy1 * w3.x : 0.f, h2[nb][3] > 0.f ? dy1 * w3.y : 0.f, nb, false, op, sm.d2);
+           h2[nb][2] > 0.f ? dy1 * w3.x : 0.f, h2[nb][3] > 0.f ? dy1 * w3.y : 0.f, nb, op, sm.d2);
     }
 #pragma unroll
     for (int nb = 0; nb < 8; ++nb) {
@@ -345,15 +360,24 @@ __global__ void __launch_bounds__(kGradThreads, 2) k_mlp_grad(const __nv_bfloat1
       layer(op, sm.w2t, nb, v);
 #pragma unroll
       for (int e = 0; e < 4; ++e) v[e] = (live1 >> (4 * nb + e)) & 1u ? v[e] : 0.f;
-      keep(v[0], v[1], v[2], v[3], nb, false, nullptr, sm.d1);
+      keep(v[0], v[1], v[2], v[3], nb, nullptr, sm.d1);
     }
     __syncthreads();
     // ---- sums over the tile's samples: rows 16 warp .. + 15
     const int ms = (lane >> 4) * 8 + (lane & 7), mc = ((lane >> 3) & 1) * 8;  // A: matrices (0, 0) (0, 8) (8, 0) (8, 8)
     const int bs = ((lane >> 3) & 1) * 8 + (lane & 7), bc = (lane >> 4) * 8;  // B: (0, 0) (8, 0) (0, 8) (8, 8)
-    constexpr uint32_t kOnes = 0x3F803F80u;
+    // sums of 16 samples' deltas (rows g, g + 8) added to a layer's bias sums
+    auto bias = [](const uint32_t (&A)[3][4], float (&sum)[2]) {
+      constexpr uint32_t kOnes = 0x3F803F80u;
+      float first[4] = {0.f, 0.f, 0.f, 0.f}, rest[4] = {0.f, 0.f, 0.f, 0.f};
+      mma_k16(first, A[0], kOnes, kOnes);
+      mma_k16(rest, A[2], kOnes, kOnes);
+      mma_k16(rest, A[1], kOnes, kOnes);
+      sum[0] += first[0] + rest[0];
+      sum[1] += first[2] + rest[2];
+    };
     {
-      float hi[8][4], lo[8][4], ones[4] = {0.f, 0.f, 0.f, 0.f};
+      float hi[8][4], lo[8][4];
 #pragma unroll
       for (int nb = 0; nb < 8; ++nb)
 #pragma unroll
@@ -363,8 +387,7 @@ __global__ void __launch_bounds__(kGradThreads, 2) k_mlp_grad(const __nv_bfloat1
         uint32_t A[3][4];
 #pragma unroll
         for (int k = 0; k < 3; ++k) ldmatrix_t(&sm.d2[k][16 * ks + ms][16 * warp + mc], A[k]);
-#pragma unroll
-        for (int k = 2; k >= 0; --k) mma_k16(ones, A[k], kOnes, kOnes);
+        bias(A, ab2);
 #pragma unroll
         for (int np = 0; np < 4; ++np) {
           uint32_t B[3][4];
@@ -386,11 +409,9 @@ __global__ void __launch_bounds__(kGradThreads, 2) k_mlp_grad(const __nv_bfloat1
       for (int nb = 0; nb < 8; ++nb)
 #pragma unroll
         for (int e = 0; e < 4; ++e) aw2[nb][e] += hi[nb][e] + lo[nb][e];
-      ab2[0] += ones[0];
-      ab2[1] += ones[2];
     }
     {
-      float hi[4] = {0.f, 0.f, 0.f, 0.f}, lo[4] = {0.f, 0.f, 0.f, 0.f}, ones[4] = {0.f, 0.f, 0.f, 0.f};
+      float hi[4] = {0.f, 0.f, 0.f, 0.f}, lo[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll
       for (int kp = 0; kp < kTile / 32; ++kp) {
         uint32_t B[3][4];  // samples 32 kp + 0, 8, 16, 24 of the features
@@ -401,8 +422,7 @@ __global__ void __launch_bounds__(kGradThreads, 2) k_mlp_grad(const __nv_bfloat1
           uint32_t A[3][4];
 #pragma unroll
           for (int k = 0; k < 3; ++k) ldmatrix_t(&sm.d1[k][32 * kp + 16 * h + ms][16 * warp + mc], A[k]);
-#pragma unroll
-          for (int k = 2; k >= 0; --k) mma_k16(ones, A[k], kOnes, kOnes);
+          bias(A, ab1);
           mma_k16(lo, A[2], B[0][2 * h], B[0][2 * h + 1]);
           mma_k16(lo, A[0], B[2][2 * h], B[2][2 * h + 1]);
           mma_k16(lo, A[1], B[1][2 * h], B[1][2 * h + 1]);
@@ -413,8 +433,6 @@ __global__ void __launch_bounds__(kGradThreads, 2) k_mlp_grad(const __nv_bfloat1
       }
 #pragma unroll
       for (int e = 0; e < 4; ++e) aw1[e] += hi[e] + lo[e];
-      ab1[0] += ones[0];
-      ab1[1] += ones[2];
     }
     __syncthreads();
   }
