@@ -15,7 +15,7 @@
 //    part T^T s_I leaves the registers with every tile and sums over the lanes of a column group,
 //    which few columns per lane make short; the row part T s_J stays in registers along a row of
 //    tiles, where few rows per lane take few registers;
-//  * fragments: the 16 x 16 blocks of mma.m16n8k16's A operand (FP32 tiles, R = 4, 8).
+//  * fragments: the 16 x 16 blocks of mma.m16n8k16's A operand (FP32 tiles, R = 8).
 //
 // FP16 storage (FP32 solvers): the same tiles as IEEE half, row by row with the 16-byte chunks of a
 // row exchanged for ldmatrix (or as patches), each tile divided by its own largest entry (kept
@@ -417,12 +417,12 @@ __device__ __forceinline__ uint32_t movmatrix(uint32_t a) {
   return d;
 }
 
-// The upper 16 bits of two floats as a pair: bf16 by truncation.
-__device__ __forceinline__ uint32_t upper_pair(float lo, float hi) {
-  return __byte_perm(__float_as_uint(lo), __float_as_uint(hi), 0x7632);
+// Two floats as a bf16 pair, rounded to nearest.
+__device__ __forceinline__ uint32_t bf16_pair(float lo, float hi) {
+  uint32_t d;
+  asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(d) : "f"(hi), "f"(lo));
+  return d;
 }
-
-__device__ __forceinline__ float bf16_part(float x) { return __uint_as_float(__float_as_uint(x) & 0xFFFF0000u); }
 
 // Where port p of a strip lies in a row of the vector operand: lane t of a column reads its eight
 // entries (k = 2t, 2t + 1, 2t + 8, 2t + 9 of both 16-row halves) in one 16-byte load.
@@ -433,8 +433,15 @@ __device__ __forceinline__ int operand_pos(int p) {
 // Columns of the MMAs' vector operand.  FP16 tiles: columns 2 r, 2 r + 1 hold the two terms of right-
 // hand side r (hi and lo of s / sigma, sigma_r a power of two at or above the segment's max |s_r|:
 // together 2^-24 of it), so one product takes both and its lane adds them; R = 8 takes two operands.
-// FP32 tiles: S and s both as three bf16 terms (8 + 8 + 8 bits, exact), columns = right-hand sides;
-// the six products of terms above 2^-24 accumulate in order of size.
+// FP32 tiles: S and s both as three bf16 terms, columns = right-hand sides.  The first two terms are
+// rounded to nearest, so their remainders are at most 2^-8 and 2^-17 of the power of two below the value, of
+// either sign, and the third term is exact; six of the nine products count, and what the others (mid lo, lo mid,
+// lo lo) leave out is at most 2^-24 of a product and nothing on average.  (Terms cut off instead have
+// remainders up to twice as large and of the value's sign: up to 2^-21, always towards zero.)  The
+// tensor core cuts its sums off too; the first terms' products of every MMA are therefore added in FP32,
+// only the others, 2^-8 of those, accumulate there.  Error of y over |S| |s|, rms, random subgraphs of
+// 300 to 1060 ports, signed / positive entries: 1.6e-8 / 9.2e-8; with cut-off terms and one accumulator
+// 2.7e-8 / 2.9e-7; an FP32 loop (SIMT products) 1.6e-8 / 7.1e-8.
 template <typename TS, int R>
 __host__ __device__ constexpr int operand_rows() {
   return sizeof(TS) == 2 ? 2 * R : 3 * R;
@@ -463,7 +470,7 @@ __host__ __device__ constexpr int sweep_threads(int mma) { return mma ? 32 * mma
 // Each lane copies its own patches one tile ahead into shared-memory slots that only it reads (cp.async, 16 bytes a piece): no registers hold loads in flight, no lane waits for
 // another, and a segment's first tile arrives while its vectors are read.
 //
-// MMA (FP16 tiles; FP32 tiles with R = 4, 8): the tile's products on the tensor cores
+// MMA (FP16 tiles; FP32 tiles with R = 8): the tile's products on the tensor cores
 // (mma.m16n8k16, FP32 accumulation, each tile's sums added in FP32), the transposed ones from
 // ldmatrix.trans or movmatrix.  The SIMT products of an FP16 tile take about 210 instructions per
 // lane (32 conversions, 64 FMAs, shuffles), of an FP32 tile at R = 8 about 980: the issue rate, not
@@ -631,10 +638,13 @@ __global__ void __launch_bounds__(sweep_threads(MMA), sizeof(T) == 8 || MMA > 8 
             o[(2 * (r + c)) * a.op_stride] = __half_as_ushort(hi);
             o[(2 * (r + c) + 1) * a.op_stride] = __half_as_ushort(__float2half_rn(x - __half2float(hi)));
           } else {
-            const float x = v[c], h = bf16_part(x), md = bf16_part(x - h), l = x - h - md;
-            o[(r + c) * a.op_stride] = (uint16_t)(__float_as_uint(h) >> 16);
-            o[(R + r + c) * a.op_stride] = (uint16_t)(__float_as_uint(md) >> 16);
-            o[(2 * R + r + c) * a.op_stride] = (uint16_t)(__float_as_uint(l) >> 16);
+            float x = v[c];
+#pragma unroll
+            for (int term = 0; term < 3; ++term) {
+              const uint32_t t = bf16_pair(x, 0.f);
+              o[(term * R + r + c) * a.op_stride] = (uint16_t)t;
+              x -= __uint_as_float(t << 16);
+            }
           }
         }
       }
@@ -729,27 +739,48 @@ __global__ void __launch_bounds__(sweep_threads(MMA), sizeof(T) == 8 || MMA > 8 
         load_patch(reinterpret_cast<const float*>(tile), lane, x);
         fetch(slot);
         slot = slot + 1 == kDepth ? 0 : slot + 1;
-        // terms of S from the smallest: a = 2 meets s_hi; a = 1 s_mid, s_hi; a = 0 s_lo, s_mid, s_hi
+        float lr[2][4], lc[2][4];  // the products of all but the first terms
 #pragma unroll
-        for (int term = 2; term >= 0; --term)
+        for (int h = 0; h < 2; ++h)
 #pragma unroll
-          for (int k = 0; k < 4; ++k) {
-            const int mi = k >> 1, ki = k & 1;
+          for (int u = 0; u < 4; ++u) lr[h][u] = lc[h][u] = 0.f;
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+          const int mi = k >> 1, ki = k & 1;
+#pragma unroll
+          for (int term = 0; term < 3; ++term) {
             uint32_t A[4], At[4];
 #pragma unroll
             for (int u = 0; u < 4; ++u) {
-              float p0 = x[8 * k + 2 * u], p1 = x[8 * k + 2 * u + 1];
-              if (term >= 1) p0 -= bf16_part(p0), p1 -= bf16_part(p1);
-              if (term >= 2) p0 -= bf16_part(p0), p1 -= bf16_part(p1);
-              A[u] = upper_pair(p0, p1);
+              A[u] = bf16_pair(x[8 * k + 2 * u], x[8 * k + 2 * u + 1]);
+              x[8 * k + 2 * u] -= __uint_as_float(A[u] << 16);
+              x[8 * k + 2 * u + 1] -= __uint_as_float(A[u] & 0xFFFF0000u);
             }
             At[0] = movmatrix(A[0]), At[1] = movmatrix(A[2]), At[2] = movmatrix(A[1]), At[3] = movmatrix(A[3]);
 #pragma unroll
-            for (int n = 2 - term; n >= 0; --n) {
-              mma16816<false>(dr[mi][0], A, bJ[n][2 * ki], bJ[n][2 * ki + 1]);
-              if (I != J) mma16816<false>(dc[ki][0], At, bI[n][2 * mi], bI[n][2 * mi + 1]);
+            for (int n = 0; n < 3 - term; ++n) {
+              if (term + n > 0) {
+                mma16816<false>(lr[mi], A, bJ[n][2 * ki], bJ[n][2 * ki + 1]);
+                if (I != J) mma16816<false>(lc[ki], At, bI[n][2 * mi], bI[n][2 * mi + 1]);
+              } else {
+                float hr[4] = {0.f, 0.f, 0.f, 0.f};
+                mma16816<false>(hr, A, bJ[0][2 * ki], bJ[0][2 * ki + 1]);
+#pragma unroll
+                for (int u = 0; u < 4; ++u) dr[mi][0][u] += hr[u];
+                if (I != J) {
+                  float hc[4] = {0.f, 0.f, 0.f, 0.f};
+                  mma16816<false>(hc, At, bI[0][2 * mi], bI[0][2 * mi + 1]);
+#pragma unroll
+                  for (int u = 0; u < 4; ++u) dc[ki][0][u] += hc[u];
+                }
+              }
             }
           }
+        }
+#pragma unroll
+        for (int h = 0; h < 2; ++h)
+#pragma unroll
+          for (int u = 0; u < 4; ++u) dr[h][0][u] += lr[h][u], dc[h][0][u] += lc[h][u];
       }
 #pragma unroll
       for (int h = 0; h < 4; ++h)
@@ -1020,9 +1051,11 @@ __global__ void __launch_bounds__(256) k_port_vec(const PortArgs<T> a, int nport
 }
 
 // Shared memory of a sweep and the kernel that goes with it.  Accumulators per warp (R <= 2) if they
-// leave room for two CTAs per SM (one in FP64); the tensor cores for FP16 tiles and for FP32 tiles with R = 4, 8 wherever their operands and
-// slots fit.  Vectors too long for that many CTAs take one, then the SIMT products, then give up
-// the gaps, the slots and the row sums.
+// leave room for two CTAs per SM (one in FP64); the tensor cores for FP16 tiles and for FP32 tiles with
+// R = 8 wherever their operands and slots fit.  FP32 tiles, SIMT and tensor-core products: R = 4, 288
+// subgraphs of 300 to 1060 ports 0.076 and 0.088 ms, 512 of 600 to 1360 0.221 and 0.250, 2500 of 40 to 130
+// 0.046 and 0.058; R = 8 0.164 and 0.108, 0.486 and 0.325, 0.073 and 0.060.  Vectors too long for that many
+// CTAs take one, then the SIMT products, then give up the gaps, the slots and the row sums.
 PortShape port_shape(size_t elem, size_t stored, int R, int max_ports) {
   const size_t npad = (size_t)((max_ports + kNB - 1) / kNB) * kNB;
   const size_t sum1 = (size_t)kNB * R * elem;  // a warp's row sums of one strip
@@ -1049,11 +1082,10 @@ PortShape port_shape(size_t elem, size_t stored, int R, int max_ports) {
     p.layout = mma && stored == 4 ? kPortFragments : R <= 2 ? kPortPatch8x4 : kPortPatch4x8;
     return p.smem <= most;
   };
-  const bool mma = stored == 2 || (stored == 4 && R >= 4);
+  const bool mma = stored == 2 || (stored == 4 && R >= 8);
   if (R <= 2 && fit(mma ? 8 : 0, true, 0, true, 0, share)) return p;
-  // tensor cores: two CTAs of 8 warps per SM where they fit, else FP32 one of 16 warps (R = 8, 439 MB,
-  // one CTA per SM: 260 k cycles with 16 warps, 283 k with 8; R = 4, where two fit: two of 8 warps
-  // 191 k, one of 16 242 k), else one of 8
+  // tensor cores: two CTAs of 8 warps per SM where they fit, else FP32 one of 16 warps (439 MB, one CTA
+  // per SM: 260 k cycles with 16 warps, 283 k with 8), else one of 8
   if (mma)
     for (int sb : {8, 4, 2, 1})
       if (fit(8, false, 0, true, sb, share)) return p;
@@ -1079,7 +1111,7 @@ PortShape port_shape(size_t elem, size_t stored, int R, int max_ports) {
 // and its waves, and a little per strip of them.  In tiles of the same kernel, from the cycles of every
 // CTA of a sweep over 288 ragged subgraphs of 1 to 33 strips (least squares):
 //   FP64 8 + 0.3 per strip (R = 1), 5 + 0.3 (R = 2); FP32 27 + 0.6 (R = 1, 2); FP16 41 + 1.2 (R = 1);
-//   tensor cores, 8 warps: FP32 44 + 0.7 (R = 4), 48 + 1.0 (R = 8), FP16 54 + 1.9 and 67 + 2.6;
+//   tensor cores, 8 warps: FP32 48 + 1.0 (R = 8), FP16 54 + 1.9 (R = 4), 67 + 2.6 (R = 8);
 //   16 warps: FP32 71 + 0.1.
 // (With 20 for R >= 4 the CTAs of many small subgraphs took 1.4 times the average.)
 PortPlan port_plan(const PieceDesc* pd, int npieces, size_t elem, size_t stored, int R, int ctas, int mma) {
@@ -1168,7 +1200,7 @@ PortPlan port_plan(const PieceDesc* pd, int npieces, size_t elem, size_t stored,
 
 template <typename T, typename TS, int R>
 static const void* port_kernel_r(bool priv, int mma) {
-  constexpr bool can_mma = sizeof(TS) == 2 || (sizeof(TS) == 4 && R >= 4);
+  constexpr bool can_mma = sizeof(TS) == 2 || (sizeof(TS) == 4 && R >= 8);
   if constexpr (can_mma) {
     if constexpr (R <= 2) {
       if (mma && priv) return (const void*)k_port_sweep<T, TS, R, true, 8>;
