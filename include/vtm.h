@@ -241,8 +241,9 @@ typedef struct vtm_setup_opts {
                               fits in shared memory (nrhs <= 8) and in device memory            */
   int32_t port_storage;    /* PORT form, FP32 solvers: storage of S_j (VTM_STORE_*).
                               nrhs <= 8: NATIVE (0) the solver precision; FP16 halves the bytes
-                              of a sweep (each 32 x 32 tile of S_j scaled by its largest entry,
-                              FP32 arithmetic; the sweeps then match the FP64 oracle to about
+                              of a sweep (each 32 x 32 tile of S_j scaled by its largest entry; the
+                              port vector keeps 2^-23 of each entry down to 2^-29 of the largest,
+                              FP32 accumulation; the sweeps then match the FP64 oracle to about
                               2^-11 per sweep and the FP64 defect correction restores the
                               tolerance; a phase on FP16 responses restarts once its inner
                               residual is below 4 x 2^-11, and with coupled lines once a check

@@ -430,9 +430,13 @@ __device__ __forceinline__ int operand_pos(int p) {
   return ((p & 7) >> 1) * 8 + ((p >> 4) * 2 + ((p >> 3) & 1)) * 2 + (p & 1);
 }
 
-// Columns of the MMAs' vector operand.  FP16 tiles: columns 2 r, 2 r + 1 hold the two terms of right-
-// hand side r (hi and lo of s / sigma, sigma_r a power of two at or above the segment's max |s_r|:
-// together 2^-24 of it), so one product takes both and its lane adds them; R = 8 takes two operands.
+// Columns of the MMAs' vector operand.
+// FP16 tiles: columns 2 r, 2 r + 1 hold the two terms of right-hand side r, x = s_r / sigma_r = t0 + 2^-11 t1, so
+// one product takes both and its lane adds them; R = 8 takes two operands.  sigma_r is the power of two
+// that puts the segment's max |s_r| just below 2^15, and t1 is what t0 leaves times 2^11: at both ends fp16's
+// exponent is used in full, and an entry keeps 2^-23 of itself down to 2^-29 of the largest, 2^-12 to 2^-38.
+// (With max |x| = 1 and t1 not scaled an entry kept 2^-25 of the largest: ports whose s was 2^-24 of it
+// were lost.)
 // FP32 tiles: S and s both as three bf16 terms, columns = right-hand sides.  The first two terms are
 // rounded to nearest, so their remainders are at most 2^-8 and 2^-17 of the power of two below the value, of
 // either sign, and the third term is exact; six of the nine products count, and what the others (mid lo, lo mid,
@@ -442,6 +446,7 @@ __device__ __forceinline__ int operand_pos(int p) {
 // only the others, 2^-8 of those, accumulate there.  Error of y over |S| |s|, rms, random subgraphs of
 // 300 to 1060 ports, signed / positive entries: 1.6e-8 / 9.2e-8; with cut-off terms and one accumulator
 // 2.7e-8 / 2.9e-7; an FP32 loop (SIMT products) 1.6e-8 / 7.1e-8.
+constexpr float kTerm1 = 4.8828125e-4f;  // 2^-11
 template <typename TS, int R>
 __host__ __device__ constexpr int operand_rows() {
   return sizeof(TS) == 2 ? 2 * R : 3 * R;
@@ -592,7 +597,7 @@ __global__ void __launch_bounds__(sweep_threads(MMA), sizeof(T) == 8 || MMA > 8 
       for (int d = 0; d < kDepth; ++d) fetch(d);
     if (!waited) grid_dep_wait();  // everything above is constant between sweeps
     waited = true;
-    float sigma[RV];  // MMA, FP16 tiles: the scale of s in the columns this thread writes out
+    float sigma[RV], inv[RV];  // MMA, FP16 tiles: the scale of s in the columns this thread writes out, its inverse
     if constexpr (MMA) {
       // s as 16-bit terms, through an FP32 copy in the accumulators' place; then y = 0
       const T* sp = a.s + (size_t)pd.port_off * R;
@@ -622,7 +627,9 @@ __global__ void __launch_bounds__(sweep_threads(MMA), sizeof(T) == 8 || MMA > 8 
           int e = 0;
           const float mm = __int_as_float(smax[r + c]);
           if (mm > 0.f && isfinite(mm)) frexpf(mm, &e);
-          sigma[c] = ldexpf(1.f, max(-120, e));
+          e = max(-110, e) - 15;
+          sigma[c] = ldexpf(1.f, e);
+          inv[c] = ldexpf(1.f, -e);
         }
       }
       for (int i = tid; i < rows * (R / RV); i += TH) {
@@ -633,10 +640,10 @@ __global__ void __launch_bounds__(sweep_threads(MMA), sizeof(T) == 8 || MMA > 8 
 #pragma unroll
         for (int c = 0; c < RV; ++c) {
           if constexpr (HALF) {
-            const float x = v[c] / sigma[c];
-            const __half hi = __float2half_rn(x);
-            o[(2 * (r + c)) * a.op_stride] = __half_as_ushort(hi);
-            o[(2 * (r + c) + 1) * a.op_stride] = __half_as_ushort(__float2half_rn(x - __half2float(hi)));
+            const float x = v[c] * inv[c];
+            const __half t0 = __float2half_rn(x);
+            o[(2 * (r + c)) * a.op_stride] = __half_as_ushort(t0);
+            o[(2 * (r + c) + 1) * a.op_stride] = __half_as_ushort(__float2half_rn((x - __half2float(t0)) / kTerm1));
           } else {
             float x = v[c];
 #pragma unroll
@@ -788,7 +795,7 @@ __global__ void __launch_bounds__(sweep_threads(MMA), sizeof(T) == 8 || MMA > 8 
         for (int k = 0; k < NV; ++k) {
           if constexpr (HALF) {
             const float* d = &dr[h >> 1][k][2 * (h & 1)];
-            rp[h][k] += (d[0] + d[1]) * sc;
+            rp[h][k] += fmaf(d[1], kTerm1, d[0]) * sc;
           } else {
             rp[h][k] += dr[h >> 1][0][2 * (h & 1) + k];
           }
@@ -801,7 +808,7 @@ __global__ void __launch_bounds__(sweep_threads(MMA), sizeof(T) == 8 || MMA > 8 
 #pragma unroll
               for (int h = 0; h < 4; ++h) {
                 const float* d = &dc[h >> 1][k][2 * (h & 1)];
-                yw[(J * kNB + 8 * h + fg) * R + out_col(k)] += (d[0] + d[1]) * sc;
+                yw[(J * kNB + 8 * h + fg) * R + out_col(k)] += fmaf(d[1], kTerm1, d[0]) * sc;
               }
         } else if (2 * ft < R) {
 #pragma unroll

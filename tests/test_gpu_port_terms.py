@@ -9,6 +9,7 @@ import numpy as np
 import pytest
 
 from paper_0807_1949_gb300 import inputs
+from test_precision_bounds import TOL_FP16
 
 pytestmark = pytest.mark.gpu
 torch = pytest.importorskip("torch")
@@ -35,6 +36,20 @@ def _two_sweeps(vtmlib, a, w, storage):
     out = np.empty_like(w)
     out[:, vertex] = got[:, 0::2]
     return out, (2.0 / (a / 2 + 1.0) - 1.0) ** 2 * w
+
+
+@pytest.mark.parametrize("nrhs", [1, 2, 4, 8])
+def test_fp16_storage_keeps_small_waves(vtmlib, nrhs):
+    """Waves of a subgraph that differ by up to 2^34: every port's next wave within the rounding of the
+    FP16 storage (S_pp within 0.9 .. 0.99 of its tile's largest entry: 2^-12 / 0.9 of S_pp, times
+    2 S_pp / (2 S_pp - 1) <= 2.25 in the wave: 6.1e-4, below TOL_FP16), the smallest included."""
+    rng = np.random.default_rng(nrhs)
+    a = rng.uniform(0.02, 0.2, N)
+    w = rng.uniform(0.5, 1.0, (nrhs, N)) * rng.choice([-1.0, 1.0], (nrhs, N))
+    w *= 2.0 ** -rng.choice([0, 7, 13, 20, 26, 34], (nrhs, N))
+    w = w.astype(np.float32).astype(np.float64)
+    got, ref = _two_sweeps(vtmlib, a, w, "fp16")
+    assert np.max(np.abs(got / ref - 1.0)) <= TOL_FP16
 
 
 @pytest.mark.parametrize("nrhs", [2, 4, 8])
