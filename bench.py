@@ -670,7 +670,13 @@ def run_vtm(args):
         if sinfo.ncouplings:
             # per coupling 4 list entries (two ports on each side): wave index, -y and one gathered wave
             alg_bytes += 4 * sinfo.ncouplings * (8 + R * elem) + sinfo.nports * 4
-        if R >= 16:
+        bound = "hbm"
+        if sinfo.port_kernel == vtm.PORT_RESIDENT:
+            # S_j stays in shared memory: a sweep moves its waves only, written once and read by the
+            # ends' twins as words of twice their size, between the SMs; what it waits for is that exchange
+            kname, ksrc, bound = "k_port_resident<float,%d>" % R, "port_resident.cu", "latency"
+            alg_bytes = 4 * sinfo.nends * R * elem
+        elif R >= 16:
             kname, ksrc = "k_port_sweep_tc<%d>" % R, "port_tc.cu"
         else:
             kname = "k_port_sweep<float,%s,%d>" % ("__half" if bits_now == 16 else "float", R)
@@ -678,6 +684,7 @@ def run_vtm(args):
     else:
         sweep_ms = band_ms
         alg_bytes = band_bytes
+        bound = "hbm"
         if R >= 16:
             kname = "k_sweep_wide<float,float,%d>" % R
         elif sinfo.sweep_variant == 1:
@@ -769,11 +776,15 @@ def run_vtm(args):
         cpu = cpu_baseline(args.workload, ks, src)
     if cdesc is not None:
         cdesc["pairs"] = int(sinfo.ncouplings)
+    if port and sinfo.port_kernel == vtm.PORT_RESIDENT:
+        l2 = "port responses resident in shared memory (%.1f MB)" % (sinfo.port_bytes / 1e6)
+    else:
+        l2 = ("inputs larger than L2 (FP32 factor %.2f GB, port responses %.2f GB)"
+              % (sinfo.factor_bytes / 1e9, (sinfo.port_bytes if port else 0) / 1e9))
     cfg = {"workload": args.workload, "nrhs": R, "rtol": w["rtol"], "z": zdesc, "coupling": cdesc,
            "pieces": sinfo.npieces,
            "parallelism": "replicas" if ws > 1 else "single",
-           "l2": "inputs larger than L2 (FP32 factor %.2f GB, port responses %.2f GB)"
-                 % (sinfo.factor_bytes / 1e9, (sinfo.port_bytes if port else 0) / 1e9),
+           "l2": l2,
            "sweeps": sweeps, "restarts": stats[-1].restarts, "final_rel_residual": rel,
            "value_with_setup_ms": round(ms + sinfo.setup_ms, 1),
            "setup_ms": round(sinfo.setup_ms, 1), "factor_ms": round(sinfo.factor_ms, 1),
@@ -796,7 +807,7 @@ def run_vtm(args):
         "vs_baseline": None, "dtype": dtype_desc, "data": "synthetic",
         "value_with_setup": round(ms + sinfo.setup_ms, 1),
         "config": cfg,
-        "roofline": {"bound": "hbm", "kernel": kname, "achieved": round(achieved, 1),
+        "roofline": {"bound": bound, "kernel": kname, "achieved": round(achieved, 1),
                      "peak": pk["hbm_gbs"], "peak_source": pk["source"], "unit": "GB/s",
                      "frac": round(achieved / pk["hbm_gbs"], 4), "traffic": traffic,
                      "alg_bytes_per_launch": int(alg_bytes), "launch_ms": round(sweep_ms, 4)},

@@ -281,6 +281,14 @@ enum {
   VTM_FORM_PORT = 2
 };
 
+enum {
+  VTM_PORT_NONE = 0,           /* band form                                                    */
+  VTM_PORT_TILES = 1,          /* nrhs <= 8: S_j streamed in 32 x 32 tiles                     */
+  VTM_PORT_RESIDENT = 2,       /* S_j in shared memory, a batch of sweeps in one launch        */
+  VTM_PORT_TC_SEPARATE = 3,    /* nrhs 16 / 32: tensor cores, port vectors in a launch of their own */
+  VTM_PORT_TC_FUSED = 4        /* nrhs 16 / 32: tensor cores, port vectors in the same launch  */
+};
+
 typedef struct vtm_solver vtm_solver;
 
 typedef struct vtm_solver_info {
@@ -304,7 +312,8 @@ typedef struct vtm_solver_info {
   int32_t sweep_variant;       /* 0: one CTA works each block step in turn; 1: pipelined (chain
                                   warps finish block k while the others prepare block k+1)    */
   int32_t sweep_form;          /* VTM_FORM_BAND or VTM_FORM_PORT (after AUTO was resolved)    */
-  int64_t port_bytes;          /* PORT: bytes of the port responses S_j one sweep streams     */
+  int64_t port_bytes;          /* PORT: bytes of the port responses S_j one sweep reads: from memory, or
+                                  with VTM_PORT_RESIDENT from shared memory, where they stay      */
   double port_setup_ms;        /* PORT: device time of computing S_j (unit-source solves)     */
   double port_sweep_ms;        /* PORT: device time of one port-form sweep                    */
   int64_t nports;              /* port copies (copies with at least one line end)             */
@@ -316,6 +325,7 @@ typedef struct vtm_solver_info {
   int32_t band_tc;             /* 1: the multi-RHS band sweep (FP32, nrhs 16 / 32) runs its
                                   products on the tensor cores (factor balanced by its row norms,
                                   fp16 hi / lo panels of 128-row groups, FP32 accumulation)     */
+  int32_t port_kernel;         /* PORT: the kernel of the port sweeps (VTM_PORT_*)             */
   int64_t band_tc_bytes;       /* bytes of that tensor-core factor (each sweep reads it twice)  */
 } vtm_solver_info;
 

@@ -1330,7 +1330,11 @@ static void choose_form(vtm_solver* s, const vtm_setup_opts* o, int64_t s_tiles,
   s->wscr.alloc(s->wzero.bytes);
   VTM_CUDA(cudaMemsetAsync(s->wzero.p, 0, s->wzero.bytes, s->stream));
   compute_port_response<T>(s, s_tiles * (tc ? 128 * 128 / (kNB * kNB) : 1));
-  s->info.port_bytes = (int64_t)s_bytes;
+  s->info.port_bytes = s->resident ? (int64_t)s->S.bytes : (int64_t)s_bytes;
+  s->info.port_kernel = s->resident            ? VTM_PORT_RESIDENT
+                        : !tc                  ? VTM_PORT_TILES
+                        : s->tc_stiles.p       ? VTM_PORT_TC_SEPARATE
+                                               : VTM_PORT_TC_FUSED;
   s->info.port_storage_bits = 8 * (int)sizeof(T);
   if constexpr (sizeof(T) == 4) {
     // FP16_AUTO only where the sweep streams S_j from HBM: responses that stay in the 126 MB L2

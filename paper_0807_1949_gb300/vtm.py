@@ -24,6 +24,7 @@ PART_GRID, PART_OWNERS, PART_EXPLICIT, PART_ELEMENTS, PART_CONFORMAL = 1, 2, 3, 
 Z_UNIFORM, Z_EXPLICIT, Z_MATCHED, Z_LEARNED = 0, 1, 2, 3
 MLP_IN, MLP_HIDDEN, MLP_PARAMS = 8, 64, 4801
 FP64, FP32 = 0, 1
+PORT_NONE, PORT_TILES, PORT_RESIDENT, PORT_TC_SEPARATE, PORT_TC_FUSED = 0, 1, 2, 3, 4
 
 
 class VTMError(RuntimeError):
@@ -72,7 +73,8 @@ class SolverInfo(C.Structure):
                 ("sweep_variant", C.c_int32), ("sweep_form", C.c_int32), ("port_bytes", C.c_int64),
                 ("port_setup_ms", C.c_double), ("port_sweep_ms", C.c_double),
                 ("nports", C.c_int64), ("port_storage_bits", C.c_int32), ("factor_tc", C.c_int32),
-                ("ncouplings", C.c_int64), ("band_tc", C.c_int32), ("band_tc_bytes", C.c_int64)]
+                ("ncouplings", C.c_int64), ("band_tc", C.c_int32), ("port_kernel", C.c_int32),
+                ("band_tc_bytes", C.c_int64)]
 
 
 class Stats(C.Structure):
