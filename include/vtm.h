@@ -221,9 +221,13 @@ typedef struct vtm_setup_opts {
                               dropped by this factor (0 = 1e-4); ignored for FP64            */
   const vtm_mlp* model;    /* LEARNED: impedance model (not retained after vtm_setup)        */
   int64_t wait_polls;      /* polls of a bounded device wait before the sweep gives up and
-                              reports VTM_ERR_TIMEOUT (0 = 4194304)                          */
-  int32_t withhold_slab;   /* testing only: the sweep never issues the copy of this factor slab
-                              of each subgraph, so that wait runs out (0 = off; k>0 = slab k-1) */
+                              reports VTM_ERR_TIMEOUT (0 = 4194304).  A poll of the resident port sweep
+                              is one load (about 1 us), so it takes at least 65536 of them, unless
+                              withhold_slab makes a wait of it run out                       */
+  int32_t withhold_slab;   /* testing only (0 = off): k > 0: the band sweep never issues the copy of
+                              factor slab k-1 of each subgraph, k < 0: the resident port sweep never
+                              publishes the first line end's wave of sweep -k of a launch, so that a
+                              wait runs out                                                  */
   int32_t sweep_variant;   /* nrhs <= 8: 0: the pipelined sweep for FP32 solvers where it is the faster
                               one (three factor slabs fit in shared memory, and nrhs > 1 or no more
                               subgraphs than SMs), else the single-block sweep; 1: single-block

@@ -273,7 +273,7 @@ __global__ void __launch_bounds__(kResThreads, 1) k_port_resident(const ResArgs<
         if (lastk) {
 #pragma unroll
           for (int c = 0; c < C; ++c) a.wout[(size_t)e * R + r + c] = w[c];
-        } else {
+        } else if (e != 0 || k != a.withhold) {
           publish<T, C>(out, (size_t)e * R + r, w, (uint32_t)k);
         }
       }

@@ -104,6 +104,7 @@ struct vtm_solver {
   int slot_elems = 0, ys_elems = 0, win_elems = 0;
   long wait_limit = 1L << 22;
   int withhold = -1;
+  int withhold_wave = 0;
   std::vector<int> stage_cands;
   // kept for re-assembly with new impedances (eq. 5.8 depends on Z)
   DevBuf d_copy_piece, d_lrowptr, d_lcol, d_lval, d_port_of_copy, d_invz64;
@@ -766,6 +767,7 @@ static void setup_typed(const vtm_partition* p, const vtm_setup_opts* o, vtm_sol
     choose_form<T>(s, o, soff, foff);
   }
   s->withhold = o->withhold_slab > 0 ? o->withhold_slab - 1 : -1;  // after tuning: only real sweeps
+  s->withhold_wave = o->withhold_slab < 0 ? -std::max(o->withhold_slab, -INT32_MAX) : 0;
 
   s->info.npieces = np;
   s->info.ncopies = C;
@@ -1140,7 +1142,9 @@ static void launch_resident(vtm_solver* s, int k) {
   a.cpl = couple_ref<T>(s);
   a.sweeps = k;
   a.status = s->status.as<int>();
-  a.wait_limit = std::max(s->wait_limit, 65536L);  // a poll is one load here (about 1 us), not a suspended wait
+  a.withhold = s->withhold_wave;
+  // a poll is one load here (about 1 us), not a suspended wait
+  a.wait_limit = s->withhold_wave ? s->wait_limit : std::max(s->wait_limit, 65536L);
   VTM_CUDA(launch_port_resident<T>(a, s->R, s->res_grid, s->res_smem, s->res_xch.bytes, s->stream));
   s->launches++;
   s->cur = (s->cur + k) & 1;
