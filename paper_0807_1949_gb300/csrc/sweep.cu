@@ -506,8 +506,8 @@ static const void* pipe_kernel(int R) {
   switch (R) {
     case 1: return (const void*)k_sweep_pipe<T, 1>;
     case 2: return (const void*)k_sweep_pipe<T, 2>;
-    case 4: return (const void*)k_sweep_pipe<T, 4>;
-    case 8: return (const void*)k_sweep_pipe<T, 8>;
+    case 4: return sizeof(T) == 4 ? (const void*)k_sweep_pipe<float, 4> : nullptr;  // FP64: up to two (sweep_variant 2)
+    case 8: return sizeof(T) == 4 ? (const void*)k_sweep_pipe<float, 8> : nullptr;
     default: return nullptr;
   }
 }
