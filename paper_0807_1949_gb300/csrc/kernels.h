@@ -345,8 +345,8 @@ cudaError_t launch_split(int64_t ncopies, int R, const int64_t* copy_vertex, con
 template <typename T>
 cudaError_t launch_assemble(int64_t n, int R, const int64_t* vc_ptr, const int64_t* vc_copy, const T* xc,
                             const double* xbase, double* xt, int64_t ld, cudaStream_t st);
-// sums_r[q] += ||b_q - A x_q||^2, sums_b[q] += ||b_q||^2 (R <= 8).
-cudaError_t launch_residual_norms(int64_t n, int R, const int64_t* rowptr, const int32_t* col, const double* val,
+// sums_r[q] += ||b_q - A x_q||^2, sums_b[q] += ||b_q||^2 (R <= 8) on a device of nsm SMs.
+cudaError_t launch_residual_norms(int nsm, int64_t n, int R, const int64_t* rowptr, const int32_t* col, const double* val,
                                   const double* b, int64_t ldb, const double* x, int64_t ldx, double* sums_r,
                                   double* sums_b, cudaStream_t st);
 // res = b - A x (res may be NULL) and squared norms with fixed-order sums (identical inputs give

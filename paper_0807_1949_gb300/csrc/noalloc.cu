@@ -28,24 +28,31 @@ static __device__ __align__(256) double g_noalloc_scratch[2 * VTM_NOALLOC_MAX_RH
 
 constexpr int kMaxDevices = 64;
 std::mutex g_mu;
-double* g_scratch_ptr[kMaxDevices] = {};  // device address of g_noalloc_scratch, per device
+struct Device {
+  double* scratch = nullptr;  // device address of g_noalloc_scratch
+  int nsm = 0;                // its SMs
+};
+Device g_devices[kMaxDevices];
 
 // In host code the name g_noalloc_scratch is only a host-side stand-in; the kernels need the
 // device address, looked up once per device with that device current.
-double* scratch_for_current_device() {
+Device current_device() {
   int dev = -1;
   cudaError_t e = cudaGetDevice(&dev);
   if (e != cudaSuccess) vtm::fail(VTM_ERR_CUDA, std::string("cudaGetDevice: ") + cudaGetErrorString(e));
   if (dev < 0 || dev >= kMaxDevices) vtm::fail(VTM_ERR_INVALID, "device ordinal out of range");
   std::lock_guard<std::mutex> lock(g_mu);
-  if (!g_scratch_ptr[dev]) {
+  if (!g_devices[dev].scratch) {
     void* p = nullptr;
     e = cudaGetSymbolAddress(&p, g_noalloc_scratch);
     if (e != cudaSuccess || !p)
       vtm::fail(VTM_ERR_CUDA, std::string("cudaGetSymbolAddress: ") + cudaGetErrorString(e));
-    g_scratch_ptr[dev] = static_cast<double*>(p);
+    int nsm = 0;
+    e = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
+    if (e != cudaSuccess) vtm::fail(VTM_ERR_CUDA, std::string("cudaDeviceGetAttribute: ") + cudaGetErrorString(e));
+    g_devices[dev] = {static_cast<double*>(p), nsm};
   }
-  return g_scratch_ptr[dev];
+  return g_devices[dev];
 }
 
 __global__ void k_noalloc_finish(int nrhs, const double* __restrict__ sums, double* __restrict__ rel) {
@@ -59,7 +66,7 @@ __global__ void k_noalloc_finish(int nrhs, const double* __restrict__ sums, doub
 
 namespace vtm {
 // Loads the array onto the current device and caches its address (called by vtm_setup).
-void noalloc_prepare_current_device() { scratch_for_current_device(); }
+void noalloc_prepare_current_device() { current_device(); }
 }  // namespace vtm
 
 extern "C" int vtm_relative_residual_noalloc(int64_t n, const int64_t* rowptr, const int32_t* col, const double* val,
@@ -73,11 +80,12 @@ extern "C" int vtm_relative_residual_noalloc(int64_t n, const int64_t* rowptr, c
                                      std::to_string(VTM_NOALLOC_MAX_RHS) + "], got " + std::to_string(nrhs));
     if (ldb < n || ldx < n) vtm::fail(VTM_ERR_INVALID, "vtm_relative_residual_noalloc: leading dimension < n");
     cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
-    double* sums = scratch_for_current_device();
+    const Device dev = current_device();
+    double* sums = dev.scratch;
     // the array keeps the previous call's sums: clear both halves before accumulating
     cudaError_t e = cudaMemsetAsync(sums, 0, 2 * VTM_NOALLOC_MAX_RHS * sizeof(double), st);
     if (e == cudaSuccess)
-      e = vtm::launch_residual_norms(n, nrhs, rowptr, col, val, b, ldb, x, ldx, sums, sums + VTM_NOALLOC_MAX_RHS, st);
+      e = vtm::launch_residual_norms(dev.nsm, n, nrhs, rowptr, col, val, b, ldb, x, ldx, sums, sums + VTM_NOALLOC_MAX_RHS, st);
     if (e == cudaSuccess) {
       k_noalloc_finish<<<1, 32, 0, st>>>(nrhs, sums, rel);
       e = cudaGetLastError();

@@ -336,14 +336,14 @@ cudaError_t launch_assemble(int64_t n, int R, const int64_t* vc_ptr, const int64
   return cudaGetLastError();
 }
 
-cudaError_t launch_residual_norms(int64_t n, int R, const int64_t* rowptr, const int32_t* col, const double* val,
+cudaError_t launch_residual_norms(int nsm, int64_t n, int R, const int64_t* rowptr, const int32_t* col, const double* val,
                                   const double* b, int64_t ldb, const double* x, int64_t ldx, double* sums_r,
                                   double* sums_b, cudaStream_t st) {
   if (R < 1 || R > 8) return cudaErrorInvalidValue;
   if (n <= 0) return cudaSuccess;
   // several rows per thread only where the GPU stays full (8 blocks per SM): a small matrix waits for
   // its loads, not for FP64
-  const int rows = (int)std::min<int64_t>(kNormRows, std::max<int64_t>(1, n / ((int64_t)kBS * 8 * 152)));
+  const int rows = (int)std::min<int64_t>(kNormRows, std::max<int64_t>(1, n / ((int64_t)kBS * 8 * nsm)));
   const unsigned bx = (unsigned)((n + (int64_t)kBS * rows - 1) / ((int64_t)kBS * rows));
   switch (R) {
     case 1: k_residual_norms<1, 1><<<bx, kBS, 0, st>>>(n, rows, rowptr, col, val, b, ldb, x, ldx, sums_r, sums_b); break;
