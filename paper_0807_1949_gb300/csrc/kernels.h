@@ -113,7 +113,7 @@ struct PortShape {
   int mma;         // warps of a CTA with its products on the tensor cores (0: SIMT products)
   int priv;        // 1: an accumulator per warp (R <= 2), 0: one for all
   int ring;        // 1: shared-memory slots for the tiles in flight (0: no room)
-  int sb;          // strips whose row sums the warps keep between barriers (0: no room)
+  int sb;          // strips whose row sums the warps keep between barriers (priv: 0)
   size_t smem;
 };
 

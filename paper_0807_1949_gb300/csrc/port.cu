@@ -933,9 +933,8 @@ __global__ void __launch_bounds__(sweep_threads(MMA), sizeof(T) == 8 || MMA > 8 
           for (int c = 0; c < RV; ++c) v[c] *= sigma[c];
       });
     } else {
-      const int sbs = sb > 0 ? sb : 1;
-      for (int Ib = I0; Ib <= I1; Ib += sbs) {
-        const int Ie = min(Ib + sbs, I1 + 1);
+      for (int Ib = I0; Ib <= I1; Ib += sb) {
+        const int Ie = min(Ib + sb, I1 + 1);
         for (int I = Ib; MMA && I < Ie; ++I) {
           uint32_t bI[NB][4];
           operand(I, bI);
@@ -966,33 +965,18 @@ __global__ void __launch_bounds__(sweep_threads(MMA), sizeof(T) == 8 || MMA > 8 
             multiply(I, J, pt, sc, rp);
           }
           reduce_scatter<T, PR, R, 1>(rp, pb);  // lane (pa, pb) ends with row PR pa + pb
-          if (sb > 0) {
-            T* o = buf + ((size_t)(warp * sb + (I - Ib)) * kNB + PR * pa + pb) * R;
+          T* o = buf + ((size_t)(warp * sb + (I - Ib)) * kNB + PR * pa + pb) * R;
 #pragma unroll
-            for (int r = 0; r < R; ++r) o[r] = rp[0][r];
-          } else {
-            // no room for the warps' row sums: they take turns
-            for (int w = 0; w < kWarps; ++w) {
-              __syncthreads();
-              if (w == warp) {
-                T* at = yv + vidx<R>(I * kNB + PR * pa + pb, pad);
-#pragma unroll
-                for (int r = 0; r < R; ++r) at[r] += rp[0][r];
-              }
-            }
-            __syncthreads();
-          }
+          for (int r = 0; r < R; ++r) o[r] = rp[0][r];
         }
-        if (sb > 0) {
-          __syncthreads();
-          for (int i = tid; i < (Ie - Ib) * kNB * R; i += TH) {
-            T v = T(0);
+        __syncthreads();
+        for (int i = tid; i < (Ie - Ib) * kNB * R; i += TH) {
+          T v = T(0);
 #pragma unroll
-            for (int w = 0; w < kWarps; ++w) v += buf[(size_t)w * sb * kNB * R + i];
-            yv[vidx<R>(Ib * kNB + i / R, pad) + i % R] += v;
-          }
-          __syncthreads();
+          for (int w = 0; w < kWarps; ++w) v += buf[(size_t)w * sb * kNB * R + i];
+          yv[vidx<R>(Ib * kNB + i / R, pad) + i % R] += v;
         }
+        __syncthreads();
       }
       finish_segment<T, R, TH>(a, sg, si, pd, rows, reinterpret_cast<int*>(sv),
                            [&](int q, int r, T(&v)[RV]) {
@@ -1062,7 +1046,7 @@ __global__ void __launch_bounds__(256) k_port_vec(const PortArgs<T> a, int nport
 // R = 8 wherever their operands and slots fit.  FP32 tiles, SIMT and tensor-core products: R = 4, 288
 // subgraphs of 300 to 1060 ports 0.076 and 0.088 ms, 512 of 600 to 1360 0.221 and 0.250, 2500 of 40 to 130
 // 0.046 and 0.058; R = 8 0.164 and 0.108, 0.486 and 0.325, 0.073 and 0.060.  Vectors too long for that many
-// CTAs take one, then the SIMT products, then give up the gaps, the slots and the row sums.
+// CTAs take one, then the SIMT products, then give up the gaps and the slots.
 PortShape port_shape(size_t elem, size_t stored, int R, int max_ports) {
   const size_t npad = (size_t)((max_ports + kNB - 1) / kNB) * kNB;
   const size_t sum1 = (size_t)kNB * R * elem;  // a warp's row sums of one strip
@@ -1107,8 +1091,8 @@ PortShape port_shape(size_t elem, size_t stored, int R, int max_ports) {
     for (int sb : {8, 4, 2, 1})
       if (fit(0, false, pad, true, sb, most)) return p;
   const size_t all_smem = 227 * 1024;
-  if (fit(0, false, 0, true, 1, all_smem) || fit(0, false, 0, false, 1, all_smem)) return p;
-  fit(0, false, 0, false, 0, all_smem);
+  if (fit(0, false, 0, true, 1, all_smem)) return p;
+  fit(0, false, 0, false, 1, all_smem);  // with more ports than this has room for the band sweep has none either
   return p;
 }
 
