@@ -217,7 +217,7 @@ cudaError_t launch_factor(const PieceDesc* pieces, int npieces, int max_w, T* ba
                           T* diag0, cudaStream_t st) {
   const size_t smem = sizeof(T) * 33 * (size_t)(kNB + (max_w > kNB ? max_w : kNB));
   if (smem > 227 * 1024) return cudaErrorInvalidValue;
-  cudaError_t e = cudaFuncSetAttribute(k_factor<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  cudaError_t e = allow_all_smem((const void*)k_factor<T>);
   if (e != cudaSuccess) return e;
   k_factor<T><<<npieces, 256, smem, st>>>(pieces, band, status, piece_flag, diag0);
   return cudaGetLastError();

@@ -328,7 +328,7 @@ cudaError_t launch_factor_tc(const PieceDesc* pieces, int npieces, int max_w, fl
                              int* piece_flag, float* diag0, long wait_limit, cudaStream_t st) {
   const size_t smem = factor_tc_smem_bytes(max_w);
   if (smem > 227 * 1024 || max_w > 3 * kTB) return cudaErrorInvalidValue;
-  cudaError_t e = cudaFuncSetAttribute(k_factor_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  cudaError_t e = allow_all_smem((const void*)k_factor_tc);
   if (e != cudaSuccess) return e;
   if (npieces > 0) k_factor_tc<<<npieces, kFactorThreads, smem, st>>>(pieces, band, status, piece_flag, diag0, max_w, wait_limit);
   return cudaGetLastError();

@@ -13,6 +13,11 @@
 
 namespace vtm {
 
+// Lets a kernel take all the dynamic shared memory that an SM has for it.  The limit belongs to the kernel and
+// not to a solver: set to what the solver at hand needs, the next one's setup would lower it for solvers
+// that are still in use, whose launches would then be refused.
+cudaError_t allow_all_smem(const void* kernel);
+
 // Arguments of one VTM sweep (Table 1 steps 3-5) over a set of subgraphs.  TF: factor and
 // substitution type; TV: type of the sources, local solutions, waves and 1/Z in global memory.
 template <typename TF, typename TV = TF>
@@ -52,7 +57,7 @@ struct SweepArgs {
 
 size_t sweep_smem_bytes(size_t elem, int R, int stages, int slot_elems, int ys_elems, int win_elems);
 template <typename TF, typename TV>
-cudaError_t sweep_configure(int R, size_t smem);
+cudaError_t sweep_configure(int R);
 template <typename TF, typename TV>
 cudaError_t sweep_occupancy(int R, size_t smem, int* ctas_per_sm);
 template <typename TF, typename TV>
@@ -86,7 +91,7 @@ cudaError_t launch_sweep_wide_tc(const SweepArgs<float, float>& a, int R, int np
 // Wide variant (R = 16, 32): vectors spill to xc, a circular window of 512 rows stays in shared memory.
 size_t sweep_wide_smem_bytes(size_t elem, int R, int stages, int slot_elems, int cap);
 template <typename TF, typename TV>
-cudaError_t sweep_wide_configure(int R, size_t smem);
+cudaError_t sweep_wide_configure(int R);
 template <typename TF, typename TV>
 cudaError_t launch_sweep_wide(const SweepArgs<TF, TV>& a, int R, int npieces, size_t smem, cudaStream_t st,
                               int batches = 1);

@@ -354,6 +354,8 @@ static void factor_typed(vtm_solver* s) {
 template <typename T>
 static void input_impedances_typed(vtm_solver* s, std::vector<double>& r_api);
 
+constexpr size_t kSweepSmemMax = 227 * 1024 - 128;  // the band sweep kernels have 128 bytes of their own
+
 // Shared-memory plan of the FP64 launch over the flagged subgraphs (FP64 factor, FP32 vectors).
 static void plan_hi(vtm_solver* s) {
   if (s->np_hi == 0) return;
@@ -372,7 +374,7 @@ static void plan_hi(vtm_solver* s) {
   s->hi_cap = 64;
   while (s->hi_cap < mWp - 1 + kNB) s->hi_cap *= 2;
   if (s->wide && s->hi_cap > kWideWindow) fail(VTM_ERR_INVALID, "flagged subgraph too wide for the multi-RHS window");
-  const size_t kSmemMax = 227 * 1024;
+  const size_t kSmemMax = kSweepSmemMax;
   s->hi_stages = 0;
   for (int st2 : {8, 6, 4, 3, 2}) {
     if (s->hi_stages) break;
@@ -384,8 +386,8 @@ static void plan_hi(vtm_solver* s) {
     }
   }
   if (!s->hi_stages) fail(VTM_ERR_INVALID, "a subgraph flagged for FP64 is too large for the FP64 sweep");
-  if (s->wide) VTM_CUDA((sweep_wide_configure<double, float>(R, s->hi_smem)));
-  else VTM_CUDA((sweep_configure<double, float>(R, s->hi_smem)));
+  if (s->wide) VTM_CUDA((sweep_wide_configure<double, float>(R)));
+  else VTM_CUDA((sweep_configure<double, float>(R)));
 }
 
 // Coupled lines (§7.2): check every pair; the diagonal of Y (1/Z_t + the line's conductances) goes
@@ -634,9 +636,8 @@ static void setup_typed(const vtm_partition* p, const vtm_setup_opts* o, vtm_sol
   s->slot_elems = kNB * max_Wp;
   s->ys_elems = (2 * (max_Wp - 1) + max_pad) * R;
   s->win_elems = std::max(1, max_ends) * R;
-  const size_t kSmemMax = 227 * 1024;
+  const size_t kSmemMax = kSweepSmemMax;
   std::vector<int> stage_cands;
-  size_t smem_cap = 0;
   if (s->wide && max_Wp - 1 + kNB > kWideWindow)
     fail(VTM_ERR_INVALID, "bandwidth too large for the multi-RHS sweep window");
   s->cap = 64;
@@ -661,7 +662,6 @@ static void setup_typed(const vtm_partition* p, const vtm_setup_opts* o, vtm_sol
     if (b <= kSmemMax) {
       stage_cands.push_back(st2);
       single.push_back({st2, false});
-      smem_cap = std::max(smem_cap, b);
     }
     if (!s->wide && st2 >= 3 && (pipe_auto || (o->sweep_variant == 2 && R <= 2)) &&
         sweep_smem_for(s, sizeof(T), st2, true) <= kPipeSmemMax) {
@@ -677,8 +677,8 @@ static void setup_typed(const vtm_partition* p, const vtm_setup_opts* o, vtm_sol
   s->stage_cands = stage_cands;
   s->stages = stage_cands.back();
   s->sweep_smem = sweep_smem_for(s, sizeof(T), s->stages);
-  if (s->wide) VTM_CUDA((sweep_wide_configure<T, T>(R, smem_cap)));
-  else VTM_CUDA((sweep_configure<T, T>(R, smem_cap)));
+  if (s->wide) VTM_CUDA((sweep_wide_configure<T, T>(R)));
+  else VTM_CUDA((sweep_configure<T, T>(R)));
   if (pipes) VTM_CUDA(sweep_pipe_configure<T>(R));
 
   // ---- vertex -> copies (for assembly)
@@ -917,7 +917,7 @@ static void compute_port_response(vtm_solver* s, int64_t s_tiles) {
   const int np = s->npieces;
   if (!s->resident) s->S.alloc((size_t)s_tiles * kNB * kNB * sizeof(T));
   VTM_CUDA(cudaMemsetAsync(s->S.p, 0, s->S.bytes, st));
-  const size_t kSmemMax = 227 * 1024;
+  const size_t kSmemMax = kSweepSmemMax;
   int st_lo = s->wide ? s->stages : 0;
   size_t sm_lo = s->wide ? s->sweep_smem : 0;
   if (!s->wide && s->cap <= kWideWindow)
@@ -963,7 +963,7 @@ static void compute_port_response(vtm_solver* s, int64_t s_tiles) {
     size_t fb = 0, tb = 0;
     VTM_CUDA(cudaMemGetInfo(&fb, &tb));
     if (!s->wide && !own) {
-      VTM_CUDA((sweep_wide_configure<T, T>(Rs, sm_lo)));
+      VTM_CUDA((sweep_wide_configure<T, T>(Rs)));
       if constexpr (sizeof(T) == 4) {
         if (s->wt_ok && (double)s->wt_bytes < 0.4 * (double)fb) {
           wt_tmp.alloc((size_t)s->wt_bytes);

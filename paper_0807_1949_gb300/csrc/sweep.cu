@@ -534,22 +534,27 @@ cudaError_t launch_sweep_pipe(const SweepArgs<T, T>& a, int R, int npieces, size
   return cudaLaunchKernel(k, dim3(npieces), dim3(kSweepThreads), av, smem, st);
 }
 
+cudaError_t allow_all_smem(const void* kernel) {
+  int dev = 0, most = 0;
+  cudaFuncAttributes fa;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&most, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+  if (e == cudaSuccess) e = cudaFuncGetAttributes(&fa, kernel);
+  if (e != cudaSuccess) return e;
+  return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, most - (int)fa.sharedSizeBytes);
+}
+
 size_t sweep_smem_bytes(size_t elem, int R, int stages, int slot_elems, int ys_elems, int win_elems) {
   return 128 + elem * ((size_t)stages * slot_elems + ys_elems + win_elems + (size_t)kNB * R);
 }
 
-template <typename TF, typename TV, int R>
-static cudaError_t configure_one(size_t smem) {
-  return cudaFuncSetAttribute(k_sweep<TF, TV, R>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-}
-
 template <typename TF, typename TV>
-cudaError_t sweep_configure(int R, size_t smem) {
+cudaError_t sweep_configure(int R) {
   switch (R) {
-    case 1: return configure_one<TF, TV, 1>(smem);
-    case 2: return configure_one<TF, TV, 2>(smem);
-    case 4: return configure_one<TF, TV, 4>(smem);
-    case 8: return configure_one<TF, TV, 8>(smem);
+    case 1: return allow_all_smem((const void*)k_sweep<TF, TV, 1>);
+    case 2: return allow_all_smem((const void*)k_sweep<TF, TV, 2>);
+    case 4: return allow_all_smem((const void*)k_sweep<TF, TV, 4>);
+    case 8: return allow_all_smem((const void*)k_sweep<TF, TV, 8>);
     default: return cudaErrorInvalidValue;
   }
 }
@@ -586,7 +591,7 @@ cudaError_t launch_sweep(const SweepArgs<TF, TV>& a, int R, int npieces, size_t 
 }
 
 #define VTM_SWEEP_INST(TF, TV)                                                                    \
-  template cudaError_t sweep_configure<TF, TV>(int, size_t);                                       \
+  template cudaError_t sweep_configure<TF, TV>(int);                                       \
   template cudaError_t sweep_occupancy<TF, TV>(int, size_t, int*);                                 \
   template cudaError_t launch_sweep<TF, TV>(const SweepArgs<TF, TV>&, int, int, size_t, cudaStream_t, int);
 VTM_SWEEP_INST(float, float)

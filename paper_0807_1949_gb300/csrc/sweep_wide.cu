@@ -343,16 +343,11 @@ __global__ void __launch_bounds__(kWideThreads, 1) k_sweep_wide(const SweepArgs<
   }
 }
 
-template <typename TF, typename TV, int R>
-static cudaError_t wide_configure_one(size_t smem) {
-  return cudaFuncSetAttribute(k_sweep_wide<TF, TV, R>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-}
-
 template <typename TF, typename TV>
-cudaError_t sweep_wide_configure(int R, size_t smem) {
+cudaError_t sweep_wide_configure(int R) {
   switch (R) {
-    case 16: return wide_configure_one<TF, TV, 16>(smem);
-    case 32: return wide_configure_one<TF, TV, 32>(smem);
+    case 16: return allow_all_smem((const void*)k_sweep_wide<TF, TV, 16>);
+    case 32: return allow_all_smem((const void*)k_sweep_wide<TF, TV, 32>);
     default: return cudaErrorInvalidValue;
   }
 }
@@ -371,7 +366,7 @@ cudaError_t launch_sweep_wide(const SweepArgs<TF, TV>& a, int R, int npieces, si
 }
 
 #define VTM_WIDE_INST(TF, TV)                                  \
-  template cudaError_t sweep_wide_configure<TF, TV>(int, size_t); \
+  template cudaError_t sweep_wide_configure<TF, TV>(int);         \
   template cudaError_t launch_sweep_wide<TF, TV>(const SweepArgs<TF, TV>&, int, int, size_t, cudaStream_t, int);
 VTM_WIDE_INST(float, float)
 VTM_WIDE_INST(double, double)
