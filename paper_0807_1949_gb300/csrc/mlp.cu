@@ -186,12 +186,13 @@ __global__ void __launch_bounds__(kFwdThreads, 3) k_mlp_forward(const __nv_bfloa
 // tiles of 64 samples, 16 per warp.  Forward as in k_mlp_forward; the layers' deltas and activations
 // (FP32 values as three exact bf16 terms) go to shared memory, where ldmatrix.trans turns them into
 // the operands of the sums over samples: warp m computes rows 16 m .. 16 m + 15 of dW2 = D2^T H1 and
-// of dW1 = D1^T X, and db2, db1 as products with a column of ones.  Of the nine products of terms (split3_nearest)
-// six count, the other three are at most 2^-24 of the whole; those of the two first terms accumulate apart from the rest, and every
-// tile's sums are added in FP32, the bias sums' after every 16 samples and first terms apart (through one
-// accumulator for all terms of a tile the tensor core cut off twelve times: 64 equal samples gave biases
-// up to 6e-7 away from one sample's, now the same bits).  Each CTA writes its partial gradient and loss; k_mlp_reduce adds
-// the CTAs' partials in their order, so the gradient is the same bit for bit from run to run.
+// of dW1 = D1^T X, and db2, db1 as products with columns of ones.  Of the nine products of terms
+// (split3_nearest) six count, the other three are at most 2^-24 of the whole; those of the two first terms
+// accumulate apart from the rest, and every tile's sums are added in FP32, the bias sums' after every 16
+// samples (through one accumulator for all terms of a tile the tensor core cut off twelve times: 64 equal
+// samples gave biases up to 6e-7 away from one sample's, now the same bits).  Each CTA writes its partial
+// gradient and loss; k_mlp_reduce adds the CTAs' partials in their order, so the gradient is the same bit for
+// bit from run to run.
 //
 // What bounds it: latency at the training loop's 16,384 samples (one or two tiles per CTA).  There
 // 115 us for the call with one thread per sample, serial sums over the tile and an atomic per
@@ -366,15 +367,16 @@ __global__ void __launch_bounds__(kGradThreads, 2) k_mlp_grad(const __nv_bfloat1
     // ---- sums over the tile's samples: rows 16 warp .. + 15
     const int ms = (lane >> 4) * 8 + (lane & 7), mc = ((lane >> 3) & 1) * 8;  // A: matrices (0, 0) (0, 8) (8, 0) (8, 8)
     const int bs = ((lane >> 3) & 1) * 8 + (lane & 7), bc = (lane >> 4) * 8;  // B: (0, 0) (8, 0) (0, 8) (8, 8)
-    // sums of 16 samples' deltas (rows g, g + 8) added to a layer's bias sums
-    auto bias = [](const uint32_t (&A)[3][4], float (&sum)[2]) {
-      constexpr uint32_t kOnes = 0x3F803F80u;
-      float first[4] = {0.f, 0.f, 0.f, 0.f}, rest[4] = {0.f, 0.f, 0.f, 0.f};
-      mma_k16(first, A[0], kOnes, kOnes);
-      mma_k16(rest, A[2], kOnes, kOnes);
-      mma_k16(rest, A[1], kOnes, kOnes);
-      sum[0] += first[0] + rest[0];
-      sum[1] += first[2] + rest[2];
+    // sums of 16 samples' deltas (rows g, g + 8) added to a layer's bias sums: first terms in the even
+    // columns, the others in the odd ones
+    const uint32_t even = (g & 1) ? 0u : 0x3F803F80u, odd = (g & 1) ? 0x3F803F80u : 0u;
+    auto bias = [&](const uint32_t (&A)[3][4], float (&sum)[2]) {
+      float d[4] = {0.f, 0.f, 0.f, 0.f};
+      mma_k16(d, A[2], odd, odd);
+      mma_k16(d, A[1], odd, odd);
+      mma_k16(d, A[0], even, even);
+      sum[0] += d[0] + d[1];
+      sum[1] += d[2] + d[3];
     };
     {
       float hi[8][4], lo[8][4];
