@@ -225,9 +225,8 @@ typedef struct vtm_setup_opts {
                               is one load (about 1 us), so it takes at least 65536 of them, unless
                               withhold_slab makes a wait of it run out                       */
   int32_t withhold_slab;   /* testing only (0 = off): k > 0: the band sweep never issues the copy of
-                              factor slab k-1 of each subgraph, k < 0: the resident port sweep never
-                              publishes the first line end's wave of sweep -k of a launch, so that a
-                              wait runs out                                                  */
+                              factor slab k-1 of each subgraph, k < 0: the first line end of the resident
+                              port sweep awaits a wave that nothing publishes, so that a wait runs out */
   int32_t sweep_variant;   /* nrhs <= 8: 0: the pipelined sweep for FP32 solvers where it is the faster
                               one (three factor slabs fit in shared memory, and nrhs > 1 or no more
                               subgraphs than SMs), else the single-block sweep; 1: single-block

@@ -218,7 +218,6 @@ struct ResArgs {
   const T* invz;
   CoupleRef<T> cpl;
   int sweeps;
-  int withhold;                // testing: sweep whose wave of line end 0 is never published (0 = none)
   int* status;
   long wait_limit;
 };

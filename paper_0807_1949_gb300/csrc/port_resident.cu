@@ -20,11 +20,11 @@
 // wait is bounded; a CTA whose wait runs out records VTM_ERR_TIMEOUT and goes on without waiting, so
 // that the launch ends.
 //
-// What bounds it: the latency of the exchange (a store, a load that sees it, about 1.5 us) and of
-// the product's three block-wide steps; S is not read from memory at all.  Measured per sweep against
-// one launch per sweep: 32^2 in 4 subgraphs, FP64 8.9 -> 2.5 us; 256^2 in 64 subgraphs, FP32
-// 6.8 -> 3.3 us; 100 finite-element subgraphs of about 100 ports, 16 right-hand sides (tensor-core
-// sweep before) 13 -> 8 us.
+// What bounds it: the latency of the exchange (a store, a load that sees it) and of the product's three
+// block-wide steps, about 2 us together; S is not read from memory at all.  Measured per sweep in batches of 160
+// (of 20), launch and clearing included, against one launch per sweep: 32^2 in 4 subgraphs, FP64 8.9 -> 2.2
+// (2.5) us; 256^2 in 64 subgraphs, FP32, coupled lines 6.8 -> 2.0 (2.3) us; 100 finite-element subgraphs of about
+// 100 ports, 16 right-hand sides (tensor-core sweep before) 13 -> 7.0 (7.3) us.
 #include <algorithm>
 #include <numeric>
 
@@ -273,7 +273,7 @@ __global__ void __launch_bounds__(kResThreads, 1) k_port_resident(const ResArgs<
         if (lastk) {
 #pragma unroll
           for (int c = 0; c < C; ++c) a.wout[(size_t)e * R + r + c] = w[c];
-        } else if (e != 0 || k != a.withhold) {
+        } else {
           publish<T, C>(out, (size_t)e * R + r, w, (uint32_t)k);
         }
       }

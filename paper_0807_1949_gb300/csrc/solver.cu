@@ -104,7 +104,7 @@ struct vtm_solver {
   int slot_elems = 0, ys_elems = 0, win_elems = 0;
   long wait_limit = 1L << 22;
   int withhold = -1;
-  int withhold_wave = 0;
+  DevBuf res_twin;                   // testing: twins of the resident sweep, one of them an end that nothing writes
   std::vector<int> stage_cands;
   // kept for re-assembly with new impedances (eq. 5.8 depends on Z)
   DevBuf d_copy_piece, d_lrowptr, d_lcol, d_lval, d_port_of_copy, d_invz64;
@@ -645,9 +645,11 @@ static void setup_typed(const vtm_partition* p, const vtm_setup_opts* o, vtm_sol
   // deeper rings for thin bands: a slab of a 2D subgraph is a few KB, and hiding DRAM latency takes
   // several of them in flight (the mbarrier area holds up to kMaxStages).  FP32 solvers
   // take the pipelined sweep (see k_sweep_pipe) where it has room for three slabs (two in work, one in
-  // flight), with one right-hand side only up to one subgraph per SM: beyond that two single-block
-  // CTAs per SM hide each other's chains (128^3 in 512 subgraphs 0.95 ms, pipelined 1.01; 64^3 in 64:
-  // 0.38 and 0.25; 288 ragged subgraphs with 8 right-hand sides 1.22 and 0.50).  In FP64 the chain warp
+  // flight), with one right-hand side only up to one subgraph per SM.  Single-block and pipelined there: 17^3
+  // subgraphs, 64 of them 0.365 and 0.220 ms, 150 0.366 and 0.261; 33^2, 64 0.064 and 0.041; eight right-hand sides,
+  // 288 ragged ones 1.22 and 0.50.  Beyond, two single-block CTAs per SM hide each other's chains and the lead
+  // depends on the band: 17^3, 252 subgraphs 0.486 and 0.468, 512 0.945 and 0.943; 11^3, 512 0.214 and 0.133; 33^2, 400
+  // 0.077 and 0.088: there the single-block sweep, which was there first, stays.  In FP64 the chain warp
   // has one quarter of the SM's FP64 units (32^2: 38 us, pipelined 81).  Only the staging depth is
   // tuned, never the variant: the variants add in different orders, and two identical solvers must
   // agree bit for bit.
@@ -742,7 +744,7 @@ static void setup_typed(const vtm_partition* p, const vtm_setup_opts* o, vtm_sol
   s->bt.alloc((size_t)C * R * sizeof(T));
   s->xc.alloc((size_t)C * R * sizeof(T));
   for (int b = 0; b < 2; ++b) {
-    s->w[b].alloc((size_t)std::max<int64_t>(1, s->E) * R * sizeof(T));
+    s->w[b].alloc((size_t)(s->E + 1) * R * sizeof(T));  // + 1: withhold_slab < 0
     VTM_CUDA(cudaMemsetAsync(s->w[b].p, 0, s->w[b].bytes, st));
   }
   VTM_CUDA(cudaMemsetAsync(s->bt.p, 0, s->bt.bytes, st));
@@ -767,7 +769,12 @@ static void setup_typed(const vtm_partition* p, const vtm_setup_opts* o, vtm_sol
     choose_form<T>(s, o, soff, foff);
   }
   s->withhold = o->withhold_slab > 0 ? o->withhold_slab - 1 : -1;  // after tuning: only real sweeps
-  s->withhold_wave = o->withhold_slab < 0 ? -std::max(o->withhold_slab, -INT32_MAX) : 0;
+  if (o->withhold_slab < 0 && s->resident) {
+    std::vector<int32_t> never = twin;
+    never[0] = (int32_t)s->E;
+    upload(s->res_twin, never, st);
+    VTM_CUDA(cudaStreamSynchronize(st));
+  }
 
   s->info.npieces = np;
   s->info.ncopies = C;
@@ -1137,14 +1144,13 @@ static void launch_resident(vtm_solver* s, int k) {
   a.wout = s->w[(s->cur + k) & 1].as<T>();
   a.xch[0] = s->res_xch.as<unsigned long long>();
   a.xch[1] = a.xch[0] + s->res_xch.bytes / 16;
-  a.twin = s->twin.as<int32_t>();
+  a.twin = (s->res_twin.p ? s->res_twin : s->twin).template as<int32_t>();
   a.invz = s->invz_t.as<T>();
   a.cpl = couple_ref<T>(s);
   a.sweeps = k;
   a.status = s->status.as<int>();
-  a.withhold = s->withhold_wave;
   // a poll is one load here (about 1 us), not a suspended wait
-  a.wait_limit = s->withhold_wave ? s->wait_limit : std::max(s->wait_limit, 65536L);
+  a.wait_limit = s->res_twin.p ? s->wait_limit : std::max(s->wait_limit, 65536L);
   VTM_CUDA(launch_port_resident<T>(a, s->R, s->res_grid, s->res_smem, s->res_xch.bytes, s->stream));
   s->launches++;
   s->cur = (s->cur + k) & 1;
@@ -1261,7 +1267,7 @@ static void choose_form(vtm_solver* s, const vtm_setup_opts* o, int64_t s_tiles,
       s->res_grid = (int)rp.ctas.size();
       s->res_pieces = (int)rp.piece_s.size();
       s->res_smem = rp.smem;
-      s->res_xch.alloc((size_t)2 * s->E * s->R * (sizeof(T) / 4) * sizeof(unsigned long long));
+      s->res_xch.alloc((size_t)2 * (s->E + 1) * s->R * (sizeof(T) / 4) * sizeof(unsigned long long));  // + 1: withhold_slab < 0
       s->S.alloc((size_t)rp.s_elems * sizeof(T));
     }
   }
@@ -1294,11 +1300,12 @@ static void choose_form(vtm_solver* s, const vtm_setup_opts* o, int64_t s_tiles,
     s->tc_tmem_cols = tmem_cols;
     s->tc_n4max = n4max;
     for (const PieceDesc& d : lo) s->tc_max_ends = std::max(s->tc_max_ends, d.nends);
-    // The port vectors: a launch of their own up to kTcSeparate items per CTA, fused beyond (there the
-    // gathers hide behind the next items' blocks, and the operand tiles would pass through HBM).
-    // 64^3 with 32 right-hand sides (1.2 items per CTA) 0.083 ms separate, 0.193 fused; 128^3 (3.4)
-    // 0.521 and 0.557; 256^3 (27) 3.86 fused, where the tiles and a second pass over the waves would
-    // add 2.3 GB to 25.
+    // The port vectors: a launch of their own up to kTcSeparate items per CTA, fused beyond, where the
+    // gathers hide behind the next items' blocks.  17^3 subgraphs, 32 right-hand sides, coupled lines, separate
+    // and fused by items per CTA: 1.2 (64^3) 0.083 and 0.193 ms, 3.4 0.515 and 0.523, 5.1 0.776 and 0.762, 6.6 1.013
+    // and 0.971, 11 1.78 and 1.65, 17 2.61 and 2.41.  Plain lines gather a fifth of the waves and cross below 3.4
+    // (0.500 and 0.480 there, 0.752 and 0.702 at 5.1), small subgraphs with coupled lines late (10^3: 15 items
+    // 0.491 and 0.505, 27 0.931 and 0.978; 6^3: 5.3 0.094 and 0.099, 13.5 0.266 and 0.244).
     constexpr double kTcSeparate = 5.0;
     const bool separate = (double)pl.items.size() <= kTcSeparate * nsm &&
                           port_vec_tc_smem_bytes(s->tc_max_ends) <= kVecTcSmemMax;

@@ -340,7 +340,7 @@ class Solver:
     def __init__(self, part: Partition, z=1.0, precision: str = "fp64", nrhs: int = 1, stream=None,
                  check_every: int = 10, inner_reduction: float = 0.0, z_init: float = 1.0,
                  wait_polls: int = 0, withhold_slab: int = -1, sweep_variant: str = "auto",
-                 form: str = "auto", port_storage: str = "native", coupling=None, withhold_wave: int = 0):
+                 form: str = "auto", port_storage: str = "native", coupling=None, withhold_wave: bool = False):
         o = _Opts()
         ckeep = None
         if coupling is not None:
@@ -374,7 +374,7 @@ class Solver:
         o.check_every = check_every
         o.inner_reduction = inner_reduction
         o.wait_polls = int(wait_polls)
-        o.withhold_slab = int(withhold_slab) + 1 if withhold_slab >= 0 else -int(withhold_wave)
+        o.withhold_slab = int(withhold_slab) + 1 if withhold_slab >= 0 else -int(bool(withhold_wave))
         self.nrhs = nrhs
         self.n = part.info().n
         h = C.c_void_p()
