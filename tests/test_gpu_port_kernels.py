@@ -92,6 +92,29 @@ def test_fused_port_vectors(vtmlib, nrhs, kind, gamma):
     _check(s, b, 4, copies, waves[:, lm], TOL[kind])
 
 
+# fused, with a subgraph that is cut between super-rows: 1512 cells of 2^3 vertices around one of 12^3 (1592 ports,
+# 91 blocks, where a CTA's share of all is 40), whose items leave partial sums
+@pytest.mark.parametrize("nrhs,kind", [(16, "fp32"), (32, "fp16")])
+def test_fused_with_a_cut_subgraph(vtmlib, nrhs, kind):
+    n, lo, hi = 24, 6, 18
+    A = inputs.grid_poisson((n, n, n), sigma=0.8, seed=7)
+    As = A.to_scipy()
+    z, y, x = np.meshgrid(*(np.arange(n),) * 3, indexing="ij")
+    cell = ((z // 2) * (n // 2) + y // 2) * (n // 2) + x // 2
+    core = (x >= lo) & (x < hi) & (y >= lo) & (y < hi) & (z >= lo) & (z < hi)
+    home = np.unique(np.where(core, -1, cell).ravel(), return_inverse=True)[1]
+    owners = [tuple(sorted({int(home[i])} | {int(h) for h in home[As.indices[As.indptr[i]:As.indptr[i + 1]]]}))
+              for i in range(A.n)]
+    lines = [(i, p, q) for i, o in enumerate(owners) for a, p in enumerate(o) for q in o[a + 1:]]
+    part = vtmlib.partition_evs(A, "owners", owners=owners, lines=lines)
+    osplit = evs.split_by_owners(As, owners, lines)
+    s = vtmlib.Solver(part, z=0.9, precision="fp32", nrhs=nrhs, form="port", port_storage="fp16" if kind == "fp16" else "native")
+    assert s.info().port_kernel == vtmlib.PORT_TC_FUSED and s.info().npieces == 1513 > 5 * NSM
+    b = inputs.rhs_uniform(A.n, nrhs, seed=7)
+    copies, waves = _oracle_after(osplit, b, 0.9, 4)
+    _check(s, b, 4, copies, waves[:, _line_map(part, osplit)], TOL[kind])
+
+
 # FP32 responses of single partial super-rows (up to 88 ports) that do not fit into shared memory: 750 subgraphs
 @pytest.mark.parametrize("nrhs", [16, 32])
 def test_tensor_core_single_super_row(vtmlib, nrhs):
