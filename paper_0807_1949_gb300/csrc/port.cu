@@ -482,13 +482,12 @@ __host__ __device__ constexpr int sweep_threads(int mma) { return mma ? 32 * mma
 // the memory, bound those sweeps.
 //
 // What bounds it (GB300): HBM at R = 1, 2 and with FP16 tiles, FP64 arithmetic in FP64 (0.9 of its
-// pipe), with three-term FP32 tiles the issue rate and the segments' latency.  Measured per sweep
-// against one CTA per subgraph with shared-memory atomics (R > 1, FP64) or an accumulator per warp
-// (FP32 / FP16, R = 1): 64^3 in 64 subgraphs 0.116 -> 0.042 ms (FP32, R = 1, 188 MB) and 0.82 -> 0.19 ms
-// (FP64, 376 MB); 101 x 67 x 83 in 288 ragged subgraphs, R = 8, 439 MB: 0.54 -> 0.16 ms (0.22 with shares
-// that counted a segment as 20 tiles, and 8 warps); 128^3 in 512 subgraphs, FP16, 1.01 GB: 0.199 ->
-// 0.183 ms (0.81 of the copy bandwidth with the port vectors' own launch; the tiles are read with an
-// evict-first hint, without it 0.198 ms).
+// pipe), with three-term FP32 tiles the issue rate and the segments' latency.  Measured per sweep, port
+// vectors included, against one CTA per subgraph with shared-memory atomics (R > 1, FP64) or an accumulator per
+// warp (FP32 / FP16, R = 1): 64^3 in 64 subgraphs 0.116 -> 0.042 ms (FP32, R = 1, 188 MB) and 0.82 -> 0.19 ms (FP64,
+// 376 MB); 101 x 67 x 83 in 288 ragged subgraphs, 439 MB: R = 8 0.54 -> 0.144 ms, R = 4 0.108; 128^3 in 512
+// subgraphs, FP16, 1.01 GB: 0.199 -> 0.178 ms (0.88 of the copy bandwidth; the tiles are read with an evict-first
+// hint, without it 8 % more), R = 2 0.223, R = 4 0.242.
 template <typename T, typename TS, int R, bool PRIV, int MMA>
 __global__ void __launch_bounds__(sweep_threads(MMA), sizeof(T) == 8 || MMA > 8 ? 1 : 2)
     k_port_sweep(const PortArgs<T> a) {
