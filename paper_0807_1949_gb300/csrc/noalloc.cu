@@ -85,7 +85,8 @@ extern "C" int vtm_relative_residual_noalloc(int64_t n, const int64_t* rowptr, c
     // the array keeps the previous call's sums: clear both halves before accumulating
     cudaError_t e = cudaMemsetAsync(sums, 0, 2 * VTM_NOALLOC_MAX_RHS * sizeof(double), st);
     if (e == cudaSuccess)
-      e = vtm::launch_residual_norms(dev.nsm, n, nrhs, rowptr, col, val, b, ldb, x, ldx, sums, sums + VTM_NOALLOC_MAX_RHS, st);
+      e = vtm::launch_residual_norms(dev.nsm, n, nrhs, rowptr, col, val, b, ldb, x, ldx, sums,
+                                     sums + VTM_NOALLOC_MAX_RHS, st);
     if (e == cudaSuccess) {
       k_noalloc_finish<<<1, 32, 0, st>>>(nrhs, sums, rel);
       e = cudaGetLastError();

@@ -1101,9 +1101,9 @@ PortShape port_shape(size_t elem, size_t stored, int R, int max_ports) {
 // and its waves, and a little per strip of them.  In tiles of the same kernel, from the cycles of every
 // CTA of a sweep over 288 ragged subgraphs of 1 to 33 strips (least squares):
 //   FP64 8 + 0.3 per strip (R = 1), 5 + 0.3 (R = 2); FP32 27 + 0.6 (R = 1, 2); FP16 41 + 1.2 (R = 1);
-//   tensor cores, 8 warps: FP32 48 + 1.0 (R = 8), FP16 54 + 1.9 (R = 4), 67 + 2.6 (R = 8);
-//   16 warps: FP32 71 + 0.1.
-// (With 20 for R >= 4 the CTAs of many small subgraphs took 1.4 times the average.)
+//   tensor cores, 8 warps: FP32 48 + 1.0 (R = 8), FP16 54 + 1.9 (R = 4), 67 + 2.6 (R = 8); 16 warps: FP32 71 + 0.1.
+// FP32 at R = 4: 20 (five sets of 64 to 2500 subgraphs: 10 is up to 24 % slower, 30 and 40 within 1 % but
+// 10 % slower with 2500 small ones).
 PortPlan port_plan(const PieceDesc* pd, int npieces, size_t elem, size_t stored, int R, int ctas, int mma) {
   constexpr int kMinSeg = 32;
   double seg = 20, strip = 0;  // SIMT products, R >= 4

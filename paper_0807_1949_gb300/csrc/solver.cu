@@ -744,7 +744,7 @@ static void setup_typed(const vtm_partition* p, const vtm_setup_opts* o, vtm_sol
   s->bt.alloc((size_t)C * R * sizeof(T));
   s->xc.alloc((size_t)C * R * sizeof(T));
   for (int b = 0; b < 2; ++b) {
-    s->w[b].alloc((size_t)(s->E + 1) * R * sizeof(T));  // + 1: withhold_slab < 0
+    s->w[b].alloc((size_t)(s->E + 1) * R * sizeof(T));  // one end more: withhold_slab < 0
     VTM_CUDA(cudaMemsetAsync(s->w[b].p, 0, s->w[b].bytes, st));
   }
   VTM_CUDA(cudaMemsetAsync(s->bt.p, 0, s->bt.bytes, st));
@@ -1267,7 +1267,8 @@ static void choose_form(vtm_solver* s, const vtm_setup_opts* o, int64_t s_tiles,
       s->res_grid = (int)rp.ctas.size();
       s->res_pieces = (int)rp.piece_s.size();
       s->res_smem = rp.smem;
-      s->res_xch.alloc((size_t)2 * (s->E + 1) * s->R * (sizeof(T) / 4) * sizeof(unsigned long long));  // + 1: withhold_slab < 0
+      // one end more than there are: withhold_slab < 0
+      s->res_xch.alloc((size_t)2 * (s->E + 1) * s->R * (sizeof(T) / 4) * sizeof(unsigned long long));
       s->S.alloc((size_t)rp.s_elems * sizeof(T));
     }
   }

@@ -70,8 +70,8 @@ def test_kernel_choice(vtmlib, dims, block, nrhs, kind, kernel):
 # fused: more than five items per SM, so that both slots of the port vectors are used again; subgraphs of 91 to
 # 152 ports, one and two super-rows.  Coupled lines: entries past the
 # fourth of a port's list (a gather record holds four)
-@pytest.mark.parametrize("nrhs,kind,gamma", [(16, "fp32", None), (32, "fp32", None), (16, "fp16", None), (32, "fp16", None),
-                                             (32, "fp32", 1.0)])
+@pytest.mark.parametrize("nrhs,kind,gamma", [(16, "fp32", None), (32, "fp32", None), (16, "fp16", None),
+                                             (32, "fp16", None), (32, "fp32", 1.0)])
 def test_fused_port_vectors(vtmlib, nrhs, kind, gamma):
     nz = 5 * NSM // 100 + 1
     dims, block = (51, 51, 5 * nz + 1), (5, 5, 5)
@@ -108,7 +108,8 @@ def test_fused_with_a_cut_subgraph(vtmlib, nrhs, kind):
     lines = [(i, p, q) for i, o in enumerate(owners) for a, p in enumerate(o) for q in o[a + 1:]]
     part = vtmlib.partition_evs(A, "owners", owners=owners, lines=lines)
     osplit = evs.split_by_owners(As, owners, lines)
-    s = vtmlib.Solver(part, z=0.9, precision="fp32", nrhs=nrhs, form="port", port_storage="fp16" if kind == "fp16" else "native")
+    s = vtmlib.Solver(part, z=0.9, precision="fp32", nrhs=nrhs, form="port",
+                      port_storage="fp16" if kind == "fp16" else "native")
     assert s.info().port_kernel == vtmlib.PORT_TC_FUSED and s.info().npieces == 1513 > 5 * NSM
     b = inputs.rhs_uniform(A.n, nrhs, seed=7)
     copies, waves = _oracle_after(osplit, b, 0.9, 4)
